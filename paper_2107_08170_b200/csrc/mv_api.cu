@@ -4,6 +4,7 @@
 #include "../../include/mv.h"
 #include "mv_device.cuh"
 #include "mv_pack.cuh"
+#include "mv_merge.cuh"
 #include "mv_render.cuh"
 
 #include <cmath>
@@ -32,7 +33,7 @@ constexpr double kCtaFixedCost = 0.15;
 #ifndef MV_MERGE_SCRATCH_MB
 #define MV_MERGE_SCRATCH_MB 1024
 #endif
-constexpr size_t kMergeScratchBytes = (size_t)MV_MERGE_SCRATCH_MB << 20;   // coverage bitmap for the envs of one merge launch
+constexpr size_t kMergeScratchBytes = (size_t)MV_MERGE_SCRATCH_MB << 20;   // bit arrays for the envs of one merge launch
 
 inline uint32_t round_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
@@ -48,7 +49,8 @@ struct mv_batch {
     uint8_t *d_mat = nullptr;
     CamRec *d_cams = nullptr;
     uint32_t *d_status = nullptr;
-    uint32_t *d_covered = nullptr;      // merge scratch: one bit per voxel for merge_chunk envs
+    uint32_t *d_merge = nullptr;        // merge scratch: MergeLayout::env_words for merge_chunk envs
+    MergeLayout merge{};
     int merge_chunk = 0;
     int4 *d_overlay = nullptr;          // [O][max_overlay_rects]
     int32_t *d_overlay_count = nullptr; // [O]
@@ -153,6 +155,10 @@ RenderFn render_fn(const mv_batch *b) {
     if (!b->occ_shared) return render_kernel<kRenderThreads, false, false>;
     return b->lay.ysh == 5 ? render_kernel<kRenderThreads, true, true> : render_kernel<kRenderThreads, true, false>;
 }
+
+// The merge sweep keeps a layer number per column: a byte for grids less than 256 high.
+using MergeFn = void (*)(const unsigned char *, const uint8_t *, EnvLayout, MergeLayout, int, uint32_t *, uint4 *, int32_t *, int);
+MergeFn merge_sweep(int grid_y) { return grid_y < 256 ? merge_sweep_kernel<uint8_t> : merge_sweep_kernel<uint16_t>; }
 
 int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, int obs_count, cudaStream_t s) {
     RenderParams p{};
@@ -552,25 +558,41 @@ int mv_merge_voxels(mv_batch *b, int env_begin, int env_count, mv_box *d_boxes_o
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t words = b->nvox / 32;
-    if (!b->d_covered) {
-        size_t chunk = kMergeScratchBytes / (words * 4 * 2);       // coverage bits + x-packed occupancy per env
-        chunk = chunk < 1 ? 1 : (chunk > (size_t)b->desc.num_envs ? (size_t)b->desc.num_envs : chunk);
-        MV_CUDA(b, cudaMalloc(&b->d_covered, chunk * words * 4 * 2));
+    if (!b->d_merge) {
+        const mv_batch_desc &d = b->desc;
+        MergeLayout ml{};
+        ml.gx = d.grid_x; ml.gy = d.grid_y; ml.gz = d.grid_z;
+        ml.W = (d.grid_x + 31) / 32;
+        ml.colw = 1 << (b->lay.ysh - 5);
+        ml.mask_words = (uint32_t)d.grid_y * d.grid_z * ml.W;
+        ml.slots = (ml.W <= 16 ? 2 * ml.W : ml.W) + 1;
+        ml.work_bytes = (uint32_t)d.grid_z * ml.slots * 16 + (uint32_t)d.grid_x * d.grid_z * (d.grid_y < 256 ? 1 : 2);
+        ml.work_off = (3 * ml.mask_words + (uint32_t)d.grid_x * d.grid_z * ml.colw + 3) / 4 * 4;
+        cudaFuncAttributes fa{};
+        const void *sweep = (const void *)merge_sweep(d.grid_y);
+        MV_CUDA(b, cudaFuncGetAttributes(&fa, sweep));
+        ml.work_in_smem = ml.work_bytes + fa.sharedSizeBytes <= (size_t)b->smem_max;
+        if (ml.work_in_smem)       // (to the device's maximum: the cap belongs to the function, not to this batch)
+            MV_CUDA(b, cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            b->smem_max - (int)fa.sharedSizeBytes));
+        ml.env_words = ((size_t)ml.work_off + (ml.work_in_smem ? 0 : ml.work_bytes / 4) + 3) / 4 * 4;
+        size_t chunk = kMergeScratchBytes / (ml.env_words * 4);
+        chunk = chunk < 1 ? 1 : (chunk > (size_t)d.num_envs ? (size_t)d.num_envs : chunk);
+        MV_CUDA(b, cudaMalloc(&b->d_merge, chunk * ml.env_words * 4));
+        b->merge = ml;
         b->merge_chunk = (int)chunk;
     }
-    const int kMergeChunk = b->merge_chunk;
-    for (int e0 = 0; e0 < env_count; e0 += kMergeChunk) {
-        const int n = env_count - e0 < kMergeChunk ? env_count - e0 : kMergeChunk;
-        uint32_t *occx = b->d_covered + (size_t)kMergeChunk * words;
-        MV_CUDA(b, cudaMemsetAsync(b->d_covered, 0, (size_t)n * words * 4, s));
-        xpack_kernel<<<(unsigned)(((size_t)n * words + 255) / 256), 256, 0, s>>>(
-            b->d_env_blocks, b->lay, env_begin + e0, n, b->desc.grid_x, b->desc.grid_y, b->desc.grid_z, occx);
+    const MergeLayout &ml = b->merge;
+    const int per_env = (ml.W + 3) / 4 * ((ml.gz + 7) / 8) * ml.colw;
+    for (int e0 = 0; e0 < env_count; e0 += b->merge_chunk) {
+        const int n = env_count - e0 < b->merge_chunk ? env_count - e0 : b->merge_chunk;
+        merge_masks_kernel<<<(unsigned)n * per_env, kMergeThreads, 0, s>>>(b->d_env_blocks, b->d_mat, b->lay, ml,
+                                                                          env_begin + e0, b->d_merge);
         b->launches++;
         MV_CUDA(b, cudaGetLastError());
-        merge_voxels_kernel<<<(n * 32 + 127) / 128, 128, 0, s>>>(
-            occx, b->d_mat, b->lay, env_begin + e0, n, b->desc.grid_x, b->desc.grid_y, b->desc.grid_z,
-            b->d_covered, reinterpret_cast<uint4 *>(d_boxes_out + (size_t)e0 * max_out), d_count_out + e0, max_out);
+        merge_sweep(b->desc.grid_y)<<<n, kMergeThreads, ml.work_in_smem ? ml.work_bytes : 0, s>>>(
+            b->d_env_blocks, b->d_mat, b->lay, ml, env_begin + e0, b->d_merge,
+            reinterpret_cast<uint4 *>(d_boxes_out + (size_t)e0 * max_out), d_count_out + e0, max_out);
         b->launches++;
         MV_CUDA(b, cudaGetLastError());
     }
@@ -713,7 +735,7 @@ int mv_destroy(mv_batch *b) {
         if (g.ok) {
             if (cudaDeviceSynchronize() != cudaSuccess) rc = MV_ERR_CUDA;
             cudaFree(b->d_env_blocks); cudaFree(b->d_mat); cudaFree(b->d_cams); cudaFree(b->d_status);
-            cudaFree(b->d_overlay); cudaFree(b->d_overlay_count); cudaFree(b->d_covered); cudaFree(b->d_env_index);
+            cudaFree(b->d_overlay); cudaFree(b->d_overlay_count); cudaFree(b->d_merge); cudaFree(b->d_env_index);
             free_host_step(b);
             cudaGetLastError();
         }

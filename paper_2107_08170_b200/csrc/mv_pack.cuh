@@ -264,120 +264,6 @@ __global__ void move_agents_kernel(int32_t *__restrict__ cams, const float4 *__r
     }
 }
 
-// Occupancy of the envs of one merge launch re-packed along x (bit v&31 of word v>>5, v = x + gx*(z + gz*y)),
-// the order in which the merge sweeps.  One thread per output word; scratch, off the per-step path.
-__global__ void xpack_kernel(const unsigned char *__restrict__ env_blocks, EnvLayout lay, int env_begin, int env_count,
-                             int gx, int gy, int gz, uint32_t *__restrict__ out)
-{
-    const size_t nwords = (size_t)gx * gy * gz / 32;
-    const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= nwords * (size_t)env_count) return;
-    const size_t e = gid / nwords, w = gid - e * nwords;
-    const uint32_t *occ = reinterpret_cast<const uint32_t *>(env_blocks + (size_t)(env_begin + e) * lay.stride);
-    uint32_t word = 0;
-    for (int b = 0; b < 32; ++b) {
-        const size_t v = w * 32 + b;
-        const int x = (int)(v % gx), r = (int)(v / gx), z = r % gz, y = r / gz;
-        const uint32_t u = voxel_index(lay.ysh, gx, x, y, z);
-        word |= ((occ[u >> 5] >> (u & 31)) & 1u) << b;
-    }
-    out[gid] = word;
-}
-
-// Greedy merging of an env's voxels into boxes (paper Section 3.3), one warp per env, in the
-// same order as a serial sweep: the warp finds the first filled, uncovered voxel in index order,
-// grows a box along +x, then +z, then +y while every cell of the new row / slab is filled,
-// uncovered and of the same material, emits it and marks it covered.  `occx` is the x-packed copy
-// of the occupancy made by xpack_kernel; `covered` is scratch in the same packing, one bit per
-// voxel per env of this launch, zeroed by the caller; it is read around L1 (ld.cg) because lanes
-// read bits that other lanes set with atomics.
-__global__ void merge_voxels_kernel(const uint32_t *__restrict__ occx, const uint8_t *__restrict__ mat,
-                                    EnvLayout lay, int env_begin, int env_count, int gx, int gy, int gz,
-                                    uint32_t *__restrict__ covered, uint4 *__restrict__ boxes_out,
-                                    int32_t *__restrict__ count_out, int max_out)
-{
-    const int lane = threadIdx.x & 31;
-    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (e >= env_count) return;
-    const size_t nvox = (size_t)gx * gy * gz;
-    const int nwords = (int)(nvox / 32);
-    const uint32_t *occ = occx + (size_t)e * nwords;
-    const uint8_t *m_env = mat + (size_t)(env_begin + e) * ((size_t)gx * gz << lay.ysh);
-    uint32_t *cov = covered + (size_t)e * nwords;
-    uint4 *out = boxes_out + (size_t)e * max_out * 2;
-    const unsigned full = 0xffffffffu;
-    auto open = [&](int i, int j, int k, int m) -> bool {
-        const int v = i + gx * (k + gz * j);
-        const uint32_t bit = 1u << (v & 31);
-        return (occ[v >> 5] & bit) && !(__ldcg(&cov[v >> 5]) & bit) && m_env[voxel_index(lay.ysh, gx, i, j, k)] == m;
-    };
-    int count = 0;
-    for (int w0 = 0; w0 < nwords; w0 += 32) {
-        // words w0..w0+31: lane owns one; handle every uncovered filled voxel in them, in order
-        // every trip covers at least one voxel of these 1024, so 1024 trips always suffice
-        for (int trip = 0; trip < 1024; ++trip) {
-            const int wi = w0 + lane;
-            const uint32_t mine = wi < nwords ? (occ[wi] & ~__ldcg(&cov[wi])) : 0u;
-            const unsigned has = __ballot_sync(full, mine != 0u);
-            if (!has) break;
-            const int src = __ffs(has) - 1;
-            const uint32_t word = __shfl_sync(full, mine, src);
-            const int v = (w0 + src) * 32 + (__ffs(word) - 1);
-            const int i = v % gx, r = v / gx, k = r % gz, j = r / gz;
-            const int m = m_env[voxel_index(lay.ysh, gx, i, j, k)];
-            int w = 1, d = 1, h = 1;
-            for (;;) {                                           // +x, 32 cells per vote
-                const int a = w + lane;
-                const bool ok = (i + a < gx) && open(i + a, j, k, m);
-                const unsigned bad = ~__ballot_sync(full, ok);
-                if (bad) { w += __ffs(bad) - 1; break; }
-                w += 32;
-            }
-            for (; k + d < gz; ++d) {                            // +z, one row per trip
-                bool ok = true;
-                for (int a = lane; a < w; a += 32) ok = ok && open(i + a, j, k + d, m);
-                if (!__all_sync(full, ok)) break;
-            }
-            for (; j + h < gy; ++h) {                            // +y, one slab per trip
-                bool ok = true;
-                for (int c = lane; c < w * d; c += 32) ok = ok && open(i + c % w, j + h, k + c / w, m);
-                if (!__all_sync(full, ok)) break;
-            }
-            __syncwarp();
-            // mark covered.  When gx is a multiple of 32, x-rows of different z or y never share a word:
-            // one lane per row does plain read-modify-writes, and the warp barrier orders them before the
-            // other lanes' later reads.  Narrower grids take atomics and a fence.
-            if ((gx & 31) == 0) {
-                for (int r = lane; r < d * h; r += 32) {
-                    const int b = r % d, cc = r / d;
-                    const int v0 = i + gx * ((k + b) + gz * (j + cc)), v1 = v0 + w;      // bits [v0, v1)
-                    for (int wd = v0 >> 5; wd <= (v1 - 1) >> 5; ++wd) {
-                        const int lo = max(v0 - 32 * wd, 0), hi = min(v1 - 32 * wd, 32);
-                        const uint32_t bits = (hi == 32 ? 0xffffffffu : ((1u << hi) - 1u)) & ~((1u << lo) - 1u);
-                        __stcg(&cov[wd], __ldcg(&cov[wd]) | bits);
-                    }
-                }
-            } else {
-                for (int c = lane; c < w * d * h; c += 32) {
-                    const int a = c % w, b = (c / w) % d, cc = c / (w * d);
-                    const int vv = (i + a) + gx * ((k + b) + gz * (j + cc));
-                    atomicOr(&cov[vv >> 5], 1u << (vv & 31));
-                }
-                __threadfence();
-            }
-            __syncwarp();
-            if (lane == 0 && count < max_out) {
-                out[2 * count] = make_uint4(__float_as_uint((float)i), __float_as_uint((float)j),
-                                            __float_as_uint((float)k), __float_as_uint((float)(i + w)));
-                out[2 * count + 1] = make_uint4(__float_as_uint((float)(j + h)), __float_as_uint((float)(k + d)),
-                                                (uint32_t)m, 0u);
-            }
-            ++count;
-        }
-    }
-    if (lane == 0) count_out[e] = count;
-}
-
 // GUI rectangles into the library's table; counts clamped to 0..max_rects.
 __global__ void copy_overlays_kernel(const int4 *__restrict__ rects, const int32_t *__restrict__ counts,
                                      int4 *__restrict__ out_rects, int32_t *__restrict__ out_counts, int num_obs,

@@ -249,3 +249,42 @@ def test_scene_generators_give_the_same_arrays_on_cpu_and_gpu():
             gpu = scenes.make_scene(cfg, device=torch.device("cuda", 0))
             for k in ("grid", "palette", "boxes", "box_count", "cams"):
                 assert torch.equal(cpu[k], gpu[k].cpu()), (name, k)
+
+
+@pytest.mark.parametrize("grid,kind,palette", [
+    ((4, 4, 4), "random", 3), ((32, 8, 12), "random", 2), ((36, 12, 20), "random", 4), ((100, 36, 24), "random", 3),
+    ((68, 68, 8), "random", 1), ((64, 32, 64), "solid", 2), ((128, 8, 128), "checker", 2), ((1024, 4, 8), "slabs", 3),
+    ((512, 4, 512), "slabs", 3)])
+def test_merge_voxels_grid_shapes(oracle, grid, kind, palette):
+    """Rows of one, several and 32 words, ragged last words, columns of several words, more new boxes in a
+    layer than are handled at a time (checker), footprints of every size, and a layer too large for shared memory."""
+    from paper_2107_08170_b200 import binding as B
+    gx, gy, gz = grid
+    rng = np.random.default_rng(gx * gy + gz)
+    E = 3
+    g = np.zeros((E, gy, gz, gx), np.uint8)
+    if kind == "solid":
+        g[:] = 1
+        g[1, 5, 7, 9] = 0
+    elif kind == "checker":
+        y, z, x = np.ogrid[:gy, :gz, :gx]
+        g[:] = ((x + z) & 1) * (1 + (y // 3 & 1))
+        g[2] = np.where((x + z + y) & 1, 1, 0)
+    elif kind == "slabs":                                # random boxes over each other: long runs, ragged ends
+        for e in range(E):
+            for _ in range(200):
+                a = rng.integers(0, [gx, gy, gz])
+                b = a + rng.integers(1, [max(gx // 3, 2), gy, max(gz // 3, 2)])
+                g[e, a[1]:b[1], a[2]:b[2], a[0]:b[0]] = rng.integers(0, palette)
+    else:
+        g[:] = np.where(rng.random(g.shape) < 0.8, rng.integers(1, palette + 2, g.shape), 0)
+        g[1, :, :, : gx // 2] = 1
+    batch = B.Batch(B.make_desc(E, 1, grid, 0, 8, 4, palette))
+    batch.upload_worlds(0, E, torch.from_numpy(g).cuda(), palette=torch.zeros(E, palette, 3, dtype=torch.uint8).cuda())
+    cap = 40000
+    boxes, counts = batch.merge_voxels(0, E, cap)
+    for e in range(E):
+        want, total = oracle.merge_voxels(g[e], palette, cap)
+        assert int(counts[e]) == total, (grid, kind, e)
+        assert (boxes[e, :len(want)].cpu().numpy() == want).all(), (grid, kind, e)
+    batch.destroy()
