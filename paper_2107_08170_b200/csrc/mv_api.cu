@@ -43,12 +43,13 @@ struct mv_batch {
     mv_batch_desc desc;
     int num_obs = 0;
     size_t nvox = 0;
-    size_t mat_bytes_per_env = 0;       // material store: one byte per voxel index (columns padded to 2^ysh)
+    size_t mat_bytes_per_env = 0;       // material store: one byte per voxel (columns padded to 2^msh)
     EnvLayout lay{};
     unsigned char *d_env_blocks = nullptr;
     uint8_t *d_mat = nullptr;
     CamRec *d_cams = nullptr;
     uint32_t *d_status = nullptr;
+    int *d_acc = nullptr;               // [E][kPackAccInts] accumulators of the uploads in flight
     uint32_t *d_merge = nullptr;        // merge scratch: MergeLayout::env_words for merge_chunk envs
     MergeLayout merge{};
     int merge_chunk = 0;
@@ -177,6 +178,7 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.palette = b->desc.palette_size;
     p.W = b->desc.width; p.H = b->desc.height;
     p.tiles_x = b->tiles_x; p.tiles_y = b->tiles_y; p.mask_words = b->mask_words;
+    p.mat_mul = 1u << (b->lay.msh - 2);
     p.sky_rgbx = b->sky_rgbx;
     p.miss_depth = b->desc.miss_depth;
     const uint32_t unstaged = b->occ_shared ? 0u : b->lay.occ_bytes;   // shared-memory offsets shift down by it
@@ -210,12 +212,31 @@ int launch_cameras(mv_batch *b, const mv_camera *d_cams, cudaStream_t s) {
     return MV_OK;
 }
 
-int launch_boxes(mv_batch *b, int env_begin, const int32_t *d_env_index, int env_count, const mv_box *d_boxes,
-                 const int32_t *d_count, cudaStream_t s) {
-    const int n = env_count * (b->desc.max_boxes + 1);
-    copy_boxes_kernel<<<(n + 255) / 256, 256, 0, s>>>(reinterpret_cast<const uint4 *>(d_boxes), d_count,
-                                                       b->d_env_blocks, b->lay, env_begin, d_env_index, env_count,
-                                                       b->desc.max_boxes, b->desc.palette_size, b->d_status);
+// One launch for whatever the upload brings (null: not in this upload).
+int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int env_count, const uint8_t *d_grid,
+                  const mv_box *d_boxes, const int32_t *d_count, const uint8_t *d_palette, cudaStream_t s) {
+    const mv_batch_desc &d = b->desc;
+    UploadArgs u{};
+    u.grid = d_grid; u.boxes = reinterpret_cast<const uint4 *>(d_boxes); u.counts = d_count; u.palette_rgb = d_palette;
+    u.env_blocks = b->d_env_blocks; u.mat = b->d_mat; u.acc = b->d_acc; u.status = b->d_status;
+    u.env_index = d_env_index; u.lay = b->lay; u.env_begin = env_begin; u.env_count = env_count;
+    u.gx = d.grid_x; u.gy = d.grid_y; u.gz = d.grid_z; u.max_boxes = d.max_boxes; u.palette = d.palette_size;
+    for (int c = 0; c < 3; ++c) u.light[c] = (double)d.light_dir[c];
+    u.ambient = (double)d.ambient;
+    auto ctas = [](size_t threads) { return (threads + kUploadThreads - 1) / kUploadThreads; };
+    u.tiles_per_word = (int)ctas((size_t)(d.grid_x / 4) * d.grid_z);
+    u.tiles_per_env = u.tiles_per_word * ((d.grid_y + 31) / 32);         // (words above grid_y stay zero)
+    // tiles a CTA packs one after the other: one, until there are four CTAs for every slot of the GPU
+    const int64_t per_slot = (int64_t)u.tiles_per_env * env_count / (3 * 4 * (int64_t)b->sms);
+    u.tiles_per_cta = (int)(per_slot < 1 ? 1 : per_slot > 8 ? 8 : per_slot);
+    u.pack_ctas_per_env = (u.tiles_per_env + u.tiles_per_cta - 1) / u.tiles_per_cta;
+    const size_t pack = d_grid ? (size_t)u.pack_ctas_per_env * env_count : 0;
+    const size_t lut = d_palette ? ctas((size_t)env_count * kFaces * d.palette_size) : 0;
+    const size_t box = d_boxes ? ctas((size_t)env_count * (d.max_boxes + 1)) : 0;
+    if (pack + lut + box == 0) return MV_OK;
+    if (pack + lut + box > 0x7fffffffull) return MV_ERR_INVALID_ARG;
+    u.pack_ctas = (unsigned)pack; u.lut_ctas = (unsigned)lut;
+    upload_kernel<<<(unsigned)(pack + lut + box), kUploadThreads, pack ? kUploadSmem : 0, s>>>(u);
     b->launches++;
     MV_CUDA(b, cudaGetLastError());
     return MV_OK;
@@ -312,41 +333,13 @@ int upload_worlds(mv_batch *b, int env_begin, const int32_t *h_env_index, int en
         MV_CUDA(b, cudaMemcpyAsync(b->d_env_index, h_env_index, (size_t)env_count * 4, cudaMemcpyHostToDevice, s));
         d_index = b->d_env_index;
     }
-    auto dst_env = [&](int i) { return h_env_index ? h_env_index[i] : env_begin + i; };
-    if (d_grid) {
-        const size_t threads = ((size_t)(b->desc.grid_x / 4) * b->desc.grid_z << (b->lay.ysh - 5)) * (size_t)env_count;
-        const size_t blocks = (threads + 255) / 256;
-        if (blocks > 0x7fffffffull) return MV_ERR_INVALID_ARG;
-        pack_grid_kernel<<<(unsigned)blocks, 256, 0, s>>>(d_grid, b->d_env_blocks, b->d_mat, b->lay, b->desc.grid_x,
-                                                           b->desc.grid_y, b->desc.grid_z, env_begin, d_index, env_count,
-                                                           b->desc.palette_size, b->d_status);
-        b->launches++;
-        MV_CUDA(b, cudaGetLastError());
-        occupied_bounds_kernel<<<env_count, 256, 0, s>>>(b->d_env_blocks, b->lay, env_begin, d_index, b->desc.grid_x,
-                                                          b->desc.grid_y, b->desc.grid_z);
-        b->launches++;
-        MV_CUDA(b, cudaGetLastError());
-        for (int i = 0; i < env_count; ++i) {
-            const int e = dst_env(i);
-            if (!b->has_grid[e]) { b->has_grid[e] = 1; b->missing_grid--; }
-        }
-    }
-    if (d_palette) {
-        const int n = env_count * kFaces * b->desc.palette_size;
-        build_lut_kernel<<<(n + 255) / 256, 256, 0, s>>>(d_palette, b->d_env_blocks, b->lay, env_begin, d_index, env_count,
-                                                          b->desc.palette_size, (double)b->desc.light_dir[0],
-                                                          (double)b->desc.light_dir[1], (double)b->desc.light_dir[2],
-                                                          (double)b->desc.ambient);
-        b->launches++;
-        MV_CUDA(b, cudaGetLastError());
-        for (int i = 0; i < env_count; ++i) {
-            const int e = dst_env(i);
-            if (!b->has_palette[e]) { b->has_palette[e] = 1; b->missing_palette--; }
-        }
-    }
-    if (d_boxes) {
-        int r = launch_boxes(b, env_begin, d_index, env_count, d_boxes, d_box_count, s);
-        if (r != MV_OK) return r;
+    int r = launch_upload(b, env_begin, d_index, env_count, d_grid, d_boxes, d_box_count, d_palette, s);
+    if (r != MV_OK) return r;
+    // (once every env has a grid and a palette there is nothing left to track)
+    for (int i = 0; i < env_count && ((d_grid && b->missing_grid > 0) || (d_palette && b->missing_palette > 0)); ++i) {
+        const int e = h_env_index ? h_env_index[i] : env_begin + i;
+        if (d_grid && !b->has_grid[e]) { b->has_grid[e] = 1; b->missing_grid--; }
+        if (d_palette && !b->has_palette[e]) { b->has_palette[e] = 1; b->missing_palette--; }
     }
     return MV_OK;
 }
@@ -396,7 +389,8 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     L.ysh = 5;                                              // bits per (x, z) column: a power of two >= grid_y, >= 32
     while ((1 << L.ysh) < d.grid_y) L.ysh++;
     L.occ_bytes = (uint32_t)(((size_t)d.grid_x * d.grid_z << L.ysh) / 8);
-    b->mat_bytes_per_env = (size_t)d.grid_x * d.grid_z << L.ysh;
+    L.msh = d.grid_y <= 16 ? 4 : L.ysh;
+    b->mat_bytes_per_env = (size_t)d.grid_x * d.grid_z << L.msh;
     L.lut_off = L.occ_bytes;
     L.box_off = L.lut_off + round_up(kFaces * d.palette_size * 4, 16);
     L.count_off = L.box_off + (uint32_t)d.max_boxes * 32;
@@ -437,6 +431,7 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
                        RenderFn(render_kernel<kRenderThreadsSmall, true, false>),
                        RenderFn(render_kernel<kRenderThreadsSmall, false, false>)})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(upload_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUploadSmem);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
     // One CTA per environment (block staged once for all its agents) when that still fills the GPU;
     // otherwise one CTA per observation.  Cost model: waves of resident CTAs x (agents + fixed part).
@@ -467,6 +462,7 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
               cudaMalloc(&b->d_mat, (size_t)d.num_envs * b->mat_bytes_per_env) == cudaSuccess &&
               cudaMalloc(&b->d_cams, (size_t)b->num_obs * sizeof(CamRec)) == cudaSuccess &&
               cudaMalloc(&b->d_status, 16) == cudaSuccess &&
+              cudaMalloc(&b->d_acc, (size_t)d.num_envs * kPackAccInts * 4) == cudaSuccess &&
               cudaMalloc(&b->d_env_index, (size_t)d.num_envs * 4) == cudaSuccess;
     if (ok && d.max_overlay_rects > 0)
         ok = cudaMalloc(&b->d_overlay, (size_t)b->num_obs * d.max_overlay_rects * 16) == cudaSuccess &&
@@ -474,6 +470,11 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
              cudaMemset(b->d_overlay_count, 0, (size_t)b->num_obs * 4) == cudaSuccess;
     if (ok) ok = cudaMemset(b->d_env_blocks, 0, blocks_bytes) == cudaSuccess &&
                  cudaMemset(b->d_status, 0, 16) == cudaSuccess;
+    if (ok) {
+        const int n = d.num_envs * kPackAccInts;
+        init_acc_kernel<<<(n + 255) / 256, 256>>>(b->d_acc, n);
+        ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(0) == cudaSuccess;
+    }
     if (!ok) {
         cudaGetLastError();
         mv_destroy(b);
@@ -626,7 +627,7 @@ int mv_step_host(mv_batch *b, const mv_camera *h_cams, const mv_box *h_boxes, co
         MV_CUDA(b, cudaMemcpyAsync(b->d_box_in, h_boxes, (size_t)E * b->desc.max_boxes * sizeof(mv_box),
                                    cudaMemcpyHostToDevice, s));
         MV_CUDA(b, cudaMemcpyAsync(b->d_count_in, h_box_count, (size_t)E * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-        int r = launch_boxes(b, 0, nullptr, E, b->d_box_in, b->d_count_in, s);
+        int r = launch_upload(b, 0, nullptr, E, nullptr, b->d_box_in, b->d_count_in, nullptr, s);
         if (r != MV_OK) return r;
     }
     int r = launch_cameras(b, b->d_cam_in, s);
@@ -734,7 +735,7 @@ int mv_destroy(mv_batch *b) {
         DeviceGuard g(b->desc.device);
         if (g.ok) {
             if (cudaDeviceSynchronize() != cudaSuccess) rc = MV_ERR_CUDA;
-            cudaFree(b->d_env_blocks); cudaFree(b->d_mat); cudaFree(b->d_cams); cudaFree(b->d_status);
+            cudaFree(b->d_env_blocks); cudaFree(b->d_mat); cudaFree(b->d_cams); cudaFree(b->d_status); cudaFree(b->d_acc);
             cudaFree(b->d_overlay); cudaFree(b->d_overlay_count); cudaFree(b->d_merge); cudaFree(b->d_env_index);
             free_host_step(b);
             cudaGetLastError();

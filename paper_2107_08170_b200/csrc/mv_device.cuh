@@ -28,7 +28,8 @@ static_assert(sizeof(CamRec) == 64, "CamRec must be 64 bytes");
 // Occupancy is packed along y: the (x, z) column owns 2^ysh consecutive bits (2^ysh >= grid_y, at
 // least 32), bit index u = ((x + grid_x*z) << ysh) | y, bit u&31 of word u>>5.  A walk along x or z
 // therefore moves by whole words and a walk along y stays inside the column's word(s); for grids
-// up to 32 voxels high a column is exactly one word.  The material store uses the same index u.
+// up to 32 voxels high a column is exactly one word.  The material store keeps a column's bytes together in the
+// same way, ((x + grid_x*z) << msh) | y; 16 bytes are enough for the low grids and halve what an upload writes.
 struct EnvLayout {
     uint32_t occ_bytes;     // grid_x*grid_z*2^ysh/8
     uint32_t lut_off;       // 7*palette_size RGBX words
@@ -38,6 +39,7 @@ struct EnvLayout {
     uint32_t block_bytes;   // bytes staged per CTA (multiple of 16)
     uint32_t stride;        // distance between envs in HBM (multiple of 128)
     uint32_t ysh;           // log2 of the bits per (x, z) column
+    uint32_t msh;           // log2 of the material bytes per column: ysh, or 4 for grids up to 16 high
 };
 
 __host__ __device__ __forceinline__ uint32_t voxel_index(uint32_t ysh, int gx, int x, int y, int z) {
@@ -46,7 +48,7 @@ __host__ __device__ __forceinline__ uint32_t voxel_index(uint32_t ysh, int gx, i
 
 struct RenderParams {
     const unsigned char *env_blocks;   // [E] EnvLayout blocks
-    const uint8_t *mat;                // [E][grid_x*grid_z << ysh] material ids by voxel index (clamped at upload)
+    const uint8_t *mat;                // [E][grid_x*grid_z << msh] material ids by column and height (clamped at upload)
     const CamRec *cams;                // [O]
     uint8_t *rgb;                      // [O][H][W][3]
     float *depth;                      // [O][H][W]
@@ -57,6 +59,7 @@ struct RenderParams {
     int gx, gy, gz;
     int max_boxes, palette;
     int W, H, tiles_x, tiles_y, mask_words;
+    uint32_t mat_mul;                  // material bytes per byte of occupancy word: 2^msh / 4 (grids up to 32 high)
     uint32_t sky_rgbx;
     float miss_depth;
     int agents_per_cta;                // observations one CTA renders: 1, or all agents of its env
@@ -73,5 +76,36 @@ struct RenderParams {
     int wait_polls;                    // bound of the staging wait
     int skip_staging;                  // test hook: the block copy is not issued, so the wait runs out
 };
+
+// Bulk asynchronous copies into shared memory and the barrier that counts their bytes.
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+// Plain (single-CTA) bulk copy global -> shared, completion counted on an mbarrier.
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Bounded wait: gives up after `limit` polls instead of spinning forever.
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, int limit) {
+    for (int i = 0; i < limit; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
+}
+constexpr int kDrainPolls = 1 << 26;               // bound of the wait for a copy known to be in flight
 
 }  // namespace mv

@@ -21,38 +21,8 @@
 
 namespace mv {
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-// Plain (single-CTA) bulk copy global -> shared, completion counted on an mbarrier.
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Bounded wait: gives up after `limit` polls instead of spinning forever.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, int limit) {
-    for (int i = 0; i < limit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-
 #define kInf (__int_as_float(0x7f800000))
 constexpr uint32_t kNoRow = 0xffffffffu;           // "no surface" marker of the traversal
-constexpr int kDrainPolls = 1 << 26;               // bound of the wait for a copy known to be in flight
 
 // Reciprocal to 1 ulp in one instruction; every use is inside toleranced intersection arithmetic.
 __device__ __forceinline__ float fast_rcp(float x) {
@@ -371,7 +341,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             rec[4] = make_float4(__uint_as_float(1u << cy0), filled ? -kInf : p.exit_scale,
                                  __uint_as_float(filled ? inside_row : kNoRow), __uint_as_float(cell_pos(cx0, cy0, cz0)));
             const unsigned long long mp = reinterpret_cast<unsigned long long>(
-                p.mat + (size_t)env * ((size_t)gx * gz << p.lay.ysh) - vi_bias);
+                p.mat + (size_t)env * ((size_t)gx * gz << p.lay.msh) -
+                (COLW ? occ_base * p.mat_mul : vi_bias >> (p.lay.ysh - p.lay.msh)));
             rec[5] = make_float4(__uint_as_float((uint32_t)mp), __uint_as_float((uint32_t)(mp >> 32)),
                                  __uint_as_float(p.sky_rgbx), p.miss_depth);
         }
@@ -517,7 +488,9 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 if (COLW) {
                     uint32_t y;
                     asm("bfind.u32 %0, %1;" : "=r"(y) : "r"(bit));
-                    vi = (pos << 3) + y;
+                    vi = pos * p.mat_mul + y;
+                } else if (p.lay.msh < p.lay.ysh) {
+                    vi = ((pos >> 1) & ~15u) | (pos & 15u);      // 16 material bytes to 32 occupancy bits
                 }
                 asm volatile("{\n"
                     " .reg .pred pv;\n"

@@ -735,3 +735,28 @@ def test_host_step_allocation_failure_is_reported_and_can_be_retried():
     from gpu_util import render_scene
     cfg = scenes.config("tiny")
     assert render_scene(cfg, scenes.make_scene(cfg))[2] == 0
+
+
+@pytest.mark.parametrize("grid,palette,envs", [((4, 4, 4), 1, 3), ((16, 16, 64), 200, 2), ((20, 20, 52), 129, 2),
+                                               ((128, 32, 36), 64, 40), ((64, 36, 20), 256, 2), ((32, 132, 68), 7, 9)])
+def test_upload_packs_every_tile(oracle, grid, palette, envs):
+    """Tiles of the upload: less than one, exact, ragged, several per CTA, several words per column, 16 and 32 material
+    bytes per column.  The voxel merge reads back what was packed (occupancy, bounds and materials)."""
+    B = _binding()
+    gx, gy, gz = grid
+    rng = np.random.default_rng(gx + gy)
+    g = np.where(rng.random((envs, gy, gz, gx)) < 0.1, rng.integers(1, palette + 3, (envs, gy, gz, gx)), 0).astype(np.uint8)
+    g[envs - 1] = 0
+    g[envs - 1, gy - 1, gz - 1, gx - 1] = 1
+    batch = B.Batch(B.make_desc(envs, 1, grid, 0, 8, 4, palette))
+    d_grid = torch.from_numpy(g).cuda()
+    for _ in range(2):                                           # (the second upload finds the accumulators as the first left them)
+        batch.upload_worlds(0, envs, d_grid)
+    assert batch.query_status() == (1 if (g >= palette).any() else 0)
+    cap = 20000
+    boxes, counts = batch.merge_voxels(0, envs, cap)
+    for e in (0, envs // 2, envs - 1):
+        want, total = oracle.merge_voxels(g[e], palette, cap)
+        assert int(counts[e]) == total
+        assert (boxes[e, :len(want)].cpu().numpy() == want).all()
+    batch.destroy()
