@@ -43,7 +43,7 @@ struct mv_batch {
     mv_batch_desc desc;
     int num_obs = 0;
     size_t nvox = 0;
-    size_t mat_bytes_per_env = 0;       // material store: one byte per voxel (columns padded to 2^msh)
+    size_t mat_bytes_per_env = 0;       // material store: one byte per voxel index (columns padded to 2^ysh)
     EnvLayout lay{};
     unsigned char *d_env_blocks = nullptr;
     uint8_t *d_mat = nullptr;
@@ -131,9 +131,6 @@ mv_batch::Smem smem_layout(const mv_batch *b, int apc) {
     m.agent_stride = m.agent_ovtile_off + round_up(((ntiles + 31) / 32) * 4, 16);
     m.misc_off = m.agent_off + (uint32_t)apc * m.agent_stride;
     m.bytes = m.misc_off + 32;
-#if defined(MV_BRICKS) && MV_BRICKS == 1
-    m.bytes += round_up((uint32_t)((d.grid_x / 4) * (d.grid_z / 4)), 16);   // experiment: one byte per column of 4x4x4 bricks
-#endif
     return m;
 }
 
@@ -178,7 +175,6 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.palette = b->desc.palette_size;
     p.W = b->desc.width; p.H = b->desc.height;
     p.tiles_x = b->tiles_x; p.tiles_y = b->tiles_y; p.mask_words = b->mask_words;
-    p.mat_mul = 1u << (b->lay.msh - 2);
     p.sky_rgbx = b->sky_rgbx;
     p.miss_depth = b->desc.miss_depth;
     const uint32_t unstaged = b->occ_shared ? 0u : b->lay.occ_bytes;   // shared-memory offsets shift down by it
@@ -389,8 +385,7 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     L.ysh = 5;                                              // bits per (x, z) column: a power of two >= grid_y, >= 32
     while ((1 << L.ysh) < d.grid_y) L.ysh++;
     L.occ_bytes = (uint32_t)(((size_t)d.grid_x * d.grid_z << L.ysh) / 8);
-    L.msh = d.grid_y <= 16 ? 4 : L.ysh;
-    b->mat_bytes_per_env = (size_t)d.grid_x * d.grid_z << L.msh;
+    b->mat_bytes_per_env = (size_t)d.grid_x * d.grid_z << L.ysh;
     L.lut_off = L.occ_bytes;
     L.box_off = L.lut_off + round_up(kFaces * d.palette_size * 4, 16);
     L.count_off = L.box_off + (uint32_t)d.max_boxes * 32;

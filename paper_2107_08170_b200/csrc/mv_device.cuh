@@ -28,8 +28,7 @@ static_assert(sizeof(CamRec) == 64, "CamRec must be 64 bytes");
 // Occupancy is packed along y: the (x, z) column owns 2^ysh consecutive bits (2^ysh >= grid_y, at
 // least 32), bit index u = ((x + grid_x*z) << ysh) | y, bit u&31 of word u>>5.  A walk along x or z
 // therefore moves by whole words and a walk along y stays inside the column's word(s); for grids
-// up to 32 voxels high a column is exactly one word.  The material store keeps a column's bytes together in the
-// same way, ((x + grid_x*z) << msh) | y; 16 bytes are enough for the low grids and halve what an upload writes.
+// up to 32 voxels high a column is exactly one word.  The material store uses the same index u.
 struct EnvLayout {
     uint32_t occ_bytes;     // grid_x*grid_z*2^ysh/8
     uint32_t lut_off;       // 7*palette_size RGBX words
@@ -39,7 +38,6 @@ struct EnvLayout {
     uint32_t block_bytes;   // bytes staged per CTA (multiple of 16)
     uint32_t stride;        // distance between envs in HBM (multiple of 128)
     uint32_t ysh;           // log2 of the bits per (x, z) column
-    uint32_t msh;           // log2 of the material bytes per column: ysh, or 4 for grids up to 16 high
 };
 
 __host__ __device__ __forceinline__ uint32_t voxel_index(uint32_t ysh, int gx, int x, int y, int z) {
@@ -48,7 +46,7 @@ __host__ __device__ __forceinline__ uint32_t voxel_index(uint32_t ysh, int gx, i
 
 struct RenderParams {
     const unsigned char *env_blocks;   // [E] EnvLayout blocks
-    const uint8_t *mat;                // [E][grid_x*grid_z << msh] material ids by column and height (clamped at upload)
+    const uint8_t *mat;                // [E][grid_x*grid_z << ysh] material ids by voxel index (clamped at upload)
     const CamRec *cams;                // [O]
     uint8_t *rgb;                      // [O][H][W][3]
     float *depth;                      // [O][H][W]
@@ -59,7 +57,6 @@ struct RenderParams {
     int gx, gy, gz;
     int max_boxes, palette;
     int W, H, tiles_x, tiles_y, mask_words;
-    uint32_t mat_mul;                  // material bytes per byte of occupancy word: 2^msh / 4 (grids up to 32 high)
     uint32_t sky_rgbx;
     float miss_depth;
     int agents_per_cta;                // observations one CTA renders: 1, or all agents of its env

@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
     const int w = 4 * wb + wi, x = 32 * w + lane, z0 = 8 * zb + 4 * half;
     const bool upper = hiy - 32 * wq > 16, in_x = x < ml.gx;
     const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk) + x * ml.colw + wq;
-    const uint8_t *m_col = mat + (size_t)(env_begin + e) * ((size_t)ml.gx * ml.gz << lay.msh) + ((size_t)x << lay.msh) + 32 * wq;
+    const uint8_t *m_col = mat + (size_t)(env_begin + e) * ((size_t)ml.gx * ml.gz << lay.ysh) + ((size_t)x << lay.ysh) + 32 * wq;
     uint32_t *ye = scratch + (size_t)e * ml.env_words + 3 * (size_t)ml.mask_words + x * ml.colw + wq;
     auto load_column = [&](const uint8_t *src, uint32_t out[8]) {
         const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src));
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
     uint32_t own[8] = {}, back[8] = {}, f_back = 0;
     if (in_x && z0 > 0 && z0 < ml.gz) {
         f_back = occ[(size_t)(z0 - 1) * ml.gx * ml.colw];
-        load_column(m_col + ((size_t)(z0 - 1) * ml.gx << lay.msh), back);
+        load_column(m_col + ((size_t)(z0 - 1) * ml.gx << lay.ysh), back);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -107,13 +107,13 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
         uint32_t f = 0, lx = 0, lz = 0;
         if (z < ml.gz && in_x) {
             const size_t row = (size_t)z * ml.gx;
-            const uint8_t *src = m_col + (row << lay.msh);
+            const uint8_t *src = m_col + (row << lay.ysh);
             f = occ[row * ml.colw];
             uint32_t other[8], f_left = 0;
             load_column(src, own);
             if (x > 0) {
                 f_left = occ[(row - 1) * ml.colw];
-                load_column(src - (1u << lay.msh), other);
+                load_column(src - (1u << lay.ysh), other);
             }
             lz = f & f_back & equal_bits(own, back);
             if (x > 0) lx = f & f_left & equal_bits(own, other);
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
     const unsigned char *blk = env_blocks + (size_t)(env_begin + e) * lay.stride;
     const int *bounds = reinterpret_cast<const int *>(blk + lay.count_off);
     const int loy = bounds[2], loz = bounds[3], hiy = bounds[5], hiz = bounds[6];
-    const uint8_t *m_env = mat + (size_t)(env_begin + e) * ((size_t)gx * gz << lay.msh);
+    const uint8_t *m_env = mat + (size_t)(env_begin + e) * ((size_t)gx * gz << lay.ysh);
     uint32_t *mine = scratch + (size_t)e * ml.env_words;
     const uint32_t *masks = mine, *ye = mine + 3 * (size_t)ml.mask_words;
     uint4 *rows = reinterpret_cast<uint4 *>(ml.work_in_smem ? s_work : reinterpret_cast<unsigned char *>(mine + ml.work_off));
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
             // a thread per box: the run in its first row, and the rows until its first cell is marked ended
             for (int b = tid; b < n; b += kMergeThreads) {
                 const int x = (int)(s_list[b] & 0xffffu), k = (int)(s_list[b] >> 16);
-                const uint8_t m = m_env[voxel_index(lay.msh, gx, x, j, k)];
+                const uint8_t m = m_env[voxel_index(lay.ysh, gx, x, j, k)];
                 int wd = x >> 5;
                 uint4 r = rows[k * slots + wd];
                 uint32_t stop = (r.y | ~r.x) & ~((2u << (x & 31)) - 1u);

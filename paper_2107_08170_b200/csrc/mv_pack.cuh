@@ -173,19 +173,12 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
         if (r >= groups) continue;
         const int z = r / xg_n, xg = r - z * xg_n;
         const uint32_t col0 = 4u * (uint32_t)r;
-        uint8_t *mdst = p.mat + env * ((size_t)layer << p.lay.msh) + ((size_t)col0 << p.lay.msh) + 32 * wq;
+        uint8_t *mdst = p.mat + env * ((size_t)layer << p.lay.ysh) + ((size_t)col0 << p.lay.ysh) + 32 * wq;
         uint32_t *occ = reinterpret_cast<uint32_t *>(blk);
-        if (p.lay.msh == 4) {                                 // grids up to 16 high keep 16 bytes a column
 #pragma unroll
-            for (int c = 0; c < 4; c += 2)
-                store32(mdst + ((size_t)c << 4), col[c][0], col[c][1], col[c][2], col[c][3],
-                        col[c + 1][0], col[c + 1][1], col[c + 1][2], col[c + 1][3]);
-        } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                store32(mdst + ((size_t)c << p.lay.msh), col[c][0], col[c][1], col[c][2], col[c][3], col[c][4], col[c][5],
-                        col[c][6], col[c][7]);
-        }
+        for (int c = 0; c < 4; ++c)
+            store32(mdst + ((size_t)c << p.lay.ysh), col[c][0], col[c][1], col[c][2], col[c][3], col[c][4], col[c][5],
+                    col[c][6], col[c][7]);
         if (colw == 1) *reinterpret_cast<uint4 *>(occ + col0) = make_uint4(bits[0], bits[1], bits[2], bits[3]);
         else
 #pragma unroll

@@ -64,21 +64,10 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 // Register names used by the macros (declared by the enclosing asm block): tx ty tz dtx dty dtz
 // (f32), sx sy sz pos bit w a it (b32), ta tb (f32), px py pz pq ph pf (pred), texit (f32); the
 // global flavour also uses ag (b64) and the operand named by MV_DDA_GBASE.
-#if defined(MV_PROBE) && MV_PROBE == 9
-#define MV_DDA_COUNT " add.f32 ns, ns, 0f3F800000;\n"
-#else
-#define MV_DDA_COUNT
-#endif
-#if defined(MV_TEST_FORM) && MV_TEST_FORM == 1
-#define MV_DDA_TESTBIT " and.b32 w, w, bit;\n setp.ne.u32 ph, w, 0;\n"
-#else
-#define MV_DDA_TESTBIT " lop3.or.b32 w|ph, w, bit, 0, 0xC0, pf;\n"
-#endif
 #define MV_DDA_HEAD(T, OUT)                          \
     " min.f32 " T ", tx, ty, tz;\n"                  \
     " setp.geu.or.f32 pq, " T ", texit, ph;\n"       \
     " @pq bra " OUT ";\n"                            \
-    MV_DDA_COUNT                                     \
     " setp.eq.f32 px, tx, " T ";\n"                  \
     " setp.eq.and.f32 py|pz, ty, " T ", !px;\n"      \
     " @px add.f32 tx, tx, dtx;\n"                    \
@@ -89,7 +78,7 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " @pz add.s32 pos, pos, sz;\n"                   \
     " @py shf.l.wrap.b32 bit, bit, bit, sy;\n"       \
     " ld.shared.u32 w, [pos];\n"                     \
-    MV_DDA_TESTBIT
+    " lop3.or.b32 w|ph, w, bit, 0, 0xC0, pf;\n"
 #define MV_DDA_STEP_IDX_TAIL                         \
     " shf.r.wrap.b32 w, w, 0, pos;\n"                \
     " lop3.or.b32 w|ph, w, 1, 0, 0xC0, pf;\n"
@@ -120,24 +109,10 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     "MV_DDA_OUT:\n"
 #define MV_DDA_DECL                                  \
     " .reg .pred px, py, pz, pq, ph, pf;\n"          \
-    " .reg .f32 tx, ty, tz, dtx, dty, dtz, ta, tb, texit, thit, ns;\n" \
+    " .reg .f32 tx, ty, tz, dtx, dty, dtz, ta, tb, texit, thit;\n" \
     " .reg .b32 sx, sy, sz, pos, bit, w, a, it;\n"   \
-    " .reg .b64 ag, gbase;\n"                        \
-    " mov.f32 ns, 0f00000000;\n"
+    " .reg .b64 ag, gbase;\n"
 
-// MV_PROBE builds are for instruction counting only (never the shipped library): 1 = every walk ends
-// at its first test, 2 = also no box tests, 3 = no tiles at all (CTA prologue alone), 9 = the depth
-// channel carries each ray's number of walk steps instead of depth.
-#ifndef MV_PROBE
-#define MV_PROBE 0
-#endif
-// MV_BRICKS builds are an experiment, never the shipped library: 1 = two-level traversal (a one-bit map
-// of 4x4x4 bricks built per CTA; empty bricks are jumped across, occupied ones walked cell by cell by
-// the same PTX loop), 2 = the flat walk through the same C++ path, as the like-for-like baseline of 1.
-// Both need grid_x to be a power of two and a grid at most 32 high.
-#ifndef MV_BRICKS
-#define MV_BRICKS 0
-#endif
 #ifndef MV_MINB
 #define MV_MINB 3
 #endif
@@ -149,11 +124,11 @@ constexpr uint32_t kAgentFilled = 4u;      // the eye's own voxel is filled
 // Per-agent block in shared memory (16-byte slots): camera record (3), {hit time a ray starts with,
 // flags, self box, overlay count} (1), {start bit mask, exit-time factor, start colour row, start position} (1), {64-bit address
 // of the env's material store, biased for the walk's positions} (1), DDA start
-// table (8 sign combinations x 3 axes), then eye-relative boxes, overlay rectangles, per-tile box
+// table (8 sign combinations x 3 axes + 2 rows for the first stretch), then eye-relative boxes, overlay rectangles, per-tile box
 // masks and per-tile overlay bits at offsets the host lays out.
 constexpr int kAgentRecVecs = 6;
-constexpr int kDdaVecs = 24;
-// byte offsets, from the agent block's start plus 48 x (sign combination), of the DDA table rows of
+constexpr int kDdaVecs = 40;                        // 8 sign combinations x 5 rows
+// byte offsets, from the agent block's start plus 80 x (sign combination), of the DDA table rows of
 // the x, y and z axis and of the colour-row word of the x row (as text, for the PTX blocks)
 // hard bound of the traversal loop: no grid allows more steps than 3 x 1024 + 3
 #define MV_STEP_BUDGET "3080"
@@ -161,6 +136,18 @@ constexpr int kDdaVecs = 24;
 #define MV_TAB_Y "112"
 #define MV_TAB_Z "128"
 #define MV_TAB_ROW "108"
+#define MV_TAB_SKIP "144"
+#define MV_TAB_SKIP2 "160"
+// The empty box that a walk starts with (see the table's construction) grows by at most this many cells an axis.
+constexpr int kSkipCells = 8, kSkipCellsY = 4;
+// Crossings are counted up to a little less than the box's exit time: 2^-16 of the count, where rounding takes 2^-20 of
+// it at most; one that falls in between is left to the walk.
+constexpr float kSkipMargin = 1.0f - 1.52587890625e-5f;
+#define MV_SKIP_MARGIN "0f3F7FFF00"
+// The count comes out of an addition of 2^23, whose float's bits are 0x4B000000 + count.
+constexpr uint32_t kSkipBias = 0x4B000000u;
+#define MV_SKIP_MAGIC "0f4B000000"
+#define MV_SKIP_UNMAGIC "0fCB000000"
 static_assert(16 * kAgentRecVecs == 96, "MV_TAB_* follow the agent record size");
 constexpr uint32_t kAgentDdaOff = 16u * kAgentRecVecs;
 constexpr uint32_t kAgentRelOff = 16u * (kAgentRecVecs + kDdaVecs);
@@ -308,13 +295,13 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         const uint32_t u = (uint32_t)(stride_x * cx + stride_z * cz + cy);
         return (s_occ[u >> 5] >> (u & 31)) & 1u;
     };
-    for (int slot = tid; slot < kDdaVecs * apc; slot += NT) {
-        // DDA start table of agent ag, entry 3*signs + axis (bit c of `signs` set: direction component c
+    for (int slot = tid; slot < 24 * apc; slot += NT) {
+        // DDA start table of agent ag, row 5*signs + axis (bit c of `signs` set: direction component c
         // negative): x = distance (>= 0) from the eye to the cell face the ray meets first, y = cells
         // left before the occupied box ends that way, z = what a step along the axis adds to the
         // position (column-word flavour: byte stride for x and z, rotate count for y), w = shared-memory
         // address of the colour-table row of the face entered by a step along this axis.
-        const int ag = slot / kDdaVecs, e = slot - ag * kDdaVecs;
+        const int ag = slot / 24, e = slot - ag * 24;
         const int signs = e / 3, ax = e - 3 * signs, neg = (signs >> ax) & 1;
         float4 *rec = agent_rec(ag);
         const float4 c0 = rec[0];
@@ -328,7 +315,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         int st;
         if (COLW) st = ax == 0 ? (neg ? -4 : 4) : (ax == 1 ? (neg ? 31 : 1) : (neg ? -4 * gx : 4 * gx));
         else st = (ax == 0 ? stride_x : (ax == 1 ? 1 : stride_z)) * (neg ? -1 : 1);
-        agent_dda(ag)[e] = make_float4(neg ? Pc - (float)cc : (float)(cc + 1) - Pc,
+        agent_dda(ag)[5 * signs + ax] = make_float4(neg ? Pc - (float)cc : (float)(cc + 1) - Pc,
                                        neg ? (float)(cc - lo_c) : (float)(hi_c - 1 - cc), __int_as_float(st),
                                        __uint_as_float(lut_base + (uint32_t)((2 * ax + neg) * P_ * 4)));
         if (e == 0) {
@@ -341,11 +328,73 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             rec[4] = make_float4(__uint_as_float(1u << cy0), filled ? -kInf : p.exit_scale,
                                  __uint_as_float(filled ? inside_row : kNoRow), __uint_as_float(cell_pos(cx0, cy0, cz0)));
             const unsigned long long mp = reinterpret_cast<unsigned long long>(
-                p.mat + (size_t)env * ((size_t)gx * gz << p.lay.msh) -
-                (COLW ? occ_base * p.mat_mul : vi_bias >> (p.lay.ysh - p.lay.msh)));
+                p.mat + (size_t)env * ((size_t)gx * gz << p.lay.ysh) - vi_bias);
             rec[5] = make_float4(__uint_as_float((uint32_t)mp), __uint_as_float((uint32_t)(mp >> 32)),
                                  __uint_as_float(p.sky_rgbx), p.miss_depth);
         }
+    }
+    // The first stretch of a walk.  For every combination of signs: a box of empty cells that begins at the eye's cell and is
+    // grown greedily the way such rays go (x, z, y in turn, while the next layer of cells is empty).  A ray crosses
+    // nothing filled before it leaves that box, so it takes all its x and z crossings up to then at once, whatever their
+    // order (three steps of seven on average; the vertical ones are too few to be worth it): 234 -> 220 instructions a tile
+    // on 128x32x128 columns, 1230 -> 1184 us for 16384 observations; 64x16x64 rooms with boxes 1126 -> 1007 us.  Rows 3 and
+    // 4 of the table:
+    // {cells to spare in x, z, y; start position, from which kSkipBias steps each way are taken off} {what is added to
+    // t |d| in x and in z to give the crossings up to time t, rounded down}.
+    for (int slot = (tid + NT - 64) % NT; slot < 8 * apc; slot += NT) {
+        const int ag = slot >> 3, signs = slot & 7;
+        const float4 c0 = agent_rec(ag)[0];
+        float4 *row = agent_dda(ag) + 5 * signs + 3;
+        const bool cam_in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
+                            (c0.y < (float)hiy) && (c0.z >= (float)loz) && (c0.z < (float)hiz);
+        if (!cam_in) continue;                       // (the table's users start elsewhere)
+        const int cx = (int)floorf(c0.x), cy = (int)floorf(c0.y), cz = (int)floorf(c0.z);
+        const int dx = (signs & 1) ? -1 : 1, dy = (signs & 2) ? -1 : 1, dz = (signs & 4) ? -1 : 1;
+        const int wsh = p.lay.ysh - 5, yb = cy & 31;
+        const uint32_t *word = s_occ + (((cx + gx * cz) << wsh) + (cy >> 5));
+        const int step_x = dx << wsh, step_z = (gx * dz) << wsh;
+        const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
+        // (an eye exactly on a cell face and looking down the axis leaves its cell at once: one more for it, so that
+        // mirrored views get mirrored boxes)
+        const int on_x = qx == 0.0f ? 1 : 0, on_z = qz == 0.0f ? 1 : 0;
+        const int lim_x = min(kSkipCells - 1 + on_x, dx < 0 ? cx - lox : hix - 1 - cx);
+        const int lim_z = min(kSkipCells - 1 + on_z, dz < 0 ? cz - loz : hiz - 1 - cz);
+        const int lim_y = min(min(kSkipCellsY, dy < 0 ? cy - loy : hiy - 1 - cy), dy < 0 ? yb : 31 - yb);
+        uint32_t seen = word[0], ys = 1u << yb;      // columns of the box or-ed together; its heights
+        int ex = 0, ey = 0, ez = 0;
+        bool gox = !(seen & ys) && lim_x > 0, goz = !(seen & ys) && lim_z > 0, goy = !(seen & ys);
+        if (gox && on_x) { const uint32_t f = word[step_x]; gox = !(f & ys); if (gox) { seen |= f; ex = 1; } }
+        if (goz && on_z) {
+            const uint32_t f = word[step_z] | (ex ? word[step_x + step_z] : 0u);
+            goz = !(f & ys);
+            if (goz) { seen |= f; ez = 1; }
+        }
+        while (gox || goy || goz) {
+            // the next layers in x and z and the corner between them, all loads of a round in flight at once
+            gox = gox && ex < lim_x;
+            goz = goz && ez < lim_z;
+            const uint32_t *px = word + (ex + 1) * step_x, *pz = word + (ez + 1) * step_z;
+            uint32_t fx = 0, fz = 0, corner = 0;
+#pragma unroll
+            for (int i = 0; i <= kSkipCells; ++i) {
+                if (gox && i <= ez) fx |= px[i * step_z];
+                if (goz && i <= ex) fz |= pz[i * step_x];
+            }
+            if (gox && goz) corner = px[(ez + 1) * step_z];
+            gox = gox && !(fx & ys);
+            if (gox) { seen |= fx; fz |= corner; ++ex; }
+            goz = goz && !(fz & ys);
+            if (goz) { seen |= fz; ++ez; }
+            const uint32_t b = 1u << ((yb + dy * (ey + 1)) & 31);
+            goy = goy && ey < lim_y && !(seen & b);
+            if (goy) { ys |= b; ++ey; }
+        }
+        int sx, sz;
+        if (COLW) { sx = 4 * dx; sz = 4 * gx * dz; }
+        else { sx = dx * stride_x; sz = dz * stride_z; }
+        row[0] = make_float4((float)ex, (float)ez, (float)ey,
+                             __uint_as_float(cell_pos(cx, cy, cz) - kSkipBias * (uint32_t)sx - kSkipBias * (uint32_t)sz));
+        row[1] = make_float4((1.0f - qx) * kSkipMargin, (1.0f - qz) * kSkipMargin, 0.0f, 0.0f);
     }
     {
         const int nb = min(s_count[0], p.max_boxes);
@@ -401,21 +450,6 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     }
         }
     }
-#if MV_BRICKS == 1
-    unsigned char *s_brick = smem + p.smem_misc_off + 32;
-    if (COLW) {
-        const int bxn = gx >> 2, bzn = gz >> 2;
-        for (int i = tid; i < bxn * bzn; i += NT) {
-            const int bx = i % bxn, bz = i / bxn;
-            uint32_t m = 0;
-            for (int j = 0; j < 4; ++j)
-                for (int k = 0; k < 4; ++k) m |= s_occ[(4 * bx + k) + gx * (4 * bz + j)];
-            uint32_t byte = 0;
-            for (int by = 0; by < 8; ++by) byte |= ((m >> (4 * by)) & 0xFu) ? (1u << by) : 0u;
-            s_brick[i] = (unsigned char)byte;
-        }
-    }
-#endif
     __syncthreads();
 
     const float flox = (float)lox, floy = (float)loy, floz = (float)loz;
@@ -437,11 +471,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     const int rgb_lane_off = st_r * W * 3 + st_j * 4;
     keep(lane_a); keep(lane_b); keep(st_sel);
     const uint32_t tile_begin = smem_addr(s_tile) + 16u * (uint32_t)warp;
-#if MV_PROBE == 3
-    uint32_t tile_end = smem_addr(s_tile);
-#else
     uint32_t tile_end = smem_addr(s_tile) + 16u * (uint32_t)ntiles;
-#endif
     uint32_t mask_step = 4u * kWarps * (uint32_t)ms;                        // bytes between a warp's consecutive tile masks
     keep(tile_end); keep(mask_step);
 
@@ -488,9 +518,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 if (COLW) {
                     uint32_t y;
                     asm("bfind.u32 %0, %1;" : "=r"(y) : "r"(bit));
-                    vi = pos * p.mat_mul + y;
-                } else if (p.lay.msh < p.lay.ysh) {
-                    vi = ((pos >> 1) & ~15u) | (pos & 15u);      // 16 material bytes to 32 occupancy bits
+                    vi = (pos << 3) + y;
                 }
                 asm volatile("{\n"
                     " .reg .pred pv;\n"
@@ -514,12 +542,6 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     : "r"(row), "r"(vi), "f"(t_hit), "r"(abase), "r"(mask_p)
                     : "memory");
             }
-#if MV_PROBE == 9
-            depth = t_hit;
-#endif
-#if MV_PROBE >= 2 && MV_PROBE < 9
-            m = 0;
-#endif
 
             // ---- the less common work, behind one test: boxes binned to this tile (or more than 32 boxes
             // per environment) and the GUI overlay.  A box wins only with a strictly smaller time.
@@ -532,7 +554,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     const float ix = __uint_as_float(__float_as_uint(dtx) | (sgn3 << 31));
                     const float iy = __uint_as_float(__float_as_uint(dty) | ((sgn3 & 2u) << 30));
                     const float iz = __uint_as_float(__float_as_uint(dtz) | ((sgn3 & 4u) << 29));
-                    const uint32_t tab = abase + 48u * sgn3;
+                    const uint32_t tab = abase + 80u * sgn3;
                     uint32_t baddr = 0;
                     for (int w = 0;;) {
                         while (m) {
@@ -605,7 +627,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 :: "r"(rgbx), "f"(depth), "r"(tile_px), "l"(depth_lane), "l"(rgb_lane), "r"(st_sel), "r"(row), "r"(mat_id)
                 : "memory");
         };
-        if (COLW && cam_in && !MV_BRICKS) {
+        if (COLW && cam_in) {
             for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
                 int tile_px;
                 uint32_t pos, bit = 0, row, sgn3;
@@ -629,7 +651,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " ld.shared.f32 Fx, [%10+12];\n"
                     " ld.shared.v4.f32 {Fy, Fz, Rx, Ry}, [%10+16];\n"
                     " ld.shared.v4.f32 {Rz, Ux, Uy, Uz}, [%10+32];\n"
-                    " ld.shared.v4.b32 {bit, esc, %4, pos}, [%10+64];\n"
+                    " ld.shared.v4.b32 {bit, esc, %4, _}, [%10+64];\n"
                     " add.f32 ca, Ta, %11;\n"
                     " sub.f32 cb, Tb, %12;\n"
                     " fma.rn.f32 dx, ca, Rx, Fx;\n"
@@ -652,7 +674,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mov.b32 u, dz;\n"
                     " shr.u32 u, u, 29;\n"
                     " lop3.b32 %8, u, 4, %8, 0xEA;\n"
-                    " mad.lo.u32 tab, %8, 48, %10;\n"
+                    " mad.lo.u32 tab, %8, 80, %10;\n"
                     " ld.shared.v4.b32 {q0, q1, sx, _}, [tab+" MV_TAB_X "];\n"
                     " ld.shared.v4.b32 {q2, q3, sy, _}, [tab+" MV_TAB_Y "];\n"
                     " ld.shared.v4.b32 {q4, q5, sz, _}, [tab+" MV_TAB_Z "];\n"
@@ -664,18 +686,31 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " fma.rn.f32 q5, q5, dtz, tz;\n"
                     " min.f32 q1, q1, q3, q5;\n"
                     " mul.f32 texit, q1, esc;\n"
-#if MV_PROBE >= 1 && MV_PROBE < 9
-                    " mov.f32 texit, 0fFF800000;\n"
-#endif
+                    " ld.shared.v4.b32 {q0, q1, q2, pos}, [tab+" MV_TAB_SKIP "];\n"
+                    " ld.shared.v2.f32 {q3, q4}, [tab+" MV_TAB_SKIP2 "];\n"
+                    " fma.rn.f32 q0, q0, dtx, tx;\n"
+                    " fma.rn.f32 q1, q1, dtz, tz;\n"
+                    " fma.rn.f32 q2, q2, dty, ty;\n"
+                    " min.f32 q0, q0, q1, q2;\n"
+                    " mul.f32 q0, q0, " MV_SKIP_MARGIN ";\n"
+                    " fma.rn.f32 q3, q0, ix, q3;\n"
+                    " fma.rn.f32 q4, q0, iz, q4;\n"
+                    " add.rm.f32 q3, q3, " MV_SKIP_MAGIC ";\n"
+                    " add.rm.f32 q4, q4, " MV_SKIP_MAGIC ";\n"
+                    " mov.b32 u, q3;\n"
+                    " mad.lo.u32 pos, u, sx, pos;\n"
+                    " mov.b32 u, q4;\n"
+                    " mad.lo.u32 pos, u, sz, pos;\n"
+                    " add.f32 q3, q3, " MV_SKIP_UNMAGIC ";\n"
+                    " add.f32 q4, q4, " MV_SKIP_UNMAGIC ";\n"
+                    " fma.rn.f32 tx, q3, dtx, tx;\n"
+                    " fma.rn.f32 tz, q4, dtz, tz;\n"
                     " ld.shared.f32 thit, [%10+48];\n"
                     " mov.s32 it, " MV_STEP_BUDGET ";\n"
                     MV_DDA_LOOP(MV_DDA_STEP_COLW)
                     " @py add.u32 tab, tab, 16;\n"
                     " @pz add.u32 tab, tab, 32;\n"
                     " @ph ld.shared.u32 %4, [tab+" MV_TAB_ROW "];\n"
-#if MV_PROBE == 9
-                    " mov.f32 thit, ns;\n"
-#endif
                     " mov.b32 %1, pos;\n"
                     " mov.b32 %2, bit;\n"
                     " mov.f32 %3, thit;\n"
@@ -713,7 +748,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 const float ix = fast_rcp(dx), iy = fast_rcp(dy), iz = fast_rcp(dz);
                 dtx = fabsf(ix); dty = fabsf(iy); dtz = fabsf(iz);
                 sgn3 = (__float_as_uint(dx) >> 31) | ((__float_as_uint(dy) >> 30) & 2u) | ((__float_as_uint(dz) >> 29) & 4u);
-                const uint32_t tab = abase + 48u * sgn3;
+                const uint32_t tab = abase + 80u * sgn3;
                 float qxx, qxy, qyx, qyy, qzx, qzy;
                 int sx, sy, sz;
                 asm volatile("ld.shared.v4.b32 {%0, %1, %2, _}, [%3+" MV_TAB_X "];" : "=f"(qxx), "=f"(qxy), "=r"(sx) : "r"(tab));
@@ -727,6 +762,17 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     t0y = qyx * dty;
                     t0z = qzx * dtz;
                     t_exit = min3f(fmaf(qxy, dtx, t0x), fmaf(qyy, dty, t0y), fmaf(qzy, dtz, t0z)) * esc;
+                    if (!COLW) {                  // the first stretch, as in the block above
+                        float ex, ez, ey, kx, kz;
+                        uint32_t at;
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4+" MV_TAB_SKIP "];" : "=f"(ex), "=f"(ez), "=f"(ey), "=r"(at) : "r"(tab));
+                        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2+" MV_TAB_SKIP2 "];" : "=f"(kx), "=f"(kz) : "r"(tab));
+                        const float ts = min3f(fmaf(ex, dtx, t0x), fmaf(ez, dtz, t0z), fmaf(ey, dty, t0y)) * kSkipMargin;
+                        const float nx = __fadd_rd(fmaf(ts, fabsf(dx), kx), 8388608.0f), nz = __fadd_rd(fmaf(ts, fabsf(dz), kz), 8388608.0f);
+                        pos = at + __float_as_uint(nx) * (uint32_t)sx + __float_as_uint(nz) * (uint32_t)sz;
+                        t0x = fmaf(nx - 8388608.0f, dtx, t0x);
+                        t0z = fmaf(nz - 8388608.0f, dtz, t0z);
+                    }
                 } else {
                     // eye outside the occupied box: clip the ray to it, start in the entry cell
                     const bool ngx = dx < 0.0f, ngy = dy < 0.0f, ngz = dz < 0.0f;
@@ -762,9 +808,6 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     }
                     if (!alive || filled) t_exit = -kInf;
                 }
-#if MV_PROBE >= 1 && MV_PROBE < 9
-                t_exit = -kInf;
-#endif
 #define MV_DDA_IO                                                                                         \
                     : "+r"(pos), "+r"(bit), "+f"(t_hit), "+r"(row)                                                  \
                     : "f"(t0x), "f"(t0y), "f"(t0z), "f"(dtx), "f"(dty), "f"(dtz), "r"(sx), "r"(sy), "r"(sz), "f"(t_exit), \
@@ -778,61 +821,6 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
 #define MV_DDA_OUTS                                                                                       \
                     " selp.u32 a, 16, 32, py;\n selp.u32 a, 0, a, px;\n add.u32 a, a, %15;\n"                        \
                     " @ph ld.shared.u32 %3, [a+" MV_TAB_ROW "];\n mov.b32 %0, pos;\n mov.b32 %1, bit;\n mov.f32 %2, thit;\n"
-#if MV_BRICKS == 1
-                if (COLW && cam_in) {
-                    // two-level traversal: per brick, its exit time; occupied bricks are walked by the PTX
-                    // loop up to that time, then every axis is advanced past its crossings up to it (one
-                    // crossing after a walked brick, several across an empty one) and the arrival cell tested
-                    const int lgx = 31 - __clz(gx);
-                    const float adx = fabsf(dx), ady = fabsf(dy), adz = fabsf(dz);
-                    const float t_exit_all = t_exit;
-                    for (int guard = 0; guard < 3 * 256 + 8 && row == kNoRow; ++guard) {
-                        const uint32_t col = (pos - occ_base) >> 2;
-                        const int cx = (int)(col & (uint32_t)(gx - 1)), cz = (int)(col >> lgx), cy = 31 - __clz(bit);
-                        const int nbx = (sgn3 & 1u) ? (cx & 3) : 3 - (cx & 3), nby = (sgn3 & 2u) ? (cy & 3) : 3 - (cy & 3);
-                        const int nbz = (sgn3 & 4u) ? (cz & 3) : 3 - (cz & 3);
-                        const float tbk = min3f(fmaf((float)nbx, dtx, t0x), fmaf((float)nby, dty, t0y), fmaf((float)nbz, dtz, t0z));
-                        if ((s_brick[(cx >> 2) + (gx >> 2) * (cz >> 2)] >> (cy >> 2)) & 1u) {
-                            t_exit = fminf(tbk, t_exit_all);
-                            asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_COLW) MV_DDA_OUTS
-                                         " mov.f32 %4, tx;\n mov.f32 %5, ty;\n mov.f32 %6, tz;\n}\n"
-                                         : "+r"(pos), "+r"(bit), "+f"(t_hit), "+r"(row), "+f"(t0x), "+f"(t0y), "+f"(t0z)
-                                         : "f"(dtx), "f"(dty), "f"(dtz), "r"(sx), "r"(sy), "r"(sz), "f"(t_exit), "r"(p.max_steps),
-                                           "r"(tab), "l"(s_occ)
-                                         : "memory");
-                            if (row != kNoRow) break;
-                        }
-                        if (tbk >= t_exit_all) break;
-                        // crossings of each axis up to the brick's exit time (with a tolerance: the exit
-                        // time is a product, the crossing times are sums)
-                        const float tol = fmaf(tbk, 1e-5f, 1e-6f);
-                        const int mx = t0x <= tbk + tol ? (int)floorf(fmaxf(tbk - t0x, 0.0f) * adx + 1e-3f) + 1 : 0;
-                        const int my = t0y <= tbk + tol ? (int)floorf(fmaxf(tbk - t0y, 0.0f) * ady + 1e-3f) + 1 : 0;
-                        const int mz = t0z <= tbk + tol ? (int)floorf(fmaxf(tbk - t0z, 0.0f) * adz + 1e-3f) + 1 : 0;
-                        // nothing to cross: the walk itself took the step out of the brick (its crossing times are
-                        // sums, the brick's exit time a product); look at the new brick
-                        if (mx + my + mz == 0) continue;
-                        // never past the occupied cell box (integer test, so the position stays valid)
-                        const int rx = (sgn3 & 1u) ? cx - lox : hix - 1 - cx, ry = (sgn3 & 2u) ? cy - loy : hiy - 1 - cy;
-                        const int rz = (sgn3 & 4u) ? cz - loz : hiz - 1 - cz;
-                        if (mx > rx || my > ry || mz > rz) break;
-                        t0x = fmaf((float)mx, dtx, t0x); t0y = fmaf((float)my, dty, t0y); t0z = fmaf((float)mz, dtz, t0z);
-                        pos += (uint32_t)(mx * sx + mz * sz);
-                        bit = __funnelshift_l(bit, bit, (uint32_t)(my * sy) & 31u);
-                        if (pos - occ_base >= p.lay.occ_bytes) break;        // (cannot happen; guards the load below)
-                        uint32_t w;
-                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(pos));
-                        if (w & bit) {
-                            t_hit = tbk;
-                            const float lastx = t0x - dtx, lasty = t0y - dty, lastz = t0z - dtz;     // the latest crossing taken
-                            const float lx_ = mx ? lastx : -kInf, ly_ = my ? lasty : -kInf, lz_ = mz ? lastz : -kInf;
-                            const float latest = fmaxf(lx_, fmaxf(ly_, lz_));
-                            asm volatile("ld.shared.u32 %0, [%1+" MV_TAB_ROW "];" : "=r"(row)
-                                         : "r"(tab + (lx_ == latest ? 0u : (ly_ == latest ? 16u : 32u))));
-                        }
-                    }
-                } else
-#endif
                 if constexpr (COLW) {
                     asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_COLW) MV_DDA_OUTS "}\n" MV_DDA_IO);
                 } else if constexpr (OCC_SHARED) {
@@ -843,9 +831,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
 #undef MV_DDA_IO
 #undef MV_DDA_IN
 #undef MV_DDA_OUTS
-#if MV_PROBE != 9
                 if (row == kNoRow) t_hit = kInf;          // no voxel hit
-#endif
                 finish_tile(tile_p, mask_p, tile_px, pos, bit, row, sgn3, t_hit, dtx, dty, dtz);
             }
         }

@@ -760,3 +760,36 @@ def test_upload_packs_every_tile(oracle, grid, palette, envs):
         assert int(counts[e]) == total
         assert (boxes[e, :len(want)].cpu().numpy() == want).all()
     batch.destroy()
+
+
+@pytest.mark.parametrize("grid", [(24, 12, 20), (40, 36, 24), (100, 32, 12)])
+def test_first_stretch_of_a_walk(oracle, grid):
+    """Eyes in empty boxes of every size from a single cell to more than a walk takes at once, at cell centres and exactly
+    on cell faces and edges, close to the grid's border and to its corners; one-word and two-word columns."""
+    gx, gy, gz = grid
+    rng = np.random.default_rng(gx)
+    E = 10
+    g = np.where(rng.random((E, gy, gz, gx)) < 0.25, rng.integers(1, 6, (E, gy, gz, gx)), 0).astype(np.uint8)
+    g[:, 0] = 1
+    cams = []
+    for e in range(E):
+        at = np.array([rng.integers(2, gx - 2), rng.integers(3, min(gy, 12) - 2), rng.integers(2, gz - 2)])
+        if e == 7:
+            at = np.array([1, 2, 1])
+        if e == 8:
+            at = np.array([gx - 2, gy - 3, gz - 2])
+        r = rng.integers(0, 12, 6) if e < 7 else np.array([1, 1, 1, 1, 1, 1])
+        if e == 6:
+            r = np.zeros(6, int)
+        on_face = e in (2, 3, 4)                               # (there the oracle wants the cells next to the face empty)
+        if on_face:
+            r = np.maximum(r, 1)
+        lo, hi = np.maximum(at - r[:3], [0, 1, 0]), at + r[3:] + 1
+        g[e, lo[1]:hi[1], lo[2]:hi[2], lo[0]:hi[0]] = 0
+        p = at + rng.uniform(0.05, 0.95, 3)
+        if on_face:
+            p = np.where([e != 3, False, e != 2], at, p)
+        cams.append(cam_row(*p, rng.uniform(0, 6.28), rng.uniform(-0.5, 0.5)))
+    _, _, status, st = _render_custom(oracle, g, _pal(E, 6), np.stack(cams), 64, 36)
+    assert status == 0
+    parity.assert_parity(st, f"first stretch {grid}")
