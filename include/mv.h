@@ -265,6 +265,49 @@ int mv_step_host(mv_batch *batch, const mv_camera *h_cams, const mv_box *h_boxes
 int mv_step_host_static(mv_batch *batch, const mv_camera *h_cams, uint8_t *h_rgb, float *h_depth,
                         void *cuda_stream);
 
+/* Seeded synthetic scenes (the package's generator; no counterpart in the paper, whose layouts are not published).  An
+ * upload wants worlds that exist already; a program without a simulator of its own makes them with these two calls.
+ * The arrays are those of the package's Python generator, bit for bit. */
+typedef struct mv_scene_desc {
+    uint64_t seed;
+    int32_t world;                      /* 0 wall segments, 1 rooms, 2 columns */
+    int32_t grid_x, grid_y, grid_z;     /* as in mv_batch_desc */
+    int32_t palette_size;
+    int32_t count;                      /* rectangles (segments, columns), or wall lines per axis (rooms; up to 1024) */
+    int32_t line_pitch, pillars;        /* rooms only */
+    int32_t agents, movable_boxes;
+    int32_t body_boxes;                 /* != 0: a box per agent after the movable ones */
+    int32_t step;                       /* which of the seeded camera placements */
+    int32_t cam_y_is_fixed;             /* != 0: eyes at cam_y above the column's own height */
+    float cam_y;
+} mv_scene_desc;
+
+/* Worlds of the scene ids d_env_ids.
+ *   desc        HOST pointer       d_env_ids  DEVICE int64 [env_count]
+ *   d_grid      DEVICE uint8 [env_count][grid_y][grid_z][grid_x]      d_palette  DEVICE uint8 [env_count][palette_size][3]
+ *   d_height    DEVICE int64 [env_count][grid_z][grid_x], height of the solid stack over the floor layer
+ * Errors: INVALID_ARG, CUDA. */
+int mv_scene_worlds(const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, uint8_t *d_grid,
+                    uint8_t *d_palette, int64_t *d_height, int device, void *cuda_stream);
+
+/* Movable boxes, cameras and bodies for the same ids and the heights of their worlds.
+ *   d_slots     DEVICE int32 [env_count] or NULL: env i's cameras go to d_cams[slots[i]] (NULL: to d_cams[i])
+ *   d_boxes     DEVICE mv_box [env_count][movable_boxes + (body_boxes ? agents : 0)]   d_box_count  DEVICE int32 [env_count]
+ *   d_cams      DEVICE mv_camera [...][agents]
+ * Errors: INVALID_ARG, CUDA. */
+int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int64_t *d_height,
+                      const int32_t *d_slots, mv_box *d_boxes, int32_t *d_box_count, mv_camera *d_cams, int device,
+                      void *cuda_stream);
+
+/* One step of the batch's episode clocks (paper Appendix A.1: episodes end on their own; A.2: time-left bar).  With
+ * advance != 0: t += 1; where t >= length, done = 1, t = 0 and episode += 1.  Then, if bar_rows > 0, every agent's overlay
+ * becomes one bar: bar_rows rows, width * (length - t) / length pixels.
+ *   d_t, d_episode, d_length  DEVICE int64 [num_envs]     d_done  DEVICE uint8 [num_envs], needed when advance != 0
+ *   bar_rgb     HOST uint8 [3]
+ * Errors: INVALID_ARG (bars without max_overlay_rects), CUDA. */
+int mv_advance_episodes(mv_batch *batch, int64_t *d_t, int64_t *d_episode, const int64_t *d_length, uint8_t *d_done,
+                        int advance, int bar_rows, const uint8_t *bar_rgb, void *cuda_stream);
+
 /* Synchronise the stream and return the device status word: a negative mv_status if a CUDA
  * error or device timeout occurred, else the OR of the MV_FLAG_* bits seen so far (0 = clean).
  * clear != 0 resets the sticky bits. */

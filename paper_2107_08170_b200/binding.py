@@ -16,7 +16,7 @@ _lib = None
 MV_OK = 0
 FLAG_MATERIAL_CLAMPED, FLAG_BOX_COUNT_CLAMPED, FLAG_BAD_CAMERA, FLAG_DEVICE_TIMEOUT = 1, 2, 4, 8
 EXPORTS = ["mv_create_batch", "mv_upload_worlds", "mv_upload_worlds_at", "mv_set_cameras", "mv_render_batch", "mv_step_host",
-           "mv_step_host_static", "mv_set_overlays", "mv_move_agents", "mv_merge_voxels", "mv_debug_staging", "mv_debug_occupancy_in_global", "mv_debug_agents_per_cta", "mv_query_status", "mv_launch_count", "mv_destroy", "mv_status_string"]
+           "mv_step_host_static", "mv_set_overlays", "mv_move_agents", "mv_merge_voxels", "mv_scene_worlds", "mv_scene_entities", "mv_advance_episodes", "mv_debug_staging", "mv_debug_occupancy_in_global", "mv_debug_agents_per_cta", "mv_query_status", "mv_launch_count", "mv_destroy", "mv_status_string"]
 
 
 class BatchDesc(C.Structure):
@@ -26,6 +26,13 @@ class BatchDesc(C.Structure):
                 ("palette_size", C.c_int32), ("hfov_rad", C.c_float), ("light_dir", C.c_float * 3),
                 ("ambient", C.c_float), ("sky_rgb", C.c_uint8 * 3), ("pad", C.c_uint8),
                 ("miss_depth", C.c_float), ("device", C.c_int32), ("max_overlay_rects", C.c_int32)]
+
+
+class SceneDesc(C.Structure):
+    _fields_ = [("seed", C.c_uint64), ("world", C.c_int32), ("grid_x", C.c_int32), ("grid_y", C.c_int32),
+                ("grid_z", C.c_int32), ("palette_size", C.c_int32), ("count", C.c_int32), ("line_pitch", C.c_int32),
+                ("pillars", C.c_int32), ("agents", C.c_int32), ("movable_boxes", C.c_int32), ("body_boxes", C.c_int32),
+                ("step", C.c_int32), ("cam_y_is_fixed", C.c_int32), ("cam_y", C.c_float)]
 
 
 class MvError(RuntimeError):
@@ -53,6 +60,9 @@ def lib() -> C.CDLL:
         L.mv_set_overlays.argtypes = [vp, vp, vp, vp]
         L.mv_move_agents.argtypes = [vp, vp, vp, vp, vp]
         L.mv_merge_voxels.argtypes = [vp, i, i, vp, vp, i, vp]
+        L.mv_scene_worlds.argtypes = [C.POINTER(SceneDesc), vp, i, vp, vp, vp, i, vp]
+        L.mv_scene_entities.argtypes = [C.POINTER(SceneDesc), vp, i, vp, vp, vp, vp, vp, i, vp]
+        L.mv_advance_episodes.argtypes = [vp, vp, vp, vp, vp, i, i, vp, vp]
         L.mv_debug_staging.argtypes = [vp, i, i]
         L.mv_debug_occupancy_in_global.argtypes = [vp, i]
         L.mv_debug_agents_per_cta.argtypes = [vp, i]
@@ -132,6 +142,21 @@ def _stream(stream):
     return C.c_void_p(stream.cuda_stream)
 
 
+def scene_worlds(desc: SceneDesc, env_ids, grid, palette, height):
+    """Worlds of the seeded ids `env_ids` (CUDA int64) into the given CUDA arrays, on the current stream."""
+    _check(lib().mv_scene_worlds(C.byref(desc), _dptr(env_ids, torch.int64), env_ids.numel(), _dptr(grid, torch.uint8),
+                                 _dptr(palette, torch.uint8), _dptr(height, torch.int64), grid.device.index,
+                                 _stream(torch.cuda.current_stream(grid.device))), "mv_scene_worlds")
+
+
+def scene_entities(desc: SceneDesc, env_ids, height, boxes, box_count, cams, slots=None):
+    """Boxes and cameras of the same ids; env i's cameras go to row slots[i] (default i) of `cams`."""
+    _check(lib().mv_scene_entities(C.byref(desc), _dptr(env_ids, torch.int64), env_ids.numel(), _dptr(height, torch.int64),
+                                   _dptr(slots, torch.int32), _dptr(boxes, torch.int32), _dptr(box_count, torch.int32),
+                                   _dptr(cams, torch.int32), height.device.index,
+                                   _stream(torch.cuda.current_stream(height.device))), "mv_scene_entities")
+
+
 class Batch:
     """Handle to one mv_batch.  Methods mirror the C entry points one to one."""
 
@@ -188,6 +213,13 @@ class Batch:
         _check(lib().mv_merge_voxels(self._h, env_begin, env_count, _dptr(boxes), _dptr(counts), max_out,
                                      _stream(stream)), "mv_merge_voxels")
         return boxes, counts
+
+    def advance_episodes(self, t, episode, length, done=None, bar_rows=0, bar_rgb=(0, 0, 0), stream=None):
+        """Episode clocks one step on (done, CUDA bool [num_envs], is written) or, without `done`, as they are; then the
+        time-left bars if bar_rows > 0.  t, episode, length: CUDA int64 [num_envs]."""
+        _check(lib().mv_advance_episodes(self._h, _dptr(t, torch.int64), _dptr(episode, torch.int64), _dptr(length, torch.int64),
+                                         _dptr(done, torch.bool), int(done is not None), bar_rows, bytes(bar_rgb),
+                                         _stream(stream)), "mv_advance_episodes")
 
     def step_host_static(self, cams, rgb, depth, stream=None):
         """The never-allocating host step (fixed 8 MiB device array inside the library): for callers

@@ -6,6 +6,7 @@
 #include "mv_pack.cuh"
 #include "mv_merge.cuh"
 #include "mv_render.cuh"
+#include "mv_scene.cuh"
 
 #include <cmath>
 #include <cstdio>
@@ -312,6 +313,23 @@ int static_scratch_for_device(mv_batch *b, int device, unsigned char **out) {
 }  // namespace
 
 namespace {
+// Checks a scene descriptor and spells it out for the kernels.
+bool scene_args(const mv_scene_desc *d, const int64_t *d_env_ids, int env_count, SceneArgs *a) {
+    auto dim_ok = [](int g) { return g >= 4 && g <= 1024 && (g % 4) == 0; };
+    if (!d || !d_env_ids || env_count < 0 || d->world < 0 || d->world > 2 || !dim_ok(d->grid_x) || !dim_ok(d->grid_y) ||
+        !dim_ok(d->grid_z) || d->palette_size < 1 || d->palette_size > 256 || d->count < 0 || d->count > (d->world == 1 ? 1024 : 1 << 24) ||
+        d->line_pitch < 0 || d->line_pitch > 1024 || d->pillars < 0 || d->pillars > 1 << 24 || d->agents < 1 || d->agents > 1 << 16 ||
+        d->movable_boxes < 0 || d->movable_boxes > 1 << 16 || d->step < 0 ||
+        (int64_t)env_count * d->grid_x * d->grid_z / 4 > (1ll << 38) || (int64_t)env_count * (d->world == 1 ? 1 : d->count) > (1ll << 38))
+        return false;
+    *a = SceneArgs{};
+    a->seed = d->seed; a->world = d->world; a->gx = d->grid_x; a->gy = d->grid_y; a->gz = d->grid_z; a->palette = d->palette_size;
+    a->count = d->count; a->pitch = d->line_pitch; a->pillars = d->pillars; a->agents = d->agents; a->boxes = d->movable_boxes;
+    a->bodies = d->body_boxes ? 1 : 0; a->max_boxes = d->movable_boxes + (d->body_boxes ? d->agents : 0); a->step = d->step;
+    a->cam_y_is_fixed = d->cam_y_is_fixed ? 1 : 0; a->cam_y = d->cam_y; a->env_count = env_count; a->env = d_env_ids;
+    return true;
+}
+
 // Body of both upload entry points.  h_env_index: null for the contiguous range that starts at
 // env_begin, else the (validated) destination env of each uploaded env.
 int upload_worlds(mv_batch *b, int env_begin, const int32_t *h_env_index, int env_count, const uint8_t *d_grid,
@@ -677,6 +695,63 @@ int mv_step_host_static(mv_batch *b, const mv_camera *h_cams, uint8_t *h_rgb, fl
     MV_CUDA(b, cudaMemcpyAsync(h_rgb, d_rgb, O * px * 3, cudaMemcpyDeviceToHost, s));
     MV_CUDA(b, cudaMemcpyAsync(h_depth, d_depth, O * px * 4, cudaMemcpyDeviceToHost, s));
     return finish_host_step(b, s);
+}
+
+int mv_scene_worlds(const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, uint8_t *d_grid,
+                    uint8_t *d_palette, int64_t *d_height, int device, void *cuda_stream) {
+    SceneArgs a;
+    if (!scene_args(desc, d_env_ids, env_count, &a) || !d_grid || !d_palette || !d_height || !aligned16(d_height) || !aligned16(d_grid))
+        return MV_ERR_INVALID_ARG;
+    if (env_count == 0) return MV_OK;
+    DeviceGuard g(device);
+    if (!g.ok) return MV_ERR_CUDA;
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    auto ctas = [](size_t threads) { return (threads + kSceneThreads - 1) / kSceneThreads; };
+    const size_t cells = (size_t)a.gx * a.gz;
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(d_height);
+    if (a.world == kWorldRooms) {
+        scene_rooms_kernel<<<env_count, kSceneThreads, (4 * (size_t)a.count + a.gx + a.gz) * 4, s>>>(a, keys);
+    } else {
+        MV_CUDA(nullptr, cudaMemsetAsync(keys, 0, env_count * cells * 8, s));
+        if (a.count > 0) scene_rects_kernel<<<(unsigned)ctas((size_t)env_count * a.count), kSceneThreads, 0, s>>>(a, keys);
+    }
+    MV_CUDA(nullptr, cudaGetLastError());
+    const size_t columns = ctas(env_count * cells / 4), colours = ctas((size_t)env_count * 3 * a.palette);
+    scene_expand_kernel<<<(unsigned)(columns + colours), kSceneThreads, 0, s>>>(a, keys, d_grid, d_palette, (long long)columns);
+    MV_CUDA(nullptr, cudaGetLastError());
+    return MV_OK;
+}
+
+int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int64_t *d_height,
+                      const int32_t *d_slots, mv_box *d_boxes, int32_t *d_box_count, mv_camera *d_cams, int device,
+                      void *cuda_stream) {
+    SceneArgs a;
+    if (!scene_args(desc, d_env_ids, env_count, &a) || !d_height || !d_box_count || !d_cams || (a.max_boxes > 0 && !d_boxes))
+        return MV_ERR_INVALID_ARG;
+    if (env_count == 0) return MV_OK;
+    DeviceGuard g(device);
+    if (!g.ok) return MV_ERR_CUDA;
+    scene_entities_kernel<<<env_count, kSceneThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+        a, reinterpret_cast<const long long *>(d_height), d_slots, reinterpret_cast<uint32_t *>(d_boxes), d_box_count,
+        reinterpret_cast<uint32_t *>(d_cams));
+    MV_CUDA(nullptr, cudaGetLastError());
+    return MV_OK;
+}
+
+int mv_advance_episodes(mv_batch *b, int64_t *d_t, int64_t *d_episode, const int64_t *d_length, uint8_t *d_done, int advance,
+                        int bar_rows, const uint8_t *bar_rgb, void *cuda_stream) {
+    if (!b || !d_t || !d_episode || !d_length || (advance && !d_done) || bar_rows < 0 || bar_rows > 4096 ||
+        (bar_rows > 0 && (!bar_rgb || b->desc.max_overlay_rects == 0)))
+        return MV_ERR_INVALID_ARG;
+    DeviceGuard g(b->desc.device);
+    if (!g.ok) return MV_ERR_CUDA;
+    const uint32_t rgb = bar_rows > 0 ? (uint32_t)bar_rgb[0] | (uint32_t)bar_rgb[1] << 8 | (uint32_t)bar_rgb[2] << 16 : 0u;
+    episode_clocks_kernel<<<(b->desc.num_envs + 127) / 128, 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+        d_t, d_episode, d_length, d_done, b->desc.num_envs, b->desc.agents_per_env, advance ? 1 : 0, b->desc.width, bar_rows, rgb,
+        bar_rows > 0 ? b->d_overlay : nullptr, b->d_overlay_count, b->desc.max_overlay_rects);
+    b->launches++;
+    MV_CUDA(b, cudaGetLastError());
+    return MV_OK;
 }
 
 int mv_query_status(mv_batch *b, int clear, void *cuda_stream) {

@@ -8,7 +8,8 @@ whose generators are not published in the paper text.
 
 Everything is derived from a counter-based integer hash (a splitmix64-style finaliser on
 int64 tensors), so a generator gives the same arrays on the CPU and on a CUDA device and
-any environment range can be generated on its own (chunked generation of large batches).
+any environment range can be generated on its own (chunked generation of large batches).  CUDA arrays come from
+the library's kernels, which give the same bits as the torch code below; that code serves the CPU.
 
 Array conventions (these are the C ABI's conventions, see include/mv.h):
   grid     uint8  [E][gy][gz][gx]   material id per voxel, 0 = empty, x fastest
@@ -129,6 +130,53 @@ def config(name: str, **over) -> SceneConfig:
     return SceneConfig(name=name, **kw)
 
 
+# --------------------------------------------------------------------------- on the device
+
+_WORLDS = {"segments": 0, "rooms": 1, "columns": 2}
+
+
+def _native_desc(cfg: SceneConfig, step: int = 0):
+    """The configuration as the CUDA library's generator takes it, or None where it does not."""
+    gx, gy, gz = cfg.grid
+    counts = {"rooms": {"n_lines", "pitch", "n_pillars"}}.get(cfg.world, {"n_rects"})
+    if cfg.world not in _WORLDS or not set(cfg.extra) <= counts or any(g % 4 or not 4 <= g <= 1024 for g in cfg.grid) \
+            or not 1 <= cfg.palette_size <= 256 or cfg.extra.get("n_lines", 6) > 1024 or step < 0:
+        return None
+    from . import binding
+    d = binding.SceneDesc()
+    d.seed, d.world, (d.grid_x, d.grid_y, d.grid_z) = cfg.seed & _MASK64, _WORLDS[cfg.world], cfg.grid
+    d.palette_size, d.agents, d.movable_boxes, d.body_boxes = cfg.palette_size, cfg.agents, cfg.movable_boxes, int(cfg.body_boxes)
+    if cfg.world == "rooms":
+        d.count, d.line_pitch, d.pillars = cfg.extra.get("n_lines", 6), cfg.extra.get("pitch", 9), cfg.extra.get("n_pillars", 24)
+    else:
+        d.count = cfg.extra.get("n_rects", 9 if cfg.world == "segments" else 1050)
+    d.step, d.cam_y_is_fixed, d.cam_y = step, int(cfg.cam_y_fixed is not None), cfg.cam_y_fixed or 0.0
+    return d
+
+
+def _native_worlds(cfg: SceneConfig, desc, env: torch.Tensor):
+    from . import binding
+    gx, gy, gz = cfg.grid
+    E, dev = env.numel(), env.device
+    grid = torch.empty(E, gy, gz, gx, dtype=torch.uint8, device=dev)
+    palette = torch.empty(E, cfg.palette_size, 3, dtype=torch.uint8, device=dev)
+    height = torch.empty(E, gz, gx, dtype=torch.int64, device=dev)
+    binding.scene_worlds(desc, env.contiguous(), grid, palette, height)
+    return {"grid": grid, "palette": palette, "height": height, "env": env}
+
+
+def _native_entities(cfg: SceneConfig, desc, env: torch.Tensor, height: torch.Tensor, cams=None, slots=None):
+    """With `cams` and `slots` (CUDA int32) the cameras go straight to those environments' rows of an existing array."""
+    from . import binding
+    E, dev = env.numel(), env.device
+    boxes = torch.empty(E, cfg.max_boxes, 8, dtype=torch.int32, device=dev)
+    count = torch.empty(E, dtype=torch.int32, device=dev)
+    if cams is None:
+        cams = torch.empty(E * cfg.agents, 6, dtype=torch.int32, device=dev)
+    binding.scene_entities(desc, env.contiguous(), height.contiguous(), boxes, count, cams, slots)
+    return {"boxes": boxes, "box_count": count, "cams": cams}
+
+
 # --------------------------------------------------------------------------- worlds
 
 def _scatter_rects(rng: Rng, stream: int, env: torch.Tensor, n_rects: int, gx: int, gz: int,
@@ -241,6 +289,8 @@ def make_worlds(cfg: SceneConfig, env_begin: int = 0, env_count: int | None = No
     else:
         env_count = cfg.num_envs - env_begin if env_count is None else env_count
         env = torch.arange(env_begin, env_begin + env_count, device=rng.device)
+    if env.is_cuda and (desc := _native_desc(cfg)) is not None:
+        return _native_worlds(cfg, desc, env)
     gx, gy, gz = cfg.grid
     P = cfg.palette_size
     if cfg.world == "rooms":
@@ -274,6 +324,8 @@ def make_boxes_and_cameras(cfg: SceneConfig, worlds: dict, step: int = 0):
     dev = rng.device
     env = worlds["env"]
     height = worlds["height"]                       # solid cells above the floor layer
+    if height.is_cuda and (desc := _native_desc(cfg, step)) is not None:
+        return _native_entities(cfg, desc, env, height)
     E = env.numel()
     gx, gy, gz = cfg.grid
     P = cfg.palette_size

@@ -288,3 +288,21 @@ def test_merge_voxels_grid_shapes(oracle, grid, kind, palette):
         assert int(counts[e]) == total, (grid, kind, e)
         assert (boxes[e, :len(want)].cpu().numpy() == want).all(), (grid, kind, e)
     batch.destroy()
+
+
+@pytest.mark.parametrize("world,grid,extra", [("rooms", (16, 16, 16), {"n_lines": 1, "n_pillars": 3}), ("rooms", (192, 20, 44), {"n_lines": 3}),
+                                              ("columns", (20, 12, 128), {"n_rects": 160}), ("segments", (16, 4, 24), {})])
+def test_scene_kernels_give_the_generators_arrays(world, grid, extra):
+    """The device generator against the CPU one where it can go wrong: few cells, ragged grids, no boxes, more agents than
+    a round takes, one material, later steps, scattered scene ids."""
+    for seed, palette, nb, agents, bodies in ((3, 1, 0, 1, False), (-5, 17, 70, 9, True), (1 << 40, 256, 300, 2, True)):
+        cfg = scenes.SceneConfig(name="x", num_envs=5, agents=agents, grid=grid, width=8, height=4, palette_size=palette, world=world,
+                                 movable_boxes=nb, body_boxes=bodies, cam_y_fixed=1.5 if palette == 17 else None, seed=seed, extra=extra)
+        ids = torch.tensor([7, 0, 123456789, 4])
+        for step in (0, 3):
+            out = []
+            for dev in ("cpu", "cuda"):
+                w = scenes.make_worlds(cfg, device=dev, env_ids=ids)
+                out.append({**w, **scenes.make_boxes_and_cameras(cfg, w, step)})
+            for k, v in out[0].items():
+                assert v.dtype == out[1][k].dtype and torch.equal(v, out[1][k].cpu()), (world, seed, step, k)
