@@ -116,14 +116,16 @@ def desc_from_config(cfg, device=0, max_overlay_rects=0) -> BatchDesc:
                      cfg.miss_depth, device, max_overlay_rects)
 
 
+# (Small batches wait for this file, not for the GPU: pointers go to ctypes as plain integers, and the current stream's
+# handle is asked for without building a Stream object, which costs 3 us.)
 def _dptr(t, dtype=None):
     if t is None:
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise ValueError(f"expected dtype {dtype}, got {t.dtype}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _hptr(t, dtype=None):
@@ -131,15 +133,25 @@ def _hptr(t, dtype=None):
         return None
     if t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CPU tensor")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise ValueError(f"expected dtype {dtype}, got {t.dtype}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+_initialized = False
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    global _initialized
+    if stream is not None:
+        return stream.cuda_stream
+    if _initialized:
+        return _raw_stream(_device())
+    handle = torch.cuda.current_stream().cuda_stream          # (sets torch's CUDA state up on its first use)
+    _initialized = _raw_stream is not None and _device is not None
+    return handle
 
 
 def scene_worlds(desc: SceneDesc, env_ids, grid, palette, height):

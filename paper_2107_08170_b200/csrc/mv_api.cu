@@ -104,12 +104,12 @@ int cuda_fail(mv_batch *b, cudaError_t e) {
 
 struct DeviceGuard {
     int prev = -1;
-    bool ok = false;
+    bool ok = false, changed = false;
     explicit DeviceGuard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) return;
-        ok = (prev == dev) || (cudaSetDevice(dev) == cudaSuccess);
+        ok = prev == dev || (changed = cudaSetDevice(dev) == cudaSuccess);
     }
-    ~DeviceGuard() { if (ok && prev >= 0) cudaSetDevice(prev); }
+    ~DeviceGuard() { if (changed) cudaSetDevice(prev); }
 };
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
