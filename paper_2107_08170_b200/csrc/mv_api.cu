@@ -27,6 +27,10 @@ constexpr int kRenderThreadsSmall = MV_NT / 2; // ...and for CTAs with few tiles
 // (measured: 64x36 images +10 %; 128x72 -2 %; four CTAs alone on the GPU -20 %: fewer warps per CTA, longer CTA).
 constexpr int kSmallCtaTiles = 192;
 constexpr int kHostChunks = 8;
+// CTAs that split the tiles of an observation between them, when the occupancy is not staged: enough to fill the GPU twice
+// (512 observations of 128x72 on 192x48x192: 112, 109, 115, 127 us with 1, 2, 4, 8 times); staged: once, as each one stages
+// the block again (4 of 64x36: 20.6 us with a CTA each, 12 with 6).
+constexpr int kPartWaves = 2;
 // Staging + set-up of a CTA, in units of one observation's render time, as measured on B200 at 128x72:
 // 0.15 to 0.18 for 64x16x64 grids, 0.10 for 128x32x128 grids (where a second agent's tables usually cost
 // the third resident CTA per SM, which the occupancy query below sees).
@@ -63,7 +67,7 @@ struct mv_batch {
     bool has_cams = false;
     double kr = 0, ku = 0;
     uint32_t sky_rgbx = 0;
-    struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, agent_ovtile_off, misc_off, bytes; };
+    struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, agent_ovtile_off, agent_near_off, misc_off, bytes; };
     Smem smem{};                        // shared-memory layout of the render kernel for agents_per_cta
     int agents_per_cta = 1;             // observations one CTA renders: 1, or every agent of its env
     int threads = MV_NT;                // threads per CTA of the render kernel (fewer for CTAs with few tiles)
@@ -115,21 +119,27 @@ struct DeviceGuard {
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Shared-memory layout of the render kernel when one CTA renders `apc` observations of an env:
-// staged env block, tile table, then one block per agent (camera record and DDA start table,
+// staged env block (without the occupancy when that stays in global memory), tile table, then one block per agent (camera record and DDA start table,
 // eye-relative boxes, overlay rectangles, per-tile box masks, per-tile overlay bits), then the
 // barrier and flag words.
-mv_batch::Smem smem_layout(const mv_batch *b, int apc) {
+mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     const mv_batch_desc &d = b->desc;
     const uint32_t ntiles = (uint32_t)(b->tiles_x * b->tiles_y);
     mv_batch::Smem m{};
-    m.tile_off = round_up(b->lay.block_bytes, 16);
+    m.tile_off = round_up(b->lay.block_bytes - (occ_shared ? 0u : b->lay.occ_bytes), 16);
     m.agent_off = m.tile_off + ntiles * 16;
     m.agent_ov_off = kAgentRelOff + (uint32_t)(d.max_boxes > 0 ? d.max_boxes : 1) * 32;
     m.agent_mask_off = m.agent_ov_off + (uint32_t)(d.max_overlay_rects > 0 ? d.max_overlay_rects : 1) * 32;
     // per tile: the box-mask words, preceded by a summary word when there is more than one
     const uint32_t words_per_tile = b->mask_words > 1 ? (uint32_t)b->mask_words + 1 : 1u;
     m.agent_ovtile_off = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
-    m.agent_stride = m.agent_ovtile_off + round_up(((ntiles + 31) / 32) * 4, 16);
+    m.agent_near_off = m.agent_ovtile_off + round_up(((ntiles + 31) / 32) * 4, 16);
+    m.agent_stride = m.agent_near_off;
+    if (!occ_shared) {                  // the columns around the eye, if there is room for them
+        const uint32_t near_bytes = round_up((2 * kSkipCells + 1) * (2 * kSkipCells + 1) * 4, 16);
+        if ((int64_t)m.agent_off + (int64_t)apc * (m.agent_stride + near_bytes) + 32 <= b->smem_max) m.agent_stride += near_bytes;
+        else m.agent_near_off = 0;
+    }
     m.misc_off = m.agent_off + (uint32_t)apc * m.agent_stride;
     m.bytes = m.misc_off + 32;
     return m;
@@ -141,6 +151,17 @@ int pick_threads(const mv_batch *b, int apc) {
     const bool few_tiles = b->tiles_x * b->tiles_y * apc < kSmallCtaTiles;
     const bool fills = (int64_t)b->num_obs / apc >= (int64_t)6 * b->sms;
     return few_tiles && fills ? kRenderThreadsSmall : kRenderThreads;
+}
+
+// CTAs per observation (or environment) in a batch with few of them: as many as fill the GPU kPartWaves times over, but
+// each with a tile for every warp.
+int pick_parts(const mv_batch *b, int64_t ctas) {
+    const int per_sm = b->threads == kRenderThreads ? 3 : 6;
+    const int64_t slots = (int64_t)per_sm * b->sms * (b->occ_shared ? 1 : kPartWaves);
+    const int64_t most = b->tiles_x * b->tiles_y / (b->threads / 32);
+    int64_t parts = slots / ctas;
+    parts = parts > most ? most : parts;
+    return parts < 1 ? 1 : (int)parts;
 }
 
 // The three instantiations of the render kernel: column-word walk (grid at most 32 high, occupancy
@@ -178,11 +199,9 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.tiles_x = b->tiles_x; p.tiles_y = b->tiles_y; p.mask_words = b->mask_words;
     p.sky_rgbx = b->sky_rgbx;
     p.miss_depth = b->desc.miss_depth;
-    const uint32_t unstaged = b->occ_shared ? 0u : b->lay.occ_bytes;   // shared-memory offsets shift down by it
-    p.smem_tile_off = b->smem.tile_off - unstaged; p.smem_agent_off = b->smem.agent_off - unstaged;
-    p.smem_misc_off = b->smem.misc_off - unstaged;
+    p.smem_tile_off = b->smem.tile_off; p.smem_agent_off = b->smem.agent_off; p.smem_misc_off = b->smem.misc_off;
     p.agent_stride = b->smem.agent_stride; p.agent_ov_off = b->smem.agent_ov_off;
-    p.agent_mask_off = b->smem.agent_mask_off; p.agent_ovtile_off = b->smem.agent_ovtile_off;
+    p.agent_mask_off = b->smem.agent_mask_off; p.agent_ovtile_off = b->smem.agent_ovtile_off; p.agent_near_off = b->smem.agent_near_off;
     p.agents_per_cta = b->agents_per_cta;
     p.max_steps = b->desc.grid_x + b->desc.grid_y + b->desc.grid_z + 3;
     // accumulated crossing times drift from the exact products by at most one rounding per step
@@ -192,8 +211,10 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.max_overlay = b->desc.max_overlay_rects;
     p.wait_polls = b->wait_polls;
     p.skip_staging = b->skip_staging;
-    const int ctas = obs_count / b->agents_per_cta;   // callers pass whole environments when a CTA renders one
-    render_fn(b)<<<ctas, b->threads, b->smem.bytes - unstaged, s>>>(p);
+    const int64_t ctas = obs_count / b->agents_per_cta;   // callers pass whole environments when a CTA renders one
+    const int ntiles = b->tiles_x * b->tiles_y, parts = pick_parts(b, ctas);
+    p.part_tiles = (ntiles + parts - 1) / parts;
+    render_fn(b)<<<dim3((unsigned)ctas, (unsigned)((ntiles + p.part_tiles - 1) / p.part_tiles)), b->threads, b->smem.bytes, s>>>(p);
     b->launches++;
     MV_CUDA(b, cudaGetLastError());
     return MV_OK;
@@ -413,7 +434,6 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     b->tiles_x = d.width / 8;
     b->tiles_y = d.height / 4;
     b->mask_words = d.max_boxes > 0 ? (d.max_boxes + 31) / 32 : 1;
-    b->smem = smem_layout(b, 1);
 
     // kr = tan(hfov/2)/W, ku = (tan(hfov/2)*H/W)/H in double (scalar set-up for the camera kernel)
     const double tx = std::tan((double)d.hfov_rad / 2.0);
@@ -434,9 +454,9 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     b->smem_max = smem_max;
     // the occupancy normally rides in shared memory with the rest of the env block; a grid too large
     // for that keeps it in global memory and stages only the block's tail
-    b->occ_fits_shared = (int)b->smem.bytes <= smem_max;
-    b->occ_shared = b->occ_fits_shared;
-    if ((int)(b->smem.bytes - L.occ_bytes) > smem_max) { delete b; return MV_ERR_UNSUPPORTED; }
+    b->occ_fits_shared = b->occ_shared = (int64_t)smem_layout(b, 1, true).bytes <= smem_max;
+    b->smem = smem_layout(b, 1, b->occ_shared);
+    if ((int64_t)b->smem.bytes > smem_max) { delete b; return MV_ERR_UNSUPPORTED; }
     // The dynamic shared-memory cap is a property of the kernel function on this device, shared by
     // every batch: raise it to the device's maximum once, never to one batch's own size.
     for (RenderFn f : {RenderFn(render_kernel<kRenderThreads, true, true>), RenderFn(render_kernel<kRenderThreads, true, false>),
@@ -449,13 +469,11 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     // One CTA per environment (block staged once for all its agents) when that still fills the GPU;
     // otherwise one CTA per observation.  Cost model: waves of resident CTAs x (agents + fixed part).
     if (d.agents_per_env > 1) {
-        const mv_batch::Smem all = smem_layout(b, d.agents_per_env);
-        const uint32_t unstaged = b->occ_shared ? 0u : L.occ_bytes;   // never give up staged occupancy for it
-        if ((int)(all.bytes - unstaged) <= smem_max) {
+        const mv_batch::Smem all = smem_layout(b, d.agents_per_env, b->occ_shared);    // (never give up staged occupancy for it)
+        if ((int64_t)all.bytes <= smem_max) {
             auto waves_cost = [&](const mv_batch::Smem &m, int apc) {
                 int per_sm = 0;
-                cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_fn(b), kRenderThreads,
-                                                                              m.bytes - unstaged);
+                cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_fn(b), kRenderThreads, m.bytes);
                 if (q != cudaSuccess || per_sm < 1) return 1e30;
                 const double slots = (double)per_sm * sms, ctas = (double)b->num_obs / apc;
                 return std::ceil(ctas / slots) * (apc + kCtaFixedCost);
@@ -773,6 +791,7 @@ int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     if (!b) return MV_ERR_INVALID_ARG;
     if (!on && !b->occ_fits_shared) return MV_ERR_UNSUPPORTED;
     b->occ_shared = !on;
+    b->smem = smem_layout(b, b->agents_per_cta, b->occ_shared);
     return MV_OK;
 }
 
@@ -781,11 +800,10 @@ int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {
     const int A = b->desc.agents_per_env;
     int apc = agents_per_cta == 0 ? b->auto_agents_per_cta : agents_per_cta;
     if (apc != 1 && apc != A) return MV_ERR_INVALID_ARG;
-    const mv_batch::Smem m = smem_layout(b, apc);
-    if ((int)(m.bytes - b->lay.occ_bytes) > b->smem_max) return MV_ERR_UNSUPPORTED;
-    b->occ_fits_shared = (int)m.bytes <= b->smem_max;
+    if ((int64_t)smem_layout(b, apc, false).bytes > b->smem_max) return MV_ERR_UNSUPPORTED;
+    b->occ_fits_shared = (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max;
     if (!b->occ_fits_shared) b->occ_shared = false;
-    b->smem = m;
+    b->smem = smem_layout(b, apc, b->occ_shared);
     b->agents_per_cta = apc;
     b->threads = pick_threads(b, apc);
     return MV_OK;

@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int apc = p.agents_per_cta;
+    constexpr int kWarps = NT / 32;
     const int obs0 = p.obs_begin + blockIdx.x * apc;
     const int env = p.agents == 1 ? obs0 : obs0 / p.agents;
     const int W = p.W, H = p.H;
@@ -200,6 +201,9 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     auto agent_ovtile = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_ovtile_off); };
     const int ovt_words = (ntiles + 31) / 32;
 
+    // (in a batch with few observations each one's tiles are split between the CTAs of a grid column)
+    const int tile0 = blockIdx.y * p.part_tiles, tile1 = min(tile0 + p.part_tiles, ntiles);
+
     // ---- stage the environment block
     if (tid == 0) mbar_init(s_bar, 1);
     __syncthreads();
@@ -210,10 +214,10 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     // ---- meanwhile: tile table, cleared masks, camera records, GUI rectangles
     for (int ag = 0; ag < apc; ++ag) {
         uint32_t *mk = agent_mask(ag);
-        for (int i = tid; i < ntiles * ms; i += NT) mk[i] = 0u;
+        for (int i = tile0 * ms + tid; i < tile1 * ms; i += NT) mk[i] = 0u;
     }
     const float inv_tiles_x = 1.0f / (float)p.tiles_x;
-    for (int i = tid; i < ntiles; i += NT) {
+    for (int i = tile0 + tid; i < tile1; i += NT) {
         // (i + 0.5) / tiles_x is at least 1 / (2 tiles_x) away from an integer: exact in float for any image
         const int ty = (int)(((float)i + 0.5f) * inv_tiles_x), tx = i - ty * p.tiles_x;
         // a = 2px+1-W and b = H-1-2py of the tile's first pixel (small integers: exact as floats)
@@ -333,6 +337,20 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                                  __uint_as_float(p.sky_rgbx), p.miss_depth);
         }
     }
+    // (with the occupancy in global memory the columns around the eye are fetched first, all at once)
+    constexpr int kNear = 2 * kSkipCells + 1;
+    auto agent_near = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_near_off); };
+    if (!OCC_SHARED && p.agent_near_off) {
+        for (int i = tid; i < apc * kNear * kNear; i += NT) {
+            const int ag = i / (kNear * kNear), c = i - ag * kNear * kNear, dz = c / kNear - kSkipCells, dx = c % kNear - kSkipCells;
+            const float4 c0 = agent_rec(ag)[0];
+            if (!(c0.x >= 0.0f && c0.x < (float)gx && c0.y >= 0.0f && c0.y < (float)p.gy && c0.z >= 0.0f && c0.z < (float)gz)) continue;
+            const int x = (int)floorf(c0.x) + dx, z = (int)floorf(c0.z) + dz;
+            if (x >= 0 && x < gx && z >= 0 && z < gz)
+                agent_near(ag)[c] = s_occ[((size_t)(x + gx * z) << (p.lay.ysh - 5)) + ((int)floorf(c0.y) >> 5)];
+        }
+        __syncthreads();
+    }
     // The first stretch of a walk.  For every combination of signs: a box of empty cells that begins at the eye's cell and is
     // grown greedily the way such rays go (x, z, y in turn, while the next layer of cells is empty).  A ray crosses
     // nothing filled before it leaves that box, so it takes all its x and z crossings up to then at once, whatever their
@@ -351,8 +369,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         const int cx = (int)floorf(c0.x), cy = (int)floorf(c0.y), cz = (int)floorf(c0.z);
         const int dx = (signs & 1) ? -1 : 1, dy = (signs & 2) ? -1 : 1, dz = (signs & 4) ? -1 : 1;
         const int wsh = p.lay.ysh - 5, yb = cy & 31;
-        const uint32_t *word = s_occ + (((cx + gx * cz) << wsh) + (cy >> 5));
-        const int step_x = dx << wsh, step_z = (gx * dz) << wsh;
+        const uint32_t *word = OCC_SHARED ? s_occ + (((cx + gx * cz) << wsh) + (cy >> 5)) : agent_near(ag) + kSkipCells * (kNear + 1);
+        const int step_x = OCC_SHARED ? dx << wsh : dx, step_z = OCC_SHARED ? (gx * dz) << wsh : kNear * dz;
         const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
         // (an eye exactly on a cell face and looking down the axis leaves its cell at once: one more for it, so that
         // mirrored views get mirrored boxes)
@@ -360,7 +378,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         const int lim_x = min(kSkipCells - 1 + on_x, dx < 0 ? cx - lox : hix - 1 - cx);
         const int lim_z = min(kSkipCells - 1 + on_z, dz < 0 ? cz - loz : hiz - 1 - cz);
         const int lim_y = min(min(kSkipCellsY, dy < 0 ? cy - loy : hiy - 1 - cy), dy < 0 ? yb : 31 - yb);
-        uint32_t seen = word[0], ys = 1u << yb;      // columns of the box or-ed together; its heights
+        const bool blind = !OCC_SHARED && !p.agent_near_off;       // (no room for them: the box stays a single cell)
+        uint32_t seen = blind ? ~0u : word[0], ys = 1u << yb;      // columns of the box or-ed together; its heights
         int ex = 0, ey = 0, ez = 0;
         bool gox = !(seen & ys) && lim_x > 0, goz = !(seen & ys) && lim_z > 0, goy = !(seen & ys);
         if (gox && on_x) { const uint32_t f = word[step_x]; gox = !(f & ys); if (gox) { seen |= f; ex = 1; } }
@@ -462,7 +481,6 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     // packed colour and its right neighbour's; the lanes of pixels 3 and 7 store no RGB word.  keep()
     // pins the constants in registers: recomputing them per tile costs more issue slots than the
     // registers are worth.
-    constexpr int kWarps = NT / 32;
     float lane_a = (float)(2 * (lane & 7)), lane_b = (float)(2 * (lane >> 3));
     const int st_r = lane >> 3, st_q = lane & 7, st_j = st_q - (st_q >> 2), st_byte = st_q & 3;
     // bytes st_byte.. of the own pixel (3 of them at most), then the neighbour's from its byte 0 (selector 4..)
@@ -470,8 +488,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     const int depth_lane_off = (lane >> 3) * W + (lane & 7);
     const int rgb_lane_off = st_r * W * 3 + st_j * 4;
     keep(lane_a); keep(lane_b); keep(st_sel);
-    const uint32_t tile_begin = smem_addr(s_tile) + 16u * (uint32_t)warp;
-    uint32_t tile_end = smem_addr(s_tile) + 16u * (uint32_t)ntiles;
+    const uint32_t tile_begin = smem_addr(s_tile) + 16u * (uint32_t)(tile0 + warp);
+    uint32_t tile_end = smem_addr(s_tile) + 16u * (uint32_t)tile1;
     uint32_t mask_step = 4u * kWarps * (uint32_t)ms;                        // bytes between a warp's consecutive tile masks
     keep(tile_end); keep(mask_step);
 
@@ -492,7 +510,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         uint32_t rare = (ov_count > 0 && p.max_boxes >= 32) ? 2u : 0u;
         keep(rare);
         uint32_t abase = smem_addr(agent_rec(ag));
-        uint32_t mask_p = smem_addr(agent_mask(ag) + (size_t)warp * ms);
+        uint32_t mask_p = smem_addr(agent_mask(ag) + (size_t)(tile0 + warp) * ms);
         // (store addresses as global-space addresses for the PTX store block)
         unsigned long long depth_lane = (unsigned long long)__cvta_generic_to_global(depth_obs + depth_lane_off);
         unsigned long long rgb_lane = (unsigned long long)__cvta_generic_to_global(rgb_obs + rgb_lane_off);
