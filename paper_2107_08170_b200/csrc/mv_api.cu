@@ -67,7 +67,7 @@ struct mv_batch {
     bool has_cams = false;
     double kr = 0, ku = 0;
     uint32_t sky_rgbx = 0;
-    struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, agent_ovtile_off, agent_near_off, misc_off, bytes; };
+    struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, agent_near_off, misc_off, bytes; };
     Smem smem{};                        // shared-memory layout of the render kernel for agents_per_cta
     int agents_per_cta = 1;             // observations one CTA renders: 1, or every agent of its env
     int threads = MV_NT;                // threads per CTA of the render kernel (fewer for CTAs with few tiles)
@@ -127,19 +127,19 @@ mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     const uint32_t ntiles = (uint32_t)(b->tiles_x * b->tiles_y);
     mv_batch::Smem m{};
     m.tile_off = round_up(b->lay.block_bytes - (occ_shared ? 0u : b->lay.occ_bytes), 16);
-    m.agent_off = m.tile_off + ntiles * 16;
-    m.agent_ov_off = kAgentRelOff + (uint32_t)(d.max_boxes > 0 ? d.max_boxes : 1) * 32;
-    m.agent_mask_off = m.agent_ov_off + (uint32_t)(d.max_overlay_rects > 0 ? d.max_overlay_rects : 1) * 32;
+    m.agent_off = round_up(m.tile_off + ntiles * 16, kAgentAlign);
+    m.agent_ov_off = kAgentRelOff + (uint32_t)d.max_boxes * 32;
+    m.agent_mask_off = m.agent_ov_off + (uint32_t)d.max_overlay_rects * 32;
     // per tile: the box-mask words, preceded by a summary word when there is more than one
     const uint32_t words_per_tile = b->mask_words > 1 ? (uint32_t)b->mask_words + 1 : 1u;
-    m.agent_ovtile_off = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
-    m.agent_near_off = m.agent_ovtile_off + round_up(((ntiles + 31) / 32) * 4, 16);
-    m.agent_stride = m.agent_near_off;
+    m.agent_near_off = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
+    uint32_t agent_bytes = m.agent_near_off;
     if (!occ_shared) {                  // the columns around the eye, if there is room for them
         const uint32_t near_bytes = round_up((2 * kSkipCells + 1) * (2 * kSkipCells + 1) * 4, 16);
-        if ((int64_t)m.agent_off + (int64_t)apc * (m.agent_stride + near_bytes) + 32 <= b->smem_max) m.agent_stride += near_bytes;
+        if ((int64_t)m.agent_off + (int64_t)apc * round_up(agent_bytes + near_bytes, kAgentAlign) + 32 <= b->smem_max) agent_bytes += near_bytes;
         else m.agent_near_off = 0;
     }
+    m.agent_stride = apc > 1 ? round_up(agent_bytes, kAgentAlign) : round_up(agent_bytes, 16);
     m.misc_off = m.agent_off + (uint32_t)apc * m.agent_stride;
     m.bytes = m.misc_off + 32;
     return m;
@@ -183,7 +183,7 @@ MergeFn merge_sweep(int grid_y) { return grid_y < 256 ? merge_sweep_kernel<uint8
 int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, int obs_count, cudaStream_t s) {
     RenderParams p{};
     p.env_blocks = b->d_env_blocks;
-    p.mat = b->d_mat;
+    p.mat = b->d_mat; p.mat_stride = b->mat_bytes_per_env;
     p.cams = b->d_cams;
     p.rgb = d_rgb;
     p.depth = d_depth;
@@ -201,7 +201,7 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.miss_depth = b->desc.miss_depth;
     p.smem_tile_off = b->smem.tile_off; p.smem_agent_off = b->smem.agent_off; p.smem_misc_off = b->smem.misc_off;
     p.agent_stride = b->smem.agent_stride; p.agent_ov_off = b->smem.agent_ov_off;
-    p.agent_mask_off = b->smem.agent_mask_off; p.agent_ovtile_off = b->smem.agent_ovtile_off; p.agent_near_off = b->smem.agent_near_off;
+    p.agent_mask_off = b->smem.agent_mask_off; p.agent_near_off = b->smem.agent_near_off;
     p.agents_per_cta = b->agents_per_cta;
     p.max_steps = b->desc.grid_x + b->desc.grid_y + b->desc.grid_z + 3;
     // accumulated crossing times drift from the exact products by at most one rounding per step
@@ -236,7 +236,7 @@ int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int en
     const mv_batch_desc &d = b->desc;
     UploadArgs u{};
     u.grid = d_grid; u.boxes = reinterpret_cast<const uint4 *>(d_boxes); u.counts = d_count; u.palette_rgb = d_palette;
-    u.env_blocks = b->d_env_blocks; u.mat = b->d_mat; u.acc = b->d_acc; u.status = b->d_status;
+    u.env_blocks = b->d_env_blocks; u.mat = b->d_mat; u.mat_stride = b->mat_bytes_per_env; u.acc = b->d_acc; u.status = b->d_status;
     u.env_index = d_env_index; u.lay = b->lay; u.env_begin = env_begin; u.env_count = env_count;
     u.gx = d.grid_x; u.gy = d.grid_y; u.gz = d.grid_z; u.max_boxes = d.max_boxes; u.palette = d.palette_size;
     for (int c = 0; c < 3; ++c) u.light[c] = (double)d.light_dir[c];
@@ -423,8 +423,11 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     EnvLayout &L = b->lay;
     L.ysh = 5;                                              // bits per (x, z) column: a power of two >= grid_y, >= 32
     while ((1 << L.ysh) < d.grid_y) L.ysh++;
-    L.occ_bytes = (uint32_t)(((size_t)d.grid_x * d.grid_z << L.ysh) / 8);
-    b->mat_bytes_per_env = (size_t)d.grid_x * d.grid_z << L.ysh;
+    L.pitch = (uint32_t)d.grid_x + 1;
+    L.origin = L.pitch + 1;                                 // a fence row, and the fence column before x = 0
+    const size_t columns = (size_t)L.pitch * (d.grid_z + 2) + 1;
+    L.occ_bytes = (uint32_t)(((columns << L.ysh) / 8 + 15) / 16 * 16);
+    b->mat_bytes_per_env = (columns << L.ysh);
     L.lut_off = L.occ_bytes;
     L.box_off = L.lut_off + round_up(kFaces * d.palette_size * 4, 16);
     L.count_off = L.box_off + (uint32_t)d.max_boxes * 32;
@@ -433,7 +436,9 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
 
     b->tiles_x = d.width / 8;
     b->tiles_y = d.height / 4;
-    b->mask_words = d.max_boxes > 0 ? (d.max_boxes + 31) / 32 : 1;
+    // a bit per box, and one behind them for "a GUI rectangle touches the tile"
+    b->mask_words = (d.max_boxes + (d.max_overlay_rects > 0 ? 1 : 0) + 31) / 32;
+    if (b->mask_words < 1) b->mask_words = 1;
 
     // kr = tan(hfov/2)/W, ku = (tan(hfov/2)*H/W)/H in double (scalar set-up for the camera kernel)
     const double tx = std::tan((double)d.hfov_rad / 2.0);
@@ -504,6 +509,8 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     if (ok) {
         const int n = d.num_envs * kPackAccInts;
         init_acc_kernel<<<(n + 255) / 256, 256>>>(b->d_acc, n);
+        const size_t words = (size_t)d.num_envs * (L.occ_bytes / 4);
+        fence_kernel<<<(unsigned)((words + 255) / 256), 256>>>(b->d_env_blocks, L, d.grid_x, d.grid_z, d.num_envs);
         ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(0) == cudaSuccess;
     }
     if (!ok) {
@@ -594,6 +601,7 @@ int mv_merge_voxels(mv_batch *b, int env_begin, int env_count, mv_box *d_boxes_o
         const mv_batch_desc &d = b->desc;
         MergeLayout ml{};
         ml.gx = d.grid_x; ml.gy = d.grid_y; ml.gz = d.grid_z;
+        ml.mat_stride = b->mat_bytes_per_env;
         ml.W = (d.grid_x + 31) / 32;
         ml.colw = 1 << (b->lay.ysh - 5);
         ml.mask_words = (uint32_t)d.grid_y * d.grid_z * ml.W;

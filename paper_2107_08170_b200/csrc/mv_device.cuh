@@ -26,11 +26,14 @@ static_assert(sizeof(CamRec) == 64, "CamRec must be 64 bytes");
 // One environment's render inputs, contiguous in HBM so that a single bulk copy stages them
 // into shared memory:  [occupancy bits | shade LUT | boxes | box count + occupied bounds].
 // Occupancy is packed along y: the (x, z) column owns 2^ysh consecutive bits (2^ysh >= grid_y, at
-// least 32), bit index u = ((x + grid_x*z) << ysh) | y, bit u&31 of word u>>5.  A walk along x or z
+// least 32), bit index u = ((origin + x + pitch*z) << ysh) | y, bit u&31 of word u>>5.  A walk along x or z
 // therefore moves by whole words and a walk along y stays inside the column's word(s); for grids
 // up to 32 voxels high a column is exactly one word.  The material store uses the same index u.
+// The grid is fenced in: one column between each row and the next (pitch = grid_x + 1) and a row before the first and
+// after the last are all ones, written once when the batch is made, so a walk in x and z that leaves the grid hits
+// something at once instead of having to be stopped by a test at every step.
 struct EnvLayout {
-    uint32_t occ_bytes;     // grid_x*grid_z*2^ysh/8
+    uint32_t occ_bytes;     // (pitch*(grid_z + 2) + 1) columns of 2^ysh bits, rounded up to 16
     uint32_t lut_off;       // 7*palette_size RGBX words
     uint32_t box_off;       // max_boxes * 32 bytes
     uint32_t count_off;     // 32 bytes: {box count, lo x,y,z, hi x,y,z, pad}; [lo, hi) = cell box
@@ -38,15 +41,20 @@ struct EnvLayout {
     uint32_t block_bytes;   // bytes staged per CTA (multiple of 16)
     uint32_t stride;        // distance between envs in HBM (multiple of 128)
     uint32_t ysh;           // log2 of the bits per (x, z) column
+    uint32_t pitch, origin; // columns from one row to the next; column of (0, 0)
 };
 
-__host__ __device__ __forceinline__ uint32_t voxel_index(uint32_t ysh, int gx, int x, int y, int z) {
-    return ((uint32_t)(x + gx * z) << ysh) | (uint32_t)y;
+__host__ __device__ __forceinline__ uint32_t column_index(const EnvLayout &lay, int x, int z) {
+    return lay.origin + (uint32_t)x + lay.pitch * (uint32_t)z;
+}
+__host__ __device__ __forceinline__ uint32_t voxel_index(const EnvLayout &lay, int x, int y, int z) {
+    return (column_index(lay, x, z) << lay.ysh) | (uint32_t)y;
 }
 
 struct RenderParams {
     const unsigned char *env_blocks;   // [E] EnvLayout blocks
-    const uint8_t *mat;                // [E][grid_x*grid_z << ysh] material ids by voxel index (clamped at upload)
+    const uint8_t *mat;                // [E][mat_stride] material ids by voxel index (clamped at upload)
+    size_t mat_stride;
     const CamRec *cams;                // [O]
     uint8_t *rgb;                      // [O][H][W][3]
     float *depth;                      // [O][H][W]
@@ -63,11 +71,10 @@ struct RenderParams {
     int part_tiles;                    // tiles of one observation that a CTA renders
     int max_steps;                     // most steps a walk can take: grid_x + grid_y + grid_z + 3 (sizes the exit margin)
     float exit_scale;                  // 1 - (bound on the rounding drift of accumulated crossing times)
-    // shared-memory offsets after the staged env block: tile table, per-agent blocks (camera record,
-    // DDA start table, eye-relative boxes, then overlay rectangles, per-tile box masks and per-tile
-    // overlay bits at the offsets below), barrier and flag words
+    // shared-memory offsets after the staged env block: tile table, per-agent blocks (ray table, camera record,
+    // eye-relative boxes, then overlay rectangles and per-tile box masks at the offsets below), barrier and flag words
     uint32_t smem_tile_off, smem_agent_off, smem_misc_off;
-    uint32_t agent_stride, agent_ov_off, agent_mask_off, agent_ovtile_off, agent_near_off;
+    uint32_t agent_stride, agent_ov_off, agent_mask_off, agent_near_off;
     const int4 *overlay;               // [O][max_overlay] 16-byte records, or null
     const int32_t *overlay_count;      // [O]
     int max_overlay;

@@ -38,6 +38,7 @@ struct MergeLayout {
     uint32_t work_off;        // word offset of the work area in the env's scratch
     int work_in_smem;
     size_t env_words;         // words between envs
+    size_t mat_stride;        // bytes between envs in the material store
 };
 
 // 32 x 32 bit transpose over a warp: bit i of lane l becomes bit l of lane i.
@@ -73,8 +74,8 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
     const int lane = threadIdx.x & 31, wi = (threadIdx.x >> 5) & 3, half = threadIdx.x >> 7;
     const int w = 4 * wb + wi, x = 32 * w + lane, z0 = 8 * zb + 4 * half;
     const bool upper = hiy - 32 * wq > 16, in_x = x < ml.gx;
-    const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk) + x * ml.colw + wq;
-    const uint8_t *m_col = mat + (size_t)(env_begin + e) * ((size_t)ml.gx * ml.gz << lay.ysh) + ((size_t)x << lay.ysh) + 32 * wq;
+    const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk) + (lay.origin + x) * ml.colw + wq;
+    const uint8_t *m_col = mat + (size_t)(env_begin + e) * ml.mat_stride + ((size_t)(lay.origin + x) << lay.ysh) + 32 * wq;
     uint32_t *ye = scratch + (size_t)e * ml.env_words + 3 * (size_t)ml.mask_words + x * ml.colw + wq;
     auto load_column = [&](const uint8_t *src, uint32_t out[8]) {
         const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src));
@@ -98,15 +99,15 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
     };
     uint32_t own[8] = {}, back[8] = {}, f_back = 0;
     if (in_x && z0 > 0 && z0 < ml.gz) {
-        f_back = occ[(size_t)(z0 - 1) * ml.gx * ml.colw];
-        load_column(m_col + ((size_t)(z0 - 1) * ml.gx << lay.ysh), back);
+        f_back = occ[(size_t)(z0 - 1) * lay.pitch * ml.colw];
+        load_column(m_col + ((size_t)(z0 - 1) * lay.pitch << lay.ysh), back);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int z = z0 + i;
         uint32_t f = 0, lx = 0, lz = 0;
         if (z < ml.gz && in_x) {
-            const size_t row = (size_t)z * ml.gx;
+            const size_t row = (size_t)z * lay.pitch;
             const uint8_t *src = m_col + (row << lay.ysh);
             f = occ[row * ml.colw];
             uint32_t other[8], f_left = 0;
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
 #pragma unroll
             for (int q = 0; q < 7; ++q) other[q] = __funnelshift_r(own[q], own[q + 1], 8);     // one height up
             other[7] = (own[7] >> 8) | (above << 24);
-            ye[row * ml.colw] = f & ((f >> 1) | (f_above << 31)) & equal_bits(own, other);
+            ye[(size_t)z * ml.gx * ml.colw] = f & ((f >> 1) | (f_above << 31)) & equal_bits(own, other);
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q) back[q] = own[q];
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
     const unsigned char *blk = env_blocks + (size_t)(env_begin + e) * lay.stride;
     const int *bounds = reinterpret_cast<const int *>(blk + lay.count_off);
     const int loy = bounds[2], loz = bounds[3], hiy = bounds[5], hiz = bounds[6];
-    const uint8_t *m_env = mat + (size_t)(env_begin + e) * ((size_t)gx * gz << lay.ysh);
+    const uint8_t *m_env = mat + (size_t)(env_begin + e) * ml.mat_stride;
     uint32_t *mine = scratch + (size_t)e * ml.env_words;
     const uint32_t *masks = mine, *ye = mine + 3 * (size_t)ml.mask_words;
     uint4 *rows = reinterpret_cast<uint4 *>(ml.work_in_smem ? s_work : reinterpret_cast<unsigned char *>(mine + ml.work_off));
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
             // a thread per box: the run in its first row, and the rows until its first cell is marked ended
             for (int b = tid; b < n; b += kMergeThreads) {
                 const int x = (int)(s_list[b] & 0xffffu), k = (int)(s_list[b] >> 16);
-                const uint8_t m = m_env[voxel_index(lay.ysh, gx, x, j, k)];
+                const uint8_t m = m_env[voxel_index(lay, x, j, k)];
                 int wd = x >> 5;
                 uint4 r = rows[k * slots + wd];
                 uint32_t stop = (r.y | ~r.x) & ~((2u << (x & 31)) - 1u);

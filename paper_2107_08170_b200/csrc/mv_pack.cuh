@@ -49,6 +49,19 @@ constexpr int kUploadThreads = 256;
 constexpr int kUploadPolls = 1 << 18, kUploadStages = 2;
 constexpr int kUploadSmem = kUploadStages * 32 * kUploadThreads * 4;
 
+// The fence around the columns of every env (see EnvLayout); grid columns keep their zeros.
+__global__ void fence_kernel(unsigned char *env_blocks, EnvLayout lay, int gx, int gz, int num_envs)
+{
+    const int colw = 1 << (lay.ysh - 5);
+    const int words = (int)(lay.occ_bytes / 4);
+    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long e = gid / words;
+    if (e >= num_envs) return;
+    const int w = (int)(gid - e * words), c = w / colw - 1, z = c < 0 ? -1 : c / (int)lay.pitch - 1;
+    const int x = c - (z + 1) * (int)lay.pitch;
+    if (z < 0 || z >= gz || x < 0 || x >= gx) reinterpret_cast<uint32_t *>(env_blocks + (size_t)e * lay.stride)[w] = 0xffffffffu;
+}
+
 __global__ void init_acc_kernel(int *acc, int n)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, k = i % kPackAccInts;
@@ -62,6 +75,7 @@ struct UploadArgs {
     const uint8_t *palette_rgb;        // null: no palettes
     unsigned char *env_blocks;
     uint8_t *mat;
+    size_t mat_stride;
     int *acc;                          // [E][kPackAccInts]
     uint32_t *status;
     const int32_t *env_index;          // destination envs, or null for the range from env_begin
@@ -172,17 +186,15 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
         if (threadIdx.x < 32 && tile + kUploadStages < tile_end) fetch(tile + kUploadStages);
         if (r >= groups) continue;
         const int z = r / xg_n, xg = r - z * xg_n;
-        const uint32_t col0 = 4u * (uint32_t)r;
-        uint8_t *mdst = p.mat + env * ((size_t)layer << p.lay.ysh) + ((size_t)col0 << p.lay.ysh) + 32 * wq;
+        const uint32_t col0 = column_index(p.lay, 4 * xg, z);
+        uint8_t *mdst = p.mat + env * p.mat_stride + ((size_t)col0 << p.lay.ysh) + 32 * wq;
         uint32_t *occ = reinterpret_cast<uint32_t *>(blk);
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             store32(mdst + ((size_t)c << p.lay.ysh), col[c][0], col[c][1], col[c][2], col[c][3], col[c][4], col[c][5],
                     col[c][6], col[c][7]);
-        if (colw == 1) *reinterpret_cast<uint4 *>(occ + col0) = make_uint4(bits[0], bits[1], bits[2], bits[3]);
-        else
 #pragma unroll
-            for (int c = 0; c < 4; ++c) occ[(col0 + c) * colw + wq] = bits[c];
+        for (int c = 0; c < 4; ++c) occ[(col0 + c) * colw + wq] = bits[c];
         const uint32_t any = bits[0] | bits[1] | bits[2] | bits[3];
         if (any) {
             lo[0] = min(lo[0], 4 * xg + (bits[0] ? 0 : bits[1] ? 1 : bits[2] ? 2 : 3));
@@ -311,7 +323,7 @@ __global__ void camera_kernel(const int32_t *__restrict__ cams, CamRec *__restri
 
 // True iff the body box around (x, y, z) lies inside the grid and touches no filled voxel
 // (cells floor(lo)..floor(hi) on every axis, ends included).
-__device__ __forceinline__ bool body_free(const uint32_t *occ, uint32_t ysh, int gx, int gy, int gz, float x, float y,
+__device__ __forceinline__ bool body_free(const uint32_t *occ, const EnvLayout &lay, int gx, int gy, int gz, float x, float y,
                                           float z, float hw, float below, float above)
 {
     const float lx = __fsub_rn(x, hw), hx = __fadd_rn(x, hw);
@@ -325,7 +337,7 @@ __device__ __forceinline__ bool body_free(const uint32_t *occ, uint32_t ysh, int
     for (int j = j0; j <= j1; ++j)
         for (int k = k0; k <= k1; ++k)
             for (int i = i0; i <= i1; ++i) {
-                const uint32_t v = voxel_index(ysh, gx, i, j, k);
+                const uint32_t v = voxel_index(lay, i, j, k);
                 if ((occ[v >> 5] >> (v & 31)) & 1u) return false;
             }
     return true;
@@ -357,8 +369,8 @@ __global__ void move_agents_kernel(int32_t *__restrict__ cams, const float4 *__r
     unsigned char *blk = env_blocks + (size_t)(o / agents) * lay.stride;
     const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk);
     float nx = x, nz = z;
-    if (body_free(occ, lay.ysh, gx, gy, gz, x_try, y, nz, hw, below, above)) nx = x_try;
-    if (body_free(occ, lay.ysh, gx, gy, gz, nx, y, z_try, hw, below, above)) nz = z_try;
+    if (body_free(occ, lay, gx, gy, gz, x_try, y, nz, hw, below, above)) nx = x_try;
+    if (body_free(occ, lay, gx, gy, gz, nx, y, z_try, hw, below, above)) nz = z_try;
     c[0] = __float_as_int(nx); c[2] = __float_as_int(nz);
     c[3] = __float_as_int(yaw); c[4] = __float_as_int(pitch);
     const int self_box = c[5];

@@ -79,6 +79,23 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " @py shf.l.wrap.b32 bit, bit, bit, sy;\n"       \
     " ld.shared.u32 w, [pos];\n"                     \
     " lop3.or.b32 w|ph, w, bit, 0, 0xC0, pf;\n"
+// The common case's step: nothing but a filled cell stops it.  What lies outside the occupied box counts as filled here
+// (the fence in x and z, `guard` = the heights outside it); afterwards w, the last column read, tells which it was.
+// The fence keeps the walk in bounds, and with a guard bit in every column it ends by itself: it only ever moves on,
+// along x, y and z, and each of them ends at something filled.
+#define MV_DDA_STEP_SEALED(T, OUT)                   \
+    " min.f32 " T ", tx, ty, tz;\n"                  \
+    " @ph bra " OUT ";\n"                            \
+    " setp.eq.f32 px, tx, " T ";\n"                  \
+    " setp.eq.and.f32 py|pz, ty, " T ", !px;\n"      \
+    " @px add.f32 tx, tx, dtx;\n"                    \
+    " @py add.f32 ty, ty, dty;\n"                    \
+    " @pz add.f32 tz, tz, dtz;\n"                    \
+    " @px add.s32 pos, pos, sx;\n"                   \
+    " @pz add.s32 pos, pos, sz;\n"                   \
+    " @py shf.l.wrap.b32 bit, bit, bit, sy;\n"       \
+    " ld.shared.u32 w, [pos];\n"                     \
+    " lop3.or.b32 a|ph, w, bit, guard, 0xC8, pf;\n"
 #define MV_DDA_STEP_IDX_TAIL                         \
     " shf.r.wrap.b32 w, w, 0, pos;\n"                \
     " lop3.or.b32 w|ph, w, 1, 0, 0xC0, pf;\n"
@@ -107,37 +124,59 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     "MV_DDA_OUT_B:\n"                                \
     " @ph mov.f32 thit, ta;\n"                       \
     "MV_DDA_OUT:\n"
+// Loop of the sealed walk.  On leaving: ph set, thit = when the filled cell was entered, px/py/pz say along which axis.
+#define MV_DDA_SEALED                                \
+    " setp.ne.u32 pf, 0, 0;\n"                       \
+    " setp.ne.u32 ph, 0, 0;\n"                       \
+    "MV_DDA_LOOP_TOP:\n"                             \
+    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
+    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
+    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
+    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
+    " bra MV_DDA_LOOP_TOP;\n"                        \
+    "MV_DDA_OUT_A:\n"                                \
+    " mov.f32 thit, tb;\n"                           \
+    " bra MV_DDA_OUT;\n"                             \
+    "MV_DDA_OUT_B:\n"                                \
+    " mov.f32 thit, ta;\n"                           \
+    "MV_DDA_OUT:\n"
 #define MV_DDA_DECL                                  \
     " .reg .pred px, py, pz, pq, ph, pf;\n"          \
     " .reg .f32 tx, ty, tz, dtx, dty, dtz, ta, tb, texit, thit;\n" \
-    " .reg .b32 sx, sy, sz, pos, bit, w, a, it;\n"   \
+    " .reg .b32 sx, sy, sz, pos, bit, guard, w, a, it;\n"   \
     " .reg .b64 ag, gbase;\n"
 
 #ifndef MV_MINB
 #define MV_MINB 3
 #endif
 
-constexpr uint32_t kOverlayTileBit = 0x80000000u;   // in a tile's box mask word (only when max_boxes < 32)
 constexpr uint32_t kAgentInside = 1u;      // eye inside the occupied cell box
 constexpr uint32_t kAgentBad = 2u;         // non-finite camera: sky frame
 constexpr uint32_t kAgentFilled = 4u;      // the eye's own voxel is filled
-// Per-agent block in shared memory (16-byte slots): camera record (3), {hit time a ray starts with,
-// flags, self box, overlay count} (1), {start bit mask, exit-time factor, start colour row, start position} (1), {64-bit address
-// of the env's material store, biased for the walk's positions} (1), DDA start
-// table (8 sign combinations x 3 axes + 2 rows for the first stretch), then eye-relative boxes, overlay rectangles, per-tile box
-// masks and per-tile overlay bits at offsets the host lays out.
-constexpr int kAgentRecVecs = 6;
-constexpr int kDdaVecs = 40;                        // 8 sign combinations x 5 rows
-// byte offsets, from the agent block's start plus 80 x (sign combination), of the DDA table rows of
-// the x, y and z axis and of the colour-row word of the x row (as text, for the PTX blocks)
+constexpr uint32_t kAgentSealed = 8u;      // eye inside, not in a filled voxel, and some height lies outside the box: the common case
+// Per-agent block in shared memory.  First the ray table, one 64-byte entry per combination of direction signs (x negative:
+// +64, y: +128, z: +256; the block is 512-byte aligned, so an entry's address is the block's OR-ed with the sign bits):
+//   {distance (>= 0) from the eye to the cell face met first, in x and z; what a step in x and z adds to the position}
+//   {first stretch: cells to spare in x, z, y; start position, from which kSkipBias steps each way are taken off}
+//   {first stretch: what is added to t |d| in x and z to give the crossings up to time t, rounded down; distance and step
+//    in y (the step is a rotate count in the column-word flavour)}
+//   {colour-table row of the face entered by an x, z, y step; -}
+// then the record {Fx, Rx, Fz, Rz} {Ux, Uz, Fy, Uy} {start bit mask, heights outside the occupied box, flags, self box} {eye
+// x, y, z, overlay count} {64-bit address of the env's material store, biased for the walk's positions; sky colour; miss
+// depth}, eye-relative boxes, overlay rectangles and per-tile box masks at offsets the host lays out.
+constexpr uint32_t kAgentTabBytes = 512, kAgentAlign = 512;
+constexpr uint32_t kAgentRecVecs = 5;
+constexpr uint32_t kAgentRelOff = kAgentTabBytes + 16u * kAgentRecVecs;
+// (as text, for the PTX blocks)
+#define MV_TAB_SKIP "16"
+#define MV_TAB_SKIP2 "32"
+#define MV_TAB_ROW "48"
+#define MV_REC_FR "512"
+#define MV_REC_UY "528"
+#define MV_REC_START "544"
+#define MV_REC_MAT "576"
 // hard bound of the traversal loop: no grid allows more steps than 3 x 1024 + 3
 #define MV_STEP_BUDGET "3080"
-#define MV_TAB_X "96"
-#define MV_TAB_Y "112"
-#define MV_TAB_Z "128"
-#define MV_TAB_ROW "108"
-#define MV_TAB_SKIP "144"
-#define MV_TAB_SKIP2 "160"
 // The empty box that a walk starts with (see the table's construction) grows by at most this many cells an axis.
 constexpr int kSkipCells = 8, kSkipCellsY = 4;
 // Crossings are counted up to a little less than the box's exit time: 2^-16 of the count, where rounding takes 2^-20 of
@@ -148,9 +187,6 @@ constexpr float kSkipMargin = 1.0f - 1.52587890625e-5f;
 constexpr uint32_t kSkipBias = 0x4B000000u;
 #define MV_SKIP_MAGIC "0f4B000000"
 #define MV_SKIP_UNMAGIC "0fCB000000"
-static_assert(16 * kAgentRecVecs == 96, "MV_TAB_* follow the agent record size");
-constexpr uint32_t kAgentDdaOff = 16u * kAgentRecVecs;
-constexpr uint32_t kAgentRelOff = 16u * (kAgentRecVecs + kDdaVecs);
 
 // One thread's share of a sky frame (non-finite camera).
 template <int NT>
@@ -167,7 +203,7 @@ template <int NT, bool OCC_SHARED, bool COLW>
 __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const RenderParams p)
 {
     static_assert(OCC_SHARED || !COLW, "the column-word walk reads shared memory");
-    extern __shared__ __align__(128) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int apc = p.agents_per_cta;
     constexpr int kWarps = NT / 32;
@@ -193,14 +229,11 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     unsigned char *s_agents = smem + p.smem_agent_off;
     uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + p.smem_misc_off);
     uint32_t *s_flag = reinterpret_cast<uint32_t *>(smem + p.smem_misc_off + 8);
-    auto agent_rec = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride); };
-    auto agent_dda = [&](int ag) { return agent_rec(ag) + kAgentRecVecs; };
-    auto agent_rel = [&](int ag) { return agent_rec(ag) + kAgentRecVecs + kDdaVecs; };
+    auto agent_tab = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride); };
+    auto agent_rec = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentTabBytes); };
+    auto agent_rel = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentRelOff); };
     auto agent_ov = [&](int ag) { return reinterpret_cast<int4 *>(s_agents + (size_t)ag * p.agent_stride + p.agent_ov_off); };
     auto agent_mask = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_mask_off); };
-    auto agent_ovtile = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_ovtile_off); };
-    const int ovt_words = (ntiles + 31) / 32;
-
     // (in a batch with few observations each one's tiles are split between the CTAs of a grid column)
     const int tile0 = blockIdx.y * p.part_tiles, tile1 = min(tile0 + p.part_tiles, ntiles);
 
@@ -226,19 +259,17 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     }
     for (int ag = tid; ag < apc; ag += NT) {
         const float4 *cq = reinterpret_cast<const float4 *>(p.cams + obs0 + ag);
-        const float4 c3 = __ldg(cq + 3);
-        float4 *rec = agent_rec(ag);
-        rec[0] = __ldg(cq);
-        rec[1] = __ldg(cq + 1);
-        rec[2] = __ldg(cq + 2);
+        const float4 c0 = __ldg(cq), c1 = __ldg(cq + 1), c2 = __ldg(cq + 2), c3 = __ldg(cq + 3);   // P F | F R | R U | self, flags
         const int ovc = p.overlay ? min(max(__ldg(p.overlay_count + obs0 + ag), 0), p.max_overlay) : 0;
-        rec[3] = make_float4(0.0f, __uint_as_float((__float_as_uint(c3.y) & kFlagBadCamera) ? kAgentBad : 0u), c3.x,
-                             __int_as_float(ovc));
+        float4 *rec = agent_rec(ag);
+        rec[0] = make_float4(c0.w, c1.z, c1.y, c2.x);
+        rec[1] = make_float4(c2.y, c2.w, c1.x, c2.z);
+        rec[2] = make_float4(0.0f, 0.0f, __uint_as_float((__float_as_uint(c3.y) & kFlagBadCamera) ? kAgentBad : 0u), c3.x);
+        rec[3] = make_float4(c0.x, c0.y, c0.z, __int_as_float(ovc));
     }
     if (p.overlay) {
-        // GUI rectangles of each observation (unpacked to x0,y0,x1,y1 / colour in two slots) and one
-        // bit per tile that any rectangle touches, so untouched tiles pay a single bit test
-        for (int i = tid; i < apc * ovt_words; i += NT) agent_ovtile(i / ovt_words)[i % ovt_words] = 0u;
+        // GUI rectangles of each observation (unpacked to x0,y0,x1,y1 / colour in two slots); the tiles any of them touches
+        // carry the bit behind the boxes'
         __syncthreads();
         for (int i = tid; i < apc * p.max_overlay; i += NT) {
             const int ag = i / p.max_overlay, r = i - ag * p.max_overlay;
@@ -254,10 +285,9 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 for (int ty = cy0 >> 2; ty <= ((cy1 - 1) >> 2); ++ty)
                     for (int tx = cx0 >> 3; tx <= ((cx1 - 1) >> 3); ++tx) {
                         const int t = ty * p.tiles_x + tx;
-                        atomicOr(&agent_ovtile(ag)[t >> 5], 1u << (t & 31));
-                        // with fewer than 32 boxes the top bit of the tile's box mask is free: it sends
-                        // exactly the touched tiles down the slow branch
-                        if (p.max_boxes < 32) atomicOr(&agent_mask(ag)[t], kOverlayTileBit);
+                        uint32_t *tm = agent_mask(ag) + t * ms;
+                        atomicOr(tm + m0 + (p.max_boxes >> 5), 1u << (p.max_boxes & 31));
+                        if (mw > 1) atomicOr(tm, 1u);
                     }
         }
     }
@@ -280,7 +310,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     // ---- per-agent traversal set-up and box binning
     const int gx = p.gx, gz = p.gz;
     // voxel-index strides of the y-packed layout: x and z move by whole columns, y by single bits
-    const int stride_x = 1 << p.lay.ysh, stride_z = gx << p.lay.ysh;
+    const int pitch = (int)p.lay.pitch, stride_x = 1 << p.lay.ysh, stride_z = pitch << p.lay.ysh;
     // Traversal is confined to the cell box [lo, hi) that holds every filled voxel of this env
     // (nothing outside it can be hit), so rays that leave it, e.g. into the sky, stop there.
     const int lox = s_count[1], loy = s_count[2], loz = s_count[3];
@@ -293,92 +323,87 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     const uint32_t inside_row = lut_base + (uint32_t)(kFaceInside * P_ * 4);
     // position of cell (cx, cy, cz) in the walk's own terms (see MV_DDA_*)
     auto cell_pos = [&](int cx, int cy, int cz) -> uint32_t {
-        return COLW ? occ_base + 4u * (uint32_t)(cx + gx * cz) : vi_bias + (uint32_t)(stride_x * cx + stride_z * cz + cy);
+        return COLW ? occ_base + 4u * column_index(p.lay, cx, cz) : vi_bias + voxel_index(p.lay, cx, cy, cz);
     };
     auto cell_filled = [&](int cx, int cy, int cz) -> bool {
-        const uint32_t u = (uint32_t)(stride_x * cx + stride_z * cz + cy);
+        const uint32_t u = voxel_index(p.lay, cx, cy, cz);
         return (s_occ[u >> 5] >> (u & 31)) & 1u;
     };
-    for (int slot = tid; slot < 24 * apc; slot += NT) {
-        // DDA start table of agent ag, row 5*signs + axis (bit c of `signs` set: direction component c
-        // negative): x = distance (>= 0) from the eye to the cell face the ray meets first, y = cells
-        // left before the occupied box ends that way, z = what a step along the axis adds to the
-        // position (column-word flavour: byte stride for x and z, rotate count for y), w = shared-memory
-        // address of the colour-table row of the face entered by a step along this axis.
-        const int ag = slot / 24, e = slot - ag * 24;
-        const int signs = e / 3, ax = e - 3 * signs, neg = (signs >> ax) & 1;
-        float4 *rec = agent_rec(ag);
-        const float4 c0 = rec[0];
-        const float Pc = ax == 0 ? c0.x : (ax == 1 ? c0.y : c0.z);
-        const bool cam_in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
-                            (c0.y < (float)hiy) && (c0.z >= (float)loz) && (c0.z < (float)hiz);
-        int cx0 = 0, cy0 = 0, cz0 = 0;
-        if (cam_in) { cx0 = (int)floorf(c0.x); cy0 = (int)floorf(c0.y); cz0 = (int)floorf(c0.z); }
-        const int cc = ax == 0 ? cx0 : (ax == 1 ? cy0 : cz0);
-        const int lo_c = ax == 0 ? lox : (ax == 1 ? loy : loz), hi_c = ax == 0 ? hix : (ax == 1 ? hiy : hiz);
-        int st;
-        if (COLW) st = ax == 0 ? (neg ? -4 : 4) : (ax == 1 ? (neg ? 31 : 1) : (neg ? -4 * gx : 4 * gx));
-        else st = (ax == 0 ? stride_x : (ax == 1 ? 1 : stride_z)) * (neg ? -1 : 1);
-        agent_dda(ag)[5 * signs + ax] = make_float4(neg ? Pc - (float)cc : (float)(cc + 1) - Pc,
-                                       neg ? (float)(cc - lo_c) : (float)(hi_c - 1 - cc), __int_as_float(st),
-                                       __uint_as_float(lut_base + (uint32_t)((2 * ax + neg) * P_ * 4)));
-        if (e == 0) {
-            const bool filled = cam_in && cell_filled(cx0, cy0, cz0);
-            rec[3].x = filled ? 0.0f : kInf;     // hit time a ray starts with: the eye's own voxel, or none yet
-            rec[3].y = __uint_as_float(__float_as_uint(rec[3].y) | (cam_in ? kAgentInside : 0u) | (filled ? kAgentFilled : 0u));
-            // exit-time factor: pulls the exit in by the rounding drift of the accumulated crossing
-            // times; -inf (the product is then -inf or NaN and the first test ends the walk) when the
-            // eye sits in a filled voxel
-            rec[4] = make_float4(__uint_as_float(1u << cy0), filled ? -kInf : p.exit_scale,
-                                 __uint_as_float(filled ? inside_row : kNoRow), __uint_as_float(cell_pos(cx0, cy0, cz0)));
-            const unsigned long long mp = reinterpret_cast<unsigned long long>(
-                p.mat + (size_t)env * ((size_t)gx * gz << p.lay.ysh) - vi_bias);
-            rec[5] = make_float4(__uint_as_float((uint32_t)mp), __uint_as_float((uint32_t)(mp >> 32)),
-                                 __uint_as_float(p.sky_rgbx), p.miss_depth);
-        }
-    }
     // (with the occupancy in global memory the columns around the eye are fetched first, all at once)
     constexpr int kNear = 2 * kSkipCells + 1;
     auto agent_near = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_near_off); };
     if (!OCC_SHARED && p.agent_near_off) {
         for (int i = tid; i < apc * kNear * kNear; i += NT) {
             const int ag = i / (kNear * kNear), c = i - ag * kNear * kNear, dz = c / kNear - kSkipCells, dx = c % kNear - kSkipCells;
-            const float4 c0 = agent_rec(ag)[0];
+            const float4 c0 = agent_rec(ag)[3];
             if (!(c0.x >= 0.0f && c0.x < (float)gx && c0.y >= 0.0f && c0.y < (float)p.gy && c0.z >= 0.0f && c0.z < (float)gz)) continue;
             const int x = (int)floorf(c0.x) + dx, z = (int)floorf(c0.z) + dz;
             if (x >= 0 && x < gx && z >= 0 && z < gz)
-                agent_near(ag)[c] = s_occ[((size_t)(x + gx * z) << (p.lay.ysh - 5)) + ((int)floorf(c0.y) >> 5)];
+                agent_near(ag)[c] = s_occ[((size_t)column_index(p.lay, x, z) << (p.lay.ysh - 5)) + ((int)floorf(c0.y) >> 5)];
         }
         __syncthreads();
+    }
+    // Where the eye is, in the terms of the walk's tables.
+    auto eye_cell = [&](const float4 &c0, int &cx, int &cy, int &cz) -> bool {
+        const bool in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
+                        (c0.y < (float)hiy) && (c0.z >= (float)loz) && (c0.z < (float)hiz);
+        cx = cy = cz = 0;
+        if (in) { cx = (int)floorf(c0.x); cy = (int)floorf(c0.y); cz = (int)floorf(c0.z); }
+        return in;
+    };
+    // The ray tables but for the first stretch, and the state a walk starts in: a thread per combination of signs.
+    for (int slot = tid; slot < 8 * apc; slot += NT) {
+        const int ag = slot >> 3, signs = slot & 7;
+        float4 *entry = agent_tab(ag) + 4 * signs, *rec = agent_rec(ag);
+        const float4 c0 = rec[3];
+        int cx, cy, cz;
+        const bool cam_in = eye_cell(c0, cx, cy, cz);
+        const int dx = (signs & 1) ? -1 : 1, dy = (signs & 2) ? -1 : 1, dz = (signs & 4) ? -1 : 1;
+        const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
+        const float qy = dy < 0 ? c0.y - (float)cy : (float)(cy + 1) - c0.y;
+        const int sx = COLW ? 4 * dx : dx * stride_x, sz = COLW ? 4 * pitch * dz : dz * stride_z, sy = COLW ? (dy < 0 ? 31 : 1) : dy;
+        entry[0] = make_float4(qx, qz, __int_as_float(sx), __int_as_float(sz));
+        entry[2] = make_float4((1.0f - qx) * kSkipMargin, (1.0f - qz) * kSkipMargin, qy, __int_as_float(sy));
+        entry[3] = make_float4(__uint_as_float(lut_base + (uint32_t)((dx < 0 ? 1 : 0) * P_ * 4)),
+                               __uint_as_float(lut_base + (uint32_t)((4 + (dz < 0 ? 1 : 0)) * P_ * 4)),
+                               __uint_as_float(lut_base + (uint32_t)((2 + (dy < 0 ? 1 : 0)) * P_ * 4)), 0.0f);
+        if (signs == 0) {
+            const bool filled = cam_in && cell_filled(cx, cy, cz);
+            const uint32_t guard = ~(hiy >= 32 ? 0xffffffffu : (1u << hiy) - 1u) | ((1u << min(loy, 31)) - 1u);
+            rec[2].x = __uint_as_float(1u << (cy & 31));
+            rec[2].y = __uint_as_float(guard);                   // heights outside the occupied box
+            rec[2].z = __uint_as_float(__float_as_uint(rec[2].z) | (cam_in ? kAgentInside : 0u) | (filled ? kAgentFilled : 0u) |
+                                       (cam_in && !filled && guard ? kAgentSealed : 0u));
+            const unsigned long long mp = reinterpret_cast<unsigned long long>(p.mat + (size_t)env * p.mat_stride - vi_bias);
+            rec[4] = make_float4(__uint_as_float((uint32_t)mp), __uint_as_float((uint32_t)(mp >> 32)),
+                                 __uint_as_float(p.sky_rgbx), p.miss_depth);
+        }
     }
     // The first stretch of a walk.  For every combination of signs: a box of empty cells that begins at the eye's cell and is
     // grown greedily the way such rays go (x, z, y in turn, while the next layer of cells is empty).  A ray crosses
     // nothing filled before it leaves that box, so it takes all its x and z crossings up to then at once, whatever their
     // order (three steps of seven on average; the vertical ones are too few to be worth it): 234 -> 220 instructions a tile
-    // on 128x32x128 columns, 1230 -> 1184 us for 16384 observations; 64x16x64 rooms with boxes 1126 -> 1007 us.  Rows 3 and
-    // 4 of the table:
-    // {cells to spare in x, z, y; start position, from which kSkipBias steps each way are taken off} {what is added to
-    // t |d| in x and in z to give the crossings up to time t, rounded down}.
-    for (int slot = (tid + NT - 64) % NT; slot < 8 * apc; slot += NT) {
-        const int ag = slot >> 3, signs = slot & 7;
-        const float4 c0 = agent_rec(ag)[0];
-        float4 *row = agent_dda(ag) + 5 * signs + 3;
-        const bool cam_in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
-                            (c0.y < (float)hiy) && (c0.z >= (float)loz) && (c0.z < (float)hiz);
-        if (!cam_in) continue;                       // (the table's users start elsewhere)
-        const int cx = (int)floorf(c0.x), cy = (int)floorf(c0.y), cz = (int)floorf(c0.z);
+    // on 128x32x128 columns, 1230 -> 1184 us for 16384 observations; 64x16x64 rooms with boxes 1126 -> 1007 us.
+    // A warp per agent, four lanes per combination: a layer's cells are read by all four, and votes tell whether it is empty (the
+    // rounds depend on one another, so their latency is what counts; each lane keeps the columns that it has seen).
+    for (int ag = (warp + kWarps - 2) % kWarps; ag < apc; ag += kWarps) {
+        const int signs = lane >> 2, part = lane & 3;
+        const unsigned group = 0xfu << (lane & 28);
+        const float4 c0 = agent_rec(ag)[3];
+        int cx, cy, cz;
+        const bool cam_in = eye_cell(c0, cx, cy, cz);
         const int dx = (signs & 1) ? -1 : 1, dy = (signs & 2) ? -1 : 1, dz = (signs & 4) ? -1 : 1;
         const int wsh = p.lay.ysh - 5, yb = cy & 31;
-        const uint32_t *word = OCC_SHARED ? s_occ + (((cx + gx * cz) << wsh) + (cy >> 5)) : agent_near(ag) + kSkipCells * (kNear + 1);
-        const int step_x = OCC_SHARED ? dx << wsh : dx, step_z = OCC_SHARED ? (gx * dz) << wsh : kNear * dz;
-        const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
+        const uint32_t *word = OCC_SHARED ? s_occ + ((column_index(p.lay, cx, cz) << wsh) + (cy >> 5)) : agent_near(ag) + kSkipCells * (kNear + 1);
+        const int step_x = OCC_SHARED ? dx << wsh : dx, step_z = OCC_SHARED ? (pitch * dz) << wsh : kNear * dz;
         // (an eye exactly on a cell face and looking down the axis leaves its cell at once: one more for it, so that
         // mirrored views get mirrored boxes)
-        const int on_x = qx == 0.0f ? 1 : 0, on_z = qz == 0.0f ? 1 : 0;
+        const int on_x = dx < 0 && c0.x == (float)cx ? 1 : 0, on_z = dz < 0 && c0.z == (float)cz ? 1 : 0;
         const int lim_x = min(kSkipCells - 1 + on_x, dx < 0 ? cx - lox : hix - 1 - cx);
         const int lim_z = min(kSkipCells - 1 + on_z, dz < 0 ? cz - loz : hiz - 1 - cz);
         const int lim_y = min(min(kSkipCellsY, dy < 0 ? cy - loy : hiy - 1 - cy), dy < 0 ? yb : 31 - yb);
-        const bool blind = !OCC_SHARED && !p.agent_near_off;       // (no room for them: the box stays a single cell)
+        // (eye outside or in a filled voxel, or no room for the columns: the box stays a single cell)
+        const bool blind = !cam_in || (!OCC_SHARED && !p.agent_near_off);
         uint32_t seen = blind ? ~0u : word[0], ys = 1u << yb;      // columns of the box or-ed together; its heights
         int ex = 0, ey = 0, ez = 0;
         bool gox = !(seen & ys) && lim_x > 0, goz = !(seen & ys) && lim_z > 0, goy = !(seen & ys);
@@ -388,32 +413,34 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             goz = !(f & ys);
             if (goz) { seen |= f; ez = 1; }
         }
-        while (gox || goy || goz) {
+        while (__any_sync(0xffffffffu, gox || goy || goz)) {
             // the next layers in x and z and the corner between them, all loads of a round in flight at once
             gox = gox && ex < lim_x;
             goz = goz && ez < lim_z;
             const uint32_t *px = word + (ex + 1) * step_x, *pz = word + (ez + 1) * step_z;
             uint32_t fx = 0, fz = 0, corner = 0;
 #pragma unroll
-            for (int i = 0; i <= kSkipCells; ++i) {
-                if (gox && i <= ez) fx |= px[i * step_z];
-                if (goz && i <= ex) fz |= pz[i * step_x];
+            for (int i = 0; i <= kSkipCells; i += 4) {
+                if (gox && i + part <= ez) fx |= px[(i + part) * step_z];
+                if (goz && i + part <= ex) fz |= pz[(i + part) * step_x];
             }
             if (gox && goz) corner = px[(ez + 1) * step_z];
-            gox = gox && !(fx & ys);
+            const unsigned full_x = __ballot_sync(0xffffffffu, (fx & ys) != 0u);
+            gox = gox && !(full_x & group);
             if (gox) { seen |= fx; fz |= corner; ++ex; }
-            goz = goz && !(fz & ys);
+            const unsigned full_z = __ballot_sync(0xffffffffu, (fz & ys) != 0u);
+            goz = goz && !(full_z & group);
             if (goz) { seen |= fz; ++ez; }
             const uint32_t b = 1u << ((yb + dy * (ey + 1)) & 31);
-            goy = goy && ey < lim_y && !(seen & b);
+            const unsigned full_y = __ballot_sync(0xffffffffu, (seen & b) != 0u);
+            goy = goy && ey < lim_y && !(full_y & group);
             if (goy) { ys |= b; ++ey; }
         }
-        int sx, sz;
-        if (COLW) { sx = 4 * dx; sz = 4 * gx * dz; }
-        else { sx = dx * stride_x; sz = dz * stride_z; }
-        row[0] = make_float4((float)ex, (float)ez, (float)ey,
-                             __uint_as_float(cell_pos(cx, cy, cz) - kSkipBias * (uint32_t)sx - kSkipBias * (uint32_t)sz));
-        row[1] = make_float4((1.0f - qx) * kSkipMargin, (1.0f - qz) * kSkipMargin, 0.0f, 0.0f);
+        if (part == 0) {
+            const int sx = COLW ? 4 * dx : dx * stride_x, sz = COLW ? 4 * pitch * dz : dz * stride_z;
+            agent_tab(ag)[4 * signs + 1] = make_float4((float)ex, (float)ez, (float)ey, __uint_as_float(cell_pos(cx, cy, cz) -
+                                                       kSkipBias * (uint32_t)sx - kSkipBias * (uint32_t)sz));
+        }
     }
     {
         const int nb = min(s_count[0], p.max_boxes);
@@ -422,10 +449,10 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         for (int i = NT - 1 - tid; i < apc * p.max_boxes; i += NT) {
             const int ag = i / p.max_boxes, b = i - ag * p.max_boxes;
             const float4 *rec = agent_rec(ag);
-            const float4 c0 = rec[0], c1 = rec[1], c2 = rec[2];
-            const float Px = c0.x, Py = c0.y, Pz = c0.z, Fx = c0.w, Fy = c1.x, Fz = c1.y;
-            const float Rx = c1.z, Ry = c1.w, Rz = c2.x, Ux = c2.y, Uy = c2.z, Uz = c2.w;
-            const int self_box = __float_as_int(rec[3].z);
+            const float4 c0 = rec[0], c1 = rec[1], P4 = rec[3];
+            const float Px = P4.x, Py = P4.y, Pz = P4.z, Fx = c0.x, Fy = c1.z, Fz = c0.z;
+            const float Rx = c0.y, Ry = 0.0f, Rz = c0.w, Ux = c1.x, Uy = c1.w, Uz = c1.y;       // (cameras do not roll)
+            const int self_box = __float_as_int(rec[2].w);
             const float r2 = Rx * Rx + Ry * Ry + Rz * Rz, u2 = Ux * Ux + Uy * Uy + Uz * Uz;
             const float ir2 = 1.0f / r2, iu2 = 1.0f / u2;
             const float4 A = s_box[2 * b], B = s_box[2 * b + 1];
@@ -497,19 +524,12 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         const int obs = obs0 + ag;
         uint8_t *rgb_obs = p.rgb + (size_t)obs * H * W * 3;
         float *depth_obs = p.depth + (size_t)obs * H * W;
-        const float4 c0 = agent_rec(ag)[0], c3 = agent_rec(ag)[3];
-        const uint32_t aflags = __float_as_uint(c3.y);
+        const uint32_t aflags = __float_as_uint(agent_rec(ag)[2].z);
         if (aflags & kAgentBad) {                   // non-finite camera: a sky frame
             write_sky<NT>(rgb_obs, depth_obs, W * H, p.sky_rgbx, p.miss_depth);
             continue;
         }
-        const float Px = c0.x, Py = c0.y, Pz = c0.z;
-        const bool cam_in = (aflags & kAgentInside) != 0;
-        const int ov_count = __float_as_int(c3.w);
-        // non-zero: every tile takes the slow branch (an overlay that cannot flag its tiles in the box mask)
-        uint32_t rare = (ov_count > 0 && p.max_boxes >= 32) ? 2u : 0u;
-        keep(rare);
-        uint32_t abase = smem_addr(agent_rec(ag));
+        uint32_t abase = smem_addr(agent_tab(ag));
         uint32_t mask_p = smem_addr(agent_mask(ag) + (size_t)(tile0 + warp) * ms);
         // (store addresses as global-space addresses for the PTX store block)
         unsigned long long depth_lane = (unsigned long long)__cvta_generic_to_global(depth_obs + depth_lane_off);
@@ -521,8 +541,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         // that the choice between the common case and the rest is taken per agent, not per tile; what
         // follows the walk is the same for both.  The warp-wide reduction and shuffle in it name all 32
         // lanes, so they wait by themselves for lanes whose walk ran longer.
-        auto finish_tile = [&](uint32_t tile_p, uint32_t mask_p, int tile_px, uint32_t pos, uint32_t bit, uint32_t row,
-                               uint32_t sgn3, float t_hit, float dtx, float dty, float dtz) {
+        auto finish_tile = [&](uint32_t mask_p, int tile_px, uint32_t pos, uint32_t bit, uint32_t row,
+                               uint32_t tab, float t_hit, float dtx, float dty, float dtz) {
             // ---- the hit voxel's material byte is asked for from global memory (its colour is looked up
             // in the shaded table only in the store block, after everything that does not need it), this
             // tile's first box-mask word is read, and the latest voxel hit of the warp is found (boxes wholly
@@ -530,7 +550,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             // material store's address in the agent block.  (Column-word flavour: the voxel index is rebuilt from
             // the column's address and the bit.)
             uint32_t rgbx, m, mat_id;
-            float depth, tb, wmax;
+            float depth;
             {
                 uint32_t vi = pos;
                 if (COLW) {
@@ -540,41 +560,42 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 }
                 asm volatile("{\n"
                     " .reg .pred pv;\n"
-                    " .reg .b32 skyb, missb, tbb, wmb;\n"
+                    " .reg .b32 skyb, missb;\n"
                     " .reg .b64 mp, sm;\n"
-                    " ld.shared.v2.b64 {mp, sm}, [%9+80];\n"
-                    " ld.shared.u32 %2, [%10];\n"
+                    " ld.shared.v2.b64 {mp, sm}, [%7+" MV_REC_MAT "];\n"
+                    " ld.shared.u32 %2, [%8];\n"
                     " mov.b64 {skyb, missb}, sm;\n"
                     " mov.b32 %0, skyb;\n"
                     " mov.b32 %1, missb;\n"
-                    " setp.ne.u32 pv, %6, 0xffffffff;\n"
-                    " mad.wide.u32 mp, %7, 1, mp;\n"
-                    " mov.b32 tbb, %8;\n"
-                    " @pv ld.global.nc.u8 %5, [mp];\n"
-                    " redux.sync.max.u32 wmb, tbb, 0xffffffff;\n"
-                    " mov.b32 %3, tbb;\n"
-                    " mov.b32 %4, wmb;\n"
-                    " @pv mov.f32 %1, %8;\n"
+                    " setp.ne.u32 pv, %4, 0xffffffff;\n"
+                    " mad.wide.u32 mp, %5, 1, mp;\n"
+                    " @pv ld.global.nc.u8 %3, [mp];\n"
+                    " @pv mov.f32 %1, %6;\n"
                     "}\n"
-                    : "=&r"(rgbx), "=&f"(depth), "=&r"(m), "=&f"(tb), "=&f"(wmax), "=&r"(mat_id)
+                    : "=&r"(rgbx), "=&f"(depth), "=&r"(m), "=&r"(mat_id)
                     : "r"(row), "r"(vi), "f"(t_hit), "r"(abase), "r"(mask_p)
                     : "memory");
             }
 
-            // ---- the less common work, behind one test: boxes binned to this tile (or more than 32 boxes
-            // per environment) and the GUI overlay.  A box wins only with a strictly smaller time.
-            if ((m | rare) != 0u) {
-                if (p.max_boxes < 32) m &= ~kOverlayTileBit;
-                if (m != 0u) {
-                    // (more than 32 boxes per env: m was the summary; start with the first real word)
+            // ---- the less common work, behind one test: boxes binned to this tile, and the GUI overlay (the bit behind the
+            // boxes').  A box wins only with a strictly smaller time; boxes wholly behind the warp's latest voxel hit are skipped.
+            if (m != 0u) {
+                {
+                    const float wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(t_hit)));
+                    float tb = t_hit;
+                    bool gui = false;
+                    // (more than one word: m was the summary; start with the first real word)
                     if (mw > 1) asm volatile("ld.shared.u32 %0, [%1+4];" : "=r"(m) : "r"(mask_p));
-                    // signed reciprocals again, and the ray's rows of the DDA table for the faces
-                    const float ix = __uint_as_float(__float_as_uint(dtx) | (sgn3 << 31));
-                    const float iy = __uint_as_float(__float_as_uint(dty) | ((sgn3 & 2u) << 30));
-                    const float iz = __uint_as_float(__float_as_uint(dtz) | ((sgn3 & 4u) << 29));
-                    const uint32_t tab = abase + 80u * sgn3;
+                    // signed reciprocals again, from the signs in the table entry's address
+                    const float ix = __uint_as_float(__float_as_uint(dtx) | ((tab & 64u) << 25));
+                    const float iy = __uint_as_float(__float_as_uint(dty) | ((tab & 128u) << 24));
+                    const float iz = __uint_as_float(__float_as_uint(dtz) | ((tab & 256u) << 23));
                     uint32_t baddr = 0;
                     for (int w = 0;;) {
+                        if (p.overlay && w == (p.max_boxes >> 5)) {
+                            gui = (m >> (p.max_boxes & 31)) & 1u;
+                            m &= ~(1u << (p.max_boxes & 31));
+                        }
                         while (m) {
                             const int b = (__ffs(m) - 1) + 32 * w;
                             m &= m - 1;
@@ -594,24 +615,22 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                                 uint32_t r = inside_row;
                                 if (!(tn < 0.0f))
                                     asm volatile("ld.shared.u32 %0, [%1+" MV_TAB_ROW "];" : "=r"(r)
-                                                 : "r"(tab + ((nx == tn) ? 0u : ((ny == tn) ? 16u : 32u))));
+                                                 : "r"(tab + ((nx == tn) ? 0u : ((ny == tn) ? 8u : 4u))));
                                 baddr = r + 4u * __float_as_uint(hi.w);
                             }
                         }
                         if (++w >= mw) break;
-                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(m) : "r"(mask_p + 4u * (uint32_t)(w + m0)));
+                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(m) : "r"(mask_p + 4u * (uint32_t)(w + 1)));
                     }
                     if (baddr) {
                         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(rgbx) : "r"(baddr));
                         depth = tb + 0.0f;
                         row = kNoRow;                            // the voxel behind the box is not looked up
                     }
-                }
-                // GUI overlay: rectangles in list order, later ones on top; depth is left alone
-                if (ov_count > 0) {
-                    const uint32_t tile_no = (tile_p - smem_addr(s_tile)) >> 4;
-                    if ((agent_ovtile(ag)[tile_no >> 5] >> (tile_no & 31)) & 1u) {
+                    // GUI overlay: rectangles in list order, later ones on top; depth is left alone
+                    if (gui) {
                         const int4 *ov = agent_ov(ag);
+                        const int ov_count = __float_as_int(agent_rec(ag)[3].w);
                         const int px = (tile_px % W) + (lane & 7), py = (tile_px / W) + (lane >> 3);
                         if (row != kNoRow) {                     // the rectangles go over the voxel colour: look it up now
                             asm volatile("ld.shared.u32 %0, [%1];" : "=r"(rgbx) : "r"(row + 4u * mat_id));
@@ -645,38 +664,36 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 :: "r"(rgbx), "f"(depth), "r"(tile_px), "l"(depth_lane), "l"(rgb_lane), "r"(st_sel), "r"(row), "r"(mat_id)
                 : "memory");
         };
-        if (COLW && cam_in) {
+        if (COLW && (aflags & kAgentSealed)) {
             for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
                 int tile_px;
-                uint32_t pos, bit = 0, row, sgn3;
+                uint32_t pos, bit = 0, row, tab;
                 float t_hit, dtx, dty, dtz;
                 // ---- the common case in one block of PTX: tile record, ray through the pixel centre
                 // (d = F + a*Rs + b*Us, a = 2px+1-W, b = H-1-2py, two chained FMAs per component),
                 // reciprocals, the DDA table rows for the ray's signs
-                // {distance to the first face, cells left, step, colour row} per axis, first crossing
+                // the table entry for the ray's signs, first crossing
                 // times, exit time, then the walk.  The basis is re-read from shared memory per tile:
                 // three broadcast loads cost less than nine registers held across the walk.
                 // A direction component that is exactly zero needs no special case here: its reciprocal
                 // is +-inf, so its crossing time is +inf (or NaN when the eye sits exactly on the face,
                 // which min and the compares ignore) and that axis is never stepped, which is the rule
-                // for such rays; the exit time ignores the axis the same way.
+                // for such rays.
                 asm volatile("{\n"
                     MV_DDA_DECL
-                    " .reg .f32 Ta, Tb, Fx, Fy, Fz, Rx, Ry, Rz, Ux, Uy, Uz, ca, cb, dx, dy, dz, ix, iy, iz;\n"
-                    " .reg .f32 q0, q1, q2, q3, q4, q5, esc;\n"
-                    " .reg .b32 u, tab;\n"
+                    " .reg .f32 Ta, Tb, Fx, Fy, Fz, Rx, Rz, Ux, Uy, Uz, ca, cb, dx, dy, dz, ix, iy, iz;\n"
+                    " .reg .f32 q0, q1, q2, q3, q4;\n"
+                    " .reg .b32 u, v;\n"
                     " ld.shared.v4.b32 {Ta, Tb, %0, _}, [%9];\n"
-                    " ld.shared.f32 Fx, [%10+12];\n"
-                    " ld.shared.v4.f32 {Fy, Fz, Rx, Ry}, [%10+16];\n"
-                    " ld.shared.v4.f32 {Rz, Ux, Uy, Uz}, [%10+32];\n"
-                    " ld.shared.v4.b32 {bit, esc, %4, _}, [%10+64];\n"
+                    " ld.shared.v4.f32 {Fx, Rx, Fz, Rz}, [%10+" MV_REC_FR "];\n"
+                    " ld.shared.v4.f32 {Ux, Uz, Fy, Uy}, [%10+" MV_REC_UY "];\n"
+                    " ld.shared.v2.b32 {bit, guard}, [%10+" MV_REC_START "];\n"
                     " add.f32 ca, Ta, %11;\n"
                     " sub.f32 cb, Tb, %12;\n"
                     " fma.rn.f32 dx, ca, Rx, Fx;\n"
-                    " fma.rn.f32 dy, ca, Ry, Fy;\n"
                     " fma.rn.f32 dz, ca, Rz, Fz;\n"
+                    " fma.rn.f32 dy, cb, Uy, Fy;\n"
                     " fma.rn.f32 dx, cb, Ux, dx;\n"
-                    " fma.rn.f32 dy, cb, Uy, dy;\n"
                     " fma.rn.f32 dz, cb, Uz, dz;\n"
                     " abs.f32 ix, dx;\n"
                     " abs.f32 iy, dy;\n"
@@ -685,27 +702,18 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " rcp.approx.ftz.f32 dty, iy;\n"
                     " rcp.approx.ftz.f32 dtz, iz;\n"
                     " mov.b32 u, dx;\n"
-                    " shr.u32 %8, u, 31;\n"
+                    " mov.b32 v, dz;\n"
+                    " prmt.b32 u, u, v, 0x00FB;\n"                  // byte 0: sign of dx, byte 1: sign of dz
+                    " lop3.b32 %8, u, 0x140, %10, 0xEA;\n"
                     " mov.b32 u, dy;\n"
-                    " shr.u32 u, u, 30;\n"
-                    " lop3.b32 %8, u, 2, %8, 0xEA;\n"
-                    " mov.b32 u, dz;\n"
-                    " shr.u32 u, u, 29;\n"
-                    " lop3.b32 %8, u, 4, %8, 0xEA;\n"
-                    " mad.lo.u32 tab, %8, 80, %10;\n"
-                    " ld.shared.v4.b32 {q0, q1, sx, _}, [tab+" MV_TAB_X "];\n"
-                    " ld.shared.v4.b32 {q2, q3, sy, _}, [tab+" MV_TAB_Y "];\n"
-                    " ld.shared.v4.b32 {q4, q5, sz, _}, [tab+" MV_TAB_Z "];\n"
-                    " mul.f32 tx, q0, dtx;\n"
-                    " mul.f32 ty, q2, dty;\n"
-                    " mul.f32 tz, q4, dtz;\n"
-                    " fma.rn.f32 q1, q1, dtx, tx;\n"
-                    " fma.rn.f32 q3, q3, dty, ty;\n"
-                    " fma.rn.f32 q5, q5, dtz, tz;\n"
-                    " min.f32 q1, q1, q3, q5;\n"
-                    " mul.f32 texit, q1, esc;\n"
-                    " ld.shared.v4.b32 {q0, q1, q2, pos}, [tab+" MV_TAB_SKIP "];\n"
-                    " ld.shared.v2.f32 {q3, q4}, [tab+" MV_TAB_SKIP2 "];\n"
+                    " shr.u32 u, u, 24;\n"
+                    " lop3.b32 %8, u, 0x80, %8, 0xEA;\n"
+                    " ld.shared.v4.b32 {tx, tz, sx, sz}, [%8];\n"
+                    " ld.shared.v4.b32 {q0, q1, q2, pos}, [%8+" MV_TAB_SKIP "];\n"
+                    " ld.shared.v4.b32 {q3, q4, ty, sy}, [%8+" MV_TAB_SKIP2 "];\n"
+                    " mul.f32 tx, tx, dtx;\n"
+                    " mul.f32 ty, ty, dty;\n"
+                    " mul.f32 tz, tz, dtz;\n"
                     " fma.rn.f32 q0, q0, dtx, tx;\n"
                     " fma.rn.f32 q1, q1, dtz, tz;\n"
                     " fma.rn.f32 q2, q2, dty, ty;\n"
@@ -723,12 +731,17 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " add.f32 q4, q4, " MV_SKIP_UNMAGIC ";\n"
                     " fma.rn.f32 tx, q3, dtx, tx;\n"
                     " fma.rn.f32 tz, q4, dtz, tz;\n"
-                    " ld.shared.f32 thit, [%10+48];\n"
-                    " mov.s32 it, " MV_STEP_BUDGET ";\n"
-                    MV_DDA_LOOP(MV_DDA_STEP_COLW)
-                    " @py add.u32 tab, tab, 16;\n"
-                    " @pz add.u32 tab, tab, 32;\n"
-                    " @ph ld.shared.u32 %4, [tab+" MV_TAB_ROW "];\n"
+                    MV_DDA_SEALED
+                    // a miss if the cell is fence (its guard bits are set) or lies at a height outside the box
+                    " or.b32 w, w, bit;\n"
+                    " and.b32 w, w, guard;\n"
+                    " setp.eq.u32 ph, w, 0;\n"
+                    " mov.b32 %4, 0xffffffff;\n"
+                    " @!ph mov.f32 thit, 0f7F800000;\n"
+                    " mov.b32 u, %8;\n"
+                    " @py add.u32 u, u, 8;\n"
+                    " @pz add.u32 u, u, 4;\n"
+                    " @ph ld.shared.u32 %4, [u+" MV_TAB_ROW "];\n"
                     " mov.b32 %1, pos;\n"
                     " mov.b32 %2, bit;\n"
                     " mov.f32 %3, thit;\n"
@@ -736,64 +749,62 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mov.f32 %6, dty;\n"
                     " mov.f32 %7, dtz;\n"
                     "}\n"
-                    : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(sgn3)
+                    : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab)
                     : "r"(tile_p), "r"(abase), "f"(lane_a), "f"(lane_b)
                     : "memory");
-                finish_tile(tile_p, mask_p, tile_px, pos, bit, row, sgn3, t_hit, dtx, dty, dtz);
+                finish_tile(mask_p, tile_px, pos, bit, row, tab, t_hit, dtx, dty, dtz);
             }
         } else {
+            const float4 P4 = agent_rec(ag)[3];
+            const float Px = P4.x, Py = P4.y, Pz = P4.z;
+            const bool cam_in = (aflags & kAgentInside) != 0;
             for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
                 int tile_px;
-                uint32_t pos, bit = 0, row, sgn3;
+                uint32_t pos, bit = 0, row, tab;
                 float t_hit, dtx, dty, dtz;
                 // ---- every other case: the same steps in C++, with the eye possibly outside the
                 // occupied box and either flavour of the walk
                 float Ta, Tb;
                 asm volatile("ld.shared.v4.b32 {%0, %1, %2, _}, [%3];" : "=f"(Ta), "=f"(Tb), "=r"(tile_px) : "r"(tile_p));
-                float Fx, Fy, Fz, Rx, Ry, Rz, Ux, Uy, Uz, esc;
-                uint32_t pos0, row0, bit0;
-                asm volatile("ld.shared.f32 %0, [%1+12];" : "=f"(Fx) : "r"(abase));
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4+16];" : "=f"(Fy), "=f"(Fz), "=f"(Rx), "=f"(Ry) : "r"(abase));
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4+32];" : "=f"(Rz), "=f"(Ux), "=f"(Uy), "=f"(Uz) : "r"(abase));
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4+64];" : "=r"(bit0), "=f"(esc), "=r"(row0), "=r"(pos0) : "r"(abase));
+                const float4 FR = agent_rec(ag)[0], UY = agent_rec(ag)[1];
+                const uint32_t bit0 = __float_as_uint(agent_rec(ag)[2].x);
                 const float a = Ta + lane_a, bb = Tb - lane_b;
-                float dx = fmaf(bb, Ux, fmaf(a, Rx, Fx));
-                float dy = fmaf(bb, Uy, fmaf(a, Ry, Fy));
-                float dz = fmaf(bb, Uz, fmaf(a, Rz, Fz));
+                float dx = fmaf(bb, UY.x, fmaf(a, FR.y, FR.x));
+                float dy = fmaf(bb, UY.w, UY.z);
+                float dz = fmaf(bb, UY.y, fmaf(a, FR.w, FR.z));
                 dx = dx == 0.0f ? 1e-30f : dx;
                 dy = dy == 0.0f ? 1e-30f : dy;
                 dz = dz == 0.0f ? 1e-30f : dz;
                 const float ix = fast_rcp(dx), iy = fast_rcp(dy), iz = fast_rcp(dz);
                 dtx = fabsf(ix); dty = fabsf(iy); dtz = fabsf(iz);
-                sgn3 = (__float_as_uint(dx) >> 31) | ((__float_as_uint(dy) >> 30) & 2u) | ((__float_as_uint(dz) >> 29) & 4u);
-                const uint32_t tab = abase + 80u * sgn3;
-                float qxx, qxy, qyx, qyy, qzx, qzy;
+                tab = abase | ((__float_as_uint(dx) >> 25) & 64u) | ((__float_as_uint(dy) >> 24) & 128u) | ((__float_as_uint(dz) >> 23) & 256u);
+                float qx, qy, qz, ex, ey, ez, kx, kz;
                 int sx, sy, sz;
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, _}, [%3+" MV_TAB_X "];" : "=f"(qxx), "=f"(qxy), "=r"(sx) : "r"(tab));
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, _}, [%3+" MV_TAB_Y "];" : "=f"(qyx), "=f"(qyy), "=r"(sy) : "r"(tab));
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, _}, [%3+" MV_TAB_Z "];" : "=f"(qzx), "=f"(qzy), "=r"(sz) : "r"(tab));
+                uint32_t at;
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(qx), "=f"(qz), "=r"(sx), "=r"(sz) : "r"(tab));
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4+" MV_TAB_SKIP "];" : "=f"(ex), "=f"(ez), "=f"(ey), "=r"(at) : "r"(tab));
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4+" MV_TAB_SKIP2 "];" : "=f"(kx), "=f"(kz), "=f"(qy), "=r"(sy) : "r"(tab));
+                const bool ngx = dx < 0.0f, ngy = dy < 0.0f, ngz = dz < 0.0f;
                 float t0x, t0y, t0z, t_exit;
                 t_hit = 0.0f;
-                pos = pos0; bit = bit0; row = row0;
+                pos = 0; bit = bit0; row = kNoRow;
                 if (cam_in) {
-                    t0x = qxx * dtx;
-                    t0y = qyx * dty;
-                    t0z = qzx * dtz;
-                    t_exit = min3f(fmaf(qxy, dtx, t0x), fmaf(qyy, dty, t0y), fmaf(qzy, dtz, t0z)) * esc;
-                    if (!COLW) {                  // the first stretch, as in the block above
-                        float ex, ez, ey, kx, kz;
-                        uint32_t at;
-                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4+" MV_TAB_SKIP "];" : "=f"(ex), "=f"(ez), "=f"(ey), "=r"(at) : "r"(tab));
-                        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2+" MV_TAB_SKIP2 "];" : "=f"(kx), "=f"(kz) : "r"(tab));
-                        const float ts = min3f(fmaf(ex, dtx, t0x), fmaf(ez, dtz, t0z), fmaf(ey, dty, t0y)) * kSkipMargin;
-                        const float nx = __fadd_rd(fmaf(ts, fabsf(dx), kx), 8388608.0f), nz = __fadd_rd(fmaf(ts, fabsf(dz), kz), 8388608.0f);
-                        pos = at + __float_as_uint(nx) * (uint32_t)sx + __float_as_uint(nz) * (uint32_t)sz;
-                        t0x = fmaf(nx - 8388608.0f, dtx, t0x);
-                        t0z = fmaf(nz - 8388608.0f, dtz, t0z);
-                    }
+                    // (crossing times are sums: the exit time is pulled in by the rounding that can pile up in them)
+                    t0x = qx * dtx;
+                    t0y = qy * dty;
+                    t0z = qz * dtz;
+                    const int cx = (int)floorf(Px), cy = (int)floorf(Py), cz = (int)floorf(Pz);
+                    t_exit = min3f(fmaf((float)(ngx ? cx - lox : hix - 1 - cx), dtx, t0x), fmaf((float)(ngy ? cy - loy : hiy - 1 - cy), dty, t0y),
+                                   fmaf((float)(ngz ? cz - loz : hiz - 1 - cz), dtz, t0z)) * p.exit_scale;
+                    // the first stretch, as in the block above
+                    const float ts = min3f(fmaf(ex, dtx, t0x), fmaf(ez, dtz, t0z), fmaf(ey, dty, t0y)) * kSkipMargin;
+                    const float nx = __fadd_rd(fmaf(ts, fabsf(dx), kx), 8388608.0f), nz = __fadd_rd(fmaf(ts, fabsf(dz), kz), 8388608.0f);
+                    pos = at + __float_as_uint(nx) * (uint32_t)sx + __float_as_uint(nz) * (uint32_t)sz;
+                    t0x = fmaf(nx - 8388608.0f, dtx, t0x);
+                    t0z = fmaf(nz - 8388608.0f, dtz, t0z);
+                    if (aflags & kAgentFilled) { row = inside_row; t_exit = -kInf; }
                 } else {
                     // eye outside the occupied box: clip the ray to it, start in the entry cell
-                    const bool ngx = dx < 0.0f, ngy = dy < 0.0f, ngz = dz < 0.0f;
                     const float x1 = (flox - Px) * ix, x2 = (fhix - Px) * ix;
                     const float y1 = (floy - Py) * iy, y2 = (fhiy - Py) * iy;
                     const float z1 = (floz - Pz) * iz, z2 = (fhiz - Pz) * iz;
@@ -822,14 +833,14 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     // entered through the box face of axis eaxis, or the eye is inside a solid
                     if (filled) {
                         if (eaxis < 0) row = inside_row;
-                        else asm volatile("ld.shared.u32 %0, [%1+" MV_TAB_ROW "];" : "=r"(row) : "r"(tab + 16u * (uint32_t)eaxis));
+                        else asm volatile("ld.shared.u32 %0, [%1+" MV_TAB_ROW "];" : "=r"(row) : "r"(tab + (eaxis == 0 ? 0u : (eaxis == 1 ? 8u : 4u))));
                     }
                     if (!alive || filled) t_exit = -kInf;
                 }
 #define MV_DDA_IO                                                                                         \
                     : "+r"(pos), "+r"(bit), "+f"(t_hit), "+r"(row)                                                  \
                     : "f"(t0x), "f"(t0y), "f"(t0z), "f"(dtx), "f"(dty), "f"(dtz), "r"(sx), "r"(sy), "r"(sz), "f"(t_exit), \
-                      "r"(p.max_steps), "r"(tab), "l"(s_occ)                                                       \
+                      "r"(0), "r"(tab), "l"(s_occ)                                                       \
                     : "memory"
 #define MV_DDA_IN                                                                                         \
                     " mov.b32 pos, %0;\n mov.b32 bit, %1;\n mov.f32 thit, %2;\n"                                    \
@@ -837,7 +848,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mov.f32 dtz, %9;\n mov.b32 sx, %10;\n mov.b32 sy, %11;\n mov.b32 sz, %12;\n mov.f32 texit, %13;\n" \
                     " mov.s32 it, " MV_STEP_BUDGET ";\n mov.b64 gbase, %16;\n"
 #define MV_DDA_OUTS                                                                                       \
-                    " selp.u32 a, 16, 32, py;\n selp.u32 a, 0, a, px;\n add.u32 a, a, %15;\n"                        \
+                    " selp.u32 a, 8, 4, py;\n selp.u32 a, 0, a, px;\n add.u32 a, a, %15;\n"                        \
                     " @ph ld.shared.u32 %3, [a+" MV_TAB_ROW "];\n mov.b32 %0, pos;\n mov.b32 %1, bit;\n mov.f32 %2, thit;\n"
                 if constexpr (COLW) {
                     asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_COLW) MV_DDA_OUTS "}\n" MV_DDA_IO);
@@ -850,7 +861,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
 #undef MV_DDA_IN
 #undef MV_DDA_OUTS
                 if (row == kNoRow) t_hit = kInf;          // no voxel hit
-                finish_tile(tile_p, mask_p, tile_px, pos, bit, row, sgn3, t_hit, dtx, dty, dtz);
+                finish_tile(mask_p, tile_px, pos, bit, row, tab, t_hit, dtx, dty, dtz);
             }
         }
     }
