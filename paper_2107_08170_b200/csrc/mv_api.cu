@@ -67,7 +67,7 @@ struct mv_batch {
     bool has_cams = false;
     double kr = 0, ku = 0;
     uint32_t sky_rgbx = 0;
-    struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, agent_near_off, misc_off, bytes; };
+    struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, misc_off, bytes; };
     Smem smem{};                        // shared-memory layout of the render kernel for agents_per_cta
     int agents_per_cta = 1;             // observations one CTA renders: 1, or every agent of its env
     int threads = MV_NT;                // threads per CTA of the render kernel (fewer for CTAs with few tiles)
@@ -132,14 +132,8 @@ mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     m.agent_mask_off = m.agent_ov_off + (uint32_t)d.max_overlay_rects * 32;
     // per tile: the box-mask words, preceded by a summary word when there is more than one
     const uint32_t words_per_tile = b->mask_words > 1 ? (uint32_t)b->mask_words + 1 : 1u;
-    m.agent_near_off = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
-    uint32_t agent_bytes = m.agent_near_off;
-    if (!occ_shared) {                  // the columns around the eye, if there is room for them
-        const uint32_t near_bytes = round_up((2 * kSkipCells + 1) * (2 * kSkipCells + 1) * 4, 16);
-        if ((int64_t)m.agent_off + (int64_t)apc * round_up(agent_bytes + near_bytes, kAgentAlign) + 32 <= b->smem_max) agent_bytes += near_bytes;
-        else m.agent_near_off = 0;
-    }
-    m.agent_stride = apc > 1 ? round_up(agent_bytes, kAgentAlign) : round_up(agent_bytes, 16);
+    const uint32_t agent_bytes = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
+    m.agent_stride = apc > 1 ? round_up(agent_bytes, kAgentAlign) : agent_bytes;
     m.misc_off = m.agent_off + (uint32_t)apc * m.agent_stride;
     m.bytes = m.misc_off + 32;
     return m;
@@ -201,7 +195,7 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.miss_depth = b->desc.miss_depth;
     p.smem_tile_off = b->smem.tile_off; p.smem_agent_off = b->smem.agent_off; p.smem_misc_off = b->smem.misc_off;
     p.agent_stride = b->smem.agent_stride; p.agent_ov_off = b->smem.agent_ov_off;
-    p.agent_mask_off = b->smem.agent_mask_off; p.agent_near_off = b->smem.agent_near_off;
+    p.agent_mask_off = b->smem.agent_mask_off;
     p.agents_per_cta = b->agents_per_cta;
     p.max_steps = b->desc.grid_x + b->desc.grid_y + b->desc.grid_z + 3;
     // accumulated crossing times drift from the exact products by at most one rounding per step

@@ -74,7 +74,7 @@ struct RenderParams {
     // shared-memory offsets after the staged env block: tile table, per-agent blocks (ray table, camera record,
     // eye-relative boxes, then overlay rectangles and per-tile box masks at the offsets below), barrier and flag words
     uint32_t smem_tile_off, smem_agent_off, smem_misc_off;
-    uint32_t agent_stride, agent_ov_off, agent_mask_off, agent_near_off;
+    uint32_t agent_stride, agent_ov_off, agent_mask_off;
     const int4 *overlay;               // [O][max_overlay] 16-byte records, or null
     const int32_t *overlay_count;      // [O]
     int max_overlay;

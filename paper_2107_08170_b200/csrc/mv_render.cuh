@@ -33,6 +33,11 @@ __device__ __forceinline__ float fast_rcp(float x) {
 // Makes a value opaque to the optimiser at this point, so that it is held in a register from
 // here on instead of being recomputed at every use.
 template <typename T> __device__ __forceinline__ void keep(T &v) { asm volatile("" : "+r"(reinterpret_cast<uint32_t &>(v))); }
+// The same for the assembler, which would rebuild a cheap value at every use: a shuffle it has to take as it comes.
+template <typename T> __device__ __forceinline__ void opaque(T &v, int lane) {
+    uint32_t &u = reinterpret_cast<uint32_t &>(v);
+    asm volatile("shfl.sync.idx.b32 %0, %0, %1, 31, 0xffffffff;" : "+r"(u) : "r"(lane));
+}
 template <typename T> __device__ __forceinline__ void keep64(T *&v) { asm volatile("" : "+l"(v)); }
 __device__ __forceinline__ float min3f(float a, float b, float c) {
     float r;
@@ -153,7 +158,7 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 constexpr uint32_t kAgentInside = 1u;      // eye inside the occupied cell box
 constexpr uint32_t kAgentBad = 2u;         // non-finite camera: sky frame
 constexpr uint32_t kAgentFilled = 4u;      // the eye's own voxel is filled
-constexpr uint32_t kAgentSealed = 8u;      // eye inside, not in a filled voxel, and some height lies outside the box: the common case
+constexpr uint32_t kAgentSealed = 8u;      // the common case: eye inside, not in a filled voxel, some height outside the box, not too large a grid
 // Per-agent block in shared memory.  First the ray table, one 64-byte entry per combination of direction signs (x negative:
 // +64, y: +128, z: +256; the block is 512-byte aligned, so an entry's address is the block's OR-ed with the sign bits):
 //   {distance (>= 0) from the eye to the cell face met first, in x and z; what a step in x and z adds to the position}
@@ -163,9 +168,9 @@ constexpr uint32_t kAgentSealed = 8u;      // eye inside, not in a filled voxel,
 //   {colour-table row of the face entered by an x, z, y step; -}
 // then the record {Fx, Rx, Fz, Rz} {Ux, Uz, Fy, Uy} {start bit mask, heights outside the occupied box, flags, self box} {eye
 // x, y, z, overlay count} {64-bit address of the env's material store, biased for the walk's positions; sky colour; miss
-// depth}, eye-relative boxes, overlay rectangles and per-tile box masks at offsets the host lays out.
+// depth} {lower corner of the occupied box, -} {upper corner, -}, eye-relative boxes, overlay rectangles and per-tile box masks at offsets the host lays out.
 constexpr uint32_t kAgentTabBytes = 512, kAgentAlign = 512;
-constexpr uint32_t kAgentRecVecs = 5;
+constexpr uint32_t kAgentRecVecs = 7;
 constexpr uint32_t kAgentRelOff = kAgentTabBytes + 16u * kAgentRecVecs;
 // (as text, for the PTX blocks)
 #define MV_TAB_SKIP "16"
@@ -175,6 +180,9 @@ constexpr uint32_t kAgentRelOff = kAgentTabBytes + 16u * kAgentRecVecs;
 #define MV_REC_UY "528"
 #define MV_REC_START "544"
 #define MV_REC_MAT "576"
+// a hit is looked at again if the ray leaves the cell within this factor of the time of the hit (1 - 2^-13)
+#define MV_GRAZE "0f3F7FF800"
+constexpr float kSealedScale = 1.0f - 1e-4f;       // least exit_scale for which that factor is wide enough
 // hard bound of the traversal loop: no grid allows more steps than 3 x 1024 + 3
 #define MV_STEP_BUDGET "3080"
 // The empty box that a walk starts with (see the table's construction) grows by at most this many cells an axis.
@@ -287,7 +295,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                         const int t = ty * p.tiles_x + tx;
                         uint32_t *tm = agent_mask(ag) + t * ms;
                         atomicOr(tm + m0 + (p.max_boxes >> 5), 1u << (p.max_boxes & 31));
-                        if (mw > 1) atomicOr(tm, 1u);
+                        if (mw > 1) *tm = 1u;
                     }
         }
     }
@@ -329,20 +337,6 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         const uint32_t u = voxel_index(p.lay, cx, cy, cz);
         return (s_occ[u >> 5] >> (u & 31)) & 1u;
     };
-    // (with the occupancy in global memory the columns around the eye are fetched first, all at once)
-    constexpr int kNear = 2 * kSkipCells + 1;
-    auto agent_near = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_near_off); };
-    if (!OCC_SHARED && p.agent_near_off) {
-        for (int i = tid; i < apc * kNear * kNear; i += NT) {
-            const int ag = i / (kNear * kNear), c = i - ag * kNear * kNear, dz = c / kNear - kSkipCells, dx = c % kNear - kSkipCells;
-            const float4 c0 = agent_rec(ag)[3];
-            if (!(c0.x >= 0.0f && c0.x < (float)gx && c0.y >= 0.0f && c0.y < (float)p.gy && c0.z >= 0.0f && c0.z < (float)gz)) continue;
-            const int x = (int)floorf(c0.x) + dx, z = (int)floorf(c0.z) + dz;
-            if (x >= 0 && x < gx && z >= 0 && z < gz)
-                agent_near(ag)[c] = s_occ[((size_t)column_index(p.lay, x, z) << (p.lay.ysh - 5)) + ((int)floorf(c0.y) >> 5)];
-        }
-        __syncthreads();
-    }
     // Where the eye is, in the terms of the walk's tables.
     auto eye_cell = [&](const float4 &c0, int &cx, int &cy, int &cz) -> bool {
         const bool in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
@@ -373,109 +367,116 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             rec[2].x = __uint_as_float(1u << (cy & 31));
             rec[2].y = __uint_as_float(guard);                   // heights outside the occupied box
             rec[2].z = __uint_as_float(__float_as_uint(rec[2].z) | (cam_in ? kAgentInside : 0u) | (filled ? kAgentFilled : 0u) |
-                                       (cam_in && !filled && guard ? kAgentSealed : 0u));
+                                       (cam_in && !filled && guard && p.exit_scale > kSealedScale ? kAgentSealed : 0u));
             const unsigned long long mp = reinterpret_cast<unsigned long long>(p.mat + (size_t)env * p.mat_stride - vi_bias);
             rec[4] = make_float4(__uint_as_float((uint32_t)mp), __uint_as_float((uint32_t)(mp >> 32)),
                                  __uint_as_float(p.sky_rgbx), p.miss_depth);
+            rec[5] = make_float4((float)lox, (float)loy, (float)loz, 0.0f);
+            rec[6] = make_float4((float)hix, (float)hiy, (float)hiz, 0.0f);
         }
     }
-    // The first stretch of a walk.  For every combination of signs: a box of empty cells that begins at the eye's cell and is
-    // grown greedily the way such rays go (x, z, y in turn, while the next layer of cells is empty).  A ray crosses
-    // nothing filled before it leaves that box, so it takes all its x and z crossings up to then at once, whatever their
-    // order (three steps of seven on average; the vertical ones are too few to be worth it): 234 -> 220 instructions a tile
-    // on 128x32x128 columns, 1230 -> 1184 us for 16384 observations; 64x16x64 rooms with boxes 1126 -> 1007 us.
-    // A warp per agent, four lanes per combination: a layer's cells are read by all four, and votes tell whether it is empty (the
-    // rounds depend on one another, so their latency is what counts; each lane keeps the columns that it has seen).
+    // The first stretch of a walk.  For every combination of signs: a box of empty cells that begins at the eye's cell.  A ray
+    // crosses nothing filled before it leaves that box, so it takes all its x and z crossings up to then at once, whatever
+    // their order (three steps of seven on average; the vertical ones are too few to be worth it): 234 -> 220
+    // instructions a tile on 128x32x128 columns, 1230 -> 1184 us for 16384 observations; 64x16x64 rooms with boxes
+    // 1126 -> 1007 us.
+    // A warp per agent, eight lanes per quadrant, each with a row of cells at the eye's height: the empty cells at its
+    // beginning, the least of them over the rows up to it, and of those rectangles the one with the longest shorter side; then
+    // as many layers above and below as are empty over all of it.  (Growing the boxes layer by layer gives the same ones
+    // within 1 %, but ten rounds that depend on one another were the longest part of a CTA's set-up: 5000 to 7000 cycles.)
     for (int ag = (warp + kWarps - 2) % kWarps; ag < apc; ag += kWarps) {
-        const int signs = lane >> 2, part = lane & 3;
-        const unsigned group = 0xfu << (lane & 28);
+        const int j = lane & 7, dx = (lane & 8) ? -1 : 1, dz = (lane & 16) ? -1 : 1;
         const float4 c0 = agent_rec(ag)[3];
         int cx, cy, cz;
         const bool cam_in = eye_cell(c0, cx, cy, cz);
-        const int dx = (signs & 1) ? -1 : 1, dy = (signs & 2) ? -1 : 1, dz = (signs & 4) ? -1 : 1;
-        const int wsh = p.lay.ysh - 5, yb = cy & 31;
-        const uint32_t *word = OCC_SHARED ? s_occ + ((column_index(p.lay, cx, cz) << wsh) + (cy >> 5)) : agent_near(ag) + kSkipCells * (kNear + 1);
-        const int step_x = OCC_SHARED ? dx << wsh : dx, step_z = OCC_SHARED ? (pitch * dz) << wsh : kNear * dz;
-        // (an eye exactly on a cell face and looking down the axis leaves its cell at once: one more for it, so that
-        // mirrored views get mirrored boxes)
+        // (an eye exactly on a cell face and looking down the axis leaves its cell at once: the rectangle begins a cell
+        // further on, so that mirrored views get mirrored boxes)
         const int on_x = dx < 0 && c0.x == (float)cx ? 1 : 0, on_z = dz < 0 && c0.z == (float)cz ? 1 : 0;
-        const int lim_x = min(kSkipCells - 1 + on_x, dx < 0 ? cx - lox : hix - 1 - cx);
-        const int lim_z = min(kSkipCells - 1 + on_z, dz < 0 ? cz - loz : hiz - 1 - cz);
-        const int lim_y = min(min(kSkipCellsY, dy < 0 ? cy - loy : hiy - 1 - cy), dy < 0 ? yb : 31 - yb);
-        // (eye outside or in a filled voxel, or no room for the columns: the box stays a single cell)
-        const bool blind = !cam_in || (!OCC_SHARED && !p.agent_near_off);
-        uint32_t seen = blind ? ~0u : word[0], ys = 1u << yb;      // columns of the box or-ed together; its heights
-        int ex = 0, ey = 0, ez = 0;
-        bool gox = !(seen & ys) && lim_x > 0, goz = !(seen & ys) && lim_z > 0, goy = !(seen & ys);
-        if (gox && on_x) { const uint32_t f = word[step_x]; gox = !(f & ys); if (gox) { seen |= f; ex = 1; } }
-        if (goz && on_z) {
-            const uint32_t f = word[step_z] | (ex ? word[step_x + step_z] : 0u);
-            goz = !(f & ys);
-            if (goz) { seen |= f; ez = 1; }
-        }
-        while (__any_sync(0xffffffffu, gox || goy || goz)) {
-            // the next layers in x and z and the corner between them, all loads of a round in flight at once
-            gox = gox && ex < lim_x;
-            goz = goz && ez < lim_z;
-            const uint32_t *px = word + (ex + 1) * step_x, *pz = word + (ez + 1) * step_z;
-            uint32_t fx = 0, fz = 0, corner = 0;
+        const int bx = cx + dx * on_x, bz = cz + dz * on_z;
+        const int lim_x = min(kSkipCells - 1, dx < 0 ? bx - lox : hix - 1 - bx), lim_z = dz < 0 ? bz - loz : hiz - 1 - bz;
+        const int wsh = p.lay.ysh - 5, yb = cy & 31;
+        const uint32_t *word = s_occ + (((int)column_index(p.lay, bx, bz + dz * j) << wsh) + (cy >> 5));
+        const bool row_in = cam_in && j <= lim_z;
+        uint32_t col[kSkipCells], filled = ~0u << kSkipCells, seen = 0;
 #pragma unroll
-            for (int i = 0; i <= kSkipCells; i += 4) {
-                if (gox && i + part <= ez) fx |= px[(i + part) * step_z];
-                if (goz && i + part <= ex) fz |= pz[(i + part) * step_x];
-            }
-            if (gox && goz) corner = px[(ez + 1) * step_z];
-            const unsigned full_x = __ballot_sync(0xffffffffu, (fx & ys) != 0u);
-            gox = gox && !(full_x & group);
-            if (gox) { seen |= fx; fz |= corner; ++ex; }
-            const unsigned full_z = __ballot_sync(0xffffffffu, (fz & ys) != 0u);
-            goz = goz && !(full_z & group);
-            if (goz) { seen |= fz; ++ez; }
-            const uint32_t b = 1u << ((yb + dy * (ey + 1)) & 31);
-            const unsigned full_y = __ballot_sync(0xffffffffu, (seen & b) != 0u);
-            goy = goy && ey < lim_y && !(full_y & group);
-            if (goy) { ys |= b; ++ey; }
+        for (int i = 0; i < kSkipCells; ++i) {
+            col[i] = row_in && i <= lim_x ? word[(dx * i) * (1 << wsh)] : ~0u;
+            filled |= ((col[i] >> yb) & 1u) << i;
         }
-        if (part == 0) {
+        int w = __ffs(filled) - 1;                               // empty cells at the row's beginning
+#pragma unroll
+        for (int s = 1; s < 8; s <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, w, s, 8);
+            if (j >= s) w = min(w, o);
+        }
+        // longest shorter side first, then the longer one; the extents ride along
+        int key = w > 0 ? min(w - 1, j) << 12 | max(w - 1, j) << 8 | (w - 1) << 4 | j : -1;
+#pragma unroll
+        for (int s = 1; s < 8; s <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, s));
+        const bool any = key >= 0;
+        const int rx = any ? (key >> 4) & 15 : 0, rz = any ? key & 15 : 0;
+#pragma unroll
+        for (int i = 0; i < kSkipCells; ++i)
+            if (i <= rx && j <= rz) seen |= col[i];
+#pragma unroll
+        for (int s = 1; s < 8; s <<= 1) seen |= __shfl_xor_sync(0xffffffffu, seen, s);
+        if (j < 2) {                                             // lane 0 of the quadrant: upward, lane 1: downward
+            const int dy = j ? -1 : 1;
+            // empty layers next to the eye's, from the columns or-ed together (the bit beyond the word counts as filled)
+            const uint32_t beyond = dy > 0 ? (yb < 31 ? seen >> (yb + 1) | 0x80000000u >> yb : 1u)
+                                           : (yb > 0 ? __brev(seen << (32 - yb)) | 1u << yb : 1u);
+            const int ey = any ? min(min(kSkipCellsY, __ffs(beyond) - 1), dy < 0 ? cy - loy : hiy - 1 - cy) : 0;
+            const int ex = any ? rx + on_x : 0, ez = any ? rz + on_z : 0;
             const int sx = COLW ? 4 * dx : dx * stride_x, sz = COLW ? 4 * pitch * dz : dz * stride_z;
+            const int signs = (dx < 0 ? 1 : 0) | (dy < 0 ? 2 : 0) | (dz < 0 ? 4 : 0);
             agent_tab(ag)[4 * signs + 1] = make_float4((float)ex, (float)ez, (float)ey, __uint_as_float(cell_pos(cx, cy, cz) -
                                                        kSkipBias * (uint32_t)sx - kSkipBias * (uint32_t)sz));
         }
     }
+    // Boxes: relative to the eye, and binned by the bounding rectangle of their projected corners (conservative, so every box
+    // that a pixel's ray can touch is tested for that pixel).  Four lanes to a box, two corners and every fourth row of
+    // tiles each; dealt from the last warp down, away from the warps that build the tables above.
     {
-        const int nb = min(s_count[0], p.max_boxes);
-        // (dealt from the last thread down, so that the warps that build the DDA tables above are not
-        // the ones that bin the boxes)
-        for (int i = NT - 1 - tid; i < apc * p.max_boxes; i += NT) {
-            const int ag = i / p.max_boxes, b = i - ag * p.max_boxes;
+        const int nb = min(s_count[0], p.max_boxes), part = lane & 3;
+        for (int i0 = 0; i0 < 4 * apc * p.max_boxes; i0 += NT) {
+            const int i = (i0 + (kWarps - 1 - warp) * 32 + lane) >> 2;
+            if ((i & ~7) >= apc * p.max_boxes) break;            // (the whole warp)
+            const int ag = apc == 1 ? 0 : min(i / p.max_boxes, apc - 1), b = min(i - ag * p.max_boxes, p.max_boxes - 1);
             const float4 *rec = agent_rec(ag);
             const float4 c0 = rec[0], c1 = rec[1], P4 = rec[3];
             const float Px = P4.x, Py = P4.y, Pz = P4.z, Fx = c0.x, Fy = c1.z, Fz = c0.z;
-            const float Rx = c0.y, Ry = 0.0f, Rz = c0.w, Ux = c1.x, Uy = c1.w, Uz = c1.y;       // (cameras do not roll)
+            const float Rx = c0.y, Rz = c0.w, Ux = c1.x, Uy = c1.w, Uz = c1.y;       // (cameras do not roll: Ry = 0)
             const int self_box = __float_as_int(rec[2].w);
-            const float r2 = Rx * Rx + Ry * Ry + Rz * Rz, u2 = Ux * Ux + Uy * Uy + Uz * Uz;
-            const float ir2 = 1.0f / r2, iu2 = 1.0f / u2;
+            const float ir2 = fast_rcp(Rx * Rx + Rz * Rz), iu2 = fast_rcp(Ux * Ux + Uy * Uy + Uz * Uz);
             const float4 A = s_box[2 * b], B = s_box[2 * b + 1];
             const float lx = A.x - Px, ly = A.y - Py, lz = A.z - Pz;
             const float hx = A.w - Px, hy = B.x - Py, hz = B.y - Pz;
-            const bool valid = (b < nb) && (b != self_box) && (A.x < A.w) && (A.y < B.x) && (A.z < B.y);
+            const bool valid = (b < nb) && (b != self_box) && (A.x < A.w) && (A.y < B.x) && (A.z < B.y) && i < apc * p.max_boxes;
             float tmin = kInf, tmax = -kInf, fxmin = kInf, fxmax = -kInf, fymin = kInf, fymax = -kInf;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float vx = (c & 1) ? hx : lx, vy = (c & 2) ? hy : ly, vz = (c & 4) ? hz : lz;
+            for (int c = 0; c < 2; ++c) {
+                const float vx = (part & 1) ? hx : lx, vy = c ? hy : ly, vz = (part & 2) ? hz : lz;
                 const float t = vx * Fx + vy * Fy + vz * Fz;
-                const float u = (vx * Rx + vy * Ry + vz * Rz) * ir2;
+                const float u = (vx * Rx + vz * Rz) * ir2;
                 const float w = (vx * Ux + vy * Uy + vz * Uz) * iu2;
                 tmin = fminf(tmin, t); tmax = fmaxf(tmax, t);
-                const float it = 1.0f / fmaxf(t, 1e-3f);
+                const float it = fast_rcp(fmaxf(t, 1e-3f));
                 const float fx = (u * it + (float)(W - 1)) * 0.5f;     // pixel column of the projection
                 const float fy = ((float)(H - 1) - w * it) * 0.5f;     // pixel row
                 fxmin = fminf(fxmin, fx); fxmax = fmaxf(fxmax, fx);
                 fymin = fminf(fymin, fy); fymax = fmaxf(fymax, fy);
             }
+#pragma unroll
+            for (int s = 1; s < 4; s <<= 1) {
+                tmin = fminf(tmin, __shfl_xor_sync(0xffffffffu, tmin, s)); tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, s));
+                fxmin = fminf(fxmin, __shfl_xor_sync(0xffffffffu, fxmin, s)); fxmax = fmaxf(fxmax, __shfl_xor_sync(0xffffffffu, fxmax, s));
+                fymin = fminf(fymin, __shfl_xor_sync(0xffffffffu, fymin, s)); fymax = fmaxf(fymax, __shfl_xor_sync(0xffffffffu, fymax, s));
+            }
             const bool front = tmin > 0.05f;                 // whole box safely in front of the eye plane
-            agent_rel(ag)[2 * b] = make_float4(lx, ly, lz, front ? tmin * 0.9999f : 0.0f);
-            agent_rel(ag)[2 * b + 1] = make_float4(hx, hy, hz, B.z);
+            if (part == 0 && valid) {
+                agent_rel(ag)[2 * b] = make_float4(lx, ly, lz, front ? tmin * 0.9999f : 0.0f);
+                agent_rel(ag)[2 * b + 1] = make_float4(hx, hy, hz, B.z);
+            }
             if (!valid || tmax < -1e-3f) continue;           // ignored, or wholly behind the eye
             int px0 = 0, px1 = W - 1, py0 = 0, py1 = H - 1;
             if (front) {
@@ -487,13 +488,12 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             }
             const uint32_t bit = 1u << (b & 31);
             uint32_t *mask = agent_mask(ag);
-            for (int ty = py0 >> 2; ty <= (py1 >> 2); ++ty)
-                for (int tx = px0 >> 3; tx <= (px1 >> 3); ++tx)
-                    {
-                        uint32_t *tm = mask + (ty * p.tiles_x + tx) * ms;
-                        atomicOr(tm + m0 + (b >> 5), bit);
-                        if (mw > 1) atomicOr(tm, bit);          // the summary word only has to be non-zero
-                    }
+            for (int ty = (py0 >> 2) + part; ty <= (py1 >> 2); ty += 4)
+                for (int tx = px0 >> 3; tx <= (px1 >> 3); ++tx) {
+                    uint32_t *tm = mask + (ty * p.tiles_x + tx) * ms;
+                    atomicOr(tm + m0 + (b >> 5), bit);
+                    if (mw > 1) *tm = 1u;                           // the summary word only has to be non-zero
+                }
         }
     }
     __syncthreads();
@@ -514,11 +514,11 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     uint32_t st_sel = st_byte == 0 ? 0x4210u : (st_byte == 1 ? 0x5421u : (st_byte == 2 ? 0x6542u : 0xffffffffu));
     const int depth_lane_off = (lane >> 3) * W + (lane & 7);
     const int rgb_lane_off = st_r * W * 3 + st_j * 4;
-    keep(lane_a); keep(lane_b); keep(st_sel);
+    opaque(lane_a, lane); opaque(lane_b, lane); opaque(st_sel, lane);
     const uint32_t tile_begin = smem_addr(s_tile) + 16u * (uint32_t)(tile0 + warp);
     uint32_t tile_end = smem_addr(s_tile) + 16u * (uint32_t)tile1;
     uint32_t mask_step = 4u * kWarps * (uint32_t)ms;                        // bytes between a warp's consecutive tile masks
-    keep(tile_end); keep(mask_step);
+    opaque(tile_end, lane); opaque(mask_step, lane);
 
     for (int ag = 0; ag < apc; ++ag) {
         const int obs = obs0 + ag;
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         // follows the walk is the same for both.  The warp-wide reduction and shuffle in it name all 32
         // lanes, so they wait by themselves for lanes whose walk ran longer.
         auto finish_tile = [&](uint32_t mask_p, int tile_px, uint32_t pos, uint32_t bit, uint32_t row,
-                               uint32_t tab, float t_hit, float dtx, float dty, float dtz) {
+                               uint32_t tab, uint32_t graze, float t_hit, float dtx, float dty, float dtz) {
             // ---- the hit voxel's material byte is asked for from global memory (its colour is looked up
             // in the shaded table only in the store block, after everything that does not need it), this
             // tile's first box-mask word is read, and the latest voxel hit of the warp is found (boxes wholly
@@ -579,8 +579,17 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
 
             // ---- the less common work, behind one test: boxes binned to this tile, and the GUI overlay (the bit behind the
             // boxes').  A box wins only with a strictly smaller time; boxes wholly behind the warp's latest voxel hit are skipped.
-            if (m != 0u) {
-                {
+            if ((m | graze) != 0u) {
+                // A voxel that the ray enters within the rounding of crossing times before it leaves the occupied box does not
+                // count (see exit_scale).  The ray leaves the box no earlier than the voxel, so that can only be where it leaves
+                // the voxel again almost at once: one ray in a thousand, and only for those the exit time is worked out.
+                if (graze) {
+                    const float4 eye = agent_rec(ag)[3], lo = agent_rec(ag)[5], hi = agent_rec(ag)[6];
+                    const float t_exit = min3f(((tab & 64u) ? eye.x - lo.x : hi.x - eye.x) * dtx, ((tab & 128u) ? eye.y - lo.y : hi.y - eye.y) * dty,
+                                               ((tab & 256u) ? eye.z - lo.z : hi.z - eye.z) * dtz) * p.exit_scale;
+                    if (!(t_hit < t_exit)) { row = kNoRow; t_hit = kInf; rgbx = p.sky_rgbx; depth = p.miss_depth; }
+                }
+                if (m != 0u) {
                     const float wmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(t_hit)));
                     float tb = t_hit;
                     bool gui = false;
@@ -667,7 +676,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         if (COLW && (aflags & kAgentSealed)) {
             for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
                 int tile_px;
-                uint32_t pos, bit = 0, row, tab;
+                uint32_t pos, bit = 0, row, tab, graze;
                 float t_hit, dtx, dty, dtz;
                 // ---- the common case in one block of PTX: tile record, ray through the pixel centre
                 // (d = F + a*Rs + b*Us, a = 2px+1-W, b = H-1-2py, two chained FMAs per component),
@@ -684,12 +693,12 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " .reg .f32 Ta, Tb, Fx, Fy, Fz, Rx, Rz, Ux, Uy, Uz, ca, cb, dx, dy, dz, ix, iy, iz;\n"
                     " .reg .f32 q0, q1, q2, q3, q4;\n"
                     " .reg .b32 u, v;\n"
-                    " ld.shared.v4.b32 {Ta, Tb, %0, _}, [%9];\n"
-                    " ld.shared.v4.f32 {Fx, Rx, Fz, Rz}, [%10+" MV_REC_FR "];\n"
-                    " ld.shared.v4.f32 {Ux, Uz, Fy, Uy}, [%10+" MV_REC_UY "];\n"
-                    " ld.shared.v2.b32 {bit, guard}, [%10+" MV_REC_START "];\n"
-                    " add.f32 ca, Ta, %11;\n"
-                    " sub.f32 cb, Tb, %12;\n"
+                    " ld.shared.v4.b32 {Ta, Tb, %0, _}, [%10];\n"
+                    " ld.shared.v4.f32 {Fx, Rx, Fz, Rz}, [%11+" MV_REC_FR "];\n"
+                    " ld.shared.v4.f32 {Ux, Uz, Fy, Uy}, [%11+" MV_REC_UY "];\n"
+                    " ld.shared.v2.b32 {bit, guard}, [%11+" MV_REC_START "];\n"
+                    " add.f32 ca, Ta, %12;\n"
+                    " sub.f32 cb, Tb, %13;\n"
                     " fma.rn.f32 dx, ca, Rx, Fx;\n"
                     " fma.rn.f32 dz, ca, Rz, Fz;\n"
                     " fma.rn.f32 dy, cb, Uy, Fy;\n"
@@ -704,7 +713,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mov.b32 u, dx;\n"
                     " mov.b32 v, dz;\n"
                     " prmt.b32 u, u, v, 0x00FB;\n"                  // byte 0: sign of dx, byte 1: sign of dz
-                    " lop3.b32 %8, u, 0x140, %10, 0xEA;\n"
+                    " lop3.b32 %8, u, 0x140, %11, 0xEA;\n"
                     " mov.b32 u, dy;\n"
                     " shr.u32 u, u, 24;\n"
                     " lop3.b32 %8, u, 0x80, %8, 0xEA;\n"
@@ -736,6 +745,11 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " or.b32 w, w, bit;\n"
                     " and.b32 w, w, guard;\n"
                     " setp.eq.u32 ph, w, 0;\n"
+                    // (a hit that may be too close to the ray's exit from the box: see below)
+                    " min.f32 ta, tx, ty, tz;\n"
+                    " mul.f32 ta, ta, " MV_GRAZE ";\n"
+                    " setp.ge.and.f32 pq, thit, ta, ph;\n"
+                    " selp.u32 %9, 1, 0, pq;\n"
                     " mov.b32 %4, 0xffffffff;\n"
                     " @!ph mov.f32 thit, 0f7F800000;\n"
                     " mov.b32 u, %8;\n"
@@ -749,10 +763,10 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mov.f32 %6, dty;\n"
                     " mov.f32 %7, dtz;\n"
                     "}\n"
-                    : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab)
+                    : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze)
                     : "r"(tile_p), "r"(abase), "f"(lane_a), "f"(lane_b)
                     : "memory");
-                finish_tile(mask_p, tile_px, pos, bit, row, tab, t_hit, dtx, dty, dtz);
+                finish_tile(mask_p, tile_px, pos, bit, row, tab, graze, t_hit, dtx, dty, dtz);
             }
         } else {
             const float4 P4 = agent_rec(ag)[3];
@@ -861,7 +875,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
 #undef MV_DDA_IN
 #undef MV_DDA_OUTS
                 if (row == kNoRow) t_hit = kInf;          // no voxel hit
-                finish_tile(mask_p, tile_px, pos, bit, row, tab, t_hit, dtx, dty, dtz);
+                finish_tile(mask_p, tile_px, pos, bit, row, tab, 0u, t_hit, dtx, dty, dtz);
             }
         }
     }
