@@ -139,6 +139,22 @@ mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     return m;
 }
 
+// Launch of a per-step kernel (see launch_dependents).
+template <typename... Params, typename... Args>
+cudaError_t launch_step(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Args &...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute overlap{};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Threads per CTA: the small shape for CTAs with few tiles, if the batch has CTAs enough to fill the GPU
 // six to an SM.
 int pick_threads(const mv_batch *b, int apc) {
@@ -208,18 +224,17 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     const int64_t ctas = obs_count / b->agents_per_cta;   // callers pass whole environments when a CTA renders one
     const int ntiles = b->tiles_x * b->tiles_y, parts = pick_parts(b, ctas);
     p.part_tiles = (ntiles + parts - 1) / parts;
-    render_fn(b)<<<dim3((unsigned)ctas, (unsigned)((ntiles + p.part_tiles - 1) / p.part_tiles)), b->threads, b->smem.bytes, s>>>(p);
+    MV_CUDA(b, launch_step(render_fn(b), dim3((unsigned)ctas, (unsigned)((ntiles + p.part_tiles - 1) / p.part_tiles)), dim3((unsigned)b->threads),
+                           b->smem.bytes, s, p));
     b->launches++;
-    MV_CUDA(b, cudaGetLastError());
     return MV_OK;
 }
 
 int launch_cameras(mv_batch *b, const mv_camera *d_cams, cudaStream_t s) {
     const int n = b->num_obs;
-    camera_kernel<<<(n + 127) / 128, 128, 0, s>>>(reinterpret_cast<const int32_t *>(d_cams), b->d_cams, n,
-                                                   b->kr, b->ku, b->d_status);
+    MV_CUDA(b, launch_step(camera_kernel, dim3((n + 127) / 128), dim3(128), 0, s, reinterpret_cast<const int32_t *>(d_cams), b->d_cams, n,
+                           b->kr, b->ku, b->d_status));
     b->launches++;
-    MV_CUDA(b, cudaGetLastError());
     b->has_cams = true;
     return MV_OK;
 }
@@ -248,9 +263,8 @@ int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int en
     if (pack + lut + box == 0) return MV_OK;
     if (pack + lut + box > 0x7fffffffull) return MV_ERR_INVALID_ARG;
     u.pack_ctas = (unsigned)pack; u.lut_ctas = (unsigned)lut;
-    upload_kernel<<<(unsigned)(pack + lut + box), kUploadThreads, pack ? kUploadSmem : 0, s>>>(u);
+    MV_CUDA(b, launch_step(upload_kernel, dim3((unsigned)(pack + lut + box)), dim3(kUploadThreads), pack ? kUploadSmem : 0, s, u));
     b->launches++;
-    MV_CUDA(b, cudaGetLastError());
     return MV_OK;
 }
 
@@ -551,10 +565,9 @@ int mv_set_overlays(mv_batch *b, const mv_overlay_rect *d_rects, const int32_t *
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
     const int n = b->num_obs * (m + 1);
-    copy_overlays_kernel<<<(n + 255) / 256, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        reinterpret_cast<const int4 *>(d_rects), d_count, b->d_overlay, b->d_overlay_count, b->num_obs, m);
+    MV_CUDA(b, launch_step(copy_overlays_kernel, dim3((n + 255) / 256), dim3(256), 0, static_cast<cudaStream_t>(cuda_stream),
+                           reinterpret_cast<const int4 *>(d_rects), d_count, b->d_overlay, b->d_overlay_count, b->num_obs, m));
     b->launches++;
-    MV_CUDA(b, cudaGetLastError());
     return MV_OK;
 }
 
@@ -570,12 +583,11 @@ int mv_move_agents(mv_batch *b, mv_camera *d_cams_inout, const mv_agent_move *d_
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
     const int n = b->num_obs;
-    move_agents_kernel<<<(n + 127) / 128, 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        reinterpret_cast<int32_t *>(d_cams_inout), reinterpret_cast<const float4 *>(d_moves), b->d_cams,
-        b->d_env_blocks, b->lay, n, b->desc.agents_per_env, b->desc.grid_x, b->desc.grid_y, b->desc.grid_z,
-        b->desc.max_boxes, sh.half_width, sh.below_eye, sh.above_eye, sh.max_pitch, b->kr, b->ku, b->d_status);
+    MV_CUDA(b, launch_step(move_agents_kernel, dim3((n + 127) / 128), dim3(128), 0, static_cast<cudaStream_t>(cuda_stream),
+                           reinterpret_cast<int32_t *>(d_cams_inout), reinterpret_cast<const float4 *>(d_moves), b->d_cams, b->d_env_blocks,
+                           b->lay, n, b->desc.agents_per_env, b->desc.grid_x, b->desc.grid_y, b->desc.grid_z, b->desc.max_boxes,
+                           sh.half_width, sh.below_eye, sh.above_eye, sh.max_pitch, b->kr, b->ku, b->d_status));
     b->launches++;
-    MV_CUDA(b, cudaGetLastError());
     b->has_cams = true;
     return MV_OK;
 }

@@ -113,4 +113,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 }
 constexpr int kDrainPolls = 1 << 26;               // bound of the wait for a copy known to be in flight
 
+// Programmatic dependent launch.  Every per-step kernel begins with launch_dependents, which lets the next kernel of the
+// stream that was launched with the attribute start once all CTAs of this one run, and waits for the previous kernel before it
+// touches global memory; so launch latency and CTA set-up overlap with what is still running, and nothing else changes.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 }  // namespace mv

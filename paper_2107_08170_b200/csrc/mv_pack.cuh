@@ -283,6 +283,8 @@ __device__ __forceinline__ void copy_boxes(const UploadArgs &p, unsigned cta)
 // Everything one upload brings, in one launch: the CTAs are dealt to the three jobs by number.
 __global__ void __launch_bounds__(kUploadThreads, 3) upload_kernel(const UploadArgs p)
 {
+    launch_dependents();
+    wait_for_previous();
     if (blockIdx.x < p.pack_ctas) pack_columns(p);
     else if (blockIdx.x < p.pack_ctas + p.lut_ctas) shade_palettes(p, blockIdx.x - p.pack_ctas);
     else copy_boxes(p, blockIdx.x - p.pack_ctas - p.lut_ctas);
@@ -314,6 +316,8 @@ __device__ __forceinline__ void write_camrec(CamRec *out, float px, float py, fl
 __global__ void camera_kernel(const int32_t *__restrict__ cams, CamRec *__restrict__ out, int num_obs,
                               double kr, double ku, uint32_t *status)
 {
+    launch_dependents();
+    wait_for_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= num_obs) return;
     const int32_t *c = cams + (size_t)o * 6;
@@ -351,6 +355,8 @@ __global__ void move_agents_kernel(int32_t *__restrict__ cams, const float4 *__r
                                    float hw, float below, float above, float max_pitch, double kr, double ku,
                                    uint32_t *status)
 {
+    launch_dependents();
+    wait_for_previous();
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= num_obs) return;
     int32_t *c = cams + (size_t)o * 6;
@@ -388,6 +394,8 @@ __global__ void copy_overlays_kernel(const int4 *__restrict__ rects, const int32
                                      int4 *__restrict__ out_rects, int32_t *__restrict__ out_counts, int num_obs,
                                      int max_rects)
 {
+    launch_dependents();
+    wait_for_previous();
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= num_obs * (max_rects + 1)) return;
     const int o = gid / (max_rects + 1), r = gid - o * (max_rects + 1);

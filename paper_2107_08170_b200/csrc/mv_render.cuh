@@ -194,7 +194,7 @@ constexpr float kSkipMargin = 1.0f - 1.52587890625e-5f;
 // The count comes out of an addition of 2^23, whose float's bits are 0x4B000000 + count.
 constexpr uint32_t kSkipBias = 0x4B000000u;
 #define MV_SKIP_MAGIC "0f4B000000"
-#define MV_SKIP_UNMAGIC "0fCB000000"
+#define MV_SKIP_UNMAGIC1 "0fCB000001"            // -(2^23 + 1)
 
 // One thread's share of a sky frame (non-finite camera).
 template <int NT>
@@ -245,14 +245,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     // (in a batch with few observations each one's tiles are split between the CTAs of a grid column)
     const int tile0 = blockIdx.y * p.part_tiles, tile1 = min(tile0 + p.part_tiles, ntiles);
 
-    // ---- stage the environment block
+    // ---- tile table, cleared masks (this much needs nothing from the kernels before)
     if (tid == 0) mbar_init(s_bar, 1);
-    __syncthreads();
-    if (tid == 0 && !p.skip_staging) {
-        mbar_expect_tx(s_bar, p.lay.block_bytes - unstaged);
-        bulk_load(smem, env_block + unstaged, p.lay.block_bytes - unstaged, s_bar);
-    }
-    // ---- meanwhile: tile table, cleared masks, camera records, GUI rectangles
     for (int ag = 0; ag < apc; ++ag) {
         uint32_t *mk = agent_mask(ag);
         for (int i = tile0 * ms + tid; i < tile1 * ms; i += NT) mk[i] = 0u;
@@ -265,6 +259,14 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         s_tile[i] = make_float4((float)(16 * tx + 1 - W), (float)(H - 1 - 8 * ty), __int_as_float(ty * 4 * W + tx * 8),
                                 __int_as_float(i));
     }
+    wait_for_previous();
+    // ---- stage the environment block
+    if (tid == 0 && !p.skip_staging) {
+        mbar_expect_tx(s_bar, p.lay.block_bytes - unstaged);
+        bulk_load(smem, env_block + unstaged, p.lay.block_bytes - unstaged, s_bar);
+    }
+    __syncthreads();
+    // ---- meanwhile: camera records, GUI rectangles
     for (int ag = tid; ag < apc; ag += NT) {
         const float4 *cq = reinterpret_cast<const float4 *>(p.cams + obs0 + ag);
         const float4 c0 = __ldg(cq), c1 = __ldg(cq + 1), c2 = __ldg(cq + 2), c3 = __ldg(cq + 3);   // P F | F R | R U | self, flags
@@ -736,10 +738,16 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mad.lo.u32 pos, u, sx, pos;\n"
                     " mov.b32 u, q4;\n"
                     " mad.lo.u32 pos, u, sz, pos;\n"
-                    " add.f32 q3, q3, " MV_SKIP_UNMAGIC ";\n"
-                    " add.f32 q4, q4, " MV_SKIP_UNMAGIC ";\n"
-                    " fma.rn.f32 tx, q3, dtx, tx;\n"
-                    " fma.rn.f32 tz, q4, dtz, tz;\n"
+                    // (the first crossing by an addition as in the walk and only the rest by a product, so that up to two crossings
+                    // give the bits that the walk would give and ties between axes go the same way)
+                    " setp.gt.f32 px, q3, " MV_SKIP_MAGIC ";\n"
+                    " setp.gt.f32 pz, q4, " MV_SKIP_MAGIC ";\n"
+                    " add.f32 q3, q3, " MV_SKIP_UNMAGIC1 ";\n"
+                    " add.f32 q4, q4, " MV_SKIP_UNMAGIC1 ";\n"
+                    " @px add.f32 tx, tx, dtx;\n"
+                    " @pz add.f32 tz, tz, dtz;\n"
+                    " @px fma.rn.f32 tx, q3, dtx, tx;\n"
+                    " @pz fma.rn.f32 tz, q4, dtz, tz;\n"
                     MV_DDA_SEALED
                     // a miss if the cell is fence (its guard bits are set) or lies at a height outside the box
                     " or.b32 w, w, bit;\n"
@@ -814,8 +822,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     const float ts = min3f(fmaf(ex, dtx, t0x), fmaf(ez, dtz, t0z), fmaf(ey, dty, t0y)) * kSkipMargin;
                     const float nx = __fadd_rd(fmaf(ts, fabsf(dx), kx), 8388608.0f), nz = __fadd_rd(fmaf(ts, fabsf(dz), kz), 8388608.0f);
                     pos = at + __float_as_uint(nx) * (uint32_t)sx + __float_as_uint(nz) * (uint32_t)sz;
-                    t0x = fmaf(nx - 8388608.0f, dtx, t0x);
-                    t0z = fmaf(nz - 8388608.0f, dtz, t0z);
+                    if (nx > 8388608.0f) t0x = fmaf(nx - 8388609.0f, dtx, t0x + dtx);
+                    if (nz > 8388608.0f) t0z = fmaf(nz - 8388609.0f, dtz, t0z + dtz);
                     if (aflags & kAgentFilled) { row = inside_row; t_exit = -kInf; }
                 } else {
                     // eye outside the occupied box: clip the ray to it, start in the entry cell
