@@ -31,10 +31,8 @@ constexpr int kHostChunks = 8;
 // (512 observations of 128x72 on 192x48x192: 112, 109, 115, 127 us with 1, 2, 4, 8 times); staged: once, as each one stages
 // the block again (4 of 64x36: 20.6 us with a CTA each, 12 with 6).
 constexpr int kPartWaves = 2;
-// Staging + set-up of a CTA, in units of one observation's render time, as measured on B200 at 128x72:
-// 0.15 to 0.18 for 64x16x64 grids, 0.10 for 128x32x128 grids (where a second agent's tables usually cost
-// the third resident CTA per SM, which the occupancy query below sees).
-constexpr double kCtaFixedCost = 0.15;
+// Staging + set-up of a CTA, in units of one observation's render time at 128x72 (measured: about 0.1).
+constexpr double kCtaFixedCost = 0.1;
 #ifndef MV_MERGE_SCRATCH_MB
 #define MV_MERGE_SCRATCH_MB 1024
 #endif
@@ -205,7 +203,7 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.gx = b->desc.grid_x; p.gy = b->desc.grid_y; p.gz = b->desc.grid_z;
     p.max_boxes = b->desc.max_boxes;
     p.palette = b->desc.palette_size;
-    p.W = b->desc.width; p.H = b->desc.height;
+    p.W = b->desc.width; p.H = b->desc.height; p.inv_W = 1.0f / (float)b->desc.width;
     p.tiles_x = b->tiles_x; p.tiles_y = b->tiles_y; p.mask_words = b->mask_words;
     p.sky_rgbx = b->sky_rgbx;
     p.miss_depth = b->desc.miss_depth;
@@ -253,8 +251,9 @@ int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int en
     auto ctas = [](size_t threads) { return (threads + kUploadThreads - 1) / kUploadThreads; };
     u.tiles_per_word = (int)ctas((size_t)(d.grid_x / 4) * d.grid_z);
     u.tiles_per_env = u.tiles_per_word * ((d.grid_y + 31) / 32);         // (words above grid_y stay zero)
-    // tiles a CTA packs one after the other: one, until there are four CTAs for every slot of the GPU
-    const int64_t per_slot = (int64_t)u.tiles_per_env * env_count / (3 * 4 * (int64_t)b->sms);
+    // tiles a CTA packs one after the other: one, until there are two CTAs for every slot of the GPU (164 / 512 envs of
+    // 128x32x128: 62 / 119 us with three CTAs of 256 threads per SM and four for every slot, 53 / 114 like this)
+    const int64_t per_slot = (int64_t)u.tiles_per_env * env_count / (12 * 2 * (int64_t)b->sms);
     u.tiles_per_cta = (int)(per_slot < 1 ? 1 : per_slot > 8 ? 8 : per_slot);
     u.pack_ctas_per_env = (u.tiles_per_env + u.tiles_per_cta - 1) / u.tiles_per_cta;
     const size_t pack = d_grid ? (size_t)u.pack_ctas_per_env * env_count : 0;
@@ -480,18 +479,19 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(upload_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUploadSmem);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
     // One CTA per environment (block staged once for all its agents) when that still fills the GPU;
-    // otherwise one CTA per observation.  Cost model: waves of resident CTAs x (agents + fixed part).
+    // otherwise one CTA per observation.  Cost model: work per slot and the wait for the last CTAs.
     if (d.agents_per_env > 1) {
         const mv_batch::Smem all = smem_layout(b, d.agents_per_env, b->occ_shared);    // (never give up staged occupancy for it)
         if ((int64_t)all.bytes <= smem_max) {
-            auto waves_cost = [&](const mv_batch::Smem &m, int apc) {
+            auto shape_cost = [&](const mv_batch::Smem &m, int apc) {
                 int per_sm = 0;
                 cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_fn(b), kRenderThreads, m.bytes);
                 if (q != cudaSuccess || per_sm < 1) return 1e30;
-                const double slots = (double)per_sm * sms, ctas = (double)b->num_obs / apc;
-                return std::ceil(ctas / slots) * (apc + kCtaFixedCost);
+                // CTAs of different length drift apart, so there are no waves: what the slots have to do, and on average half a
+                // CTA of waiting for the last ones (777 envs x 3 agents: 121 us by environment, 115 by observation)
+                return ((double)b->num_obs / apc / ((double)per_sm * sms) + 0.5) * (apc + kCtaFixedCost);
             };
-            if (waves_cost(all, d.agents_per_env) < waves_cost(b->smem, 1)) {
+            if (shape_cost(all, d.agents_per_env) < shape_cost(b->smem, 1)) {
                 b->smem = all;
                 b->agents_per_cta = b->auto_agents_per_cta = d.agents_per_env;
             }

@@ -65,6 +65,7 @@ struct RenderParams {
     int gx, gy, gz;
     int max_boxes, palette;
     int W, H, tiles_x, tiles_y, mask_words;
+    float inv_W;                       // 1 / W
     uint32_t sky_rgbx;
     float miss_depth;
     int agents_per_cta;                // observations one CTA renders: 1, or all agents of its env

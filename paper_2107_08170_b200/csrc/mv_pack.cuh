@@ -45,7 +45,7 @@ __device__ __forceinline__ size_t upload_env(const int32_t *__restrict__ env_ind
 // Per-env accumulators of an upload in flight: lo x,y,z, hi x,y,z (inclusive), CTAs done, pad.  Idle between uploads:
 // lo = 2^30, hi = -1, done = 0 (the CTA that finishes an env puts them back).
 constexpr int kPackAccInts = 8;
-constexpr int kUploadThreads = 256;
+constexpr int kUploadThreads = 64;
 constexpr int kUploadPolls = 1 << 18, kUploadStages = 2;
 constexpr int kUploadSmem = kUploadStages * 32 * kUploadThreads * 4;
 
@@ -82,20 +82,20 @@ struct UploadArgs {
     EnvLayout lay;
     int env_begin, env_count;
     int gx, gy, gz, max_boxes, palette;
-    int tiles_per_word, tiles_per_env, tiles_per_cta, pack_ctas_per_env;     // tiles of 1024 columns x 32 heights
+    int tiles_per_word, tiles_per_env, tiles_per_cta, pack_ctas_per_env;     // tiles of 256 columns x 32 heights
     // CTAs [0, pack_ctas) pack, the next lut_ctas shade, the rest copy boxes
     unsigned pack_ctas, lut_ctas;
     double light[3], ambient;
 };
 
-// A CTA packs a few tiles of one env, a tile being 1024 consecutive columns, 32 heights of them: each height is 1 KB of
+// A CTA packs a few tiles of one env, a tile being 256 consecutive columns, 32 heights of them: each height is 256 bytes of
 // the grid in a row, fetched by one bulk copy into shared memory, the next tile's while this one is packed (two
-// buffers, three CTAs per SM: about 200 KB per SM on the way without holding a register).  A thread takes four
+// buffers, twelve small CTAs per SM: about 190 KB per SM on the way without holding a register, and loads, packing and stores of different CTAs overlap).  A thread takes four
 // neighbouring columns: four occupancy words and four columns of material bytes (ids clamped to the palette; what
 // is not filled is never read, but comes out as 0), a column's 32 bytes as one 32-byte store, a whole sector.  Also
 // grows the cell box [lo, hi) that contains every filled voxel of the env; the last CTA of an env writes it next to
 // the box count (an empty grid gives lo > hi).  512 envs of 128x32x128 (268 MB in, 302 MB out): 150 us, then 42 us to
-// read the bits back for the bounds, with four-byte loads into registers and 16-byte stores; 114 us now (4.6 TB/s).
+// read the bits back for the bounds, with four-byte loads into registers and 16-byte stores; 114 us now (5.0 TB/s).
 __device__ __forceinline__ void pack_columns(const UploadArgs &p)
 {
     extern __shared__ __align__(128) uint32_t s_tile[];       // [kUploadStages][32][kUploadThreads]
@@ -281,7 +281,7 @@ __device__ __forceinline__ void copy_boxes(const UploadArgs &p, unsigned cta)
 }
 
 // Everything one upload brings, in one launch: the CTAs are dealt to the three jobs by number.
-__global__ void __launch_bounds__(kUploadThreads, 3) upload_kernel(const UploadArgs p)
+__global__ void __launch_bounds__(kUploadThreads, 12) upload_kernel(const UploadArgs p)
 {
     launch_dependents();
     wait_for_previous();

@@ -642,7 +642,9 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     if (gui) {
                         const int4 *ov = agent_ov(ag);
                         const int ov_count = __float_as_int(agent_rec(ag)[3].w);
-                        const int px = (tile_px % W) + (lane & 7), py = (tile_px / W) + (lane >> 3);
+                        // (tile_px / W, exact: tile rows begin at multiples of 4 W, so the quotient is 8 / W away from the next integer or more)
+                        const int row0 = (int)(((float)tile_px + 4.0f) * p.inv_W);
+                        const int px = tile_px - row0 * W + (lane & 7), py = row0 + (lane >> 3);
                         if (row != kNoRow) {                     // the rectangles go over the voxel colour: look it up now
                             asm volatile("ld.shared.u32 %0, [%1];" : "=r"(rgbx) : "r"(row + 4u * mat_id));
                             row = kNoRow;
