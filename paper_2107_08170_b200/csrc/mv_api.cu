@@ -45,7 +45,6 @@ inline uint32_t round_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 struct mv_batch {
     mv_batch_desc desc;
     int num_obs = 0;
-    size_t nvox = 0;
     size_t mat_bytes_per_env = 0;       // material store: one byte per voxel index (columns padded to 2^ysh)
     EnvLayout lay{};
     unsigned char *d_env_blocks = nullptr;
@@ -198,9 +197,8 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.status = b->d_status;
     p.lay = b->lay;
     p.obs_begin = obs_begin;
-    p.obs_count = obs_count;
     p.agents = b->desc.agents_per_env;
-    p.gx = b->desc.grid_x; p.gy = b->desc.grid_y; p.gz = b->desc.grid_z;
+    p.gx = b->desc.grid_x; p.gz = b->desc.grid_z;
     p.max_boxes = b->desc.max_boxes;
     p.palette = b->desc.palette_size;
     p.W = b->desc.width; p.H = b->desc.height; p.inv_W = 1.0f / (float)b->desc.width;
@@ -211,7 +209,6 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.agent_stride = b->smem.agent_stride; p.agent_ov_off = b->smem.agent_ov_off;
     p.agent_mask_off = b->smem.agent_mask_off;
     p.agents_per_cta = b->agents_per_cta;
-    p.max_steps = b->desc.grid_x + b->desc.grid_y + b->desc.grid_z + 3;
     // accumulated crossing times drift from the exact products by at most one rounding per step
     p.exit_scale = 1.0f - (float)(b->desc.grid_x + b->desc.grid_y + b->desc.grid_z + 3) * 1.1920929e-7f;
     p.overlay = b->d_overlay;
@@ -422,7 +419,6 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     if (!b) return MV_ERR_OUT_OF_MEMORY;
     b->desc = d;
     b->num_obs = d.num_envs * d.agents_per_env;
-    b->nvox = (size_t)d.grid_x * d.grid_y * d.grid_z;
     b->has_grid.assign(d.num_envs, 0);
     b->has_palette.assign(d.num_envs, 0);
     b->missing_grid = b->missing_palette = d.num_envs;

@@ -60,9 +60,9 @@ struct RenderParams {
     float *depth;                      // [O][H][W]
     uint32_t *status;
     EnvLayout lay;
-    int obs_begin, obs_count;
+    int obs_begin;
     int agents;
-    int gx, gy, gz;
+    int gx, gz;
     int max_boxes, palette;
     int W, H, tiles_x, tiles_y, mask_words;
     float inv_W;                       // 1 / W
@@ -70,7 +70,6 @@ struct RenderParams {
     float miss_depth;
     int agents_per_cta;                // observations one CTA renders: 1, or all agents of its env
     int part_tiles;                    // tiles of one observation that a CTA renders
-    int max_steps;                     // most steps a walk can take: grid_x + grid_y + grid_z + 3 (sizes the exit margin)
     float exit_scale;                  // 1 - (bound on the rounding drift of accumulated crossing times)
     // shared-memory offsets after the staged env block: tile table, per-agent blocks (ray table, camera record,
     // eye-relative boxes, then overlay rectangles and per-tile box masks at the offsets below), barrier and flag words

@@ -38,7 +38,6 @@ template <typename T> __device__ __forceinline__ void opaque(T &v, int lane) {
     uint32_t &u = reinterpret_cast<uint32_t &>(v);
     asm volatile("shfl.sync.idx.b32 %0, %0, %1, 31, 0xffffffff;" : "+r"(u) : "r"(lane));
 }
-template <typename T> __device__ __forceinline__ void keep64(T *&v) { asm volatile("" : "+l"(v)); }
 __device__ __forceinline__ float min3f(float a, float b, float c) {
     float r;
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
