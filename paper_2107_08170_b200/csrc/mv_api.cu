@@ -759,7 +759,7 @@ int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int e
     if (env_count == 0) return MV_OK;
     DeviceGuard g(device);
     if (!g.ok) return MV_ERR_CUDA;
-    scene_entities_kernel<<<env_count, kSceneThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+    scene_entities_kernel<<<env_count, kEntityThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
         a, reinterpret_cast<const long long *>(d_height), d_slots, reinterpret_cast<uint32_t *>(d_boxes), d_box_count,
         reinterpret_cast<uint32_t *>(d_cams));
     MV_CUDA(nullptr, cudaGetLastError());

@@ -61,15 +61,18 @@ class VecRenderEnv:
         A = self.cfg.agents
         for c0 in range(0, len(envs), _GEN_CHUNK):
             chunk = envs[c0:c0 + _GEN_CHUNK]
-            # ids and destinations in one pinned copy that nothing waits for
-            host = torch.from_numpy(np.stack([chunk + self._episode[chunk] * self.cfg.num_envs, chunk])).pin_memory()
-            ids, dst = host.to(self.device, non_blocking=True)
+            # ids and destinations (as int32) in one pinned copy that nothing waits for
+            host = np.empty((2, len(chunk)), np.int64)
+            host[0] = chunk + self._episode[chunk] * self.cfg.num_envs
+            host[1].view(np.int32)[:len(chunk)] = chunk
+            ids, dst = torch.from_numpy(host).pin_memory().to(self.device, non_blocking=True)
+            dst = dst.view(torch.int32)[:len(chunk)]
             w = scenes.make_worlds(self.cfg, device=self.device, env_ids=ids)
             if self._native is not None:
-                e = scenes._native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst.to(torch.int32))
+                e = scenes._native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst)
             else:
                 e = scenes.make_boxes_and_cameras(self.cfg, w)
-                self.cams.view(-1, A, 6)[dst] = e["cams"].view(-1, A, 6)
+                self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
             boxes = count = None
             if self.cfg.max_boxes > 0:
                 boxes, count = e["boxes"], e["box_count"]
