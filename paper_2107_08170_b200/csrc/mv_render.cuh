@@ -166,7 +166,7 @@ constexpr uint32_t kAgentSealed = 8u;      // the common case: eye inside, not i
 // Per-agent block in shared memory.  First the ray table, one 64-byte entry per combination of direction signs (x negative:
 // +64, y: +128, z: +256; the block is 512-byte aligned, so an entry's address is the block's OR-ed with the sign bits):
 //   {distance (>= 0) from the eye to the cell face met first, in x and z; what a step in x and z adds to the position}
-//   {first stretch: cells to spare in x, z, y; start position, from which kSkipBias steps each way are taken off}
+//   {first stretch: from the eye to its end in x, z, y, a little less (kSkipMargin); start position, from which kSkipBias steps each way are taken off}
 //   {first stretch: what is added to t |d| in x and z to give the crossings up to time t, rounded down; distance and step
 //    in y (the step is a rotate count in the column-word flavour)}
 //   {colour-table row of the face entered by an x, z, y step; -}
@@ -194,7 +194,6 @@ constexpr int kSkipCells = 8, kSkipCellsY = 4;
 // Crossings are counted up to a little less than the box's exit time: 2^-16 of the count, where rounding takes 2^-20 of
 // it at most; one that falls in between is left to the walk.
 constexpr float kSkipMargin = 1.0f - 1.52587890625e-5f;
-#define MV_SKIP_MARGIN "0f3F7FFF00"
 // The count comes out of an addition of 2^23, whose float's bits are 0x4B000000 + count.
 constexpr uint32_t kSkipBias = 0x4B000000u;
 #define MV_SKIP_MAGIC "0f4B000000"
@@ -436,7 +435,10 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
             const int ex = any ? rx + on_x : 0, ez = any ? rz + on_z : 0;
             const int sx = COLW ? 4 * dx : dx * stride_x, sz = COLW ? 4 * pitch * dz : dz * stride_z;
             const int signs = (dx < 0 ? 1 : 0) | (dy < 0 ? 2 : 0) | (dz < 0 ? 4 : 0);
-            agent_tab(ag)[4 * signs + 1] = make_float4((float)ex, (float)ez, (float)ey, __uint_as_float(cell_pos(cx, cy, cz) -
+            const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
+            const float qy = dy < 0 ? c0.y - (float)cy : (float)(cy + 1) - c0.y;
+            agent_tab(ag)[4 * signs + 1] = make_float4(((float)ex + qx) * kSkipMargin, ((float)ez + qz) * kSkipMargin,
+                                                       ((float)ey + qy) * kSkipMargin, __uint_as_float(cell_pos(cx, cy, cz) -
                                                        kSkipBias * (uint32_t)sx - kSkipBias * (uint32_t)sz));
         }
     }
@@ -700,7 +702,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                 // Where two components take the same operation and their operands lie side by side as loaded, one
                 // instruction does both (f32x2: the same roundings, one issue slot): 1079 -> 1065 us for 16384
                 // observations, 3194 -> 3118 for 16384 of 256x144.  Packing the products with dt as well is slower: the
-                // pairs it wants do not outlive the walk's own use of the registers, and are moved.
+                // pairs it wants do not outlive the walk's own use of the registers, and are moved.  (The end of the first
+                // stretch as one product, packed: 3121 -> 3095.)
                 // A direction component that is exactly zero needs no special case here: its reciprocal
                 // is +-inf, so its crossing time is +inf (or NaN when the eye sits exactly on the face,
                 // which min and the compares ignore) and that axis is never stepped, which is the rule
@@ -744,11 +747,12 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mul.f32 tx, tx, dtx;\n"
                     " mul.f32 ty, ty, dty;\n"
                     " mul.f32 tz, tz, dtz;\n"
-                    " fma.rn.f32 q0, q0, dtx, tx;\n"
-                    " fma.rn.f32 q1, q1, dtz, tz;\n"
-                    " fma.rn.f32 q2, q2, dty, ty;\n"
+                    " mov.b64 Q2, {q0, q1};\n"
+                    " mov.b64 D2, {dtx, dtz};\n"
+                    " mul.rn.f32x2 Q2, Q2, D2;\n"
+                    " mov.b64 {q0, q1}, Q2;\n"
+                    " mul.f32 q2, q2, dty;\n"
                     " min.f32 q0, q0, q1, q2;\n"
-                    " mul.f32 q0, q0, " MV_SKIP_MARGIN ";\n"
                     " fma.rn.f32 q3, q0, ix, q3;\n"
                     " fma.rn.f32 q4, q0, iz, q4;\n"
                     " mov.b64 Q2, {q3, q4};\n"
@@ -842,7 +846,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     t_exit = min3f(fmaf((float)(ngx ? cx - lox : hix - 1 - cx), dtx, t0x), fmaf((float)(ngy ? cy - loy : hiy - 1 - cy), dty, t0y),
                                    fmaf((float)(ngz ? cz - loz : hiz - 1 - cz), dtz, t0z)) * p.exit_scale;
                     // the first stretch, as in the block above
-                    const float ts = min3f(fmaf(ex, dtx, t0x), fmaf(ez, dtz, t0z), fmaf(ey, dty, t0y)) * kSkipMargin;
+                    const float ts = min3f(ex * dtx, ez * dtz, ey * dty);
                     const float nx = __fadd_rd(fmaf(ts, fabsf(dx), kx), 8388608.0f), nz = __fadd_rd(fmaf(ts, fabsf(dz), kz), 8388608.0f);
                     pos = at + __float_as_uint(nx) * (uint32_t)sx + __float_as_uint(nz) * (uint32_t)sz;
                     if (nx > 8388608.0f) t0x = fmaf(nx - 8388609.0f, dtx, t0x + dtx);
