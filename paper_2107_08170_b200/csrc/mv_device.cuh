@@ -113,9 +113,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 }
 constexpr int kDrainPolls = 1 << 26;               // bound of the wait for a copy known to be in flight
 
-// Programmatic dependent launch.  Every per-step kernel begins with launch_dependents, which lets the next kernel of the
-// stream that was launched with the attribute start once all CTAs of this one run, and waits for the previous kernel before it
-// touches global memory; so launch latency and CTA set-up overlap with what is still running, and nothing else changes.
+// Programmatic dependent launch.  Every per-step kernel waits for the previous kernel before it touches global memory, and
+// every one but the render kernel begins with launch_dependents, which lets the next kernel of the stream that was launched
+// with the attribute start once all CTAs of this one run; so launch latency and CTA set-up overlap with what is still
+// running, and nothing else changes.  (Nothing starts before the end of a render.)
+// A kernel launched like this is alive while the one before it still writes, so none of its global loads may promise
+// read-only data: no __ldg or ld.global.nc, and no const __restrict__ parameter, from which the compiler infers one and
+// which it may then move across the wait.  Ordinary loads stay behind the wait's memory clobber.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -38,8 +38,8 @@ __device__ __forceinline__ void transpose4x4(const uint32_t in[4], uint32_t out[
 }
 
 // Destination env of the e-th env of an upload: a contiguous range, or an index list.
-__device__ __forceinline__ size_t upload_env(const int32_t *__restrict__ env_index, int env_begin, size_t e) {
-    return env_index ? (size_t)__ldg(env_index + e) : (size_t)env_begin + e;
+__device__ __forceinline__ size_t upload_env(const int32_t *env_index, int env_begin, size_t e) {
+    return env_index ? (size_t)env_index[e] : (size_t)env_begin + e;
 }
 
 // Per-env accumulators of an upload in flight: lo x,y,z, hi x,y,z (inclusive), CTAs done, pad.  Idle between uploads:
@@ -313,7 +313,7 @@ __device__ __forceinline__ void write_camrec(CamRec *out, float px, float py, fl
     if (!ok) atomicOr(status, kFlagBadCamera);
 }
 
-__global__ void camera_kernel(const int32_t *__restrict__ cams, CamRec *__restrict__ out, int num_obs,
+__global__ void camera_kernel(const int32_t *cams, CamRec *out, int num_obs,
                               double kr, double ku, uint32_t *status)
 {
     launch_dependents();
@@ -349,8 +349,7 @@ __device__ __forceinline__ bool body_free(const uint32_t *occ, const EnvLayout &
 
 // Agent motion with voxel collision; one thread per agent.  Updates the caller's camera array,
 // the ray-basis table and the agent's own body box inside its env block.
-__global__ void move_agents_kernel(int32_t *__restrict__ cams, const float4 *__restrict__ moves,
-                                   CamRec *__restrict__ recs, unsigned char *__restrict__ env_blocks,
+__global__ void move_agents_kernel(int32_t *cams, const float4 *moves, CamRec *recs, unsigned char *env_blocks,
                                    EnvLayout lay, int num_obs, int agents, int gx, int gy, int gz, int max_boxes,
                                    float hw, float below, float above, float max_pitch, double kr, double ku,
                                    uint32_t *status)
@@ -390,9 +389,8 @@ __global__ void move_agents_kernel(int32_t *__restrict__ cams, const float4 *__r
 }
 
 // GUI rectangles into the library's table; counts clamped to 0..max_rects.
-__global__ void copy_overlays_kernel(const int4 *__restrict__ rects, const int32_t *__restrict__ counts,
-                                     int4 *__restrict__ out_rects, int32_t *__restrict__ out_counts, int num_obs,
-                                     int max_rects)
+__global__ void copy_overlays_kernel(const int4 *rects, const int32_t *counts, int4 *out_rects, int32_t *out_counts,
+                                     int num_obs, int max_rects)
 {
     launch_dependents();
     wait_for_previous();

@@ -115,7 +115,7 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 #define MV_DDA_STEP_IDX(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_STEP_IDX_ADV \
     " shr.u32 a, pos, 3;\n and.b32 a, a, 0xfffffffc;\n ld.shared.u32 w, [a];\n" MV_DDA_STEP_IDX_TAIL
 #define MV_DDA_STEP_IDX_GLOBAL(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_STEP_IDX_ADV \
-    " shr.u32 a, pos, 5;\n mad.wide.u32 ag, a, 4, gbase;\n ld.global.nc.u32 w, [ag];\n" MV_DDA_STEP_IDX_TAIL
+    " shr.u32 a, pos, 5;\n mad.wide.u32 ag, a, 4, gbase;\n ld.global.u32 w, [ag];\n" MV_DDA_STEP_IDX_TAIL
 // Loop around eight steps.  On leaving: ph = a filled cell was entered, thit = when, and px/py
 // still say along which axis.
 #define MV_DDA_LOOP(STEP)                            \
@@ -209,7 +209,7 @@ __device__ __forceinline__ void write_sky(uint8_t *rgb_obs, float *depth_obs, in
 
 // OCC_SHARED: the occupancy bits are staged in shared memory with the rest of the env block (the
 // normal case); otherwise only the block's tail (colour table, boxes, bounds) is staged and the
-// occupancy is read from global memory through the read-only path.
+// occupancy is read from global memory.
 // COLW: column-word flavour of the walk (grid at most 32 high and occupancy staged).
 template <int NT, bool OCC_SHARED, bool COLW>
 __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const RenderParams p)
@@ -273,8 +273,8 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
     // ---- meanwhile: camera records, GUI rectangles
     for (int ag = tid; ag < apc; ag += NT) {
         const float4 *cq = reinterpret_cast<const float4 *>(p.cams + obs0 + ag);
-        const float4 c0 = __ldg(cq), c1 = __ldg(cq + 1), c2 = __ldg(cq + 2), c3 = __ldg(cq + 3);   // P F | F R | R U | self, flags
-        const int ovc = p.overlay ? min(max(__ldg(p.overlay_count + obs0 + ag), 0), p.max_overlay) : 0;
+        const float4 c0 = cq[0], c1 = cq[1], c2 = cq[2], c3 = cq[3];   // P F | F R | R U | self, flags
+        const int ovc = p.overlay ? min(max(p.overlay_count[obs0 + ag], 0), p.max_overlay) : 0;
         float4 *rec = agent_rec(ag);
         rec[0] = make_float4(c0.w, c1.x, c1.z, c2.z);
         rec[1] = make_float4(c2.y, c2.w, c1.y, c2.x);
@@ -287,9 +287,9 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
         __syncthreads();
         for (int i = tid; i < apc * p.max_overlay; i += NT) {
             const int ag = i / p.max_overlay, r = i - ag * p.max_overlay;
-            const int ovc = min(max(__ldg(p.overlay_count + obs0 + ag), 0), p.max_overlay);
+            const int ovc = min(max(p.overlay_count[obs0 + ag], 0), p.max_overlay);
             if (r >= ovc) continue;
-            const int4 q = __ldg(p.overlay + (size_t)(obs0 + ag) * p.max_overlay + r);
+            const int4 q = p.overlay[(size_t)(obs0 + ag) * p.max_overlay + r];
             const int x0 = (int)(short)(q.x & 0xffff), y0 = (int)(short)(q.x >> 16);
             const int x1 = (int)(short)(q.y & 0xffff), y1 = (int)(short)(q.y >> 16);
             agent_ov(ag)[2 * r] = make_int4(x0, y0, x1, y1);
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const 
                     " mov.b32 %1, missb;\n"
                     " setp.ne.u32 pv, %4, 0xffffffff;\n"
                     " mad.wide.u32 mp, %5, 1, mp;\n"
-                    " @pv ld.global.nc.u8 %3, [mp];\n"
+                    " @pv ld.global.u8 %3, [mp];\n"
                     " @pv mov.f32 %1, %6;\n"
                     "}\n"
                     : "=&r"(rgbx), "=&f"(depth), "=&r"(m), "=&r"(mat_id)
