@@ -60,7 +60,7 @@ typedef enum mv_status {
 #define MV_FLAG_MATERIAL_CLAMPED 0x1u   /* a voxel or box material id was >= palette_size */
 #define MV_FLAG_BOX_COUNT_CLAMPED 0x2u  /* a box count was > max_boxes or negative */
 #define MV_FLAG_BAD_CAMERA 0x4u         /* a camera had a non-finite component */
-#define MV_FLAG_DEVICE_TIMEOUT 0x8u     /* a staging wait in the render kernel timed out */
+#define MV_FLAG_DEVICE_TIMEOUT 0x8u     /* a staging wait of a render or an upload timed out */
 
 typedef struct mv_batch mv_batch;       /* opaque; owned by the library */
 
@@ -145,6 +145,8 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out);
  *   d_box_count DEVICE int32 [env_count]; required when d_boxes is given
  *   d_palette   DEVICE uint8 [env_count][palette_size][3]; the per-env shaded colour table
  *               is rebuilt from it on the device
+ * If a bounded device-side wait runs out, MV_FLAG_DEVICE_TIMEOUT is set and the envs whose grids were in this
+ * upload have to be uploaded again; nothing else is affected.
  * Errors: INVALID_ARG (range, d_boxes without d_box_count), CUDA. */
 int mv_upload_worlds(mv_batch *batch, int env_begin, int env_count, const uint8_t *d_grid,
                      const mv_box *d_boxes, const int32_t *d_box_count, const uint8_t *d_palette,
@@ -318,7 +320,7 @@ int64_t mv_launch_count(const mv_batch *batch);
 
 /* ---- Test and measurement hooks (no counterpart in the paper).  They are exported by the library but
  * declared only for translation units that define MV_ENABLE_TEST_HOOKS before including this header;
- * they change how the render kernel runs, never what it computes.  Host-only calls. */
+ * they change how the kernels run, never what a call that reports no timeout computes.  Host-only calls. */
 #ifdef MV_ENABLE_TEST_HOOKS
 
 /* on != 0 makes the render kernel read the occupancy bits from global memory instead of staging them
@@ -329,8 +331,10 @@ int mv_debug_occupancy_in_global(mv_batch *batch, int on);
 /* Failure-detection hook.  The render kernel's only device-side wait is the bounded wait for the
  * staged env block; with skip_staging != 0 the copy is not issued, so every CTA's wait runs out after
  * wait_polls polls, the kernel returns without touching the outputs and MV_FLAG_DEVICE_TIMEOUT is set
- * (mv_query_status then returns MV_ERR_DEVICE_TIMEOUT).  Nothing faults or hangs and the context stays
- * usable.  Defaults: skip_staging 0, wait_polls 2^18; wait_polls must be in 1..2^24.
+ * (mv_query_status then returns MV_ERR_DEVICE_TIMEOUT).  An upload waits in the same way for the parts of the
+ * grid that it copies; with skip_staging != 0 the last part of every env is not copied, the rest is packed,
+ * and the same flag is set: the env holds parts of two worlds until its grid is uploaded again.
+ * Nothing faults or hangs and the context stays usable.  Defaults: skip_staging 0, wait_polls 2^18; wait_polls must be in 1..2^24.
  * Errors: INVALID_ARG. */
 int mv_debug_staging(mv_batch *batch, int skip_staging, int wait_polls);
 

@@ -259,6 +259,7 @@ int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int en
     if (pack + lut + box == 0) return MV_OK;
     if (pack + lut + box > 0x7fffffffull) return MV_ERR_INVALID_ARG;
     u.pack_ctas = (unsigned)pack; u.lut_ctas = (unsigned)lut;
+    u.wait_polls = b->wait_polls; u.skip_staging = b->skip_staging;
     MV_CUDA(b, launch_step(upload_kernel, dim3((unsigned)(pack + lut + box)), dim3(kUploadThreads), pack ? kUploadSmem : 0, s, u));
     b->launches++;
     return MV_OK;

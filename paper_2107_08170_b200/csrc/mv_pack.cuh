@@ -46,7 +46,7 @@ __device__ __forceinline__ size_t upload_env(const int32_t *env_index, int env_b
 // lo = 2^30, hi = -1, done = 0 (the CTA that finishes an env puts them back).
 constexpr int kPackAccInts = 8;
 constexpr int kUploadThreads = 64;
-constexpr int kUploadPolls = 1 << 18, kUploadStages = 2;
+constexpr int kUploadStages = 2;
 constexpr int kUploadSmem = kUploadStages * 32 * kUploadThreads * 4;
 
 // The fence around the columns of every env (see EnvLayout); grid columns keep their zeros.
@@ -85,6 +85,8 @@ struct UploadArgs {
     int tiles_per_word, tiles_per_env, tiles_per_cta, pack_ctas_per_env;     // tiles of 256 columns x 32 heights
     // CTAs [0, pack_ctas) pack, the next lut_ctas shade, the rest copy boxes
     unsigned pack_ctas, lut_ctas;
+    int wait_polls;                    // bound of the wait for a tile's copies
+    int skip_staging;                  // test hook: the last CTA of every env issues no copies, so its wait runs out
     double light[3], ambient;
 };
 
@@ -94,7 +96,8 @@ struct UploadArgs {
 // neighbouring columns: four occupancy words and four columns of material bytes (ids clamped to the palette; what
 // is not filled is never read, but comes out as 0), a column's 32 bytes as one 32-byte store, a whole sector.  Also
 // grows the cell box [lo, hi) that contains every filled voxel of the env; the last CTA of an env writes it next to
-// the box count (an empty grid gives lo > hi).  512 envs of 128x32x128 (268 MB in, 302 MB out): 150 us, then 42 us to
+// the box count (an empty grid gives lo > hi).  A CTA whose wait runs out counts like the others, so that the env's
+// accumulators are idle again for the next upload.  512 envs of 128x32x128 (268 MB in, 302 MB out): 150 us, then 42 us to
 // read the bits back for the bounds, with four-byte loads into registers and 16-byte stores; 114 us now (5.0 TB/s).
 __device__ __forceinline__ void pack_columns(const UploadArgs &p)
 {
@@ -113,7 +116,9 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
     if (threadIdx.x < 6) s_acc[threadIdx.x] = threadIdx.x < 3 ? 1 << 30 : -1;
     if (threadIdx.x == 6) s_bad = 0;
     __syncthreads();
+    const bool withheld = p.skip_staging && part == p.pack_ctas_per_env - 1;
     auto fetch = [&](int tile) {                              // one warp
+        if (withheld) return;
         const int stage = (tile - tile_begin) % kUploadStages, wq = tile / p.tiles_per_word;
         const int r0 = (tile - wq * p.tiles_per_word) * kUploadThreads, heights = min(p.gy - 32 * wq, 32);
         const uint32_t bytes = 4u * (uint32_t)min(groups - r0, kUploadThreads);
@@ -131,15 +136,15 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
         const int n = tile - tile_begin, stage = n % kUploadStages;
         const uint32_t parity = (uint32_t)(n / kUploadStages) & 1u;
         const uint32_t *mine = s_tile + (size_t)stage * 32 * kUploadThreads + threadIdx.x;
-        if (!mbar_wait_bounded(&s_bar[stage], parity, kUploadPolls)) s_bad = 1;
+        if (!mbar_wait_bounded(&s_bar[stage], parity, p.wait_polls)) s_bad = 1;
         __syncthreads();
-        if (s_bad) {                                          // (as in the render kernel: report, drain, leave)
+        if (s_bad) {                                          // (as in the render kernel: report, drain, pack no more)
             if (threadIdx.x == 0) {
                 atomicOr(p.status, kFlagTimeout);
-                for (int m = n; m < min(n + kUploadStages, tile_end - tile_begin); ++m)
+                for (int m = n; m < min(n + kUploadStages, tile_end - tile_begin) && !withheld; ++m)
                     mbar_wait_bounded(&s_bar[m % kUploadStages], (uint32_t)(m / kUploadStages) & 1u, kDrainPolls);
             }
-            return;
+            break;
         }
         const int wq = tile / p.tiles_per_word, heights = min(p.gy - 32 * wq, 32);
         const int r = (tile - wq * p.tiles_per_word) * kUploadThreads + (int)threadIdx.x;

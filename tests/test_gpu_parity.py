@@ -507,6 +507,35 @@ def test_bounded_wait_runs_out_and_reports_a_status():
     batch.destroy()
 
 
+@pytest.mark.parametrize("grid,envs", [((64, 16, 64), 3), ((64, 48, 64), 2), ((64, 16, 64), 480)])
+def test_upload_whose_wait_runs_out_leaves_nothing_behind(grid, envs):
+    """The last part of every env is withheld from an upload of empty worlds: the status says so, and the next upload
+    gives the frames that a new batch gives (its occupied bounds come from all of its parts and from no others).
+    Envs with several CTAs of one tile, two words per column, and several tiles per CTA."""
+    B = _binding()
+    cfg = scenes.config("rooms", num_envs=envs, agents=1, grid=grid, width=64, height=36)
+    sc = scenes.make_scene(cfg, device="cuda")
+    frames = []
+    for interrupted in (False, True):
+        batch = B.Batch(B.desc_from_config(cfg))
+        if interrupted:
+            batch.upload_worlds(0, envs, sc["grid"], None, None, sc["palette"])
+            batch.debug_staging(True, 64)
+            batch.upload_worlds(0, envs, torch.zeros_like(sc["grid"]), None, None, None)
+            with pytest.raises(B.MvError) as ei:
+                batch.query_status(clear=True)
+            assert ei.value.code == -5
+            batch.debug_staging(False)
+        batch.upload_worlds(0, envs, sc["grid"], None, None, sc["palette"])
+        batch.set_cameras(sc["cams"])
+        rgb, depth = batch.alloc_outputs()
+        batch.render_batch(rgb, depth)
+        assert batch.query_status() == 0
+        frames.append((rgb, depth))
+        batch.destroy()
+    assert torch.equal(frames[0][0], frames[1][0]) and torch.equal(frames[0][1], frames[1][1])
+
+
 def test_translation_and_occlusion_invariants_on_gpu(oracle):
     """Shifting world, boxes and camera by whole voxels leaves the frames bit-identical; geometry added
     strictly behind a wall changes nothing."""
