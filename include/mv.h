@@ -345,6 +345,16 @@ int mv_debug_staging(mv_batch *batch, int skip_staging, int wait_polls);
  * memory). */
 int mv_debug_agents_per_cta(mv_batch *batch, int agents_per_cta);
 
+/* How many CTAs of the render kernel share the tiles of one observation (or environment); 0 restores the library's own
+ * choice.  At most as many as leave a tile for every warp.  Results are identical.
+ * Returns the number that a render of the whole batch now uses (>= 1), or INVALID_ARG. */
+int mv_debug_parts(mv_batch *batch, int parts);
+
+/* How many CTAs of the render kernel share the tiles of one observation (or environment); 0 restores the library's own
+ * choice.  At most as many as leave a tile for every warp.  Results are identical.
+ * Returns the number that a render of the whole batch now uses (>= 1), or INVALID_ARG. */
+int mv_debug_parts(mv_batch *batch, int parts);
+
 #endif /* MV_ENABLE_TEST_HOOKS */
 
 /* Free everything mv_create_batch allocated (synchronises the device). NULL is accepted. */

@@ -27,9 +27,8 @@ constexpr int kRenderThreadsSmall = MV_NT / 2; // ...and for CTAs with few tiles
 // (measured: 64x36 images +10 %; 128x72 -2 %; four CTAs alone on the GPU -20 %: fewer warps per CTA, longer CTA).
 constexpr int kSmallCtaTiles = 192;
 constexpr int kHostChunks = 8;
-// CTAs that split the tiles of an observation between them, when the occupancy is not staged: enough to fill the GPU twice
-// (512 observations of 128x72 on 192x48x192: 112, 109, 115, 127 us with 1, 2, 4, 8 times); staged: once, as each one stages
-// the block again (4 of 64x36: 20.6 us with a CTA each, 12 with 6).
+// CTAs that split the tiles of an observation between them, in a batch with few of them (see pick_parts): this many times
+// what fills the GPU where the occupancy is not staged; once where it is, as each CTA stages the block again.
 constexpr int kPartWaves = 2;
 // Staging + set-up of a CTA, in units of one observation's render time at 128x72 (measured: about 0.1).
 constexpr double kCtaFixedCost = 0.1;
@@ -69,6 +68,7 @@ struct mv_batch {
     int agents_per_cta = 1;             // observations one CTA renders: 1, or every agent of its env
     int threads = MV_NT;                // threads per CTA of the render kernel (fewer for CTAs with few tiles)
     int sms = 0;
+    int forced_parts = 0;               // test hook: CTAs per observation (0: pick_parts decides)
     int tiles_x = 0, tiles_y = 0, mask_words = 0;
     int64_t launches = 0;
     int wait_polls = 1 << 18;
@@ -160,13 +160,24 @@ int pick_threads(const mv_batch *b, int apc) {
     return few_tiles && fills ? kRenderThreadsSmall : kRenderThreads;
 }
 
-// CTAs per observation (or environment) in a batch with few of them: as many as fill the GPU kPartWaves times over, but
-// each with a tile for every warp.
+// CTAs per observation (or environment) in a batch with few of them: as many as make three CTAs to an SM (six of the small
+// shape), kPartWaves times as many where the occupancy is not staged, but each with a tile for every warp.  Below, us of a
+// render by CTAs per observation; * is this rule.
+//   staged, 128x72: 16 observations of 128x32x128 columns 24.0 with 1, 13.3 with 4, 9.2 with 24*; 148: 37.4 33.3 32.3* 30.2
+//   with 1 to 4; 300: 59.3* 50.1 43.4 40.4.  4 observations of 64x36: 9.2 with 1, 5.6 with 6*.
+//   not staged, 128x72: 148 observations of 192x48x192 columns 75.3 with 1, 58.8 with 6*; 300: 89.6 98.3* 100.9 86.0 with
+//   1 to 4; 512: 107.0* 114.7 118.3 107.5; 192x36x192 rooms, 300: 79.9 60.9* 52.5 45.0; 512: 85.0* 69.0 60.9 64.5.
+// Three to an SM also where the staged block leaves room for one or two: the parts stage it several times over, but they
+// even out how long observations take.  As many as are resident instead: 192x32x192 columns (150 KB, one to an SM), 128x72,
+// 74 observations 31.2 against 26.6*, 148: 50.7 against 46.1*, 220: 51.2 against 55.8*; 160x32x160 (two), 220: 47.6 against
+// 38.2*.  Where it is worse: images below 128x72 with one CTA to an SM and about as many observations, if those are alike
+// (columns: 148 of 64x36 on 160x64x160 27.6*, unsplit 23.0); in rooms it is the other way round (180 of 64x36 on 192x32x192:
+// 23.0*, unsplit 29.2).
 int pick_parts(const mv_batch *b, int64_t ctas) {
     const int per_sm = b->threads == kRenderThreads ? 3 : 6;
     const int64_t slots = (int64_t)per_sm * b->sms * (b->occ_shared ? 1 : kPartWaves);
     const int64_t most = b->tiles_x * b->tiles_y / (b->threads / 32);
-    int64_t parts = slots / ctas;
+    int64_t parts = b->forced_parts > 0 ? b->forced_parts : slots / ctas;
     parts = parts > most ? most : parts;
     return parts < 1 ? 1 : (int)parts;
 }
@@ -804,6 +815,12 @@ int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     b->occ_shared = !on;
     b->smem = smem_layout(b, b->agents_per_cta, b->occ_shared);
     return MV_OK;
+}
+
+int mv_debug_parts(mv_batch *b, int parts) {
+    if (!b || parts < 0) return MV_ERR_INVALID_ARG;
+    b->forced_parts = parts;
+    return pick_parts(b, b->num_obs / b->agents_per_cta);
 }
 
 int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {

@@ -630,6 +630,43 @@ def test_cta_per_environment_equals_cta_per_observation():
     batch.destroy()
 
 
+@pytest.mark.parametrize("grid,size,agents,occ_in_global", [((128, 32, 128), (128, 72), 1, False), ((40, 48, 40), (104, 60), 3, False),
+                                                            ((64, 16, 64), (72, 52), 2, True), ((16, 8, 16), (8, 4), 1, False)])
+def test_ctas_that_share_an_observation_write_the_same_bytes(grid, size, agents, occ_in_global):
+    """The tiles of an observation may be split between CTAs, evenly or not, up to a tile per warp; with the block staged
+    or not, one observation or all of an environment per CTA, overlays and a bad camera included."""
+    B = _binding()
+    cfg = scenes.config("rooms", num_envs=5, agents=agents, grid=grid, width=size[0], height=size[1], movable_boxes=6,
+                        extra={"n_lines": max(1, grid[0] // 11)})
+    sc = scenes.make_scene(cfg, device="cuda")
+    batch = B.Batch(B.desc_from_config(cfg, 0, max_overlay_rects=1))
+    batch.upload_worlds(0, 5, sc["grid"], sc["boxes"], sc["box_count"], sc["palette"])
+    if occ_in_global:
+        batch.debug_occupancy_in_global(True)
+    sc["cams"][2, 3] = torch.tensor([float("nan")]).view(torch.int32).item()
+    rects = torch.zeros(cfg.num_obs, 1, 4, dtype=torch.int32)
+    rects[..., 1], rects[..., 2] = size[0] // 2 | ((size[1] // 2) << 16), 0x20C0FF
+    batch.set_overlays(rects.cuda(), torch.ones(cfg.num_obs, dtype=torch.int32, device="cuda"))
+    most = max(1, (size[0] // 8) * (size[1] // 4) // 12)
+    assert batch.debug_parts(0) == most                                      # so few observations: as many CTAs as can be
+    for apc in sorted({1, agents}):
+        batch.debug_agents_per_cta(apc)
+        want = None
+        for parts in (1, 2, 3, 5, 7, most, most + 1):
+            assert batch.debug_parts(parts) == min(parts, most)
+            batch.set_cameras(sc["cams"])
+            rgb, depth = batch.alloc_outputs()
+            rgb.fill_(9); depth.fill_(-3.0)
+            batch.render_batch(rgb, depth)
+            assert batch.query_status(clear=True) == B.FLAG_BAD_CAMERA
+            want = want or (rgb, depth)
+            assert torch.equal(rgb, want[0]) and torch.equal(depth, want[1]), (apc, parts)
+        assert bool((want[1] >= 0).all())
+    with pytest.raises(B.MvError):
+        batch.debug_parts(-1)
+    batch.destroy()
+
+
 def test_twenty_agents_in_one_cta(oracle):
     """More agents per CTA than one pass of the CTA's threads over the per-agent set-up covers
     (20 x 24 table slots > 384 threads): every agent's frame must still equal the per-observation
