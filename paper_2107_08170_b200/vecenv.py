@@ -8,8 +8,8 @@ time-left bar of Appendix A.2 is drawn through the GUI overlay.  Observations ar
 tensors owned by this object (Section 3.2: frames exposed directly as GPU-side tensors).
 
 Built for thousands of environments: episode clocks, time-left bars, agent state and the generation of new worlds
-all run on the GPU.  Episode lengths are fixed, so the host keeps its own copy of the clocks and knows which
-environments end without asking: a step enqueues its work and reads nothing back."""
+all run on the GPU.  The host keeps its own copy of the clocks and so knows which environments end without asking: a step
+enqueues its work and reads nothing back, unless the caller has changed a clock since the last one."""
 from __future__ import annotations
 
 import numpy as np
@@ -36,18 +36,53 @@ def time_bar_rects(steps_left, episode_len, width, agents):
     return rec
 
 
+class _Clock:
+    """A per-env counter on the device that callers may change, and the host's copy of it."""
+
+    def __init__(self, values: torch.Tensor, device):
+        with torch.inference_mode(False):           # (an inference tensor does not count its changes)
+            self.tensor, self.host = values.to(device, copy=True), values.numpy().copy()
+        self._seen = self._version()
+
+    def _version(self):
+        return None if self.tensor.is_inference() else self.tensor._version
+
+    def assign(self, value):
+        """`value` (a tensor of the right kind is taken as it is, not copied) instead of the present tensor."""
+        like = self.tensor
+        self.tensor = torch.as_tensor(value, dtype=like.dtype, device=like.device).expand(like.shape).contiguous()
+        self._seen = None
+
+    def refresh(self):
+        """Brings the host's copy up to date if the tensor was changed since it was read."""
+        version = self._version()
+        if version is None or version != self._seen:
+            self.host, self._seen = self.tensor.cpu().numpy().copy(), version
+
+
+def _clock_property(name, doc):
+    return property(lambda self: self._clocks[name].tensor, lambda self, value: self._clocks[name].assign(value), doc=doc)
+
+
 class VecRenderEnv:
+    """The clocks t, episode and episode_len (CUDA int64 [num_envs]) may be changed between steps, in place by torch
+    operations or by assignment, for instance t[i] = episode_len[i] - 1 to end an episode with the next step; that step then
+    reads them back once.  (A write that torch does not see, through `.data` or another library's pointer, is made known
+    by assigning the tensor to its own name: env.t = env.t.)"""
+
+    t = _clock_property("t", "steps taken in the present episode")
+    episode = _clock_property("episode", "episodes finished; env e in its k-th episode shows the seeded scene e + k * num_envs")
+    episode_len = _clock_property("episode_len", "steps per episode")
+
     def __init__(self, cfg: scenes.SceneConfig, episode_len, device: int = 0, time_bar: bool = True, phase=None):
         """episode_len: steps per episode (scalar or one per env).  phase: optional initial value of each
         env's step clock (so that episodes end at different times from the start)."""
         self.cfg, self.device = cfg, torch.device("cuda", device)
         E = cfg.num_envs
         host = lambda v: torch.as_tensor(v, dtype=torch.int64).expand(E).cpu().clone()
-        length, t = host(episode_len), host(0 if phase is None else phase)
-        self.episode_len, self.t = length.to(self.device), t.to(self.device)
-        self.episode = torch.zeros(E, dtype=torch.int64, device=self.device)
-        # the host's copies of the three clocks above, which it advances by itself
-        self._length, self._t, self._episode = length.numpy(), t.numpy(), np.zeros(E, np.int64)
+        self._clocks = {"t": _Clock(host(0 if phase is None else phase), self.device),
+                        "episode": _Clock(torch.zeros(E, dtype=torch.int64), self.device),
+                        "episode_len": _Clock(host(episode_len), self.device)}
         self.time_bar = time_bar
         self.batch = binding.Batch(binding.desc_from_config(cfg, device, max_overlay_rects=1 if time_bar else 0))
         self.cams = torch.zeros(cfg.num_obs, 6, dtype=torch.int32, device=self.device)
@@ -63,7 +98,7 @@ class VecRenderEnv:
             chunk = envs[c0:c0 + _GEN_CHUNK]
             # ids and destinations (as int32) in one pinned copy that nothing waits for
             host = np.empty((2, len(chunk)), np.int64)
-            host[0] = chunk + self._episode[chunk] * self.cfg.num_envs
+            host[0] = chunk + self._clocks["episode"].host[chunk] * self.cfg.num_envs
             host[1].view(np.int32)[:len(chunk)] = chunk
             ids, dst = torch.from_numpy(host).pin_memory().to(self.device, non_blocking=True)
             dst = dst.view(torch.int32)[:len(chunk)]
@@ -78,17 +113,22 @@ class VecRenderEnv:
                 boxes, count = e["boxes"], e["box_count"]
             self.batch.upload_worlds_at(chunk.astype(np.int32), w["grid"], boxes, count, w["palette"])
 
-    def _clocks(self, done=None):
+    def _refresh(self):
+        for clock in self._clocks.values():
+            clock.refresh()
+
+    def _advance(self, done=None):
         """Advance the clocks (with `done`) and draw the time-left bars."""
         if done is not None or self.time_bar:
             self.batch.advance_episodes(self.t, self.episode, self.episode_len, done, BAR_ROWS if self.time_bar else 0, BAR_RGB)
 
     def reset(self):
         """Only needed once, right after construction."""
+        self._refresh()
         self._load_envs(np.arange(self.cfg.num_envs))
         self.batch.set_cameras(self.cams)
         self._started = True
-        self._clocks()
+        self._advance()
         self.batch.render_batch(self.rgb, self.depth)
         return self.rgb, self.depth
 
@@ -99,12 +139,14 @@ class VecRenderEnv:
         assert self._started, "call reset() once before step()"
         self.batch.move_agents(self.cams, moves.contiguous())
         done = torch.empty(self.cfg.num_envs, dtype=torch.bool, device=self.device)
-        self._clocks(done)
-        self._t += 1
-        finished = np.flatnonzero(self._t >= self._length)
+        self._refresh()
+        self._advance(done)
+        t = self._clocks["t"].host
+        t += 1
+        finished = np.flatnonzero(t >= self._clocks["episode_len"].host)
         if len(finished):
-            self._episode[finished] += 1
-            self._t[finished] = 0
+            self._clocks["episode"].host[finished] += 1
+            t[finished] = 0
             self._load_envs(finished)
             self.batch.set_cameras(self.cams)
         self.batch.render_batch(self.rgb, self.depth)

@@ -71,3 +71,77 @@ def test_step_loop_with_auto_reset_matches_oracle(oracle):
     bar_len = int(bars[0].view(np.int16).reshape(-1)[2])
     assert (g_rgb[0, :2, :bar_len] == np.array(vecenv.BAR_RGB, np.uint8)).all()
     env.close()
+
+
+@pytest.mark.parametrize("inference", [False, True])
+def test_host_copy_of_a_clock_follows_every_change(inference):
+    with torch.inference_mode(inference):
+        clock = vecenv._Clock(torch.arange(6), "cpu")
+        assert not clock.tensor.is_inference()
+
+        def follows():
+            clock.refresh()
+            return clock.host.tolist() == clock.tensor.tolist()
+
+        assert follows()
+        quiet = clock.host
+        clock.refresh()
+        assert clock.host is quiet                                     # nothing changed: nothing is read
+        for change in (lambda t: t.__setitem__(2, 40), lambda t: t.fill_(3), lambda t: t[1:4].add_(2),
+                       lambda t: t.masked_fill_(t > 4, 0), lambda t: torch.add(t, 1, out=t), lambda t: t.view(2, 3).zero_()):
+            before = clock.tensor.tolist()
+            change(clock.tensor)
+            assert clock.tensor.tolist() != before and follows()
+            assert clock.host is not quiet
+        mine = torch.arange(6) * 7                                     # (under inference mode one that counts no changes)
+        clock.assign(mine)
+        assert follows() and clock.host.tolist() == [0, 7, 14, 21, 28, 35]
+        mine[0] = 9
+        assert clock.tensor[0] == 9 and follows()                      # taken as it is, not copied
+        clock.assign(5)
+        assert clock.tensor.tolist() == [5] * 6 and clock.tensor.dtype == torch.int64 and follows()
+        clock.host += 1                                                # the host's own step leaves the device's tensor alone
+        assert clock.tensor.tolist() == [5] * 6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("inference", [False, True])
+def test_clocks_set_by_the_caller_end_episodes(inference):
+    """t, episode and episode_len belong to the caller too: whatever is put there between steps decides which
+    environments the next step resets, and to which world."""
+    from gpu_util import render_scene
+    cfg = scenes.config("rooms_boxes", num_envs=4, agents=2)
+    E, A = cfg.num_envs, cfg.agents
+    first = lambda scene_id: [torch.from_numpy(v) for v in render_scene(scenes.config("rooms_boxes", num_envs=1, agents=2),
+                                                                       scenes.make_scene(cfg, scene_id, 1))[:2]]
+    still = torch.zeros(cfg.num_obs, 4, device="cuda")
+    with torch.inference_mode(inference):
+        env = vecenv.VecRenderEnv(cfg, 10, time_bar=False)
+        env.reset()
+
+        def step(ended):
+            rgb, depth, done = env.step(still)
+            assert done.tolist() == [e in ended for e in range(E)]
+            for e, k in ended.items():
+                want = first(e + k * E)
+                assert torch.equal(rgb[e * A:e * A + A].cpu(), want[0]) and torch.equal(depth[e * A:e * A + A].cpu(), want[1])
+                assert int(env.episode[e]) == k and int(env.t[e]) == 0
+            env._refresh()
+            assert all(c.host.tolist() == c.tensor.tolist() for c in env._clocks.values())
+
+        step({})
+        env.t[1] = 9                                                   # early termination
+        step({1: 1})
+        step({})
+        env.episode[2] = 5
+        env.t[2:4] = 100
+        step({2: 6, 3: 1})
+        env.episode_len[0] = int(env.t[0]) + 1
+        step({0: 1})
+        env.episode_len = 1
+        env.t = torch.zeros(E, dtype=torch.int64, device="cuda")
+        step({0: 2, 1: 2, 2: 7, 3: 2})
+        env.t.data[0] = -1                                             # not seen by torch, so said by hand
+        env.t = env.t
+        step({1: 3, 2: 8, 3: 3})
+    env.close()
