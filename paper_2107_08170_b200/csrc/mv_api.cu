@@ -572,8 +572,8 @@ int mv_set_overlays(mv_batch *b, const mv_overlay_rect *d_rects, const int32_t *
     if (d_rects && !aligned16(d_rects)) return MV_ERR_INVALID_ARG;
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
-    const int n = b->num_obs * (m + 1);
-    MV_CUDA(b, launch_step(copy_overlays_kernel, dim3((n + 255) / 256), dim3(256), 0, static_cast<cudaStream_t>(cuda_stream),
+    const int64_t n = (int64_t)b->num_obs * (m + 1);
+    MV_CUDA(b, launch_step(copy_overlays_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, static_cast<cudaStream_t>(cuda_stream),
                            reinterpret_cast<const int4 *>(d_rects), d_count, b->d_overlay, b->d_overlay_count, b->num_obs, m));
     b->launches++;
     return MV_OK;

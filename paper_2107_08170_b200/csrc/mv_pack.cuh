@@ -238,9 +238,9 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
 // Shaded colour table per env: lut[face][m] = RGBX of floor(palette*I_face + 0.5), in double.
 __device__ __forceinline__ void shade_palettes(const UploadArgs &p, unsigned cta)
 {
-    const int gid = (int)(cta * kUploadThreads + threadIdx.x), P = p.palette;
-    if (gid >= p.env_count * kFaces * P) return;
-    const int e = gid / (kFaces * P), r = gid - e * kFaces * P;
+    const long long gid = (long long)cta * kUploadThreads + threadIdx.x;     // (1.2 million envs of 256 colours are 2^31 entries)
+    const int P = p.palette, e = (int)(gid / (kFaces * P)), r = (int)(gid - (long long)e * (kFaces * P));
+    if (e >= p.env_count) return;
     const int f = r / P, m = r - f * P;
     double I = p.ambient;
     if (f < 6) {
@@ -267,9 +267,9 @@ __device__ __forceinline__ void shade_palettes(const UploadArgs &p, unsigned cta
 // Box lists into the env blocks; material ids and counts are clamped.
 __device__ __forceinline__ void copy_boxes(const UploadArgs &p, unsigned cta)
 {
-    const int gid = (int)(cta * kUploadThreads + threadIdx.x), per_env = p.max_boxes + 1;
-    if (gid >= p.env_count * per_env) return;
-    const int e = gid / per_env, b = gid - e * per_env;
+    const long long gid = (long long)cta * kUploadThreads + threadIdx.x;
+    const int per_env = p.max_boxes + 1, e = (int)(gid / per_env), b = (int)(gid - (long long)e * per_env);
+    if (e >= p.env_count) return;
     unsigned char *blk = p.env_blocks + upload_env(p.env_index, p.env_begin, (size_t)e) * p.lay.stride;
     if (b == p.max_boxes) {
         int n = p.counts[e];
@@ -399,9 +399,9 @@ __global__ void copy_overlays_kernel(const int4 *rects, const int32_t *counts, i
 {
     launch_dependents();
     wait_for_previous();
-    const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= num_obs * (max_rects + 1)) return;
-    const int o = gid / (max_rects + 1), r = gid - o * (max_rects + 1);
+    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int o = (int)(gid / (max_rects + 1)), r = (int)(gid - (long long)o * (max_rects + 1));
+    if (o >= num_obs) return;
     if (r == max_rects) {
         const int n = rects ? counts[o] : 0;
         out_counts[o] = n < 0 ? 0 : (n > max_rects ? max_rects : n);

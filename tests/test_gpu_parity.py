@@ -859,3 +859,30 @@ def test_first_stretch_of_a_walk(oracle, grid):
     _, _, status, st = _render_custom(oracle, g, _pal(E, 6), np.stack(cams), 64, 36)
     assert status == 0
     parity.assert_parity(st, f"first stretch {grid}")
+
+
+def test_colour_tables_of_more_than_two_to_the_31_entries():
+    """1.2 million environments of 256 colours in one upload (12 GB on the device): the environments on either side of the
+    table entry 2^31, and the last ones, get the frames that they get in a small batch."""
+    B = _binding()
+    envs, P = (1 << 31) // (7 * 256) + 30_000, 256
+    edge = (1 << 31) // (7 * P)
+    look = torch.tensor([0, 1, edge - 1, edge, edge + 1, edge + 2, envs - 2, envs - 1], device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    grid = torch.randint(0, 256, (envs, 4, 4, 4), generator=gen, device="cuda", dtype=torch.uint8)
+    grid[torch.rand(envs, 4, 4, 4, generator=gen, device="cuda") < 0.6] = 0
+    palette = torch.randint(20, 255, (envs, P, 3), generator=gen, device="cuda", dtype=torch.uint8)
+    row = torch.from_numpy(cam_row(2.0, 2.0, -3.0, 0.1, 0.05)).cuda()
+    frames = []
+    for g, c in ((grid, palette), (grid[look], palette[look])):
+        n = g.shape[0]
+        batch = B.Batch(B.make_desc(n, 1, (4, 4, 4), 0, 16, 12, P))
+        batch.upload_worlds(0, n, g.contiguous(), None, None, c.contiguous())
+        batch.set_cameras(row.expand(n, 6).contiguous())
+        rgb, depth = batch.alloc_outputs()
+        batch.render_batch(rgb, depth)
+        assert batch.query_status() == 0
+        frames.append((rgb[look] if n == envs else rgb, depth[look] if n == envs else depth))
+        batch.destroy()
+    assert torch.equal(frames[0][0], frames[1][0]) and torch.equal(frames[0][1], frames[1][1])
+    assert len({f.tobytes() for f in frames[1][0].cpu().numpy()}) == len(look)          # eight different frames
