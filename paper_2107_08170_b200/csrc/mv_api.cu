@@ -18,11 +18,8 @@ using namespace mv;
 
 namespace {
 
-#ifndef MV_NT
-#define MV_NT 384
-#endif
-constexpr int kRenderThreads = MV_NT;          // threads per CTA of the render kernel...
-constexpr int kRenderThreadsSmall = MV_NT / 2; // ...and for CTAs with few tiles (small images): twice as many, shorter CTAs per SM
+constexpr int kRenderThreads = 384;            // threads per CTA of the render kernel...
+constexpr int kRenderThreadsSmall = 192;       // ...and for CTAs with few tiles (small images): twice as many, shorter CTAs per SM
 // Below this many tiles per CTA the small shape is faster when there are CTAs enough to fill the GPU with it
 // (measured: 64x36 images +10 %; 128x72 -2 %; four CTAs alone on the GPU -20 %: fewer warps per CTA, longer CTA).
 constexpr int kSmallCtaTiles = 192;
@@ -32,10 +29,7 @@ constexpr int kHostChunks = 8;
 constexpr int kPartWaves = 2;
 // Staging + set-up of a CTA, in units of one observation's render time at 128x72 (measured: about 0.1).
 constexpr double kCtaFixedCost = 0.1;
-#ifndef MV_MERGE_SCRATCH_MB
-#define MV_MERGE_SCRATCH_MB 1024
-#endif
-constexpr size_t kMergeScratchBytes = (size_t)MV_MERGE_SCRATCH_MB << 20;   // bit arrays for the envs of one merge launch
+constexpr size_t kMergeScratchBytes = (size_t)1 << 30;         // bit arrays for the envs of one merge launch
 
 inline uint32_t round_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
@@ -66,7 +60,7 @@ struct mv_batch {
     struct Smem { uint32_t tile_off, agent_off, agent_stride, agent_ov_off, agent_mask_off, misc_off, bytes; };
     Smem smem{};                        // shared-memory layout of the render kernel for agents_per_cta
     int agents_per_cta = 1;             // observations one CTA renders: 1, or every agent of its env
-    int threads = MV_NT;                // threads per CTA of the render kernel (fewer for CTAs with few tiles)
+    int threads = kRenderThreads;       // threads per CTA of the render kernel (fewer for CTAs with few tiles)
     int sms = 0;
     int forced_parts = 0;               // test hook: CTAs per observation (0: pick_parts decides)
     int tiles_x = 0, tiles_y = 0, mask_words = 0;

@@ -155,9 +155,9 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " .reg .b32 sx, sy, sz, pos, bit, guard, w, a, it;\n"   \
     " .reg .b64 ag, gbase;\n"
 
-#ifndef MV_MINB
-#define MV_MINB 3
-#endif
+// Threads resident per SM that the registers are laid out for: three CTAs of 384 with 56 registers (16384 observations
+// 1.42 ms when two with 69 took 1.62).
+constexpr int kThreadsPerSm = 3 * 384;
 
 constexpr uint32_t kAgentInside = 1u;      // eye inside the occupied cell box
 constexpr uint32_t kAgentBad = 2u;         // non-finite camera: sky frame
@@ -212,7 +212,7 @@ __device__ __forceinline__ void write_sky(uint8_t *rgb_obs, float *depth_obs, in
 // occupancy is read from global memory.
 // COLW: column-word flavour of the walk (grid at most 32 high and occupancy staged).
 template <int NT, bool OCC_SHARED, bool COLW>
-__global__ void __launch_bounds__(NT, (MV_MINB * 384) / NT) render_kernel(const RenderParams p)
+__global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const RenderParams p)
 {
     static_assert(OCC_SHARED || !COLW, "the column-word walk reads shared memory");
     extern __shared__ __align__(1024) unsigned char smem[];
