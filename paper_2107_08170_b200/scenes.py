@@ -135,7 +135,7 @@ def config(name: str, **over) -> SceneConfig:
 _WORLDS = {"segments": 0, "rooms": 1, "columns": 2}
 
 
-def _native_desc(cfg: SceneConfig, step: int = 0):
+def native_desc(cfg: SceneConfig, step: int = 0):
     """The configuration as the CUDA library's generator takes it, or None where it does not."""
     gx, gy, gz = cfg.grid
     counts = {"rooms": {"n_lines", "pitch", "n_pillars"}}.get(cfg.world, {"n_rects"})
@@ -154,7 +154,8 @@ def _native_desc(cfg: SceneConfig, step: int = 0):
     return d
 
 
-def _native_worlds(cfg: SceneConfig, desc, env: torch.Tensor):
+def native_worlds(cfg: SceneConfig, desc, env: torch.Tensor):
+    """The arrays of make_worlds for the CUDA ids `env`, by the library's kernels."""
     from . import binding
     gx, gy, gz = cfg.grid
     E, dev = env.numel(), env.device
@@ -165,8 +166,8 @@ def _native_worlds(cfg: SceneConfig, desc, env: torch.Tensor):
     return {"grid": grid, "palette": palette, "height": height, "env": env}
 
 
-def _native_entities(cfg: SceneConfig, desc, env: torch.Tensor, height: torch.Tensor, cams=None, slots=None):
-    """With `cams` and `slots` (CUDA int32) the cameras go straight to those environments' rows of an existing array."""
+def native_entities(cfg: SceneConfig, desc, env: torch.Tensor, height: torch.Tensor, cams=None, slots=None):
+    """The arrays of make_boxes_and_cameras, likewise.  With `cams` and `slots` (CUDA int32) the cameras go straight to those environments' rows of an existing array."""
     from . import binding
     E, dev = env.numel(), env.device
     boxes = torch.empty(E, cfg.max_boxes, 8, dtype=torch.int32, device=dev)
@@ -289,8 +290,8 @@ def make_worlds(cfg: SceneConfig, env_begin: int = 0, env_count: int | None = No
     else:
         env_count = cfg.num_envs - env_begin if env_count is None else env_count
         env = torch.arange(env_begin, env_begin + env_count, device=rng.device)
-    if env.is_cuda and (desc := _native_desc(cfg)) is not None:
-        return _native_worlds(cfg, desc, env)
+    if env.is_cuda and (desc := native_desc(cfg)) is not None:
+        return native_worlds(cfg, desc, env)
     gx, gy, gz = cfg.grid
     P = cfg.palette_size
     if cfg.world == "rooms":
@@ -324,8 +325,8 @@ def make_boxes_and_cameras(cfg: SceneConfig, worlds: dict, step: int = 0):
     dev = rng.device
     env = worlds["env"]
     height = worlds["height"]                       # solid cells above the floor layer
-    if height.is_cuda and (desc := _native_desc(cfg, step)) is not None:
-        return _native_entities(cfg, desc, env, height)
+    if height.is_cuda and (desc := native_desc(cfg, step)) is not None:
+        return native_entities(cfg, desc, env, height)
     E = env.numel()
     gx, gy, gz = cfg.grid
     P = cfg.palette_size

@@ -87,7 +87,7 @@ class VecRenderEnv:
         self.batch = binding.Batch(binding.desc_from_config(cfg, device, max_overlay_rects=1 if time_bar else 0))
         self.cams = torch.zeros(cfg.num_obs, 6, dtype=torch.int32, device=self.device)
         self.rgb, self.depth = self.batch.alloc_outputs()
-        self._native = scenes._native_desc(cfg)
+        self._native = scenes.native_desc(cfg)
         self._started = False
 
     def _load_envs(self, envs):
@@ -104,7 +104,7 @@ class VecRenderEnv:
             dst = dst.view(torch.int32)[:len(chunk)]
             w = scenes.make_worlds(self.cfg, device=self.device, env_ids=ids)
             if self._native is not None:
-                e = scenes._native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst)
+                e = scenes.native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst)
             else:
                 e = scenes.make_boxes_and_cameras(self.cfg, w)
                 self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
