@@ -41,23 +41,23 @@ class _Clock:
 
     def __init__(self, values: torch.Tensor, device):
         with torch.inference_mode(False):           # (an inference tensor does not count its changes)
-            self.tensor, self.host = values.to(device, copy=True), values.numpy().copy()
-        self._seen = self._version()
+            self._take(values.to(device, copy=True))
+        self.refresh()
 
-    def _version(self):
-        return None if self.tensor.is_inference() else self.tensor._version
+    def _take(self, tensor):
+        self.tensor, self._counts, self._seen = tensor, not tensor.is_inference(), None
 
     def assign(self, value):
         """`value` (a tensor of the right kind is taken as it is, not copied) instead of the present tensor."""
         like = self.tensor
-        self.tensor = torch.as_tensor(value, dtype=like.dtype, device=like.device).expand(like.shape).contiguous()
-        self._seen = None
+        self._take(torch.as_tensor(value, dtype=like.dtype, device=like.device).expand(like.shape).contiguous())
 
     def refresh(self):
         """Brings the host's copy up to date if the tensor was changed since it was read."""
-        version = self._version()
-        if version is None or version != self._seen:
-            self.host, self._seen = self.tensor.cpu().numpy().copy(), version
+        if self._counts and self.tensor._version == self._seen:
+            return
+        self.host = self.tensor.cpu().numpy().copy()
+        self._seen = self.tensor._version if self._counts else None
 
 
 def _clock_property(name, doc):
