@@ -35,9 +35,9 @@ WORKLOAD = "headline"
 # capture of render_kernel on a 2048-environment slice of the headline workload (summary and command in
 # profiles/render_kernel_headline_2048env_ncu_full.md); NCU_BUILD names the commit of the library they were
 # taken on.  DRAM traffic grows in proportion to the environments, so a full launch is the slice x 8.
-NCU_BUILD = "56e11ef"
+NCU_BUILD = "63d2105"
 NCU_SLICE_ENVS = 2048
-NCU_SLICE_DRAM_BYTES = 150.62e6 + 85.22e6   # dram__bytes_read.sum + dram__bytes_write.sum of one launch on the slice
+NCU_SLICE_DRAM_BYTES = 150.62e6 + 85.20e6   # dram__bytes_read.sum + dram__bytes_write.sum of one launch on the slice
 NCU_WARP_INSTRUCTIONS_PER_TILE = 198.3  # smsp__inst_executed.sum / (8x4-pixel tiles) on the slice
 
 
@@ -196,19 +196,18 @@ def time_extras(batch, cfg, cams, rgb, depth, dev):
     out["render_occupancy_in_global_ms"] = med(lambda: batch.render_batch(rgb, depth))
     batch.debug_occupancy_in_global(False)
     # the vectorised step() wrapper at this size: move + collide, auto-reset of the ~1 % of environments whose
-    # 100-step episode ends (new worlds generated and uploaded), time-left bar, render; wall clock over 20 steps
+    # 100-step episode ends (new worlds generated and uploaded), time-left bar, render; wall clock over 100 steps
     env = vecenv.VecRenderEnv(cfg, 100, device=dev.index, phase=torch.arange(E) % 100)
     env.reset()
-    for _ in range(2):
+    for _ in range(20):
         env.step(moves)
     torch.cuda.synchronize(dev)
     t0 = time.perf_counter()
-    n_steps, n_reset = 20, 0
-    for _ in range(n_steps):
-        _, _, done = env.step(moves)
-        n_reset += int(done.sum())
+    n_steps = 100
+    dones = [env.step(moves)[2] for _ in range(n_steps)]
     torch.cuda.synchronize(dev)
     dt = time.perf_counter() - t0
+    n_reset = int(torch.stack(dones).sum())
     out["vecenv_steps_per_s"] = n_steps / dt
     out["vecenv_obs_per_s"] = n_steps * cfg.num_obs / dt
     out["vecenv_envs_reset_per_step"] = n_reset / n_steps
