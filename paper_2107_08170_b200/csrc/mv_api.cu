@@ -110,9 +110,9 @@ struct DeviceGuard {
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Shared-memory layout of the render kernel when one CTA renders `apc` observations of an env:
-// staged env block (without the occupancy when that stays in global memory), tile table, then one block per agent (camera record and DDA start table,
-// eye-relative boxes, overlay rectangles, per-tile box masks, per-tile overlay bits), then the
-// barrier and flag words.
+// staged env block (without the occupancy when that stays in global memory), tile table, then one block per agent (ray
+// table, camera record, eye-relative boxes, overlay rectangles, per-tile masks of boxes and the GUI bit), then the barrier
+// and flag words.
 mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     const mv_batch_desc &d = b->desc;
     const uint32_t ntiles = (uint32_t)(b->tiles_x * b->tiles_y);

@@ -695,9 +695,8 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 float t_hit, dtx, dty, dtz;
                 // ---- the common case in one block of PTX: tile record, ray through the pixel centre
                 // (d = F + a*Rs + b*Us, a = 2px+1-W, b = H-1-2py, two chained FMAs per component),
-                // reciprocals, the DDA table rows for the ray's signs
-                // the table entry for the ray's signs, first crossing
-                // times, exit time, then the walk.  The basis is re-read from shared memory per tile:
+                // reciprocals, the table entry for the ray's signs, first crossing times, the first
+                // stretch, then the walk.  The basis is re-read from shared memory per tile:
                 // three broadcast loads cost less than nine registers held across the walk.
                 // Where two components take the same operation and their operands lie side by side as loaded, one
                 // instruction does both (f32x2: the same roundings, one issue slot): 1079 -> 1065 us for 16384
