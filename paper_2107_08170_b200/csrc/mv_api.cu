@@ -188,9 +188,14 @@ RenderFn render_fn(const mv_batch *b) {
     return b->lay.ysh == 5 ? render_kernel<kRenderThreads, true, true> : render_kernel<kRenderThreads, true, false>;
 }
 
-// The merge sweep keeps a layer number per column: a byte for grids less than 256 high.
+// The merge sweep keeps a layer number per column: a byte for grids less than 256 high.  Rows of up to 16 words (W) are held in
+// registers, one lane a row.
 using MergeFn = void (*)(const unsigned char *, const uint8_t *, EnvLayout, MergeLayout, int, uint32_t *, uint4 *, int32_t *, int);
-MergeFn merge_sweep(int grid_y) { return grid_y < 256 ? merge_sweep_kernel<uint8_t> : merge_sweep_kernel<uint16_t>; }
+template <typename Cov> MergeFn merge_sweep_of(int W) {
+    return W <= 2 ? merge_sweep_kernel<Cov, 2> : W <= 4 ? merge_sweep_kernel<Cov, 4> : W <= 8 ? merge_sweep_kernel<Cov, 8>
+           : W <= 16 ? merge_sweep_kernel<Cov, 16> : merge_sweep_kernel<Cov, 0>;
+}
+MergeFn merge_sweep(int grid_y, int W) { return grid_y < 256 ? merge_sweep_of<uint8_t>(W) : merge_sweep_of<uint16_t>(W); }
 
 int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, int obs_count, cudaStream_t s) {
     RenderParams p{};
@@ -613,11 +618,11 @@ int mv_merge_voxels(mv_batch *b, int env_begin, int env_count, mv_box *d_boxes_o
         ml.W = (d.grid_x + 31) / 32;
         ml.colw = 1 << (b->lay.ysh - 5);
         ml.mask_words = (uint32_t)d.grid_y * d.grid_z * ml.W;
-        ml.slots = (ml.W <= 16 ? 2 * ml.W : ml.W) + 1;
+        ml.slots = ml.W + 1;
         ml.work_bytes = (uint32_t)d.grid_z * ml.slots * 16 + (uint32_t)d.grid_x * d.grid_z * (d.grid_y < 256 ? 1 : 2);
         ml.work_off = (3 * ml.mask_words + (uint32_t)d.grid_x * d.grid_z * ml.colw + 3) / 4 * 4;
         cudaFuncAttributes fa{};
-        const void *sweep = (const void *)merge_sweep(d.grid_y);
+        const void *sweep = (const void *)merge_sweep(d.grid_y, ml.W);
         MV_CUDA(b, cudaFuncGetAttributes(&fa, sweep));
         ml.work_in_smem = ml.work_bytes + fa.sharedSizeBytes <= (size_t)b->smem_max;
         if (ml.work_in_smem)       // (to the device's maximum: the cap belongs to the function, not to this batch)
@@ -638,7 +643,7 @@ int mv_merge_voxels(mv_batch *b, int env_begin, int env_count, mv_box *d_boxes_o
                                                                           env_begin + e0, b->d_merge);
         b->launches++;
         MV_CUDA(b, cudaGetLastError());
-        merge_sweep(b->desc.grid_y)<<<n, kMergeThreads, ml.work_in_smem ? ml.work_bytes : 0, s>>>(
+        merge_sweep(b->desc.grid_y, ml.W)<<<n, kMergeThreads, ml.work_in_smem ? ml.work_bytes : 0, s>>>(
             b->d_env_blocks, b->d_mat, b->lay, ml, env_begin + e0, b->d_merge,
             reinterpret_cast<uint4 *>(d_boxes_out + (size_t)e0 * max_out), d_count_out + e0, max_out);
         b->launches++;

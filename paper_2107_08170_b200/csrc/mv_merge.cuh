@@ -14,7 +14,8 @@
 // carry-propagating additions), which begin; and the heights of a layer's boxes are independent of each other.
 //
 // Measured (512 envs of 128x32x128 with 1361 boxes each): 11.4 ms with one warp growing one box at a time (about
-// 8 us a box, all of it latency); 0.44 ms now, of which the bit arrays 0.12 and the sweep 0.29.
+// 8 us a box, all of it latency); 0.44 ms with the rows of a layer one after the other in one warp; 0.31 ms with all rows at
+// once (see sweep_layer), of which the bit arrays 0.12.
 #pragma once
 #include "mv_device.cuh"
 #include "mv_pack.cuh"
@@ -33,7 +34,7 @@ struct MergeLayout {
     int W;                    // words per x-row
     int colw;                 // words per (x, z) column
     uint32_t mask_words;      // words of one x-packed array
-    int slots;                // records per row of the sweep's work area: the row's words, twice if they fit half a warp, and an empty one
+    int slots;                // records per row of the sweep's work area: the row's words and one more
     uint32_t work_bytes;      // 16 bytes per record of one layer + one Cov per column
     uint32_t work_off;        // word offset of the work area in the env's scratch
     int work_in_smem;
@@ -142,51 +143,132 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
     }
 }
 
+// out = a + b over N words, least significant first.
+template <int N> __device__ __forceinline__ void add_words(const uint32_t *a, const uint32_t *b, uint32_t *out)
+{
+    uint32_t carry = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const unsigned long long t = (unsigned long long)a[i] + b[i] + carry;
+        out[i] = (uint32_t)t;
+        carry = (uint32_t)(t >> 32);
+    }
+}
+
+// What the sweep of a layer hands on when it has more rows than the CTA has threads, and the warps to each other.
+template <int N> struct SweepEdges {
+    uint32_t warp[2][kMergeThreads / 32][N];      // L of a warp's last row, by the parity of the round
+    uint32_t open[N], link[N];                    // cells and L of the last row of the 256 before
+};
+
+// Part B of the sweep (see merge_sweep_kernel) for rows of up to N words: one lane a row.  A row is ml.slots records of
+// {open cells, x links, z links, -}, which become {new cells, their first cells, first cells of boxes that end here, -}.
+// What a row needs of the row before is its open cells (every one is in some box) and L: which of them are in the same box as
+// their neighbour at x-1.  A box ends where one of its cells fails, and the fail takes its whole segment of L along: a carry
+// chain upward and one downward, an addition each, the second on the reversed row.  So a row's L is a function of the L before,
+// and instead of going down the rows one by one (230 cycles each, 195 us of the 290 that 512 worlds of 128x32x128 took) all
+// rows begin with the L they have when no box reaches in, and apply the function until nothing changes: after i + 1 times row i
+// is right whatever the guess was, so that ends.  What comes from above is forgotten where boxes end, and obstacles a few
+// cells deep take a few times.  A warp settles its 32 rows with the row above them as it was last published; then the
+// warps publish their last rows, until that changes nothing either.
+template <int N>
+__device__ __forceinline__ void sweep_layer(uint4 *rows, int slots, int W, int nrows, SweepEdges<N> &edges)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k0 = 0; k0 < nrows; k0 += kMergeThreads) {
+        const int k = k0 + tid;
+        uint4 *p = rows + (size_t)k * slots;
+        const bool works = k0 + 32 * warp < nrows;
+        uint32_t S[N], open[N], xl[N], fail[N], L[N], in[N], above[N];
+#pragma unroll
+        for (int w = 0; w < N; ++w) {
+            const uint4 r = w < W && k < nrows ? p[w] : make_uint4(0, 0, 0, 0);
+            S[w] = w < W && k < nrows && k > 0 ? (tid > 0 ? p[w - slots].x : edges.open[w]) : 0u;
+            open[w] = r.x; xl[w] = r.y;
+            fail[w] = S[w] & ~(r.x & r.z);
+            above[w] = tid == 0 && k0 > 0 ? edges.link[w] : 0u;
+        }
+#pragma unroll
+        for (int w = 0; w < N; ++w) L[w] = open[w] & __funnelshift_l(w ? open[w - 1] : 0u, open[w], 1) & xl[w];
+        // the cells of boxes that end with the row before, given what reaches in
+        auto ended = [&](uint32_t *D) {
+            uint32_t a[N], b[N], s[N];
+#pragma unroll
+            for (int w = 0; w < N; ++w) a[w] = fail[w] | in[w];
+            add_words<N>(a, fail, s);
+#pragma unroll
+            for (int w = 0; w < N; ++w) D[w] = fail[w] | (a[w] & (s[w] ^ a[w] ^ fail[w]));
+#pragma unroll
+            for (int w = 0; w < N; ++w) {
+                a[N - 1 - w] = __brev(fail[w] | __funnelshift_r(in[w], w + 1 < N ? in[w + 1] : 0u, 1));
+                b[N - 1 - w] = __brev(fail[w]);
+            }
+            add_words<N>(a, b, s);
+#pragma unroll
+            for (int w = 0; w < N; ++w) D[w] |= __brev(a[N - 1 - w] & (s[N - 1 - w] ^ a[N - 1 - w] ^ b[N - 1 - w]));
+        };
+        for (int round = 0;; ++round) {
+            bool news = false;
+            if (works) {
+                for (;;) {
+                    uint32_t D[N], A[N];
+#pragma unroll
+                    for (int w = 0; w < N; ++w) {
+                        in[w] = __shfl_up_sync(0xffffffffu, L[w], 1);
+                        if (lane == 0) in[w] = above[w];
+                    }
+                    ended(D);
+#pragma unroll
+                    for (int w = 0; w < N; ++w) A[w] = open[w] & ~(S[w] & ~D[w]);
+                    bool changed = false;
+#pragma unroll
+                    for (int w = 0; w < N; ++w) {
+                        const uint32_t l = (in[w] & ~D[w]) | (A[w] & __funnelshift_l(w ? A[w - 1] : 0u, A[w], 1) & xl[w]);
+                        changed |= l != L[w];
+                        L[w] = l;
+                    }
+                    if (!__any_sync(0xffffffffu, changed)) break;
+                }
+                if (lane == 31)
+#pragma unroll
+                    for (int w = 0; w < N; ++w) {
+                        news |= L[w] != (round ? edges.warp[~round & 1][warp][w] : 0u);      // (they began with nothing reaching in)
+                        edges.warp[round & 1][warp][w] = L[w];
+                    }
+            }
+            if (!__syncthreads_or(news)) break;
+            if (lane == 0 && warp > 0)
+#pragma unroll
+                for (int w = 0; w < N; ++w) above[w] = edges.warp[round & 1][warp - 1][w];
+        }
+        uint32_t D[N];
+        ended(D);
+#pragma unroll
+        for (int w = 0; w < N; ++w) {
+            const uint32_t A = open[w] & ~(S[w] & ~D[w]);
+            if (w < W && k < nrows) p[w] = make_uint4(A, A & ~L[w], D[w] & S[w] & ~in[w], 0u);
+        }
+        if (k0 + kMergeThreads < nrows) {
+            if (tid == kMergeThreads - 1)
+#pragma unroll
+                for (int w = 0; w < N; ++w) { edges.open[w] = open[w]; edges.link[w] = L[w]; }
+            __syncthreads();
+        }
+    }
+}
+
 // Carry chain along a row, one word a lane: gen | (prop & carry from the bit below), which is what an addition
 // computes.  Whole lanes generate (G) or propagate (P) a carry; two votes and one more addition carry it across them.
-__device__ __forceinline__ uint32_t fill(uint32_t gen, uint32_t prop, uint32_t lane_bit, uint32_t barrier)
+__device__ __forceinline__ uint32_t fill(uint32_t gen, uint32_t prop, uint32_t lane_bit)
 {
     const uint32_t a = gen | prop;
     uint32_t s = a + gen;
-    const uint32_t G = __ballot_sync(0xffffffffu, s < a) & barrier;
-    const uint32_t P = (__ballot_sync(0xffffffffu, s == 0xffffffffu) & barrier) | G;
+    const uint32_t G = __ballot_sync(0xffffffffu, s < a), P = __ballot_sync(0xffffffffu, s == 0xffffffffu) | G;
     s += ((P + G) ^ P ^ G) & lane_bit ? 1u : 0u;
     return gen | (a & (s ^ a ^ gen));
 }
 
-// Part B of the sweep (see merge_sweep_kernel): one warp goes down `nrows` rows of a layer.  A row is ml.slots
-// records of {open cells, x links, z links, -}, one per lane, which become {new cells, their first cells, first cells of
-// boxes that end here, -}; nothing else is read or written, so the next row's record is fetched a row ahead.
-// A box with a failing cell ends, so a fail has to spread both ways along its segment, and carries only run
-// upward.  Rows of up to 16 words are therefore held twice, in order in the lower lanes and mirrored (words and
-// bits) from lane 16 on: the same instructions spread a fail upward in one half and downward in the other, and
-// the halves then exchange what they found.  Per lane: S = cells of live boxes, L = those of them linked to the cell
-// before them in the lane's own direction.
-__device__ __forceinline__ void sweep_rows(uint4 *rows, int slots, int W, int nrows, int lane)
-{
-    const bool mirror = lane >= 16;
-    const int w = mirror ? W - 1 - (lane - 16) : lane;                  // the lane's word of the row
-    const int partner = w < 0 || w >= W ? lane : (mirror ? w : 16 + W - 1 - w);
-    uint4 *p = rows + (w < 0 || w >= W ? 2 * W : (mirror ? W + w : w));   // (idle lanes share an empty record)
-    const uint32_t lane_bit = 1u << lane;
-    uint32_t S = 0, L = 0;
-    uint4 r = *p;
-    for (int k = 0; k < nrows; ++k, p += slots) {
-        const uint4 next = p[k + 1 < nrows ? slots : 0];
-        uint32_t D = fill(S & ~(r.x & r.z), L, lane_bit, 0xffff7fffu);
-        D |= __brev(__shfl_sync(0xffffffffu, D, partner));
-        const uint32_t A = r.x & ~(S & ~D);
-        uint32_t prev = __shfl_up_sync(0xffffffffu, A, 1, 16);
-        prev = (lane & 15) ? prev : 0u;
-        const uint32_t link = A & __funnelshift_l(prev, A, 1) & r.y;
-        *p = make_uint4(A, A & ~link, D & S & ~L, 0u);
-        S = (S & ~D) | A;
-        L = (L & ~D) | link;
-        r = next;
-    }
-}
-
-// The same for rows of more than 16 words: one copy of the row, a fail spread by two chains.
+// The same for rows of more than 16 words: one warp, a word of the row per lane, the rows one after the other.
 __device__ __forceinline__ void sweep_wide_rows(uint4 *rows, int slots, int W, int nrows, int lane)
 {
     uint4 *p = rows + min(lane, W);
@@ -195,10 +277,10 @@ __device__ __forceinline__ void sweep_wide_rows(uint4 *rows, int slots, int W, i
     for (int k = 0; k < nrows; ++k, p += slots) {
         const uint4 r = *p;
         const uint32_t fail = S & ~(r.x & r.z);
-        uint32_t D = fill(fail, L, lane_bit, 0xffffffffu);
+        uint32_t D = fill(fail, L, lane_bit);
         // downward: bits reversed, lanes exchanged end for end
         const uint32_t g = __brev(__shfl_xor_sync(0xffffffffu, fail, 31)), pr = __brev(__shfl_xor_sync(0xffffffffu, Lup, 31));
-        D |= __brev(__shfl_xor_sync(0xffffffffu, fill(g, pr, lane_bit, 0xffffffffu), 31));
+        D |= __brev(__shfl_xor_sync(0xffffffffu, fill(g, pr, lane_bit), 31));
         const uint32_t A = r.x & ~(S & ~D);
         uint32_t prev = __shfl_up_sync(0xffffffffu, A, 1);
         prev = lane ? prev : 0u;
@@ -229,13 +311,12 @@ __device__ __forceinline__ int run_up(uint32_t e, const uint32_t *__restrict__ y
     return n;
 }
 
-// The sweep, one CTA per env, layer by layer: (A) all threads form the layer's open cells; (B) one warp runs
-// down the rows and leaves, per row, the cells of new boxes, their first cells and the first cells of boxes
-// that end there; (C) the new boxes are numbered in sweep order (a block-wide scan), measured, given their
-// heights and the layers above marked as covered, in parallel.  B is the serial part (about 230 cycles a row).  Cov
+// The sweep, one CTA per env, layer by layer: (A) all threads form the layer's open cells; (B) sweep_layer
+// leaves, per row, the cells of new boxes, their first cells and the first cells of boxes that end there; (C) the new boxes are numbered in sweep order (a block-wide scan), measured, given their
+// heights and the layers above marked as covered, in parallel.  Cov
 // holds a layer number: a byte where that is enough, so that four CTAs fit an SM at 128x128 columns.
-template <typename Cov>
-__global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const unsigned char *__restrict__ env_blocks,
+template <typename Cov, int N>
+__global__ void __launch_bounds__(kMergeThreads, N > 0 && N <= 4 ? 4 : N == 8 ? 3 : 1) merge_sweep_kernel(const unsigned char *__restrict__ env_blocks,
                                                                        const uint8_t *__restrict__ mat, EnvLayout lay, MergeLayout ml,
                                                                        int env_begin, uint32_t *__restrict__ scratch,
                                                                        uint4 *__restrict__ boxes_out, int32_t *__restrict__ count_out,
@@ -247,6 +328,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
     __shared__ uint16_t s_high[kMergeList], s_big[kMergeList];
     __shared__ uint8_t s_mat[kMergeList];
     __shared__ int s_nbig, s_part[kMergeThreads / 32];
+    __shared__ SweepEdges<N ? N : 1> s_edges;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, e = blockIdx.x;
     const int gx = ml.gx, gz = ml.gz, W = ml.W, slots = ml.slots;
     const unsigned char *blk = env_blocks + (size_t)(env_begin + e) * lay.stride;
@@ -258,9 +340,8 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
     uint4 *rows = reinterpret_cast<uint4 *>(ml.work_in_smem ? s_work : reinterpret_cast<unsigned char *>(mine + ml.work_off));
     Cov *cov = reinterpret_cast<Cov *>(rows + (size_t)gz * slots);      // per column: covered below this layer
     uint4 *out = boxes_out + (size_t)e * max_out * 2;
-    const bool mirrored = W <= 16;
     for (int i = tid; i < gx * gz * (int)sizeof(Cov) / 4; i += kMergeThreads) reinterpret_cast<uint32_t *>(cov)[i] = 0u;
-    for (int i = tid; i < gz; i += kMergeThreads) rows[i * slots + slots - 1] = make_uint4(0, 0, 0, 0);
+    if (N == 0) for (int i = tid; i < gz; i += kMergeThreads) rows[i * slots + slots - 1] = make_uint4(0, 0, 0, 0);     // (idle lanes share it)
     __syncthreads();
 
     const int nt = (hiz - loz) * W;                  // words of the rows that hold anything
@@ -275,7 +356,6 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
             const uint32_t *m = masks + ((size_t)j * gz + k) * W + w;
             uint32_t u = m[0];
             const uint32_t lx = m[ml.mask_words], lz = m[2 * (size_t)ml.mask_words];
-            const uint32_t lx_next = mirrored && w + 1 < W ? m[ml.mask_words + 1] : 0u;
             uint32_t c = 0;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -291,15 +371,12 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_sweep_kernel(const uns
             }
             u &= ~c;
             rows[k * slots + w] = make_uint4(u, lx, lz, 0u);
-            if (mirrored) rows[k * slots + W + w] = make_uint4(__brev(u), __brev(__funnelshift_r(lx, lx_next, 1)), __brev(lz), 0u);
             any |= u != 0u;
         }
         if (!__syncthreads_or(any)) continue;
         // ---- B
-        if (warp == 0) {
-            if (mirrored) sweep_rows(rows + loz * slots, slots, W, hiz - loz, lane);
-            else sweep_wide_rows(rows + loz * slots, slots, W, hiz - loz, lane);
-        }
+        if constexpr (N > 0) sweep_layer<N>(rows + loz * slots, slots, W, hiz - loz, s_edges);
+        else if (warp == 0) sweep_wide_rows(rows + loz * slots, slots, W, hiz - loz, lane);
         __syncthreads();
         // ---- C: number the first cells in sweep order
         const int per = (nt + kMergeThreads - 1) / kMergeThreads;

@@ -254,10 +254,12 @@ def test_scene_generators_give_the_same_arrays_on_cpu_and_gpu():
 @pytest.mark.parametrize("grid,kind,palette", [
     ((4, 4, 4), "random", 3), ((32, 8, 12), "random", 2), ((36, 12, 20), "random", 4), ((100, 36, 24), "random", 3),
     ((68, 68, 8), "random", 1), ((64, 32, 64), "solid", 2), ((128, 8, 128), "checker", 2), ((1024, 4, 8), "slabs", 3),
-    ((512, 4, 512), "slabs", 3)])
+    ((512, 4, 512), "slabs", 3), ((64, 4, 300), "stairs", 2), ((132, 4, 516), "stairs", 2), ((256, 4, 260), "slabs", 2),
+    ((516, 4, 36), "stairs", 2), ((528, 4, 40), "slabs", 2)])
 def test_merge_voxels_grid_shapes(oracle, grid, kind, palette):
     """Rows of one, several and 32 words, ragged last words, columns of several words, more new boxes in a
-    layer than are handled at a time (checker), footprints of every size, and a layer too large for shared memory."""
+    layer than are handled at a time (checker), footprints of every size, a layer too large for shared memory, and
+    steps a cell wide all the way down (stairs), where what a row's boxes are depends on the rows far above it."""
     from paper_2107_08170_b200 import binding as B
     gx, gy, gz = grid
     rng = np.random.default_rng(gx * gy + gz)
@@ -270,6 +272,11 @@ def test_merge_voxels_grid_shapes(oracle, grid, kind, palette):
         y, z, x = np.ogrid[:gy, :gz, :gx]
         g[:] = ((x + z) & 1) * (1 + (y // 3 & 1))
         g[2] = np.where((x + z + y) & 1, 1, 0)
+    elif kind == "stairs":                               # every row's run begins and ends a cell further on than the last
+        k, i = np.arange(gz)[:, None], np.arange(gx)[None, :]
+        g[0] = ((i - k) % 24 < 17).astype(np.uint8)
+        g[1] = 1 + ((i + k // 2) % 40 < 3)
+        g[2] = ((i - k) % 31 < 30) & ((i + 2 * k) % 57 < 55)
     elif kind == "slabs":                                # random boxes over each other: long runs, ragged ends
         for e in range(E):
             for _ in range(200):
