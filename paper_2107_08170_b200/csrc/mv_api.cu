@@ -18,10 +18,14 @@ using namespace mv;
 
 namespace {
 
-constexpr int kRenderThreads = 384;            // threads per CTA of the render kernel...
-constexpr int kRenderThreadsSmall = 192;       // ...and for CTAs with few tiles (small images): twice as many, shorter CTAs per SM
-// Below this many tiles per CTA the small shape is faster when there are CTAs enough to fill the GPU with it
-// (measured: 64x36 images +10 %; 128x72 -2 %; four CTAs alone on the GPU -20 %: fewer warps per CTA, longer CTA).
+// Threads per CTA of the render kernel, by how many CTAs the staged blocks leave room for on an SM: three (or more) of 384 threads or
+// two of 576, so that as many warps walk (2048 x 2 observations of 160x32x160 rooms, 104 KB a block: 342 us with 384, 308).
+// (Blocks that would leave one alone are staged in small batches only, see mv_create_batch.)
+constexpr int kRenderThreads = 384, kRenderThreadsTwo = 576;
+constexpr int kRenderThreadsSmall = 192;       // CTAs with few tiles (small images): twice as many, shorter CTAs per SM
+// Below this many tiles per CTA the small shape is faster when there are CTAs enough to fill the GPU with it and room for five on
+// an SM (measured: 64x36 images +10 %; 128x72 -2 %; four CTAs alone on the GPU -20 %: fewer warps per CTA, longer CTA; 48x36
+// with room for five 135.7 us, 140.2 with three of the ordinary shape).
 constexpr int kSmallCtaTiles = 192;
 constexpr int kHostChunks = 8;
 // CTAs that split the tiles of an observation between them, in a batch with few of them (see pick_parts): this many times
@@ -68,6 +72,7 @@ struct mv_batch {
     int wait_polls = 1 << 18;
     bool occ_shared = true;             // occupancy staged in shared memory (else read from global)
     bool occ_fits_shared = true;
+    int smem_sm = 0;                    // shared memory of an SM
     int smem_max = 0;                   // opt-in shared memory per CTA of the device
     int auto_agents_per_cta = 1;        // the library's own choice (a test hook can override it)
     int skip_staging = 0;
@@ -112,7 +117,7 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // Shared-memory layout of the render kernel when one CTA renders `apc` observations of an env:
 // staged env block (without the occupancy when that stays in global memory), tile table, then one block per agent (ray
 // table, camera record, eye-relative boxes, overlay rectangles, per-tile masks of boxes and the GUI bit), then the barrier
-// and flag words.
+// and flag words and the planes' guards.
 mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     const mv_batch_desc &d = b->desc;
     const uint32_t ntiles = (uint32_t)(b->tiles_x * b->tiles_y);
@@ -126,7 +131,7 @@ mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     const uint32_t agent_bytes = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
     m.agent_stride = apc > 1 ? round_up(agent_bytes, kAgentAlign) : agent_bytes;
     m.misc_off = m.agent_off + (uint32_t)apc * m.agent_stride;
-    m.bytes = m.misc_off + 32;
+    m.bytes = m.misc_off + 16 + round_up((b->lay.planes + 2) * 4, 16);
     return m;
 }
 
@@ -146,12 +151,12 @@ cudaError_t launch_step(void (*kernel)(Params...), dim3 grid, dim3 block, size_t
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
-// Threads per CTA: the small shape for CTAs with few tiles, if the batch has CTAs enough to fill the GPU
-// six to an SM.
 int pick_threads(const mv_batch *b, int apc) {
+    const int per_sm = b->smem_sm / ((int)smem_layout(b, apc, b->occ_shared).bytes + 1024);        // (1 KB of every CTA is the system's)
+    if (per_sm < 3) return kRenderThreadsTwo;
     const bool few_tiles = b->tiles_x * b->tiles_y * apc < kSmallCtaTiles;
     const bool fills = (int64_t)b->num_obs / apc >= (int64_t)6 * b->sms;
-    return few_tiles && fills ? kRenderThreadsSmall : kRenderThreads;
+    return few_tiles && fills && per_sm >= 5 ? kRenderThreadsSmall : kRenderThreads;
 }
 
 // CTAs per observation (or environment) in a batch with few of them: as many as make three CTAs to an SM (six of the small
@@ -168,7 +173,7 @@ int pick_threads(const mv_batch *b, int apc) {
 // (columns: 148 of 64x36 on 160x64x160 27.6*, unsplit 23.0); in rooms it is the other way round (180 of 64x36 on 192x32x192:
 // 23.0*, unsplit 29.2).
 int pick_parts(const mv_batch *b, int64_t ctas) {
-    const int per_sm = b->threads == kRenderThreads ? 3 : 6;
+    const int per_sm = kThreadsPerSm / b->threads;
     const int64_t slots = (int64_t)per_sm * b->sms * (b->occ_shared ? 1 : kPartWaves);
     const int64_t most = b->tiles_x * b->tiles_y / (b->threads / 32);
     int64_t parts = b->forced_parts > 0 ? b->forced_parts : slots / ctas;
@@ -176,16 +181,24 @@ int pick_parts(const mv_batch *b, int64_t ctas) {
     return parts < 1 ? 1 : (int)parts;
 }
 
-// The three instantiations of the render kernel: column-word walk (grid at most 32 high, occupancy
-// staged), indexed walk with staged occupancy, indexed walk with the occupancy in global memory.
+// The instantiations of the render kernel: by the CTA's threads, and one plane of occupancy staged, several staged, or read from
+// global memory.
 using RenderFn = void (*)(const RenderParams);
-RenderFn render_fn(const mv_batch *b) {
-    if (b->threads == kRenderThreadsSmall) {
-        if (!b->occ_shared) return render_kernel<kRenderThreadsSmall, false, false>;
-        return b->lay.ysh == 5 ? render_kernel<kRenderThreadsSmall, true, true> : render_kernel<kRenderThreadsSmall, true, false>;
-    }
-    if (!b->occ_shared) return render_kernel<kRenderThreads, false, false>;
-    return b->lay.ysh == 5 ? render_kernel<kRenderThreads, true, true> : render_kernel<kRenderThreads, true, false>;
+template <int NT> RenderFn render_fn_of(const mv_batch *b, bool occ_shared) {
+    if (!occ_shared) return render_kernel<NT, kOccGlobal>;
+    return b->lay.planes == 1 ? render_kernel<NT, kOccWord> : render_kernel<NT, kOccPlanes>;
+}
+RenderFn render_fn(const mv_batch *b, int threads, bool occ_shared) {
+    return threads == kRenderThreadsSmall ? render_fn_of<kRenderThreadsSmall>(b, occ_shared) : threads == kRenderThreads ? render_fn_of<kRenderThreads>(b, occ_shared)
+           : render_fn_of<kRenderThreadsTwo>(b, occ_shared);
+}
+RenderFn render_fn(const mv_batch *b) { return render_fn(b, b->threads, b->occ_shared); }
+
+// CTA shape of the render kernel when a CTA renders `apc` observations of an environment.
+void choose_shape(mv_batch *b, int apc) {
+    b->agents_per_cta = apc;
+    b->smem = smem_layout(b, apc, b->occ_shared);
+    b->threads = pick_threads(b, apc);
 }
 
 // The merge sweep keeps a layer number per column: a byte for grids less than 256 high.  Rows of up to 16 words (W) are held in
@@ -256,12 +269,13 @@ int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int en
     for (int c = 0; c < 3; ++c) u.light[c] = (double)d.light_dir[c];
     u.ambient = (double)d.ambient;
     auto ctas = [](size_t threads) { return (threads + kUploadThreads - 1) / kUploadThreads; };
-    u.tiles_per_word = (int)ctas((size_t)(d.grid_x / 4) * d.grid_z);
-    u.tiles_per_env = u.tiles_per_word * ((d.grid_y + 31) / 32);         // (words above grid_y stay zero)
+    u.words = (d.grid_y + 31) / 32;
+    u.tiles_per_env = (int)ctas((size_t)(d.grid_x / 4) * d.grid_z) * u.words;
     // tiles a CTA packs one after the other: one, until there are two CTAs for every slot of the GPU (164 / 512 envs of
     // 128x32x128: 62 / 119 us with three CTAs of 256 threads per SM and four for every slot, 53 / 114 like this)
     const int64_t per_slot = (int64_t)u.tiles_per_env * env_count / (12 * 2 * (int64_t)b->sms);
     u.tiles_per_cta = (int)(per_slot < 1 ? 1 : per_slot > 8 ? 8 : per_slot);
+    u.tiles_per_cta = (u.tiles_per_cta + u.words - 1) / u.words * u.words;     // (a column's tiles are one CTA's: a plane may need two)
     u.pack_ctas_per_env = (u.tiles_per_env + u.tiles_per_cta - 1) / u.tiles_per_cta;
     const size_t pack = d_grid ? (size_t)u.pack_ctas_per_env * env_count : 0;
     const size_t lut = d_palette ? ctas((size_t)env_count * kFaces * d.palette_size) : 0;
@@ -435,12 +449,14 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     b->missing_grid = b->missing_palette = d.num_envs;
 
     EnvLayout &L = b->lay;
-    L.ysh = 5;                                              // bits per (x, z) column: a power of two >= grid_y, >= 32
+    L.ysh = 5;                                              // material bytes per (x, z) column: a power of two >= grid_y, >= 32
     while ((1 << L.ysh) < d.grid_y) L.ysh++;
     L.pitch = (uint32_t)d.grid_x + 1;
     L.origin = L.pitch + 1;                                 // a fence row, and the fence column before x = 0
     const size_t columns = (size_t)L.pitch * (d.grid_z + 2) + 1;
-    L.occ_bytes = (uint32_t)(((columns << L.ysh) / 8 + 15) / 16 * 16);
+    L.planes = d.grid_y <= 32 ? 1 : (uint32_t)((d.grid_y + kPlaneHeights - 1) / kPlaneHeights);
+    L.occ_plane = round_up((uint32_t)columns * 4, 16);
+    L.occ_bytes = L.planes * L.occ_plane;
     b->mat_bytes_per_env = (columns << L.ysh);
     L.lut_off = L.occ_bytes;
     L.box_off = L.lut_off + round_up(kFaces * d.palette_size * 4, 16);
@@ -471,18 +487,24 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d.device);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
     b->smem_max = smem_max;
-    // the occupancy normally rides in shared memory with the rest of the env block; a grid too large
-    // for that keeps it in global memory and stages only the block's tail
-    b->occ_fits_shared = b->occ_shared = (int64_t)smem_layout(b, 1, true).bytes <= smem_max;
+    b->sms = sms;
+    e = cudaDeviceGetAttribute(&b->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, d.device);
+    if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
+    // The occupancy normally rides in shared memory with the rest of the env block.  It stays in global memory where it does not
+    // fit, and where it would leave one CTA on an SM with nobody to work while it is staged, if there are observations for more
+    // than a CTA an SM: of such a grid the rays see a small part, which the cache holds (2048 observations, staged in one CTA of
+    // 1024 threads, and three of 384 with global loads: 192x32x192 rooms 229 us and 200, 128x64x128 rooms 227 and 158, 64x36
+    // images of them 128 and 57; worse for 192x32x192 columns only, 227 and 260.  With room for two, 144 to 160 wide, staged is
+    // 17 to 29 % faster.  2 observations of 148x56x112: a step of 12.3 us staged, 16.3 with global loads).
+    b->occ_fits_shared = (int64_t)smem_layout(b, 1, true).bytes <= smem_max;
+    b->occ_shared = b->occ_fits_shared && (b->num_obs <= sms || 2 * ((int64_t)smem_layout(b, 1, true).bytes + 1024) <= b->smem_sm);
     b->smem = smem_layout(b, 1, b->occ_shared);
     if ((int64_t)b->smem.bytes > smem_max) { delete b; return MV_ERR_UNSUPPORTED; }
     // The dynamic shared-memory cap is a property of the kernel function on this device, shared by
     // every batch: raise it to the device's maximum once, never to one batch's own size.
-    for (RenderFn f : {RenderFn(render_kernel<kRenderThreads, true, true>), RenderFn(render_kernel<kRenderThreads, true, false>),
-                       RenderFn(render_kernel<kRenderThreads, false, false>), RenderFn(render_kernel<kRenderThreadsSmall, true, true>),
-                       RenderFn(render_kernel<kRenderThreadsSmall, true, false>),
-                       RenderFn(render_kernel<kRenderThreadsSmall, false, false>)})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    for (int threads : {kRenderThreadsSmall, kRenderThreads, kRenderThreadsTwo})
+        for (RenderFn f : {render_fn(b, threads, true), render_fn(b, threads, false)})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(upload_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUploadSmem);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
     // One CTA per environment (block staged once for all its agents) when that still fills the GPU;
@@ -492,7 +514,8 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
         if ((int64_t)all.bytes <= smem_max) {
             auto shape_cost = [&](const mv_batch::Smem &m, int apc) {
                 int per_sm = 0;
-                cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_fn(b), kRenderThreads, m.bytes);
+                const int threads = pick_threads(b, apc);
+                cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_fn(b, threads, b->occ_shared), threads, m.bytes);
                 if (q != cudaSuccess || per_sm < 1) return 1e30;
                 // CTAs of different length drift apart, so there are no waves: what the slots have to do, and on average half a
                 // CTA of waiting for the last ones (777 envs x 3 agents: 121 us by environment, 115 by observation)
@@ -505,8 +528,7 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
         }
     }
 
-    b->sms = sms;
-    b->threads = pick_threads(b, b->agents_per_cta);
+    choose_shape(b, b->agents_per_cta);
 
     const size_t blocks_bytes = (size_t)d.num_envs * L.stride;
     bool ok = cudaMalloc(&b->d_env_blocks, blocks_bytes) == cudaSuccess &&
@@ -639,7 +661,7 @@ int mv_merge_voxels(mv_batch *b, int env_begin, int env_count, mv_box *d_boxes_o
     const int per_env = (ml.W + 3) / 4 * ((ml.gz + 7) / 8) * ml.colw;
     for (int e0 = 0; e0 < env_count; e0 += b->merge_chunk) {
         const int n = env_count - e0 < b->merge_chunk ? env_count - e0 : b->merge_chunk;
-        merge_masks_kernel<<<(unsigned)n * per_env, kMergeThreads, 0, s>>>(b->d_env_blocks, b->d_mat, b->lay, ml,
+        (b->lay.planes > 1 ? merge_masks_kernel<true> : merge_masks_kernel<false>)<<<(unsigned)n * per_env, kMergeThreads, 0, s>>>(b->d_env_blocks, b->d_mat, b->lay, ml,
                                                                           env_begin + e0, b->d_merge);
         b->launches++;
         MV_CUDA(b, cudaGetLastError());
@@ -812,7 +834,7 @@ int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     if (!b) return MV_ERR_INVALID_ARG;
     if (!on && !b->occ_fits_shared) return MV_ERR_UNSUPPORTED;
     b->occ_shared = !on;
-    b->smem = smem_layout(b, b->agents_per_cta, b->occ_shared);
+    choose_shape(b, b->agents_per_cta);
     return MV_OK;
 }
 
@@ -830,9 +852,7 @@ int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {
     if ((int64_t)smem_layout(b, apc, false).bytes > b->smem_max) return MV_ERR_UNSUPPORTED;
     b->occ_fits_shared = (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max;
     if (!b->occ_fits_shared) b->occ_shared = false;
-    b->smem = smem_layout(b, apc, b->occ_shared);
-    b->agents_per_cta = apc;
-    b->threads = pick_threads(b, apc);
+    choose_shape(b, apc);
     return MV_OK;
 }
 

@@ -25,22 +25,26 @@ static_assert(sizeof(CamRec) == 64, "CamRec must be 64 bytes");
 
 // One environment's render inputs, contiguous in HBM so that a single bulk copy stages them
 // into shared memory:  [occupancy bits | shade LUT | boxes | box count + occupied bounds].
-// Occupancy is packed along y: the (x, z) column owns 2^ysh consecutive bits (2^ysh >= grid_y, at
-// least 32), bit index u = ((origin + x + pitch*z) << ysh) | y, bit u&31 of word u>>5.  A walk along x or z
-// therefore moves by whole words and a walk along y stays inside the column's word(s); for grids
-// up to 32 voxels high a column is exactly one word.  The material store uses the same index u.
+// Occupancy is packed along y: a word holds the lowest heights of an (x, z) column, a walk along x or z moves by whole words and
+// a walk along y stays inside the word.  Grids of up to 32 heights are one plane of such words.  Higher ones are several, 31
+// heights each, one plane behind the other: bit 31 of a plane is never a voxel, so a walk up or down that leaves the plane
+// meets it (as it meets the fence) and goes on in the next one, and an environment filled only low down needs only its
+// lowest planes.  Where the occupancy is not staged as a rule, the planes are the same.
+// Materials are a byte per voxel at index u = (column << ysh) | y, 2^ysh >= grid_y, at least 32.
 // The grid is fenced in: one column between each row and the next (pitch = grid_x + 1) and a row before the first and
 // after the last are all ones, written once when the batch is made, so a walk in x and z that leaves the grid hits
 // something at once instead of having to be stopped by a test at every step.
 struct EnvLayout {
-    uint32_t occ_bytes;     // (pitch*(grid_z + 2) + 1) columns of 2^ysh bits, rounded up to 16
+    uint32_t occ_bytes;     // planes * occ_plane
+    uint32_t occ_plane;     // bytes of a plane: (pitch*(grid_z + 2) + 1) words, rounded up to 16
+    uint32_t planes;        // 1, or ceil(grid_y / 31) for grids more than 32 high
     uint32_t lut_off;       // 7*palette_size RGBX words
     uint32_t box_off;       // max_boxes * 32 bytes
     uint32_t count_off;     // 32 bytes: {box count, lo x,y,z, hi x,y,z, pad}; [lo, hi) = cell box
                             // that contains every filled voxel (lo > hi when the grid is empty)
     uint32_t block_bytes;   // bytes staged per CTA (multiple of 16)
     uint32_t stride;        // distance between envs in HBM (multiple of 128)
-    uint32_t ysh;           // log2 of the bits per (x, z) column
+    uint32_t ysh;           // log2 of the material bytes per (x, z) column
     uint32_t pitch, origin; // columns from one row to the next; column of (0, 0)
 };
 
@@ -51,6 +55,16 @@ __host__ __device__ __forceinline__ uint32_t voxel_index(const EnvLayout &lay, i
     return (column_index(lay, x, z) << lay.ysh) | (uint32_t)y;
 }
 
+// Plane of height y, and the height at which a plane begins.
+constexpr uint32_t kPlaneHeights = 31, kPlaneEnd = 0x80000000u;
+__host__ __device__ __forceinline__ uint32_t plane_of(const EnvLayout &lay, int y) { return lay.planes == 1 ? 0u : (uint32_t)y / kPlaneHeights; }
+__host__ __device__ __forceinline__ int plane_begin(uint32_t plane) { return (int)(plane * kPlaneHeights); }
+// Is the voxel filled, by the occupancy at `occ` (an env block, or what is staged of it)?
+__device__ __forceinline__ bool voxel_filled(const EnvLayout &lay, const unsigned char *occ, int x, int y, int z) {
+    const uint32_t q = plane_of(lay, y);
+    const uint32_t w = *reinterpret_cast<const uint32_t *>(occ + (size_t)q * lay.occ_plane + 4u * column_index(lay, x, z));
+    return (w >> (y - plane_begin(q))) & 1u;
+}
 struct RenderParams {
     const unsigned char *env_blocks;   // [E] EnvLayout blocks
     const uint8_t *mat;                // [E][mat_stride] material ids by voxel index (clamped at upload)

@@ -58,6 +58,7 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t v, int lane)
 // four rows, so that the column at z-1 is still in registers; the y-packed results are transposed in registers and
 // leave through shared memory as runs of up to 128 bytes.  Bound by the material bytes it streams (one byte per
 // voxel, the x-1 column from L1) once the upper 16 heights are left out where nothing is filled up there.
+template <bool PLANES>
 __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsigned char *__restrict__ env_blocks,
                                                                     const uint8_t *__restrict__ mat, EnvLayout lay,
                                                                     MergeLayout ml, int env_begin, uint32_t *__restrict__ scratch)
@@ -74,8 +75,20 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
     __shared__ uint32_t s_out[3][32][8 * 4 + 1];     // (padded: the writes run down a column)
     const int lane = threadIdx.x & 31, wi = (threadIdx.x >> 5) & 3, half = threadIdx.x >> 7;
     const int w = 4 * wb + wi, x = 32 * w + lane, z0 = 8 * zb + 4 * half;
-    const bool upper = hiy - 32 * wq > 16, in_x = x < ml.gx;
-    const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk) + (lay.origin + x) * ml.colw + wq;
+    const bool upper = hiy - 32 * wq > 16, higher = hiy - 32 * wq > 32, in_x = x < ml.gx;
+    // 32 heights of a column, and the one above them (PLANES: of the two or three planes that they lie in, as far as anything is filled)
+    const uint32_t plane = PLANES ? plane_of(lay, 32 * wq) : 0u, off = 32u * (uint32_t)wq - (uint32_t)plane_begin(plane), words = lay.occ_plane / 4;
+    const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk) + (size_t)plane * words + lay.origin + x;
+    const bool second = PLANES && plane + 1 < lay.planes && hiy > plane_begin(plane + 1), third = second && off > 29 && plane + 2 < lay.planes;
+    auto bits = [&](int at, uint32_t &above) {
+        const uint32_t *w = occ + at;
+        if (!PLANES) { above = 0u; return w[0]; }
+        unsigned long long b = (w[0] & ~kPlaneEnd) >> off;
+        if (second) b |= (unsigned long long)(w[words] & ~kPlaneEnd) << (kPlaneHeights - off);
+        if (third) b |= (unsigned long long)w[2 * words] << (2 * kPlaneHeights - off);
+        above = (uint32_t)(b >> 32);
+        return (uint32_t)b;
+    };
     const uint8_t *m_col = mat + (size_t)(env_begin + e) * ml.mat_stride + ((size_t)(lay.origin + x) << lay.ysh) + 32 * wq;
     uint32_t *ye = scratch + (size_t)e * ml.env_words + 3 * (size_t)ml.mask_words + x * ml.colw + wq;
     auto load_column = [&](const uint8_t *src, uint32_t out[8]) {
@@ -98,9 +111,9 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
         if (upper) ne |= (differ8(4) << 9) | (differ8(6) << 17);
         return ~ne;
     };
-    uint32_t own[8] = {}, back[8] = {}, f_back = 0;
+    uint32_t own[8] = {}, back[8] = {}, f_back = 0, f_above = 0;
     if (in_x && z0 > 0 && z0 < ml.gz) {
-        f_back = occ[(size_t)(z0 - 1) * lay.pitch * ml.colw];
+        f_back = bits((z0 - 1) * (int)lay.pitch, f_above);
         load_column(m_col + ((size_t)(z0 - 1) * lay.pitch << lay.ysh), back);
     }
 #pragma unroll
@@ -108,19 +121,18 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
         const int z = z0 + i;
         uint32_t f = 0, lx = 0, lz = 0;
         if (z < ml.gz && in_x) {
-            const size_t row = (size_t)z * lay.pitch;
-            const uint8_t *src = m_col + (row << lay.ysh);
-            f = occ[row * ml.colw];
-            uint32_t other[8], f_left = 0;
+            const int row = z * (int)lay.pitch;
+            const uint8_t *src = m_col + ((size_t)row << lay.ysh);
+            uint32_t other[8], f_left = 0, unused;
+            f = bits(row, f_above);
             load_column(src, own);
             if (x > 0) {
-                f_left = occ[(row - 1) * ml.colw];
+                f_left = bits(row - 1, unused);
                 load_column(src - (1u << lay.ysh), other);
             }
             lz = f & f_back & equal_bits(own, back);
             if (x > 0) lx = f & f_left & equal_bits(own, other);
-            uint32_t above = 0, f_above = 0;
-            if (wq + 1 < ml.colw) { above = src[32]; f_above = occ[row * ml.colw + 1] & 1u; }
+            const uint32_t above = PLANES && higher ? src[32] : 0u;
 #pragma unroll
             for (int q = 0; q < 7; ++q) other[q] = __funnelshift_r(own[q], own[q + 1], 8);     // one height up
             other[7] = (own[7] >> 8) | (above << 24);

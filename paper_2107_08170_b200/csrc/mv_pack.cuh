@@ -52,12 +52,11 @@ constexpr int kUploadSmem = kUploadStages * 32 * kUploadThreads * 4;
 // The fence around the columns of every env (see EnvLayout); grid columns keep their zeros.
 __global__ void fence_kernel(unsigned char *env_blocks, EnvLayout lay, int gx, int gz, int num_envs)
 {
-    const int colw = 1 << (lay.ysh - 5);
     const int words = (int)(lay.occ_bytes / 4);
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long e = gid / words;
     if (e >= num_envs) return;
-    const int w = (int)(gid - e * words), c = w / colw - 1, z = c < 0 ? -1 : c / (int)lay.pitch - 1;
+    const int w = (int)(gid - e * words), c = w % (int)(lay.occ_plane / 4) - 1, z = c < 0 ? -1 : c / (int)lay.pitch - 1;
     const int x = c - (z + 1) * (int)lay.pitch;
     if (z < 0 || z >= gz || x < 0 || x >= gx) reinterpret_cast<uint32_t *>(env_blocks + (size_t)e * lay.stride)[w] = 0xffffffffu;
 }
@@ -82,7 +81,7 @@ struct UploadArgs {
     EnvLayout lay;
     int env_begin, env_count;
     int gx, gy, gz, max_boxes, palette;
-    int tiles_per_word, tiles_per_env, tiles_per_cta, pack_ctas_per_env;     // tiles of 256 columns x 32 heights
+    int words, tiles_per_env, tiles_per_cta, pack_ctas_per_env;     // tiles of 256 columns x 32 heights, `words` of them one above the other
     // CTAs [0, pack_ctas) pack, the next lut_ctas shade, the rest copy boxes
     unsigned pack_ctas, lut_ctas;
     int wait_polls;                    // bound of the wait for a tile's copies
@@ -104,7 +103,7 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
     extern __shared__ __align__(128) uint32_t s_tile[];       // [kUploadStages][32][kUploadThreads]
     __shared__ uint64_t s_bar[kUploadStages];
     __shared__ int s_acc[6], s_last, s_bad;
-    const int colw = 1 << (p.lay.ysh - 5), xg_n = p.gx / 4;   // words per column, groups of four columns per row
+    const int xg_n = p.gx / 4;                                // groups of four columns per row
     const int e = (int)(blockIdx.x / (unsigned)p.pack_ctas_per_env), part = (int)(blockIdx.x - (unsigned)e * p.pack_ctas_per_env);
     const size_t env = upload_env(p.env_index, p.env_begin, (size_t)e);
     unsigned char *blk = p.env_blocks + env * p.lay.stride;
@@ -119,8 +118,8 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
     const bool withheld = p.skip_staging && part == p.pack_ctas_per_env - 1;
     auto fetch = [&](int tile) {                              // one warp
         if (withheld) return;
-        const int stage = (tile - tile_begin) % kUploadStages, wq = tile / p.tiles_per_word;
-        const int r0 = (tile - wq * p.tiles_per_word) * kUploadThreads, heights = min(p.gy - 32 * wq, 32);
+        const int stage = (tile - tile_begin) % kUploadStages, wq = p.words == 1 ? 0 : tile % p.words;
+        const int r0 = (p.words == 1 ? tile : tile / p.words) * kUploadThreads, heights = min(p.gy - 32 * wq, 32);
         const uint32_t bytes = 4u * (uint32_t)min(groups - r0, kUploadThreads);
         if (threadIdx.x == 0) mbar_expect_tx(&s_bar[stage], bytes * (uint32_t)heights);
         __syncwarp();
@@ -131,7 +130,7 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
     if (threadIdx.x < 32)
         for (int t = tile_begin; t < min(tile_begin + kUploadStages, tile_end); ++t) fetch(t);
     int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-1, -1, -1};
-    uint32_t clamped = 0;
+    uint32_t clamped = 0, below[4] = {0, 0, 0, 0};            // the columns' 32 heights below these
     for (int tile = tile_begin; tile < tile_end; ++tile) {
         const int n = tile - tile_begin, stage = n % kUploadStages;
         const uint32_t parity = (uint32_t)(n / kUploadStages) & 1u;
@@ -146,8 +145,8 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
             }
             break;
         }
-        const int wq = tile / p.tiles_per_word, heights = min(p.gy - 32 * wq, 32);
-        const int r = (tile - wq * p.tiles_per_word) * kUploadThreads + (int)threadIdx.x;
+        const int wq = p.words == 1 ? 0 : tile % p.words, heights = min(p.gy - 32 * wq, 32);
+        const int r = (p.words == 1 ? tile : tile / p.words) * kUploadThreads + (int)threadIdx.x;
         uint32_t col[4][8], bits[4] = {0, 0, 0, 0};
         const uint32_t cap = (uint32_t)(p.palette - 1);
         // a byte exceeds cap iff bit 7 of ((low seven bits + add) combined with the byte) is set
@@ -198,8 +197,22 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
         for (int c = 0; c < 4; ++c)
             store32(mdst + ((size_t)c << p.lay.ysh), col[c][0], col[c][1], col[c][2], col[c][3], col[c][4], col[c][5],
                     col[c][6], col[c][7]);
+        // (a plane's 31 heights begin q heights down in the tile below; the last tile also fills the planes above its own)
+        const uint32_t words = p.lay.occ_plane / 4;
+        if (p.lay.planes == 1) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) occ[(col0 + c) * colw + wq] = bits[c];
+            for (int c = 0; c < 4; ++c) occ[col0 + c] = bits[c];
+        } else {
+            for (int q = wq; q == wq || (wq == p.words - 1 && q < (int)p.lay.planes); ++q)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t off = (kPlaneHeights * (uint32_t)q) & 31u;
+                    const uint32_t w = q == 0 ? bits[c] : q == wq ? __funnelshift_r(below[c], bits[c], off) : bits[c] >> off;
+                    occ[(size_t)q * words + col0 + c] = w & ~kPlaneEnd;
+                }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) below[c] = bits[c];
         const uint32_t any = bits[0] | bits[1] | bits[2] | bits[3];
         if (any) {
             lo[0] = min(lo[0], 4 * xg + (bits[0] ? 0 : bits[1] ? 1 : bits[2] ? 2 : 3));
@@ -332,7 +345,7 @@ __global__ void camera_kernel(const int32_t *cams, CamRec *out, int num_obs,
 
 // True iff the body box around (x, y, z) lies inside the grid and touches no filled voxel
 // (cells floor(lo)..floor(hi) on every axis, ends included).
-__device__ __forceinline__ bool body_free(const uint32_t *occ, const EnvLayout &lay, int gx, int gy, int gz, float x, float y,
+__device__ __forceinline__ bool body_free(const unsigned char *occ, const EnvLayout &lay, int gx, int gy, int gz, float x, float y,
                                           float z, float hw, float below, float above)
 {
     const float lx = __fsub_rn(x, hw), hx = __fadd_rn(x, hw);
@@ -345,10 +358,8 @@ __device__ __forceinline__ bool body_free(const uint32_t *occ, const EnvLayout &
     const int k0 = (int)floorf(lz), k1 = (int)floorf(hz);
     for (int j = j0; j <= j1; ++j)
         for (int k = k0; k <= k1; ++k)
-            for (int i = i0; i <= i1; ++i) {
-                const uint32_t v = voxel_index(lay, i, j, k);
-                if ((occ[v >> 5] >> (v & 31)) & 1u) return false;
-            }
+            for (int i = i0; i <= i1; ++i)
+                if (voxel_filled(lay, occ, i, j, k)) return false;
     return true;
 }
 
@@ -377,10 +388,9 @@ __global__ void move_agents_kernel(int32_t *cams, const float4 *moves, CamRec *r
     const float x_try = (float)__dadd_rn((double)x, sxd);
     const float z_try = (float)__dadd_rn((double)z, szd);
     unsigned char *blk = env_blocks + (size_t)(o / agents) * lay.stride;
-    const uint32_t *occ = reinterpret_cast<const uint32_t *>(blk);
     float nx = x, nz = z;
-    if (body_free(occ, lay, gx, gy, gz, x_try, y, nz, hw, below, above)) nx = x_try;
-    if (body_free(occ, lay, gx, gy, gz, nx, y, z_try, hw, below, above)) nz = z_try;
+    if (body_free(blk, lay, gx, gy, gz, x_try, y, nz, hw, below, above)) nx = x_try;
+    if (body_free(blk, lay, gx, gy, gz, nx, y, z_try, hw, below, above)) nz = z_try;
     c[0] = __float_as_int(nx); c[2] = __float_as_int(nz);
     c[3] = __float_as_int(yaw); c[4] = __float_as_int(pitch);
     const int self_box = c[5];

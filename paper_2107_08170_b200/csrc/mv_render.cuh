@@ -16,6 +16,11 @@
 // The walk is confined to the cell box that holds every filled voxel of the environment (built at
 // upload), so rays that leave it stop at once; GUI rectangles, if any, are painted over the colour
 // just before the store.
+//
+// Grids more than 32 high take the same path plane by plane (EnvLayout; a walk changes planes outside its loop).  Until they
+// did they were walked by voxel index, sixteen instructions a step instead of thirteen and the tile set-up in C++: 4096
+// observations of 64x36x64 rooms 317 us, now 259; 1980 x 2 of 20x52x64 462, now 373; 6005 of 144x64x136 columns, of whose three
+// planes only the lowest is used and copied, 496, now 197; 192x48x192 (global memory) 95, now 88.
 #pragma once
 #include "mv_device.cuh"
 
@@ -67,12 +72,11 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 //    shared-memory address `pos` of the (x, z) column's word and a one-bit mask `bit` of the height;
 //    x and z steps add a byte stride to the address, a y step rotates the mask by 1 or 31, and the
 //    test is one load and one AND.
-//  * indexed (any grid): the state is the voxel index `pos` (plus 8x the shared-memory byte address
-//    of the occupancy when it is staged, so that (pos >> 3) & ~3 is the word's address and pos & 31
-//    the bit); every step adds a stride.
+//  * planes (any grid, see EnvLayout): the same within a plane, bit 31 counting as filled in every column; a walk that meets it
+//    on the way up or down goes on in the next plane (MV_DDA_CROSS).  Where the occupancy is not staged, `pos` is the word's
+//    byte offset in the environment's block and the load is a global one.
 // Register names used by the macros (declared by the enclosing asm block): tx ty tz dtx dty dtz
-// (f32), sx sy sz pos bit w a it (b32), ta tb (f32), px py pz pq ph pf (pred), texit (f32); the
-// global flavour also uses ag (b64) and the operand named by MV_DDA_GBASE.
+// (f32), sx sy sz pos bit guard w a it q (b32), ta tb (f32), px py pz pq ph pf (pred), texit (f32), ag gbase (b64).
 #define MV_DDA_HEAD(T, OUT)                          \
     " min.f32 " T ", tx, ty, tz;\n"                  \
     " setp.geu.or.f32 pq, " T ", texit, ph;\n"       \
@@ -82,40 +86,32 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " @px add.f32 tx, tx, dtx;\n"                    \
     " @py add.f32 ty, ty, dty;\n"                    \
     " @pz add.f32 tz, tz, dtz;\n"
-#define MV_DDA_STEP_COLW(T, OUT) MV_DDA_HEAD(T, OUT)  \
+#define MV_DDA_MOVE                                  \
     " @px add.s32 pos, pos, sx;\n"                   \
     " @pz add.s32 pos, pos, sz;\n"                   \
-    " @py shf.l.wrap.b32 bit, bit, bit, sy;\n"       \
-    " ld.shared.u32 w, [pos];\n"                     \
+    " @py shf.l.wrap.b32 bit, bit, bit, sy;\n"
+#define MV_DDA_LOAD_SHARED " ld.shared.u32 w, [pos];\n"
+#define MV_DDA_LOAD_GLOBAL " mad.wide.u32 ag, pos, 1, gbase;\n ld.global.u32 w, [ag];\n"
+#define MV_DDA_STEP_COLW(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_MOVE MV_DDA_LOAD_SHARED \
     " lop3.or.b32 w|ph, w, bit, 0, 0xC0, pf;\n"
+// (`guard` is the plane's end here)
+#define MV_DDA_TEST " lop3.or.b32 a|ph, w, bit, guard, 0xC8, pf;\n"
+#define MV_DDA_STEP_PLANE_SHARED(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_MOVE MV_DDA_LOAD_SHARED MV_DDA_TEST
+#define MV_DDA_STEP_PLANE_GLOBAL(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_MOVE MV_DDA_LOAD_GLOBAL MV_DDA_TEST
 // The common case's step: nothing but a filled cell stops it.  What lies outside the occupied box counts as filled here
 // (the fence in x and z, `guard` = the heights outside it); afterwards w, the last column read, tells which it was.
 // The fence keeps the walk in bounds, and with a guard bit in every column it ends by itself: it only ever moves on,
 // along x, y and z, and each of them ends at something filled.
-#define MV_DDA_STEP_SEALED(T, OUT)                   \
+#define MV_DDA_SEALED_HEAD(T, OUT)                   \
     " min.f32 " T ", tx, ty, tz;\n"                  \
     " @ph bra " OUT ";\n"                            \
     " setp.eq.f32 px, tx, " T ";\n"                  \
     " setp.eq.and.f32 py|pz, ty, " T ", !px;\n"      \
     " @px add.f32 tx, tx, dtx;\n"                    \
     " @py add.f32 ty, ty, dty;\n"                    \
-    " @pz add.f32 tz, tz, dtz;\n"                    \
-    " @px add.s32 pos, pos, sx;\n"                   \
-    " @pz add.s32 pos, pos, sz;\n"                   \
-    " @py shf.l.wrap.b32 bit, bit, bit, sy;\n"       \
-    " ld.shared.u32 w, [pos];\n"                     \
-    " lop3.or.b32 a|ph, w, bit, guard, 0xC8, pf;\n"
-#define MV_DDA_STEP_IDX_TAIL                         \
-    " shf.r.wrap.b32 w, w, 0, pos;\n"                \
-    " lop3.or.b32 w|ph, w, 1, 0, 0xC0, pf;\n"
-#define MV_DDA_STEP_IDX_ADV                          \
-    " @px add.s32 pos, pos, sx;\n"                   \
-    " @py add.s32 pos, pos, sy;\n"                   \
-    " @pz add.s32 pos, pos, sz;\n"
-#define MV_DDA_STEP_IDX(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_STEP_IDX_ADV \
-    " shr.u32 a, pos, 3;\n and.b32 a, a, 0xfffffffc;\n ld.shared.u32 w, [a];\n" MV_DDA_STEP_IDX_TAIL
-#define MV_DDA_STEP_IDX_GLOBAL(T, OUT) MV_DDA_HEAD(T, OUT) MV_DDA_STEP_IDX_ADV \
-    " shr.u32 a, pos, 5;\n mad.wide.u32 ag, a, 4, gbase;\n ld.global.u32 w, [ag];\n" MV_DDA_STEP_IDX_TAIL
+    " @pz add.f32 tz, tz, dtz;\n"
+#define MV_DDA_STEP_SEALED(T, OUT) MV_DDA_SEALED_HEAD(T, OUT) MV_DDA_MOVE MV_DDA_LOAD_SHARED MV_DDA_TEST
+#define MV_DDA_STEP_SEALED_GLOBAL(T, OUT) MV_DDA_SEALED_HEAD(T, OUT) MV_DDA_MOVE MV_DDA_LOAD_GLOBAL MV_DDA_TEST
 // Loop around eight steps.  On leaving: ph = a filled cell was entered, thit = when, and px/py
 // still say along which axis.
 #define MV_DDA_LOOP(STEP)                            \
@@ -134,14 +130,12 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " @ph mov.f32 thit, ta;\n"                       \
     "MV_DDA_OUT:\n"
 // Loop of the sealed walk.  On leaving: ph set, thit = when the filled cell was entered, px/py/pz say along which axis.
-#define MV_DDA_SEALED                                \
+#define MV_DDA_SEALED(STEP)                          \
     " setp.ne.u32 pf, 0, 0;\n"                       \
     " setp.ne.u32 ph, 0, 0;\n"                       \
     "MV_DDA_LOOP_TOP:\n"                             \
-    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
-    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
-    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
-    MV_DDA_STEP_SEALED("ta", "MV_DDA_OUT_A") MV_DDA_STEP_SEALED("tb", "MV_DDA_OUT_B")  \
+    STEP("ta", "MV_DDA_OUT_A") STEP("tb", "MV_DDA_OUT_B") STEP("ta", "MV_DDA_OUT_A") STEP("tb", "MV_DDA_OUT_B") \
+    STEP("ta", "MV_DDA_OUT_A") STEP("tb", "MV_DDA_OUT_B") STEP("ta", "MV_DDA_OUT_A") STEP("tb", "MV_DDA_OUT_B") \
     " bra MV_DDA_LOOP_TOP;\n"                        \
     "MV_DDA_OUT_A:\n"                                \
     " mov.f32 thit, tb;\n"                           \
@@ -149,10 +143,33 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     "MV_DDA_OUT_B:\n"                                \
     " mov.f32 thit, ta;\n"                           \
     "MV_DDA_OUT:\n"
+// Behind either loop: a walk that met the end of its plane goes on in the next one up or down.  END: the plane's end (0 where
+// there is one plane), PLANE: bytes from plane to plane, TAB: the shared-memory address of the planes' guards, all ones for
+// planes that nothing is filled in (and so for those that are not there).  BEYOND: what happens on meeting one of those;
+// GUARD: which of the plane's heights count as filled from now on.
+#define MV_DDA_CROSS(END, PLANE, TAB, BEYOND, GUARD, LOAD) \
+    " setp.ne.b32 pq, bit, " END ";\n"               \
+    " @pq bra MV_DDA_DONE;\n"                        \
+    " setp.eq.s32 pq, sy, 1;\n"                      \
+    " selp.s32 w, 1, -1, pq;\n"                      \
+    " add.s32 q, q, w;\n"                            \
+    " mad.lo.s32 a, q, 4, " TAB ";\n"                \
+    " ld.shared.u32 a, [a];\n"                       \
+    " mad.lo.s32 pos, w, " PLANE ", pos;\n"          \
+    " mov.b32 w, 0xffffffff;\n"                      \
+    " setp.eq.u32 ph, a, 0xffffffff;\n"              \
+    BEYOND                                           \
+    " @ph bra MV_DDA_DONE;\n"                        \
+    " selp.b32 bit, 1, 0x40000000, pq;\n"            \
+    GUARD                                            \
+    LOAD                                             \
+    MV_DDA_TEST                                      \
+    " @!ph bra MV_DDA_LOOP_TOP;\n"                   \
+    "MV_DDA_DONE:\n"
 #define MV_DDA_DECL                                  \
     " .reg .pred px, py, pz, pq, ph, pf;\n"          \
     " .reg .f32 tx, ty, tz, dtx, dty, dtz, ta, tb, texit, thit;\n" \
-    " .reg .b32 sx, sy, sz, pos, bit, guard, w, a, it;\n"   \
+    " .reg .b32 sx, sy, sz, pos, bit, guard, w, a, it, q;\n"   \
     " .reg .b64 ag, gbase;\n"
 
 // Threads resident per SM that the registers are laid out for: three CTAs of 384 with 56 registers (16384 observations
@@ -172,7 +189,7 @@ constexpr uint32_t kAgentSealed = 8u;      // the common case: eye inside, not i
 //   {colour-table row of the face entered by an x, z, y step; -}
 // then the record {Fx, Fy, Rx, Uy} {Ux, Uz, Fz, Rz} {start bit mask, heights outside the occupied box, flags, self box} {eye
 // x, y, z, overlay count} {64-bit address of the env's material store, biased for the walk's positions; sky colour; miss
-// depth} {lower corner of the occupied box, -} {upper corner, -}, eye-relative boxes, overlay rectangles and per-tile box masks at offsets the host lays out.
+// depth} {lower corner of the occupied box, plane of the eye} {upper corner, -}, eye-relative boxes, overlay rectangles and per-tile box masks at offsets the host lays out.
 constexpr uint32_t kAgentTabBytes = 512, kAgentAlign = 512;
 constexpr uint32_t kAgentRecVecs = 7;
 constexpr uint32_t kAgentRelOff = kAgentTabBytes + 16u * kAgentRecVecs;
@@ -184,6 +201,7 @@ constexpr uint32_t kAgentRelOff = kAgentTabBytes + 16u * kAgentRecVecs;
 #define MV_REC_U "528"
 #define MV_REC_START "544"
 #define MV_REC_MAT "576"
+#define MV_REC_PLANE "604"
 // a hit is looked at again if the ray leaves the cell within this factor of the time of the hit (1 - 2^-13)
 #define MV_GRAZE "0f3F7FF800"
 constexpr float kSealedScale = 1.0f - 1e-4f;       // least exit_scale for which that factor is wide enough
@@ -207,18 +225,18 @@ __device__ __forceinline__ void write_sky(uint8_t *rgb_obs, float *depth_obs, in
     for (int i = threadIdx.x; i < npx * 3; i += NT) rgb_obs[i] = (uint8_t)(sky_rgbx >> (8 * (i % 3)));
 }
 
-// OCC_SHARED: the occupancy bits are staged in shared memory with the rest of the env block (the
-// normal case); otherwise only the block's tail (colour table, boxes, bounds) is staged and the
-// occupancy is read from global memory.
-// COLW: column-word flavour of the walk (grid at most 32 high and occupancy staged).
-template <int NT, bool OCC_SHARED, bool COLW>
+// OCC: how the occupancy is walked.  kOccWord: staged in shared memory with the rest of the env block, one plane (the normal
+// case).  kOccPlanes: staged, several planes, of which those up to the highest filled voxel are copied.  kOccGlobal: read from
+// global memory, any number of planes; only the rest of the block is staged.
+constexpr int kOccWord = 0, kOccPlanes = 1, kOccGlobal = 2;
+template <int NT, int OCC>
 __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const RenderParams p)
 {
-    static_assert(OCC_SHARED || !COLW, "the column-word walk reads shared memory");
+    constexpr bool COLW = OCC == kOccWord;
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int apc = p.agents_per_cta;
     constexpr int kWarps = NT / 32;
+    const int apc = p.agents_per_cta;
     const int obs0 = p.obs_begin + blockIdx.x * apc;
     const int env = p.agents == 1 ? obs0 : obs0 / p.agents;
     const int W = p.W, H = p.H;
@@ -229,11 +247,9 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     const int ms = mw > 1 ? mw + 1 : 1;              // words per tile
     const int m0 = mw > 1 ? 1 : 0;                   // position of the first real mask word
 
-    // bytes of the env block that are NOT staged (the occupancy, when it stays in global memory)
-    const uint32_t unstaged = OCC_SHARED ? 0u : p.lay.occ_bytes;
     const unsigned char *env_block = p.env_blocks + (size_t)env * p.lay.stride;
-    const uint32_t *s_occ = OCC_SHARED ? reinterpret_cast<const uint32_t *>(smem)
-                                       : reinterpret_cast<const uint32_t *>(env_block);
+    // shared memory: room for the staged planes, then the rest of the block
+    const uint32_t stage_occ = OCC == kOccGlobal ? 0u : p.lay.occ_bytes, unstaged = p.lay.occ_bytes - stage_occ;
     const unsigned char *s_lut = smem + (p.lay.lut_off - unstaged);
     const float4 *s_box = reinterpret_cast<const float4 *>(smem + (p.lay.box_off - unstaged));
     const int *s_count = reinterpret_cast<const int *>(smem + (p.lay.count_off - unstaged));
@@ -241,6 +257,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     unsigned char *s_agents = smem + p.smem_agent_off;
     uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + p.smem_misc_off);
     uint32_t *s_flag = reinterpret_cast<uint32_t *>(smem + p.smem_misc_off + 8);
+    uint32_t *s_guard = reinterpret_cast<uint32_t *>(smem + p.smem_misc_off + 16);
     auto agent_tab = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride); };
     auto agent_rec = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentTabBytes); };
     auto agent_rel = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentRelOff); };
@@ -266,8 +283,19 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     wait_for_previous();
     // ---- stage the environment block
     if (tid == 0 && !p.skip_staging) {
-        mbar_expect_tx(s_bar, p.lay.block_bytes - unstaged);
-        bulk_load(smem, env_block + unstaged, p.lay.block_bytes - unstaged, s_bar);
+        if (COLW) {
+            mbar_expect_tx(s_bar, p.lay.block_bytes);
+            bulk_load(smem, env_block, p.lay.block_bytes, s_bar);
+        } else {
+            uint32_t bytes = 0;
+            if (OCC == kOccPlanes) {
+                const int *bounds = reinterpret_cast<const int *>(env_block + p.lay.count_off);
+                bytes = bounds[2] < bounds[5] ? (plane_of(p.lay, bounds[5] - 1) + 1u) * p.lay.occ_plane : 0u;
+            }
+            mbar_expect_tx(s_bar, bytes + p.lay.block_bytes - p.lay.occ_bytes);
+            if (bytes) bulk_load(smem, env_block, bytes, s_bar);
+            bulk_load(smem + stage_occ, env_block + p.lay.occ_bytes, p.lay.block_bytes - p.lay.occ_bytes, s_bar);
+        }
     }
     __syncthreads();
     // ---- meanwhile: camera records, GUI rectangles
@@ -322,27 +350,36 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     mbar_try_wait(s_bar, 0);              // completed phase: makes the staged bytes visible to this thread
 
     // ---- per-agent traversal set-up and box binning
-    const int gx = p.gx, gz = p.gz;
-    // voxel-index strides of the y-packed layout: x and z move by whole columns, y by single bits
-    const int pitch = (int)p.lay.pitch, stride_x = 1 << p.lay.ysh, stride_z = pitch << p.lay.ysh;
+    const int pitch = (int)p.lay.pitch;
     // Traversal is confined to the cell box [lo, hi) that holds every filled voxel of this env
     // (nothing outside it can be hit), so rays that leave it, e.g. into the sky, stop there.
     const int lox = s_count[1], loy = s_count[2], loz = s_count[3];
     const int hix = s_count[4], hiy = s_count[5], hiz = s_count[6];
     const bool any_voxel = (lox < hix) && (loy < hiy) && (loz < hiz);
-    const uint32_t occ_base = OCC_SHARED ? smem_addr(smem) : 0u;
-    const uint32_t vi_bias = 8u * occ_base;
+    const uint32_t used_planes = COLW ? 1u : any_voxel ? plane_of(p.lay, hiy - 1) + 1u : 0u;
+    constexpr bool staged = OCC != kOccGlobal;
+    const uint32_t occ_base = staged ? smem_addr(smem) : 0u;
+    const unsigned char *occ = staged ? smem : env_block;
+    const uint32_t plane_end = COLW || p.lay.planes == 1 ? 0u : kPlaneEnd;
     const int P_ = p.palette;
     const uint32_t lut_base = smem_addr(s_lut);
     const uint32_t inside_row = lut_base + (uint32_t)(kFaceInside * P_ * 4);
-    // position of cell (cx, cy, cz) in the walk's own terms (see MV_DDA_*)
+    // position of cell (cx, cy, cz) in the walk's own terms (see MV_DDA_*): its word, and the plane's heights that lie outside
+    // the occupied box
+    auto cell_plane = [&](int cy) -> uint32_t { return COLW ? 0u : plane_of(p.lay, cy); };
     auto cell_pos = [&](int cx, int cy, int cz) -> uint32_t {
-        return COLW ? occ_base + 4u * column_index(p.lay, cx, cz) : vi_bias + voxel_index(p.lay, cx, cy, cz);
+        return occ_base + cell_plane(cy) * p.lay.occ_plane + 4u * column_index(p.lay, cx, cz);
     };
-    auto cell_filled = [&](int cx, int cy, int cz) -> bool {
-        const uint32_t u = voxel_index(p.lay, cx, cy, cz);
-        return (s_occ[u >> 5] >> (u & 31)) & 1u;
+    auto plane_guard = [&](uint32_t q) -> uint32_t {
+        const int lo = loy - plane_begin(q), hi = hiy - plane_begin(q);
+        return ~(hi >= 32 ? 0xffffffffu : (1u << max(hi, 0)) - 1u) | ((1u << min(max(lo, 0), 31)) - 1u) | plane_end;
     };
+    if (!COLW)                            // the planes' guards, with one for the plane below the first and the one above the last
+        for (int i = tid; i < (int)p.lay.planes + 2; i += NT) {
+            const int q = i - 1;
+            const bool in = any_voxel && q >= 0 && q < (int)used_planes && hiy > plane_begin(q) && loy < plane_begin(q + 1);
+            s_guard[i] = in ? plane_guard(q) : 0xffffffffu;
+        }
     // Where the eye is, in the terms of the walk's tables.
     auto eye_cell = [&](const float4 &c0, int &cx, int &cy, int &cz) -> bool {
         const bool in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
@@ -361,23 +398,23 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
         const int dx = (signs & 1) ? -1 : 1, dy = (signs & 2) ? -1 : 1, dz = (signs & 4) ? -1 : 1;
         const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
         const float qy = dy < 0 ? c0.y - (float)cy : (float)(cy + 1) - c0.y;
-        const int sx = COLW ? 4 * dx : dx * stride_x, sz = COLW ? 4 * pitch * dz : dz * stride_z, sy = COLW ? (dy < 0 ? 31 : 1) : dy;
+        const int sx = 4 * dx, sz = 4 * pitch * dz, sy = dy < 0 ? 31 : 1;
         entry[0] = make_float4(qx, qz, __int_as_float(sx), __int_as_float(sz));
         entry[2] = make_float4((1.0f - qx) * kSkipMargin, (1.0f - qz) * kSkipMargin, qy, __int_as_float(sy));
         entry[3] = make_float4(__uint_as_float(lut_base + (uint32_t)((dx < 0 ? 1 : 0) * P_ * 4)),
                                __uint_as_float(lut_base + (uint32_t)((4 + (dz < 0 ? 1 : 0)) * P_ * 4)),
                                __uint_as_float(lut_base + (uint32_t)((2 + (dy < 0 ? 1 : 0)) * P_ * 4)), 0.0f);
         if (signs == 0) {
-            const bool filled = cam_in && cell_filled(cx, cy, cz);
-            const uint32_t guard = ~(hiy >= 32 ? 0xffffffffu : (1u << hiy) - 1u) | ((1u << min(loy, 31)) - 1u);
-            rec[2].x = __uint_as_float(1u << (cy & 31));
+            const bool filled = cam_in && voxel_filled(p.lay, occ, cx, cy, cz);
+            const uint32_t q = cell_plane(cy), guard = plane_guard(q);
+            rec[2].x = __uint_as_float(1u << ((cy - plane_begin(q)) & 31));
             rec[2].y = __uint_as_float(guard);                   // heights outside the occupied box
             rec[2].z = __uint_as_float(__float_as_uint(rec[2].z) | (cam_in ? kAgentInside : 0u) | (filled ? kAgentFilled : 0u) |
                                        (cam_in && !filled && guard && p.exit_scale > kSealedScale ? kAgentSealed : 0u));
-            const unsigned long long mp = reinterpret_cast<unsigned long long>(p.mat + (size_t)env * p.mat_stride - vi_bias);
+            const unsigned long long mp = reinterpret_cast<unsigned long long>(p.mat + (size_t)env * p.mat_stride - ((size_t)occ_base << (p.lay.ysh - 2)));
             rec[4] = make_float4(__uint_as_float((uint32_t)mp), __uint_as_float((uint32_t)(mp >> 32)),
                                  __uint_as_float(p.sky_rgbx), p.miss_depth);
-            rec[5] = make_float4((float)lox, (float)loy, (float)loz, 0.0f);
+            rec[5] = make_float4((float)lox, (float)loy, (float)loz, __uint_as_float(q));
             rec[6] = make_float4((float)hix, (float)hiy, (float)hiz, 0.0f);
         }
     }
@@ -400,13 +437,14 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
         const int on_x = dx < 0 && c0.x == (float)cx ? 1 : 0, on_z = dz < 0 && c0.z == (float)cz ? 1 : 0;
         const int bx = cx + dx * on_x, bz = cz + dz * on_z;
         const int lim_x = min(kSkipCells - 1, dx < 0 ? bx - lox : hix - 1 - bx), lim_z = dz < 0 ? bz - loz : hiz - 1 - bz;
-        const int wsh = p.lay.ysh - 5, yb = cy & 31;
-        const uint32_t *word = s_occ + (((int)column_index(p.lay, bx, bz + dz * j) << wsh) + (cy >> 5));
+        const uint32_t q = cell_plane(cy);
+        const int yb = (cy - plane_begin(q)) & 31;
+        const uint32_t *word = reinterpret_cast<const uint32_t *>(occ + (size_t)q * p.lay.occ_plane) + (int)column_index(p.lay, bx, bz + dz * j);
         const bool row_in = cam_in && j <= lim_z;
-        uint32_t col[kSkipCells], filled = ~0u << kSkipCells, seen = 0;
+        uint32_t col[kSkipCells], filled = ~0u << kSkipCells, seen = plane_end;
 #pragma unroll
         for (int i = 0; i < kSkipCells; ++i) {
-            col[i] = row_in && i <= lim_x ? word[(dx * i) * (1 << wsh)] : ~0u;
+            col[i] = row_in && i <= lim_x ? word[dx * i] : ~0u;
             filled |= ((col[i] >> yb) & 1u) << i;
         }
         int w = __ffs(filled) - 1;                               // empty cells at the row's beginning
@@ -433,7 +471,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                                            : (yb > 0 ? __brev(seen << (32 - yb)) | 1u << yb : 1u);
             const int ey = any ? min(min(kSkipCellsY, __ffs(beyond) - 1), dy < 0 ? cy - loy : hiy - 1 - cy) : 0;
             const int ex = any ? rx + on_x : 0, ez = any ? rz + on_z : 0;
-            const int sx = COLW ? 4 * dx : dx * stride_x, sz = COLW ? 4 * pitch * dz : dz * stride_z;
+            const int sx = 4 * dx, sz = 4 * pitch * dz;
             const int signs = (dx < 0 ? 1 : 0) | (dy < 0 ? 2 : 0) | (dz < 0 ? 4 : 0);
             const float qx = dx < 0 ? c0.x - (float)cx : (float)(cx + 1) - c0.x, qz = dz < 0 ? c0.z - (float)cz : (float)(cz + 1) - c0.z;
             const float qy = dy < 0 ? c0.y - (float)cy : (float)(cy + 1) - c0.y;
@@ -507,6 +545,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     }
     __syncthreads();
 
+    uint32_t guards = smem_addr(s_guard + 1);                               // guard of plane 0
     const float flox = (float)lox, floy = (float)loy, floz = (float)loz;
     const float fhix = (float)hix, fhiy = (float)hiy, fhiz = (float)hiz;
 
@@ -552,23 +591,20 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
         // that the choice between the common case and the rest is taken per agent, not per tile; what
         // follows the walk is the same for both.  The warp-wide reduction and shuffle in it name all 32
         // lanes, so they wait by themselves for lanes whose walk ran longer.
-        auto finish_tile = [&](uint32_t mask_p, int tile_px, uint32_t pos, uint32_t bit, uint32_t row,
+        auto finish_tile = [&](uint32_t mask_p, int tile_px, uint32_t pos, uint32_t bit, uint32_t plane, uint32_t row,
                                uint32_t tab, uint32_t graze, float t_hit, float dtx, float dty, float dtz) {
             // ---- the hit voxel's material byte is asked for from global memory (its colour is looked up
             // in the shaded table only in the store block, after everything that does not need it), this
             // tile's first box-mask word is read, and the latest voxel hit of the warp is found (boxes wholly
             // behind it are skipped).  Predicated, not branched; sky colour and miss depth ride with the
-            // material store's address in the agent block.  (Column-word flavour: the voxel index is rebuilt from
-            // the column's address and the bit.)
+            // material store's address in the agent block.  (The voxel index is rebuilt from the column's
+            // address, the bit and the plane.)
             uint32_t rgbx, m, mat_id;
             float depth;
             {
-                uint32_t vi = pos;
-                if (COLW) {
-                    uint32_t y;
-                    asm("bfind.u32 %0, %1;" : "=r"(y) : "r"(bit));
-                    vi = (pos << 3) + y;
-                }
+                uint32_t y, vi;
+                asm("bfind.u32 %0, %1;" : "=r"(y) : "r"(bit));
+                vi = COLW ? (pos << 3) + y : (pos << (p.lay.ysh - 2)) + y + plane * (kPlaneHeights - (p.lay.occ_plane << (p.lay.ysh - 2)));
                 asm volatile("{\n"
                     " .reg .pred pv;\n"
                     " .reg .b32 skyb, missb;\n"
@@ -688,10 +724,10 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 :: "r"(rgbx), "f"(depth), "r"(tile_px), "l"(depth_lane), "l"(rgb_lane), "r"(st_sel), "r"(row), "r"(mat_id)
                 : "memory");
         };
-        if (COLW && (aflags & kAgentSealed)) {
+        if (aflags & kAgentSealed) {
             for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
                 int tile_px;
-                uint32_t pos, bit = 0, row, tab, graze;
+                uint32_t pos, bit = 0, plane = 0, row, tab, graze;
                 float t_hit, dtx, dty, dtz;
                 // ---- the common case in one block of PTX: tile record, ray through the pixel centre
                 // (d = F + a*Rs + b*Us, a = 2px+1-W, b = H-1-2py, two chained FMAs per component),
@@ -707,100 +743,120 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 // is +-inf, so its crossing time is +inf (or NaN when the eye sits exactly on the face,
                 // which min and the compares ignore) and that axis is never stepped, which is the rule
                 // for such rays.
-                asm volatile("{\n"
-                    MV_DDA_DECL
-                    " .reg .f32 Ta, Tb, Fx, Fy, Fz, Rx, Rz, Ux, Uy, Uz, ca, cb, dx, dy, dz, ix, iy, iz;\n"
-                    " .reg .f32 q0, q1, q2, q3, q4;\n"
-                    " .reg .b32 u, v;\n"
-                    " .reg .b64 T2, D2, Q2, C2, M2;\n"
-                    " ld.shared.v4.b32 {Ta, Tb, %0, _}, [%10];\n"
-                    " ld.shared.v4.f32 {Fx, Fy, Rx, Uy}, [%11+" MV_REC_F "];\n"
-                    " ld.shared.v4.f32 {Ux, Uz, Fz, Rz}, [%11+" MV_REC_U "];\n"
-                    " ld.shared.v2.b32 {bit, guard}, [%11+" MV_REC_START "];\n"
-                    " mov.b64 C2, {Ta, Tb};\n"
-                    " add.rn.f32x2 C2, C2, %12;\n"
-                    " mov.b64 {ca, cb}, C2;\n"
-                    " mov.b64 T2, {Fx, Fy};\n"
-                    " mov.b64 D2, {Rx, Uy};\n"
-                    " fma.rn.f32x2 T2, C2, D2, T2;\n"
-                    " mov.b64 {dx, dy}, T2;\n"
-                    " fma.rn.f32 dz, ca, Rz, Fz;\n"
-                    " fma.rn.f32 dx, cb, Ux, dx;\n"
-                    " fma.rn.f32 dz, cb, Uz, dz;\n"
-                    " abs.f32 ix, dx;\n"
-                    " abs.f32 iy, dy;\n"
-                    " abs.f32 iz, dz;\n"
-                    " rcp.approx.ftz.f32 dtx, ix;\n"
-                    " rcp.approx.ftz.f32 dty, iy;\n"
-                    " rcp.approx.ftz.f32 dtz, iz;\n"
-                    " mov.b32 u, dx;\n"
-                    " mov.b32 v, dz;\n"
-                    " prmt.b32 u, u, v, 0x00FB;\n"                  // byte 0: sign of dx, byte 1: sign of dz
-                    " lop3.b32 %8, u, 0x140, %11, 0xEA;\n"
-                    " mov.b32 u, dy;\n"
-                    " shr.u32 u, u, 24;\n"
-                    " lop3.b32 %8, u, 0x80, %8, 0xEA;\n"
-                    " ld.shared.v4.b32 {tx, tz, sx, sz}, [%8];\n"
-                    " ld.shared.v4.b32 {q0, q1, q2, pos}, [%8+" MV_TAB_SKIP "];\n"
-                    " ld.shared.v4.b32 {q3, q4, ty, sy}, [%8+" MV_TAB_SKIP2 "];\n"
-                    " mul.f32 tx, tx, dtx;\n"
-                    " mul.f32 ty, ty, dty;\n"
-                    " mul.f32 tz, tz, dtz;\n"
-                    " mov.b64 Q2, {q0, q1};\n"
-                    " mov.b64 D2, {dtx, dtz};\n"
-                    " mul.rn.f32x2 Q2, Q2, D2;\n"
-                    " mov.b64 {q0, q1}, Q2;\n"
-                    " mul.f32 q2, q2, dty;\n"
-                    " min.f32 q0, q0, q1, q2;\n"
-                    " fma.rn.f32 q3, q0, ix, q3;\n"
-                    " fma.rn.f32 q4, q0, iz, q4;\n"
-                    " mov.b64 Q2, {q3, q4};\n"
-                    " mov.b64 M2, " MV_SKIP_MAGIC2 ";\n"
-                    " add.rm.f32x2 Q2, Q2, M2;\n"
-                    " mov.b64 {q3, q4}, Q2;\n"
-                    " mov.b32 u, q3;\n"
-                    " mad.lo.u32 pos, u, sx, pos;\n"
-                    " mov.b32 u, q4;\n"
-                    " mad.lo.u32 pos, u, sz, pos;\n"
-                    // (the first crossing by an addition as in the walk and only the rest by a product, so that up to two crossings
-                    // give the bits that the walk would give and ties between axes go the same way)
-                    " setp.gt.f32 px, q3, " MV_SKIP_MAGIC ";\n"
-                    " setp.gt.f32 pz, q4, " MV_SKIP_MAGIC ";\n"
-                    " mov.b64 Q2, {q3, q4};\n"
-                    " mov.b64 M2, " MV_SKIP_UNMAGIC2 ";\n"
-                    " add.rn.f32x2 Q2, Q2, M2;\n"
-                    " mov.b64 {q3, q4}, Q2;\n"
-                    " @px add.f32 tx, tx, dtx;\n"
-                    " @pz add.f32 tz, tz, dtz;\n"
-                    " @px fma.rn.f32 tx, q3, dtx, tx;\n"
+#define MV_SEALED_RAY \
+                    MV_DDA_DECL \
+                    " .reg .f32 Ta, Tb, Fx, Fy, Fz, Rx, Rz, Ux, Uy, Uz, ca, cb, dx, dy, dz, ix, iy, iz;\n" \
+                    " .reg .f32 q0, q1, q2, q3, q4;\n" \
+                    " .reg .b32 u, v;\n" \
+                    " .reg .b64 T2, D2, Q2, C2, M2;\n" \
+                    " ld.shared.v4.b32 {Ta, Tb, %0, _}, [%10];\n" \
+                    " ld.shared.v4.f32 {Fx, Fy, Rx, Uy}, [%11+" MV_REC_F "];\n" \
+                    " ld.shared.v4.f32 {Ux, Uz, Fz, Rz}, [%11+" MV_REC_U "];\n" \
+                    " ld.shared.v2.b32 {bit, guard}, [%11+" MV_REC_START "];\n" \
+                    " mov.b64 C2, {Ta, Tb};\n" \
+                    " add.rn.f32x2 C2, C2, %12;\n" \
+                    " mov.b64 {ca, cb}, C2;\n" \
+                    " mov.b64 T2, {Fx, Fy};\n" \
+                    " mov.b64 D2, {Rx, Uy};\n" \
+                    " fma.rn.f32x2 T2, C2, D2, T2;\n" \
+                    " mov.b64 {dx, dy}, T2;\n" \
+                    " fma.rn.f32 dz, ca, Rz, Fz;\n" \
+                    " fma.rn.f32 dx, cb, Ux, dx;\n" \
+                    " fma.rn.f32 dz, cb, Uz, dz;\n" \
+                    " abs.f32 ix, dx;\n" \
+                    " abs.f32 iy, dy;\n" \
+                    " abs.f32 iz, dz;\n" \
+                    " rcp.approx.ftz.f32 dtx, ix;\n" \
+                    " rcp.approx.ftz.f32 dty, iy;\n" \
+                    " rcp.approx.ftz.f32 dtz, iz;\n" \
+                    " mov.b32 u, dx;\n" \
+                    " mov.b32 v, dz;\n" \
+                    " prmt.b32 u, u, v, 0x00FB;\n"    /* byte 0: sign of dx, byte 1: sign of dz */ \
+                    " lop3.b32 %8, u, 0x140, %11, 0xEA;\n" \
+                    " mov.b32 u, dy;\n" \
+                    " shr.u32 u, u, 24;\n" \
+                    " lop3.b32 %8, u, 0x80, %8, 0xEA;\n" \
+                    " ld.shared.v4.b32 {tx, tz, sx, sz}, [%8];\n" \
+                    " ld.shared.v4.b32 {q0, q1, q2, pos}, [%8+" MV_TAB_SKIP "];\n" \
+                    " ld.shared.v4.b32 {q3, q4, ty, sy}, [%8+" MV_TAB_SKIP2 "];\n" \
+                    " mul.f32 tx, tx, dtx;\n" \
+                    " mul.f32 ty, ty, dty;\n" \
+                    " mul.f32 tz, tz, dtz;\n" \
+                    " mov.b64 Q2, {q0, q1};\n" \
+                    " mov.b64 D2, {dtx, dtz};\n" \
+                    " mul.rn.f32x2 Q2, Q2, D2;\n" \
+                    " mov.b64 {q0, q1}, Q2;\n" \
+                    " mul.f32 q2, q2, dty;\n" \
+                    " min.f32 q0, q0, q1, q2;\n" \
+                    " fma.rn.f32 q3, q0, ix, q3;\n" \
+                    " fma.rn.f32 q4, q0, iz, q4;\n" \
+                    " mov.b64 Q2, {q3, q4};\n" \
+                    " mov.b64 M2, " MV_SKIP_MAGIC2 ";\n" \
+                    " add.rm.f32x2 Q2, Q2, M2;\n" \
+                    " mov.b64 {q3, q4}, Q2;\n" \
+                    " mov.b32 u, q3;\n" \
+                    " mad.lo.u32 pos, u, sx, pos;\n" \
+                    " mov.b32 u, q4;\n" \
+                    " mad.lo.u32 pos, u, sz, pos;\n" \
+                    /* (the first crossing by an addition as in the walk and only the rest by a product, so that up to two crossings */ \
+                    /* give the bits that the walk would give and ties between axes go the same way) */ \
+                    " setp.gt.f32 px, q3, " MV_SKIP_MAGIC ";\n" \
+                    " setp.gt.f32 pz, q4, " MV_SKIP_MAGIC ";\n" \
+                    " mov.b64 Q2, {q3, q4};\n" \
+                    " mov.b64 M2, " MV_SKIP_UNMAGIC2 ";\n" \
+                    " add.rn.f32x2 Q2, Q2, M2;\n" \
+                    " mov.b64 {q3, q4}, Q2;\n" \
+                    " @px add.f32 tx, tx, dtx;\n" \
+                    " @pz add.f32 tz, tz, dtz;\n" \
+                    " @px fma.rn.f32 tx, q3, dtx, tx;\n" \
                     " @pz fma.rn.f32 tz, q4, dtz, tz;\n"
-                    MV_DDA_SEALED
-                    // a miss if the cell is fence (its guard bits are set) or lies at a height outside the box
-                    " or.b32 w, w, bit;\n"
-                    " and.b32 w, w, guard;\n"
-                    " setp.eq.u32 ph, w, 0;\n"
-                    // (a hit that may be too close to the ray's exit from the box: see below)
-                    " min.f32 ta, tx, ty, tz;\n"
-                    " mul.f32 ta, ta, " MV_GRAZE ";\n"
-                    " setp.ge.and.f32 pq, thit, ta, ph;\n"
-                    " selp.u32 %9, 1, 0, pq;\n"
-                    " mov.b32 %4, 0xffffffff;\n"
-                    " @!ph mov.f32 thit, 0f7F800000;\n"
-                    " mov.b32 u, %8;\n"
-                    " @py add.u32 u, u, 8;\n"
-                    " @pz add.u32 u, u, 4;\n"
-                    " @ph ld.shared.u32 %4, [u+" MV_TAB_ROW "];\n"
-                    " mov.b32 %1, pos;\n"
-                    " mov.b32 %2, bit;\n"
-                    " mov.f32 %3, thit;\n"
-                    " mov.f32 %5, dtx;\n"
-                    " mov.f32 %6, dty;\n"
+#define MV_SEALED_END \
+                    /* a miss if the cell is fence (its guard bits are set) or lies at a height outside the box */ \
+                    " or.b32 w, w, bit;\n" \
+                    " and.b32 w, w, guard;\n" \
+                    " setp.eq.u32 ph, w, 0;\n" \
+                    /* (a hit that may be too close to the ray's exit from the box: see below) */ \
+                    " min.f32 ta, tx, ty, tz;\n" \
+                    " mul.f32 ta, ta, " MV_GRAZE ";\n" \
+                    " setp.ge.and.f32 pq, thit, ta, ph;\n" \
+                    " selp.u32 %9, 1, 0, pq;\n" \
+                    " mov.b32 %4, 0xffffffff;\n" \
+                    " @!ph mov.f32 thit, 0f7F800000;\n" \
+                    " mov.b32 u, %8;\n" \
+                    " @py add.u32 u, u, 8;\n" \
+                    " @pz add.u32 u, u, 4;\n" \
+                    " @ph ld.shared.u32 %4, [u+" MV_TAB_ROW "];\n" \
+                    " mov.b32 %1, pos;\n" \
+                    " mov.b32 %2, bit;\n" \
+                    " mov.f32 %3, thit;\n" \
+                    " mov.f32 %5, dtx;\n" \
+                    " mov.f32 %6, dty;\n" \
                     " mov.f32 %7, dtz;\n"
-                    "}\n"
-                    : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze)
-                    : "r"(tile_p), "r"(abase), "l"(lane_ab)
-                    : "memory");
-                finish_tile(mask_p, tile_px, pos, bit, row, tab, graze, t_hit, dtx, dty, dtz);
+                if constexpr (COLW) {
+                    asm volatile("{\n" MV_SEALED_RAY MV_DDA_SEALED(MV_DDA_STEP_SEALED) MV_SEALED_END "}\n"
+                        : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze)
+                        : "r"(tile_p), "r"(abase), "l"(lane_ab)
+                        : "memory");
+                } else {
+#define MV_SEALED_PLANE " ld.shared.u32 q, [%11+" MV_REC_PLANE "];\n"
+#define MV_SEALED_CROSS(LOAD) MV_DDA_CROSS("%14", "%15", "%16", "", " mov.b32 guard, a;\n", LOAD) " mov.b32 %13, q;\n"
+#define MV_SEALED_IO                                                                                                \
+                        : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze), \
+                          "+r"(tile_in), "+r"(abase), "+l"(lane_ab), "=&r"(plane)                                               \
+                        : "r"(plane_end), "r"(p.lay.occ_plane), "r"(guards), "l"(env_block)                                  \
+                        : "memory"
+                    uint32_t tile_in = tile_p;
+                    if constexpr (staged)
+                        asm volatile("{\n" MV_SEALED_RAY MV_SEALED_PLANE MV_DDA_SEALED(MV_DDA_STEP_SEALED) MV_SEALED_CROSS(MV_DDA_LOAD_SHARED) MV_SEALED_END "}\n" MV_SEALED_IO);
+                    else
+                        asm volatile("{\n" MV_SEALED_RAY MV_SEALED_PLANE " mov.b64 gbase, %17;\n" MV_DDA_SEALED(MV_DDA_STEP_SEALED_GLOBAL) MV_SEALED_CROSS(MV_DDA_LOAD_GLOBAL) MV_SEALED_END "}\n" MV_SEALED_IO);
+#undef MV_SEALED_PLANE
+#undef MV_SEALED_CROSS
+#undef MV_SEALED_IO
+                }
+#undef MV_SEALED_RAY
+#undef MV_SEALED_END
+                finish_tile(mask_p, tile_px, pos, bit, plane, row, tab, graze, t_hit, dtx, dty, dtz);
             }
         } else {
             const float4 P4 = agent_rec(ag)[3];
@@ -808,7 +864,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
             const bool cam_in = (aflags & kAgentInside) != 0;
             for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
                 int tile_px;
-                uint32_t pos, bit = 0, row, tab;
+                uint32_t pos, bit = 0, plane = 0, row, tab;
                 float t_hit, dtx, dty, dtz;
                 // ---- every other case: the same steps in C++, with the eye possibly outside the
                 // occupied box and either flavour of the walk
@@ -836,6 +892,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 float t0x, t0y, t0z, t_exit;
                 t_hit = 0.0f;
                 pos = 0; bit = bit0; row = kNoRow;
+                if (!COLW) plane = __float_as_uint(agent_rec(ag)[5].w);
                 if (cam_in) {
                     // (crossing times are sums: the exit time is pulled in by the rounding that can pile up in them)
                     t0x = qx * dtx;
@@ -870,14 +927,15 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     if (eaxis == 2) cz = ngz ? hiz - 1 : loz;
                     if (!alive) { cx = cy = cz = 0; }
                     pos = cell_pos(cx, cy, cz);
-                    bit = 1u << cy;
+                    plane = cell_plane(cy);
+                    bit = 1u << (cy - plane_begin(plane));
                     t0x = ((float)(cx + (ngx ? 0 : 1)) - Px) * ix;
                     t0y = ((float)(cy + (ngy ? 0 : 1)) - Py) * iy;
                     t0z = ((float)(cz + (ngz ? 0 : 1)) - Pz) * iz;
                     t_exit = min3f(fmaf(ngx ? (float)(cx - lox) : (float)(hix - 1 - cx), dtx, t0x),
                                    fmaf(ngy ? (float)(cy - loy) : (float)(hiy - 1 - cy), dty, t0y),
                                    fmaf(ngz ? (float)(cz - loz) : (float)(hiz - 1 - cz), dtz, t0z)) * p.exit_scale;
-                    const bool filled = alive && cell_filled(cx, cy, cz);
+                    const bool filled = alive && voxel_filled(p.lay, occ, cx, cy, cz);
                     // entered through the box face of axis eaxis, or the eye is inside a solid
                     if (filled) {
                         if (eaxis < 0) row = inside_row;
@@ -886,30 +944,39 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     if (!alive || filled) t_exit = -kInf;
                 }
 #define MV_DDA_IO                                                                                         \
-                    : "+r"(pos), "+r"(bit), "+f"(t_hit), "+r"(row)                                                  \
+                    : "+r"(pos), "+r"(bit), "+f"(t_hit), "+r"(row), "+r"(plane)                                     \
                     : "f"(t0x), "f"(t0y), "f"(t0z), "f"(dtx), "f"(dty), "f"(dtz), "r"(sx), "r"(sy), "r"(sz), "f"(t_exit), \
-                      "r"(0), "r"(tab), "l"(s_occ)                                                       \
+                      "r"(tab), "r"(plane_end), "r"(p.lay.occ_plane), "r"(guards), "l"(env_block)                     \
                     : "memory"
 #define MV_DDA_IN                                                                                         \
-                    " mov.b32 pos, %0;\n mov.b32 bit, %1;\n mov.f32 thit, %2;\n"                                    \
-                    " mov.f32 tx, %4;\n mov.f32 ty, %5;\n mov.f32 tz, %6;\n mov.f32 dtx, %7;\n mov.f32 dty, %8;\n"   \
-                    " mov.f32 dtz, %9;\n mov.b32 sx, %10;\n mov.b32 sy, %11;\n mov.b32 sz, %12;\n mov.f32 texit, %13;\n" \
-                    " mov.s32 it, " MV_STEP_BUDGET ";\n mov.b64 gbase, %16;\n"
+                    " mov.b32 pos, %0;\n mov.b32 bit, %1;\n mov.f32 thit, %2;\n mov.b32 q, %4;\n"                  \
+                    " mov.f32 tx, %5;\n mov.f32 ty, %6;\n mov.f32 tz, %7;\n mov.f32 dtx, %8;\n mov.f32 dty, %9;\n"   \
+                    " mov.f32 dtz, %10;\n mov.b32 sx, %11;\n mov.b32 sy, %12;\n mov.b32 sz, %13;\n mov.f32 texit, %14;\n" \
+                    " mov.b32 guard, %16;\n mov.s32 it, " MV_STEP_BUDGET ";\n mov.b64 gbase, %19;\n"
+// (a walk that ran out or left the box may stand at a plane's end all the same: only one that entered it goes on)
+#define MV_DDA_CROSS_GENERAL(LOAD)                                                                        \
+                    " @!ph bra MV_DDA_DONE;\n"                                                                   \
+                    MV_DDA_CROSS("%16", "%17", "%18", " @ph bra MV_DDA_BEYOND;\n", "", LOAD)                     \
+                    " bra MV_DDA_END;\n"                                                                         \
+                    "MV_DDA_BEYOND:\n"                                                                           \
+                    " setp.ne.u32 ph, 0, 0;\n"                                                                   \
+                    "MV_DDA_END:\n"
 #define MV_DDA_OUTS                                                                                       \
                     " selp.u32 a, 8, 4, py;\n selp.u32 a, 0, a, px;\n add.u32 a, a, %15;\n"                        \
-                    " @ph ld.shared.u32 %3, [a+" MV_TAB_ROW "];\n mov.b32 %0, pos;\n mov.b32 %1, bit;\n mov.f32 %2, thit;\n"
+                    " @ph ld.shared.u32 %3, [a+" MV_TAB_ROW "];\n mov.b32 %0, pos;\n mov.b32 %1, bit;\n mov.f32 %2, thit;\n mov.b32 %4, q;\n"
                 if constexpr (COLW) {
                     asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_COLW) MV_DDA_OUTS "}\n" MV_DDA_IO);
-                } else if constexpr (OCC_SHARED) {
-                    asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_IDX) MV_DDA_OUTS "}\n" MV_DDA_IO);
+                } else if constexpr (staged) {
+                    asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_PLANE_SHARED) MV_DDA_CROSS_GENERAL(MV_DDA_LOAD_SHARED) MV_DDA_OUTS "}\n" MV_DDA_IO);
                 } else {
-                    asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_IDX_GLOBAL) MV_DDA_OUTS "}\n" MV_DDA_IO);
+                    asm volatile("{\n" MV_DDA_DECL MV_DDA_IN MV_DDA_LOOP(MV_DDA_STEP_PLANE_GLOBAL) MV_DDA_CROSS_GENERAL(MV_DDA_LOAD_GLOBAL) MV_DDA_OUTS "}\n" MV_DDA_IO);
                 }
 #undef MV_DDA_IO
 #undef MV_DDA_IN
+#undef MV_DDA_CROSS_GENERAL
 #undef MV_DDA_OUTS
                 if (row == kNoRow) t_hit = kInf;          // no voxel hit
-                finish_tile(mask_p, tile_px, pos, bit, row, tab, 0u, t_hit, dtx, dty, dtz);
+                finish_tile(mask_p, tile_px, pos, bit, plane, row, tab, 0u, t_hit, dtx, dty, dtz);
             }
         }
     }

@@ -1,0 +1,90 @@
+"""Grids of several occupancy planes (more than 32 high) and the CTA shapes of large blocks, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import parity
+from helpers import cam_row
+from test_gpu_parity import _binding, _pal, _render_custom
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("gy", [36, 60, 64, 96, 132])
+def test_walks_that_cross_planes(oracle, gy):
+    """A plane is 31 heights: worlds filled thinly, so that walks cross planes up and down, with solid slabs that end just
+    below, at and just above a plane's first and last height; eyes in every plane, also next to its ends, looking up and
+    down; one world filled only low down, one only high up, one eye above everything, one outside the grid."""
+    rng = np.random.default_rng(gy)
+    gx, gz, E = 20, 24, 14
+    g = np.where(rng.random((E, gy, gz, gx)) < 0.01, rng.integers(1, 6, (E, gy, gz, gx)), 0).astype(np.uint8)
+    g[:, 0] = 1
+    cams = []
+    for e in range(E):
+        edge = 31 * (1 + e % ((gy - 1) // 31))                    # first height of a plane
+        y = [edge - 1, edge, edge + 1, edge - 2, 1, gy - 3, edge - 8, min(edge + 8, gy - 2)][e % 8]
+        if e < 6:                                                 # a slab with a hole, its top or bottom at the plane's edge
+            lo = min(max(edge + (e % 3) - 1, 1), gy - 2)
+            g[e, lo:lo + 2, :, :gx // 2] = 2
+        if e == 8:
+            g[e, 6:] = 0
+            y = 3
+        if e == 9:
+            g[e, :gy - 8] = 0
+            y = gy - 6
+        if e == 10:
+            g[e, gy - 20:] = 0
+            y = gy - 10
+        y = min(max(y, 1), gy - 2)
+        at = np.array([rng.integers(3, gx - 3), y, rng.integers(3, gz - 3)])
+        g[e, max(at[1] - 1, 1):at[1] + 2, at[2] - 1:at[2] + 2, at[0] - 1:at[0] + 2] = 0
+        p = at + rng.uniform(0.1, 0.9, 3)
+        if e == 11:
+            p = np.array([-4.0, gy * 0.6, gz * 0.5])
+        cams.append(cam_row(*p, rng.uniform(0, 6.28), [0.9, -0.9, 1.3, -1.3, 0.2, -0.3][e % 6]))
+    frames = _render_custom(oracle, g, _pal(E, 6), np.stack(cams), 64, 36)
+    assert frames[2] == 0
+    parity.assert_parity(frames[3], f"planes {gy}")
+    # the same bytes with the occupancy read from global memory
+    B = _binding()
+    batch = B.Batch(B.make_desc(E, 1, (gx, gy, gz), 0, 64, 36, 6))
+    batch.upload_worlds(0, E, torch.from_numpy(g).cuda(), palette=torch.from_numpy(_pal(E, 6)).cuda())
+    batch.set_cameras(torch.from_numpy(np.stack(cams)).cuda())
+    batch.debug_occupancy_in_global(True)
+    rgb, depth = batch.alloc_outputs()
+    batch.render_batch(rgb, depth)
+    assert (rgb.cpu().numpy() == frames[0]).all() and (depth.cpu().numpy() == frames[1]).all()
+    batch.destroy()
+
+
+@pytest.mark.parametrize("grid,agents", [((160, 12, 160), 1), ((192, 8, 192), 1), ((192, 8, 192), 3), ((100, 64, 120), 2)])
+def test_large_blocks_in_wide_ctas(oracle, grid, agents):
+    """Blocks that leave room for two CTAs on an SM, or for one: the oracle's frames, and the same ones staged and with the
+    occupancy in global memory."""
+    B = _binding()
+    gx, gy, gz = grid
+    rng = np.random.default_rng(gx + gy)
+    E, P, mb = 3, 9, 5
+    g = np.where(rng.random((E, gy, gz, gx)) < 0.03, rng.integers(1, P, (E, gy, gz, gx)), 0).astype(np.uint8)
+    g[:, 0] = 3
+    cams = np.stack([cam_row(*(np.array([gx, 0, gz]) * rng.uniform(0.3, 0.7, 3) + [0, rng.uniform(1.2, gy - 1.2), 0]), rng.uniform(0, 6.28),
+                             rng.uniform(-0.5, 0.5)) for _ in range(E * agents)])
+    boxes = np.zeros((E, mb, 8), np.float32)
+    lo = rng.uniform(0.2, 0.8, (E, mb, 3)) * [gx, gy, gz]
+    boxes[..., :3], boxes[..., 3:6] = lo, lo + rng.uniform(0.5, 3, (E, mb, 3))
+    boxes = boxes.view(np.int32)
+    boxes[..., 6] = rng.integers(0, P, (E, mb))
+    count = np.full(E, mb, np.int32)
+    rgb, depth, status, st = _render_custom(oracle, g, _pal(E, P), cams, 96, 52, boxes, count, agents, mb)
+    assert status == 0
+    parity.assert_parity(st, f"wide {grid}")
+    batch = B.Batch(B.make_desc(E, agents, grid, mb, 96, 52, P))
+    batch.upload_worlds(0, E, torch.from_numpy(g).cuda(), torch.from_numpy(boxes).cuda(), torch.from_numpy(count).cuda(),
+                        torch.from_numpy(_pal(E, P)).cuda())
+    batch.set_cameras(torch.from_numpy(cams).cuda())
+    for in_global in (True, False):
+        batch.debug_occupancy_in_global(in_global)
+        out = batch.alloc_outputs()
+        batch.render_batch(*out)
+        assert (out[0].cpu().numpy() == rgb).all() and (out[1].cpu().numpy() == depth).all(), in_global
+    batch.destroy()
