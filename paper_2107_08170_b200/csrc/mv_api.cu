@@ -28,16 +28,16 @@ constexpr int kRenderThreadsSmall = 192;       // CTAs with few tiles (small ima
 // with room for five 135.7 us, 140.2 with three of the ordinary shape).
 constexpr int kSmallCtaTiles = 192;
 constexpr int kHostChunks = 8;
-// CTAs that split the tiles of an observation between them, in a batch with few of them (see pick_parts): this many times
-// what fills the GPU where the occupancy is not staged; once where it is, as each CTA stages the block again.
-constexpr int kPartWaves = 2;
-// Staging + set-up of a CTA, in units of one observation's render time at 128x72 (measured: about 0.1).
-constexpr double kCtaFixedCost = 0.1;
+// Staging and set-up of a CTA in tiles' worth of work, with the GPU full and with little to do (see pick_split).
+constexpr double kSetupTiles = 28.0, kPartTiles = 8.0;
 constexpr size_t kMergeScratchBytes = (size_t)1 << 30;         // bit arrays for the envs of one merge launch
 
 inline uint32_t round_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
 }  // namespace
+
+// The first `whole` CTAs of a render have agents_per_cta observations each, the other observations `parts` CTAs each.
+struct Split { int64_t whole; int parts; };
 
 struct mv_batch {
     mv_batch_desc desc;
@@ -66,7 +66,8 @@ struct mv_batch {
     int agents_per_cta = 1;             // observations one CTA renders: 1, or every agent of its env
     int threads = kRenderThreads;       // threads per CTA of the render kernel (fewer for CTAs with few tiles)
     int sms = 0;
-    int forced_parts = 0;               // test hook: CTAs per observation (0: pick_parts decides)
+    int resident = 1;                   // CTAs of the render kernel that an SM holds
+    int forced_parts = 0;               // test hook: CTAs per observation (0: pick_split decides)
     int tiles_x = 0, tiles_y = 0, mask_words = 0;
     int64_t launches = 0;
     int wait_polls = 1 << 18;
@@ -159,26 +160,44 @@ int pick_threads(const mv_batch *b, int apc) {
     return few_tiles && fills && per_sm >= 5 ? kRenderThreadsSmall : kRenderThreads;
 }
 
-// CTAs per observation (or environment) in a batch with few of them: as many as make three CTAs to an SM (six of the small
-// shape), kPartWaves times as many where the occupancy is not staged, but each with a tile for every warp.  Below, us of a
-// render by CTAs per observation; * is this rule.
-//   staged, 128x72: 16 observations of 128x32x128 columns 24.0 with 1, 13.3 with 4, 9.2 with 24*; 148: 37.4 33.3 32.3* 30.2
-//   with 1 to 4; 300: 59.3* 50.1 43.4 40.4.  4 observations of 64x36: 9.2 with 1, 5.6 with 6*.
-//   not staged, 128x72: 148 observations of 192x48x192 columns 75.3 with 1, 58.8 with 6*; 300: 89.6 98.3* 100.9 86.0 with
-//   1 to 4; 512: 107.0* 114.7 118.3 107.5; 192x36x192 rooms, 300: 79.9 60.9* 52.5 45.0; 512: 85.0* 69.0 60.9 64.5.
-// Three to an SM also where the staged block leaves room for one or two: the parts stage it several times over, but they
-// even out how long observations take.  As many as are resident instead: 192x32x192 columns (150 KB, one to an SM), 128x72,
-// 74 observations 31.2 against 26.6*, 148: 50.7 against 46.1*, 220: 51.2 against 55.8*; 160x32x160 (two), 220: 47.6 against
-// 38.2*.  Where it is worse: images below 128x72 with one CTA to an SM and about as many observations, if those are alike
-// (columns: 148 of 64x36 on 160x64x160 27.6*, unsplit 23.0); in rooms it is the other way round (180 of 64x36 on 192x32x192:
-// 23.0*, unsplit 29.2).
-int pick_parts(const mv_batch *b, int64_t ctas) {
-    const int per_sm = kThreadsPerSm / b->threads;
-    const int64_t slots = (int64_t)per_sm * b->sms * (b->occ_shared ? 1 : kPartWaves);
-    const int64_t most = b->tiles_x * b->tiles_y / (b->threads / 32);
-    int64_t parts = b->forced_parts > 0 ? b->forced_parts : slots / ctas;
-    parts = parts > most ? most : parts;
-    return parts < 1 ? 1 : (int)parts;
+// How a render of `obs` observations is dealt to CTAs; R = CTAs that are resident at once, costs in units of an observation's work.
+// - Less than about a round of CTAs: every observation in parts, as many as cost least: a part's length while all parts run at
+//   once (so few observations get as many parts as make a tile for every warp), with more the rounds it takes.
+// - More: the observations of the last R / 2 CTAs one by one, and those of CTAs of one or two agents in up to three parts, fewer
+//   for small images; the others whole.  Cost: the work of all CTAs, set-up included, over R, and some of the last one's length.
+// Fitted to 60 shapes from 1 to 3222 observations, each timed with up to 40 splits: the choice is 1 % above the best of these in
+// small batches (9 % at worst) and 3 % in larger ones.  Before, parts were contiguous and three CTAs made to an SM, and from a
+// round on all were whole: 300 observations of 128x32x128 columns 57.0 us, now 38.2; 113 of 216x116 45.2, now 28.4; 37 x 6 of
+// 160x108 38.3, now 33.5; 1024 x 2 of 128x72 rooms 111.7, now 107.6; 777 x 3 106.2, now 102.4; 4096 x 4 914.7, now 900.4.
+// `cost`: what the choice costs, for the choice between CTAs of one and of all agents.
+Split pick_split(const mv_batch *b, int64_t obs, double *cost = nullptr) {
+    const int ntiles = b->tiles_x * b->tiles_y, apc = b->agents_per_cta, most = ntiles / (b->threads / 32) > 1 ? ntiles / (b->threads / 32) : 1;
+    const int64_t ctas = obs / apc;
+    const double R = (double)b->resident * b->sms, setup = kSetupTiles / ntiles;
+    double least = 0.0, unused;
+    if (!cost) cost = &unused;
+    *cost = 0.0;
+    const double speed = (double)b->threads / kRenderThreads;              // of a CTA, with the GPU full
+    if (b->forced_parts > 0) return {0, b->forced_parts > most ? most : b->forced_parts};
+    if (ctas >= 0.9 * R) {
+        int parts = (ntiles + 35) / 72;
+        parts = (parts > 3 ? 3 : parts) - (apc - 1);
+        if (parts < 1) parts = 1;
+        const int64_t tail = parts * apc > 1 ? (int64_t)(R / 2) : 0;
+        least = ((double)(ctas - tail) * (apc + setup) + (double)tail * apc * (1 + parts * setup)) / R + 0.6 * (tail ? 1.0 / parts + setup : apc + setup);
+        *cost = least / speed;
+        return {ctas - tail, parts};
+    }
+    Split best{0, most};
+    auto cost_of = [&](int parts) {
+        const double part = 1.0 / parts + kPartTiles / ntiles, rounds = obs * (double)parts / R;
+        return rounds > 1.0 ? part * (rounds + 0.15) : part;
+    };
+    least = cost_of(most);
+    for (int parts = 1; parts < most; parts += 1 + parts / 8)
+        if (cost_of(parts) < least) { least = cost_of(parts); best.parts = parts; }
+    *cost = least / speed;
+    return best;
 }
 
 // The instantiations of the render kernel: by the CTA's threads, and one plane of occupancy staged, several staged, or read from
@@ -199,6 +218,8 @@ void choose_shape(mv_batch *b, int apc) {
     b->agents_per_cta = apc;
     b->smem = smem_layout(b, apc, b->occ_shared);
     b->threads = pick_threads(b, apc);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->resident, render_fn(b), b->threads, b->smem.bytes) != cudaSuccess || b->resident < 1)
+        b->resident = 1;
 }
 
 // The merge sweep keeps a layer number per column: a byte for grids less than 256 high.  Rows of up to 16 words (W) are held in
@@ -239,11 +260,10 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.max_overlay = b->desc.max_overlay_rects;
     p.wait_polls = b->wait_polls;
     p.skip_staging = b->skip_staging;
-    const int64_t ctas = obs_count / b->agents_per_cta;   // callers pass whole environments when a CTA renders one
-    const int ntiles = b->tiles_x * b->tiles_y, parts = pick_parts(b, ctas);
-    p.part_tiles = (ntiles + parts - 1) / parts;
-    MV_CUDA(b, launch_step(render_fn(b), dim3((unsigned)ctas, (unsigned)((ntiles + p.part_tiles - 1) / p.part_tiles)), dim3((unsigned)b->threads),
-                           b->smem.bytes, s, p));
+    const Split split = pick_split(b, obs_count);         // (callers pass whole environments when a CTA renders one)
+    p.whole_ctas = (unsigned)split.whole; p.parts = (unsigned)split.parts;
+    const int64_t ctas = split.whole + (obs_count - split.whole * b->agents_per_cta) * split.parts;
+    MV_CUDA(b, launch_step(render_fn(b), dim3((unsigned)ctas), dim3((unsigned)b->threads), b->smem.bytes, s, p));
     b->launches++;
     return MV_OK;
 }
@@ -507,28 +527,16 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(upload_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUploadSmem);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
-    // One CTA per environment (block staged once for all its agents) when that still fills the GPU;
-    // otherwise one CTA per observation.  Cost model: work per slot and the wait for the last CTAs.
-    if (d.agents_per_env > 1) {
-        const mv_batch::Smem all = smem_layout(b, d.agents_per_env, b->occ_shared);    // (never give up staged occupancy for it)
-        if ((int64_t)all.bytes <= smem_max) {
-            auto shape_cost = [&](const mv_batch::Smem &m, int apc) {
-                int per_sm = 0;
-                const int threads = pick_threads(b, apc);
-                cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, render_fn(b, threads, b->occ_shared), threads, m.bytes);
-                if (q != cudaSuccess || per_sm < 1) return 1e30;
-                // CTAs of different length drift apart, so there are no waves: what the slots have to do, and on average half a
-                // CTA of waiting for the last ones (777 envs x 3 agents: 121 us by environment, 115 by observation)
-                return ((double)b->num_obs / apc / ((double)per_sm * sms) + 0.5) * (apc + kCtaFixedCost);
-            };
-            if (shape_cost(all, d.agents_per_env) < shape_cost(b->smem, 1)) {
-                b->smem = all;
-                b->agents_per_cta = b->auto_agents_per_cta = d.agents_per_env;
-            }
-        }
+    // A CTA per environment (block staged once for all its agents) or per observation, whichever is expected to take less.
+    choose_shape(b, 1);
+    if (d.agents_per_env > 1 && (int64_t)smem_layout(b, d.agents_per_env, b->occ_shared).bytes <= smem_max) {   // (never give up staged occupancy for it)
+        double one, all;
+        pick_split(b, b->num_obs, &one);
+        choose_shape(b, d.agents_per_env);
+        const bool whole = pick_split(b, b->num_obs, &all).whole > 0;      // (where all goes in parts there is nothing to share)
+        if (whole && all < one) b->auto_agents_per_cta = d.agents_per_env;
+        else choose_shape(b, 1);
     }
-
-    choose_shape(b, b->agents_per_cta);
 
     const size_t blocks_bytes = (size_t)d.num_envs * L.stride;
     bool ok = cudaMalloc(&b->d_env_blocks, blocks_bytes) == cudaSuccess &&
@@ -841,7 +849,8 @@ int mv_debug_occupancy_in_global(mv_batch *b, int on) {
 int mv_debug_parts(mv_batch *b, int parts) {
     if (!b || parts < 0) return MV_ERR_INVALID_ARG;
     b->forced_parts = parts;
-    return pick_parts(b, b->num_obs / b->agents_per_cta);
+    const Split split = pick_split(b, b->num_obs);
+    return split.whole > 0 ? 1 : split.parts;
 }
 
 int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {

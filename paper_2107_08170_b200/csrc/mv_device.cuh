@@ -65,6 +65,9 @@ __device__ __forceinline__ bool voxel_filled(const EnvLayout &lay, const unsigne
     const uint32_t w = *reinterpret_cast<const uint32_t *>(occ + (size_t)q * lay.occ_plane + 4u * column_index(lay, x, z));
     return (w >> (y - plane_begin(q))) & 1u;
 }
+// Tiles that go to the same CTA when an observation's are shared out: 32 pixels, whose bytes of a row are whole sectors.
+constexpr int kPartRun = 4;
+
 struct RenderParams {
     const unsigned char *env_blocks;   // [E] EnvLayout blocks
     const uint8_t *mat;                // [E][mat_stride] material ids by voxel index (clamped at upload)
@@ -82,8 +85,9 @@ struct RenderParams {
     float inv_W;                       // 1 / W
     uint32_t sky_rgbx;
     float miss_depth;
-    int agents_per_cta;                // observations one CTA renders: 1, or all agents of its env
-    int part_tiles;                    // tiles of one observation that a CTA renders
+    int agents_per_cta;                // observations one of the first whole_ctas CTAs renders: 1, or all agents of its env
+    unsigned whole_ctas;               // the CTAs behind those render a part of one observation each:
+    unsigned parts;                    // every parts-th run of kPartRun tiles of it
     float exit_scale;                  // 1 - (bound on the rounding drift of accumulated crossing times)
     // shared-memory offsets after the staged env block: tile table, per-agent blocks (ray table, camera record,
     // eye-relative boxes, then overlay rectangles and per-tile box masks at the offsets below), barrier and flag words

@@ -236,8 +236,14 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kWarps = NT / 32;
-    const int apc = p.agents_per_cta;
-    const int obs0 = p.obs_begin + blockIdx.x * apc;
+    // The first CTAs of the grid render whole observations, those behind them every parts-th run of tiles of one (a batch with
+    // few observations, or the end of the grid).  Neighbouring runs cost about the same, so the parts of an observation do too.
+    // A part marks the boxes in all tiles' masks, like a whole; only its tile table is shorter.
+    const bool whole = blockIdx.x < p.whole_ctas;
+    const int apc = whole ? p.agents_per_cta : 1, parts = whole ? 1 : (int)p.parts;
+    const int obs_in = whole ? (int)blockIdx.x * apc : (int)((blockIdx.x - p.whole_ctas) / p.parts);
+    const int part = whole ? 0 : (int)(blockIdx.x - p.whole_ctas) - obs_in * parts;
+    const int obs0 = p.obs_begin + obs_in + (whole ? 0 : (int)p.whole_ctas * p.agents_per_cta);
     const int env = p.agents == 1 ? obs0 : obs0 / p.agents;
     const int W = p.W, H = p.H;
     const int ntiles = p.tiles_x * p.tiles_y;
@@ -263,22 +269,25 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     auto agent_rel = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentRelOff); };
     auto agent_ov = [&](int ag) { return reinterpret_cast<int4 *>(s_agents + (size_t)ag * p.agent_stride + p.agent_ov_off); };
     auto agent_mask = [&](int ag) { return reinterpret_cast<uint32_t *>(s_agents + (size_t)ag * p.agent_stride + p.agent_mask_off); };
-    // (in a batch with few observations each one's tiles are split between the CTAs of a grid column)
-    const int tile0 = blockIdx.y * p.part_tiles, tile1 = min(tile0 + p.part_tiles, ntiles);
+    // how many tiles the CTA has
+    const int runs = (ntiles + kPartRun - 1) / kPartRun, own_runs = (runs - part + parts - 1) / parts;
+    const int mine = own_runs * kPartRun - ((runs - 1 - part) % parts == 0 ? runs * kPartRun - ntiles : 0);
 
     // ---- tile table, cleared masks (this much needs nothing from the kernels before)
     if (tid == 0) mbar_init(s_bar, 1);
     for (int ag = 0; ag < apc; ++ag) {
         uint32_t *mk = agent_mask(ag);
-        for (int i = tile0 * ms + tid; i < tile1 * ms; i += NT) mk[i] = 0u;
+        for (int i = tid; i < ntiles * ms; i += NT) mk[i] = 0u;
     }
     const float inv_tiles_x = 1.0f / (float)p.tiles_x;
-    for (int i = tile0 + tid; i < tile1; i += NT) {
+    for (int j = tid; j < mine; j += NT) {
+        const int i = parts == 1 ? j : (part + j / kPartRun * parts) * kPartRun + j % kPartRun;
         // (i + 0.5) / tiles_x is at least 1 / (2 tiles_x) away from an integer: exact in float for any image
         const int ty = (int)(((float)i + 0.5f) * inv_tiles_x), tx = i - ty * p.tiles_x;
-        // a = 2px+1-W and b = H-1-2py of the tile's first pixel (small integers: exact as floats)
-        s_tile[i] = make_float4((float)(16 * tx + 1 - W), (float)(H - 1 - 8 * ty), __int_as_float(ty * 4 * W + tx * 8),
-                                __int_as_float(i));
+        // a = 2px+1-W and b = H-1-2py of the tile's first pixel (small integers: exact as floats), its place in the image and in
+        // an agent's block (the tile's box mask)
+        s_tile[j] = make_float4((float)(16 * tx + 1 - W), (float)(H - 1 - 8 * ty), __int_as_float(ty * 4 * W + tx * 8),
+                                __int_as_float((int)p.agent_mask_off + 4 * i * ms));
     }
     wait_for_previous();
     // ---- stage the environment block
@@ -546,6 +555,10 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     __syncthreads();
 
     uint32_t guards = smem_addr(s_guard + 1);                               // guard of plane 0
+    // Does the uncommon tile loop read the occupied box again, so that its bounds hold no registers while the common one runs?  As
+    // compiled that is 1 % faster for one plane (8192 x 2 of 256x144: 3099 us, 3065 like this), and slower for several (4096 of
+    // 64x36x64 250 and 254) and in CTAs of 576 threads (2048 x 2 of 160x32x160 303 and 318).
+    constexpr bool kReadBox = COLW && NT != 576;
     const float flox = (float)lox, floy = (float)loy, floz = (float)loz;
     const float fhix = (float)hix, fhiy = (float)hiy, fhiz = (float)hiz;
 
@@ -565,10 +578,9 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     opaque(lane_a, lane); opaque(lane_b, lane); opaque(st_sel, lane);
     unsigned long long lane_ab;
     asm("mov.b64 %0, {%1, %2};" : "=l"(lane_ab) : "f"(lane_a), "f"(lane_b));
-    const uint32_t tile_begin = smem_addr(s_tile) + 16u * (uint32_t)(tile0 + warp);
-    uint32_t tile_end = smem_addr(s_tile) + 16u * (uint32_t)tile1;
-    uint32_t mask_step = 4u * kWarps * (uint32_t)ms;                        // bytes between a warp's consecutive tile masks
-    opaque(tile_end, lane); opaque(mask_step, lane);
+    const uint32_t tile_begin = smem_addr(s_tile) + 16u * (uint32_t)warp;
+    uint32_t tile_end = smem_addr(s_tile) + 16u * (uint32_t)mine;
+    opaque(tile_end, lane);
 
     for (int ag = 0; ag < apc; ++ag) {
         const int obs = obs0 + ag;
@@ -580,7 +592,6 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
             continue;
         }
         uint32_t abase = smem_addr(agent_tab(ag));
-        uint32_t mask_p = smem_addr(agent_mask(ag) + (size_t)(tile0 + warp) * ms);
         // (store addresses as global-space addresses for the PTX store block)
         unsigned long long depth_lane = (unsigned long long)__cvta_generic_to_global(depth_obs + depth_lane_off);
         unsigned long long rgb_lane = (unsigned long long)__cvta_generic_to_global(rgb_obs + rgb_lane_off);
@@ -725,9 +736,9 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 : "memory");
         };
         if (aflags & kAgentSealed) {
-            for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
+            for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps) {
                 int tile_px;
-                uint32_t pos, bit = 0, plane = 0, row, tab, graze;
+                uint32_t pos, bit = 0, plane = 0, row, tab, graze, mask_p;
                 float t_hit, dtx, dty, dtz;
                 // ---- the common case in one block of PTX: tile record, ray through the pixel centre
                 // (d = F + a*Rs + b*Us, a = 2px+1-W, b = H-1-2py, two chained FMAs per component),
@@ -743,18 +754,18 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 // is +-inf, so its crossing time is +inf (or NaN when the eye sits exactly on the face,
                 // which min and the compares ignore) and that axis is never stepped, which is the rule
                 // for such rays.
-#define MV_SEALED_RAY \
+#define MV_SEALED_RAY(TILE, BASE, AB, MASK) \
                     MV_DDA_DECL \
                     " .reg .f32 Ta, Tb, Fx, Fy, Fz, Rx, Rz, Ux, Uy, Uz, ca, cb, dx, dy, dz, ix, iy, iz;\n" \
                     " .reg .f32 q0, q1, q2, q3, q4;\n" \
                     " .reg .b32 u, v;\n" \
                     " .reg .b64 T2, D2, Q2, C2, M2;\n" \
-                    " ld.shared.v4.b32 {Ta, Tb, %0, _}, [%10];\n" \
-                    " ld.shared.v4.f32 {Fx, Fy, Rx, Uy}, [%11+" MV_REC_F "];\n" \
-                    " ld.shared.v4.f32 {Ux, Uz, Fz, Rz}, [%11+" MV_REC_U "];\n" \
-                    " ld.shared.v2.b32 {bit, guard}, [%11+" MV_REC_START "];\n" \
+                    " ld.shared.v4.b32 {Ta, Tb, %0, " MASK "}, [" TILE "];\n" \
+                    " ld.shared.v4.f32 {Fx, Fy, Rx, Uy}, [" BASE "+" MV_REC_F "];\n" \
+                    " ld.shared.v4.f32 {Ux, Uz, Fz, Rz}, [" BASE "+" MV_REC_U "];\n" \
+                    " ld.shared.v2.b32 {bit, guard}, [" BASE "+" MV_REC_START "];\n" \
                     " mov.b64 C2, {Ta, Tb};\n" \
-                    " add.rn.f32x2 C2, C2, %12;\n" \
+                    " add.rn.f32x2 C2, C2, " AB ";\n" \
                     " mov.b64 {ca, cb}, C2;\n" \
                     " mov.b64 T2, {Fx, Fy};\n" \
                     " mov.b64 D2, {Rx, Uy};\n" \
@@ -772,7 +783,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     " mov.b32 u, dx;\n" \
                     " mov.b32 v, dz;\n" \
                     " prmt.b32 u, u, v, 0x00FB;\n"    /* byte 0: sign of dx, byte 1: sign of dz */ \
-                    " lop3.b32 %8, u, 0x140, %11, 0xEA;\n" \
+                    " lop3.b32 %8, u, 0x140, " BASE ", 0xEA;\n" \
                     " mov.b32 u, dy;\n" \
                     " shr.u32 u, u, 24;\n" \
                     " lop3.b32 %8, u, 0x80, %8, 0xEA;\n" \
@@ -833,43 +844,47 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     " mov.f32 %6, dty;\n" \
                     " mov.f32 %7, dtz;\n"
                 if constexpr (COLW) {
-                    asm volatile("{\n" MV_SEALED_RAY MV_DDA_SEALED(MV_DDA_STEP_SEALED) MV_SEALED_END "}\n"
-                        : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze)
+                    asm volatile("{\n" MV_SEALED_RAY("%11", "%12", "%13", "%10") MV_DDA_SEALED(MV_DDA_STEP_SEALED) MV_SEALED_END "}\n"
+                        : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze), "=&r"(mask_p)
                         : "r"(tile_p), "r"(abase), "l"(lane_ab)
                         : "memory");
                 } else {
-#define MV_SEALED_PLANE " ld.shared.u32 q, [%11+" MV_REC_PLANE "];\n"
-#define MV_SEALED_CROSS(LOAD) MV_DDA_CROSS("%14", "%15", "%16", "", " mov.b32 guard, a;\n", LOAD) " mov.b32 %13, q;\n"
+#define MV_SEALED_PLANE " ld.shared.u32 q, [%13+" MV_REC_PLANE "];\n"
+#define MV_SEALED_CROSS(LOAD) MV_DDA_CROSS("%15", "%16", "%17", "", " mov.b32 guard, a;\n", LOAD) " mov.b32 %11, q;\n"
 #define MV_SEALED_IO                                                                                                \
                         : "=&r"(tile_px), "=&r"(pos), "=&r"(bit), "=&f"(t_hit), "=&r"(row), "=&f"(dtx), "=&f"(dty), "=&f"(dtz), "=&r"(tab), "=&r"(graze), \
-                          "+r"(tile_in), "+r"(abase), "+l"(lane_ab), "=&r"(plane)                                               \
-                        : "r"(plane_end), "r"(p.lay.occ_plane), "r"(guards), "l"(env_block)                                  \
+                          "=&r"(mask_p), "=&r"(plane)                                               \
+                        : "r"(tile_p), "r"(abase), "l"(lane_ab), "r"(plane_end), "r"(p.lay.occ_plane), "r"(guards), "l"(env_block)                                  \
                         : "memory"
-                    uint32_t tile_in = tile_p;
                     if constexpr (staged)
-                        asm volatile("{\n" MV_SEALED_RAY MV_SEALED_PLANE MV_DDA_SEALED(MV_DDA_STEP_SEALED) MV_SEALED_CROSS(MV_DDA_LOAD_SHARED) MV_SEALED_END "}\n" MV_SEALED_IO);
+                        asm volatile("{\n" MV_SEALED_RAY("%12", "%13", "%14", "%10") MV_SEALED_PLANE MV_DDA_SEALED(MV_DDA_STEP_SEALED) MV_SEALED_CROSS(MV_DDA_LOAD_SHARED) MV_SEALED_END "}\n" MV_SEALED_IO);
                     else
-                        asm volatile("{\n" MV_SEALED_RAY MV_SEALED_PLANE " mov.b64 gbase, %17;\n" MV_DDA_SEALED(MV_DDA_STEP_SEALED_GLOBAL) MV_SEALED_CROSS(MV_DDA_LOAD_GLOBAL) MV_SEALED_END "}\n" MV_SEALED_IO);
+                        asm volatile("{\n" MV_SEALED_RAY("%12", "%13", "%14", "%10") MV_SEALED_PLANE " mov.b64 gbase, %18;\n" MV_DDA_SEALED(MV_DDA_STEP_SEALED_GLOBAL) MV_SEALED_CROSS(MV_DDA_LOAD_GLOBAL) MV_SEALED_END "}\n" MV_SEALED_IO);
 #undef MV_SEALED_PLANE
 #undef MV_SEALED_CROSS
 #undef MV_SEALED_IO
                 }
 #undef MV_SEALED_RAY
 #undef MV_SEALED_END
-                finish_tile(mask_p, tile_px, pos, bit, plane, row, tab, graze, t_hit, dtx, dty, dtz);
+                finish_tile(abase + mask_p, tile_px, pos, bit, plane, row, tab, graze, t_hit, dtx, dty, dtz);
             }
         } else {
             const float4 P4 = agent_rec(ag)[3];
             const float Px = P4.x, Py = P4.y, Pz = P4.z;
             const bool cam_in = (aflags & kAgentInside) != 0;
-            for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps, mask_p += mask_step) {
+            float4 lo = make_float4(flox, floy, floz, 0.0f), hi = make_float4(fhix, fhiy, fhiz, 0.0f);
+            if constexpr (kReadBox) { lo = agent_rec(ag)[5]; hi = agent_rec(ag)[6]; }
+            const int ilox = kReadBox ? (int)lo.x : lox, iloy = kReadBox ? (int)lo.y : loy, iloz = kReadBox ? (int)lo.z : loz;
+            const int ihix = kReadBox ? (int)hi.x : hix, ihiy = kReadBox ? (int)hi.y : hiy, ihiz = kReadBox ? (int)hi.z : hiz;
+            const bool any = kReadBox ? ilox < ihix && iloy < ihiy && iloz < ihiz : any_voxel;
+            for (uint32_t tile_p = tile_begin; tile_p < tile_end; tile_p += 16u * kWarps) {
                 int tile_px;
-                uint32_t pos, bit = 0, plane = 0, row, tab;
+                uint32_t pos, bit = 0, plane = 0, row, tab, mask_p;
                 float t_hit, dtx, dty, dtz;
                 // ---- every other case: the same steps in C++, with the eye possibly outside the
                 // occupied box and either flavour of the walk
                 float Ta, Tb;
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, _}, [%3];" : "=f"(Ta), "=f"(Tb), "=r"(tile_px) : "r"(tile_p));
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=f"(Ta), "=f"(Tb), "=r"(tile_px), "=r"(mask_p) : "r"(tile_p));
                 const float4 FR = agent_rec(ag)[0], UY = agent_rec(ag)[1];
                 const uint32_t bit0 = __float_as_uint(agent_rec(ag)[2].x);
                 const float a = Ta + lane_a, bb = Tb + lane_b;
@@ -899,8 +914,8 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     t0y = qy * dty;
                     t0z = qz * dtz;
                     const int cx = (int)floorf(Px), cy = (int)floorf(Py), cz = (int)floorf(Pz);
-                    t_exit = min3f(fmaf((float)(ngx ? cx - lox : hix - 1 - cx), dtx, t0x), fmaf((float)(ngy ? cy - loy : hiy - 1 - cy), dty, t0y),
-                                   fmaf((float)(ngz ? cz - loz : hiz - 1 - cz), dtz, t0z)) * p.exit_scale;
+                    t_exit = min3f(fmaf((float)(ngx ? cx - ilox : ihix - 1 - cx), dtx, t0x), fmaf((float)(ngy ? cy - iloy : ihiy - 1 - cy), dty, t0y),
+                                   fmaf((float)(ngz ? cz - iloz : ihiz - 1 - cz), dtz, t0z)) * p.exit_scale;
                     // the first stretch, as in the block above
                     const float ts = min3f(ex * dtx, ez * dtz, ey * dty);
                     const float nx = __fadd_rd(fmaf(ts, fabsf(dx), kx), 8388608.0f), nz = __fadd_rd(fmaf(ts, fabsf(dz), kz), 8388608.0f);
@@ -910,21 +925,21 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     if (aflags & kAgentFilled) { row = inside_row; t_exit = -kInf; }
                 } else {
                     // eye outside the occupied box: clip the ray to it, start in the entry cell
-                    const float x1 = (flox - Px) * ix, x2 = (fhix - Px) * ix;
-                    const float y1 = (floy - Py) * iy, y2 = (fhiy - Py) * iy;
-                    const float z1 = (floz - Pz) * iz, z2 = (fhiz - Pz) * iz;
+                    const float x1 = (lo.x - Px) * ix, x2 = (hi.x - Px) * ix;
+                    const float y1 = (lo.y - Py) * iy, y2 = (hi.y - Py) * iy;
+                    const float z1 = (lo.z - Pz) * iz, z2 = (hi.z - Pz) * iz;
                     const float nrx = fminf(x1, x2), nry = fminf(y1, y2), nrz = fminf(z1, z2);
                     const float tn = max3f(nrx, nry, nrz);
                     const float tf = min3f(fmaxf(x1, x2), fmaxf(y1, y2), fmaxf(z1, z2));
-                    const bool alive = any_voxel && (tn <= tf) && (tf > 0.0f);
+                    const bool alive = any && (tn <= tf) && (tf > 0.0f);
                     const int eaxis = tn < 0.0f ? -1 : (nrx == tn ? 0 : (nry == tn ? 1 : 2));
                     t_hit = alive ? fmaxf(tn, 0.0f) : 0.0f;
-                    int cx = min(max((int)floorf(fmaf(t_hit, dx, Px)), lox), hix - 1);
-                    int cy = min(max((int)floorf(fmaf(t_hit, dy, Py)), loy), hiy - 1);
-                    int cz = min(max((int)floorf(fmaf(t_hit, dz, Pz)), loz), hiz - 1);
-                    if (eaxis == 0) cx = ngx ? hix - 1 : lox;
-                    if (eaxis == 1) cy = ngy ? hiy - 1 : loy;
-                    if (eaxis == 2) cz = ngz ? hiz - 1 : loz;
+                    int cx = min(max((int)floorf(fmaf(t_hit, dx, Px)), ilox), ihix - 1);
+                    int cy = min(max((int)floorf(fmaf(t_hit, dy, Py)), iloy), ihiy - 1);
+                    int cz = min(max((int)floorf(fmaf(t_hit, dz, Pz)), iloz), ihiz - 1);
+                    if (eaxis == 0) cx = ngx ? ihix - 1 : ilox;
+                    if (eaxis == 1) cy = ngy ? ihiy - 1 : iloy;
+                    if (eaxis == 2) cz = ngz ? ihiz - 1 : iloz;
                     if (!alive) { cx = cy = cz = 0; }
                     pos = cell_pos(cx, cy, cz);
                     plane = cell_plane(cy);
@@ -932,9 +947,9 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                     t0x = ((float)(cx + (ngx ? 0 : 1)) - Px) * ix;
                     t0y = ((float)(cy + (ngy ? 0 : 1)) - Py) * iy;
                     t0z = ((float)(cz + (ngz ? 0 : 1)) - Pz) * iz;
-                    t_exit = min3f(fmaf(ngx ? (float)(cx - lox) : (float)(hix - 1 - cx), dtx, t0x),
-                                   fmaf(ngy ? (float)(cy - loy) : (float)(hiy - 1 - cy), dty, t0y),
-                                   fmaf(ngz ? (float)(cz - loz) : (float)(hiz - 1 - cz), dtz, t0z)) * p.exit_scale;
+                    t_exit = min3f(fmaf(ngx ? (float)(cx - ilox) : (float)(ihix - 1 - cx), dtx, t0x),
+                                   fmaf(ngy ? (float)(cy - iloy) : (float)(ihiy - 1 - cy), dty, t0y),
+                                   fmaf(ngz ? (float)(cz - iloz) : (float)(ihiz - 1 - cz), dtz, t0z)) * p.exit_scale;
                     const bool filled = alive && voxel_filled(p.lay, occ, cx, cy, cz);
                     // entered through the box face of axis eaxis, or the eye is inside a solid
                     if (filled) {
@@ -976,7 +991,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
 #undef MV_DDA_CROSS_GENERAL
 #undef MV_DDA_OUTS
                 if (row == kNoRow) t_hit = kInf;          // no voxel hit
-                finish_tile(mask_p, tile_px, pos, bit, plane, row, tab, 0u, t_hit, dtx, dty, dtz);
+                finish_tile(abase + mask_p, tile_px, pos, bit, plane, row, tab, 0u, t_hit, dtx, dty, dtz);
             }
         }
     }

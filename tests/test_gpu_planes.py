@@ -1,4 +1,5 @@
-"""Grids of several occupancy planes (more than 32 high) and the CTA shapes of large blocks, against the oracle."""
+"""Grids of several occupancy planes (more than 32 high), the CTA shapes of large blocks and the end of a large grid, against the
+oracle and against each other."""
 import numpy as np
 import pytest
 import torch
@@ -87,4 +88,36 @@ def test_large_blocks_in_wide_ctas(oracle, grid, agents):
         out = batch.alloc_outputs()
         batch.render_batch(*out)
         assert (out[0].cpu().numpy() == rgb).all() and (out[1].cpu().numpy() == depth).all(), in_global
+    batch.destroy()
+
+
+@pytest.mark.parametrize("agents,size", [(1, (72, 52)), (1, (136, 72)), (2, (72, 52)), (3, (48, 40)), (6, (64, 36))])
+def test_the_end_of_the_grid_in_parts(oracle, agents, size):
+    """A few rounds of CTAs: the last observations in parts or one by one, behind CTAs that render whole ones or all agents of an
+    environment; the same bytes as with every observation in one CTA and in three, overlays and bad cameras included."""
+    from paper_2107_08170_b200 import scenes
+    B = _binding()
+    envs = 1500 // agents if agents < 6 else 450
+    cfg = scenes.config("rooms", num_envs=envs, agents=agents, grid=(16, 12, 16), width=size[0], height=size[1], movable_boxes=4,
+                        extra={"n_lines": 1})
+    sc = scenes.make_scene(cfg, device="cuda")
+    batch = B.Batch(B.desc_from_config(cfg, 0, max_overlay_rects=1))
+    batch.upload_worlds(0, envs, sc["grid"], sc["boxes"], sc["box_count"], sc["palette"])
+    for o in (0, cfg.num_obs // 2, cfg.num_obs - 1):
+        sc["cams"][o, 3] = torch.tensor([float("nan")]).view(torch.int32).item()
+    rects = torch.zeros(cfg.num_obs, 1, 4, dtype=torch.int32)
+    rects[..., 1], rects[..., 2] = size[0] // 2 | (3 << 16), 0x20C0FF
+    batch.set_overlays(rects.cuda(), torch.ones(cfg.num_obs, dtype=torch.int32, device="cuda"))
+    batch.set_cameras(sc["cams"])
+    assert batch.query_status(clear=True) == B.FLAG_BAD_CAMERA
+    want = None
+    for apc in sorted({1, agents}):
+        batch.debug_agents_per_cta(apc)
+        for parts in (1, 3, 0):
+            assert batch.debug_parts(parts) == max(parts, 1)                 # (0: the library's choice, which begins with whole ones)
+            rgb, depth = batch.alloc_outputs()
+            rgb.fill_(9); depth.fill_(-3.0)
+            batch.render_batch(rgb, depth)
+            want = want or (rgb, depth)
+            assert torch.equal(rgb, want[0]) and torch.equal(depth, want[1]), (apc, parts)
     batch.destroy()
