@@ -509,6 +509,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
             const float hx = A.w - Px, hy = B.x - Py, hz = B.y - Pz;
             const bool valid = (b < nb) && (b != self_box) && (A.x < A.w) && (A.y < B.x) && (A.z < B.y) && i < apc * p.max_boxes;
             float tmin = kInf, tmax = -kInf, fxmin = kInf, fxmax = -kInf, fymin = kInf, fymax = -kInf;
+            uint32_t beside = 15u;                            // a bit per side of the view that all corners lie beyond
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const float vx = (part & 1) ? hx : lx, vy = c ? hy : ly, vz = (part & 2) ? hz : lz;
@@ -516,6 +517,8 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 const float u = (vx * Rx + vz * Rz) * ir2;
                 const float w = (vx * Ux + vy * Uy + vz * Uz) * iu2;
                 tmin = fminf(tmin, t); tmax = fmaxf(tmax, t);
+                const float wide = ((float)W - 0.5f) * t, high = ((float)H - 0.5f) * t;      // (a quarter of a pixel beyond the outermost centres)
+                beside &= (u > wide ? 1u : 0u) | (-u > wide ? 2u : 0u) | (w > high ? 4u : 0u) | (-w > high ? 8u : 0u);
                 const float it = fast_rcp(fmaxf(t, 1e-3f));
                 const float fx = (u * it + (float)(W - 1)) * 0.5f;     // pixel column of the projection
                 const float fy = ((float)(H - 1) - w * it) * 0.5f;     // pixel row
@@ -527,13 +530,18 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 tmin = fminf(tmin, __shfl_xor_sync(0xffffffffu, tmin, s)); tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, s));
                 fxmin = fminf(fxmin, __shfl_xor_sync(0xffffffffu, fxmin, s)); fxmax = fmaxf(fxmax, __shfl_xor_sync(0xffffffffu, fxmax, s));
                 fymin = fminf(fymin, __shfl_xor_sync(0xffffffffu, fymin, s)); fymax = fmaxf(fymax, __shfl_xor_sync(0xffffffffu, fymax, s));
+                beside &= __shfl_xor_sync(0xffffffffu, beside, s);
             }
             const bool front = tmin > 0.05f;                 // whole box safely in front of the eye plane
             if (part == 0 && valid) {
                 agent_rel(ag)[2 * b] = make_float4(lx, ly, lz, front ? tmin * 0.9999f : 0.0f);
                 agent_rel(ag)[2 * b + 1] = make_float4(hx, hy, hz, B.z);
             }
-            if (!valid || tmax < -1e-3f) continue;           // ignored, or wholly behind the eye
+            // Ignored, wholly behind the eye, or wholly beside the view.  The last matters for boxes across the eye plane, which have no
+            // bounding rectangle and go to every tile: nearly all of them are off to one side, half a box an agent among 32 in a
+            // room of 64x64, and their tests in every tile were a sixth of the frame (8192 x 2 of 256x144 3040 us, now 2591;
+            // 4096 x 4 with 36 boxes 891, now 744; 16384 with 16 boxes on 128x128 1051, now 1013).
+            if (!valid || tmax < -1e-3f || beside) continue;
             int px0 = 0, px1 = W - 1, py0 = 0, py1 = H - 1;
             if (front) {
                 px0 = (int)ceilf(fmaxf(fxmin - 0.25f, 0.0f));

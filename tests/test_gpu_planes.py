@@ -121,3 +121,45 @@ def test_the_end_of_the_grid_in_parts(oracle, agents, size):
             want = want or (rgb, depth)
             assert torch.equal(rgb, want[0]) and torch.equal(depth, want[1]), (apc, parts)
     batch.destroy()
+
+
+def test_boxes_across_the_eye_plane(oracle):
+    """Boxes across the eye plane that are off to one side go to no tile, those that reach into the view to all: beside, above and
+    below the eye, touching the view's edge from outside and inside, around the eye, long ones that cross the view, and some of
+    infinite extent, at narrow and wide angles."""
+    from helpers import box_rows
+    rng = np.random.default_rng(4)
+    E, nb, gx = 12, 40, 24
+    g = np.zeros((E, 16, gx, gx), np.uint8)
+    g[:, 0] = 1
+    eye = np.array([12.3, 8.2, 12.6])
+    cams, boxes = [], []
+    for e in range(E):
+        yaw, pitch = rng.uniform(0, 6.28), rng.uniform(-0.9, 0.9)
+        cams.append(cam_row(*eye, yaw, pitch))
+        fwd = np.array([np.cos(pitch) * np.sin(yaw), np.sin(pitch), np.cos(pitch) * np.cos(yaw)])
+        right = np.array([np.cos(yaw), 0, -np.sin(yaw)])
+        up = np.cross(fwd, right)
+        items = []
+        for n in range(nb):
+            side = (right, -right, up, -up)[n % 4] * rng.uniform(0.3, 7) + fwd * rng.uniform(-1.0, 1.5)
+            half = rng.uniform(0.05, 1.5, 3)
+            if n % 10 == 9:
+                half[n // 10 % 3] = 9.0                        # a long one
+            c = eye + side
+            if n == 5:
+                c, half = eye + fwd * 0.2, np.array([0.4, 0.3, 0.5])   # around the eye
+            lo, hi = c - half, c + half
+            if n == 7:
+                lo[1] = -np.inf
+            if n == 11:
+                hi[0] = np.inf
+            items.append((lo, hi, 1 + n % 5))
+        boxes.append(box_rows(items))
+    for hfov in (0.5, 1.5707964, 2.6):
+        for only in (range(nb), [5, 7, 11], [n for n in range(nb) if n not in (5, 7, 11)]):
+            some = np.stack([b[list(only)] for b in boxes])
+            rgb, depth, status, st = _render_custom(oracle, g, _pal(E, 6), np.stack(cams), 64, 36, some, np.full(E, len(list(only)), np.int32), 1,
+                                                    some.shape[1], hfov_rad=hfov)
+            assert status == 0
+            parity.assert_parity(st, f"across the eye plane {hfov}")
