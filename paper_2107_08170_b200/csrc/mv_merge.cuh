@@ -14,8 +14,8 @@
 // carry-propagating additions), which begin; and the heights of a layer's boxes are independent of each other.
 //
 // Measured (512 envs of 128x32x128 with 1361 boxes each): 11.4 ms with one warp growing one box at a time (about
-// 8 us a box, all of it latency); 0.44 ms with the rows of a layer one after the other in one warp; 0.31 ms with all rows at
-// once (see sweep_layer), of which the bit arrays 0.12.
+// 8 us a box, all of it latency); 0.44 ms with the rows of a layer one after the other in one warp; 0.28 ms with all rows at
+// once (see sweep_layer), of which the bit arrays 0.1.
 #pragma once
 #include "mv_device.cuh"
 #include "mv_pack.cuh"
@@ -57,7 +57,8 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t v, int lane)
 // The bit arrays of a launch's envs.  One CTA: 8 z-rows x 128 x x 32 heights of one env; a warp takes 32 columns of
 // four rows, so that the column at z-1 is still in registers; the y-packed results are transposed in registers and
 // leave through shared memory as runs of up to 128 bytes.  Bound by the material bytes it streams (one byte per
-// voxel, the x-1 column from L1) once the upper 16 heights are left out where nothing is filled up there.
+// voxel, the x-1 column from L1) and by instructions, once the upper 16 heights are left out where nothing is filled up there; then
+// two rows also share a transpose (512 worlds of 128x32x128 287.5 -> 281.4 us, 1047 of 112x44x52 329.2 -> 306.6).
 template <bool PLANES>
 __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsigned char *__restrict__ env_blocks,
                                                                     const uint8_t *__restrict__ mat, EnvLayout lay,
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
         if (upper) ne |= (differ8(4) << 9) | (differ8(6) << 17);
         return ~ne;
     };
-    uint32_t own[8] = {}, back[8] = {}, f_back = 0, f_above = 0;
+    uint32_t own[8] = {}, back[8] = {}, f_back = 0, f_above = 0, f_even = 0, lx_even = 0, lz_even = 0;
     if (in_x && z0 > 0 && z0 < ml.gz) {
         f_back = bits((z0 - 1) * (int)lay.pitch, f_above);
         load_column(m_col + ((size_t)(z0 - 1) * lay.pitch << lay.ysh), back);
@@ -141,9 +142,18 @@ __global__ void __launch_bounds__(kMergeThreads) merge_masks_kernel(const unsign
 #pragma unroll
         for (int q = 0; q < 8; ++q) back[q] = own[q];
         f_back = f;
-        s_out[0][lane][(4 * half + i) * 4 + wi] = transpose32(f, lane);
-        s_out[1][lane][(4 * half + i) * 4 + wi] = transpose32(lx, lane);
-        s_out[2][lane][(4 * half + i) * 4 + wi] = transpose32(lz, lane);
+        if (upper) {
+            s_out[0][lane][(4 * half + i) * 4 + wi] = transpose32(f, lane);
+            s_out[1][lane][(4 * half + i) * 4 + wi] = transpose32(lx, lane);
+            s_out[2][lane][(4 * half + i) * 4 + wi] = transpose32(lz, lane);
+        } else if (i & 1) {                              // 16 heights of two rows in one transpose
+            const int at = (4 * half + i - 1 + (lane >> 4)) * 4 + wi;
+            s_out[0][lane & 15][at] = transpose32(f_even | f << 16, lane);
+            s_out[1][lane & 15][at] = transpose32(lx_even | lx << 16, lane);
+            s_out[2][lane & 15][at] = transpose32(lz_even | lz << 16, lane);
+        } else {
+            f_even = f & 0xffffu; lx_even = lx & 0xffffu; lz_even = lz & 0xffffu;
+        }
     }
     __syncthreads();
     uint32_t *dst = scratch + (size_t)e * ml.env_words;
@@ -323,10 +333,11 @@ __device__ __forceinline__ int run_up(uint32_t e, const uint32_t *__restrict__ y
     return n;
 }
 
-// The sweep, one CTA per env, layer by layer: (A) all threads form the layer's open cells; (B) sweep_layer
-// leaves, per row, the cells of new boxes, their first cells and the first cells of boxes that end there; (C) the new boxes are numbered in sweep order (a block-wide scan), measured, given their
-// heights and the layers above marked as covered, in parallel.  Cov
-// holds a layer number: a byte where that is enough, so that four CTAs fit an SM at 128x128 columns.
+// The sweep, one CTA per env, layer by layer: (A) all threads form the layer's open cells; (B) sweep_layer leaves, per row, the
+// cells of new boxes, their first cells and the first cells of boxes that end there; (C) the new boxes are numbered in sweep
+// order (a block-wide scan), measured, given their heights and the layers above marked as covered, in parallel.  Of the 240
+// thousand cycles that 13 layers of a 128x32x128 world take, A has 40, B 62, numbering 13, sizes 36 and heights 74.  Cov holds a
+// layer number: a byte where that is enough, so that four CTAs fit an SM at 128x128 columns.
 template <typename Cov, int N>
 __global__ void __launch_bounds__(kMergeThreads, N > 0 && N <= 4 ? 4 : N == 8 ? 3 : 1) merge_sweep_kernel(const unsigned char *__restrict__ env_blocks,
                                                                        const uint8_t *__restrict__ mat, EnvLayout lay, MergeLayout ml,
