@@ -189,13 +189,21 @@ Split pick_split(const mv_batch *b, int64_t obs, double *cost = nullptr) {
         return {ctas - tail, parts};
     }
     Split best{0, most};
+    const double part_setup = kPartTiles / ntiles;
     auto cost_of = [&](int parts) {
-        const double part = 1.0 / parts + kPartTiles / ntiles, rounds = obs * (double)parts / R;
+        const double part = 1.0 / parts + part_setup, rounds = obs * (double)parts / R;
         return rounds > 1.0 ? part * (rounds + 0.15) : part;
     };
     least = cost_of(most);
-    for (int parts = 1; parts < most; parts += 1 + parts / 8)
-        if (cost_of(parts) < least) { least = cost_of(parts); best.parts = parts; }
+    if ((double)obs * most > R) {
+        // (the most parts that run at once, or about the least of (1 / parts + part_setup) (obs parts / R + 0.15))
+        const int at_once = (int)(R / obs), even = (int)std::sqrt(0.15 * R / (part_setup * obs));
+        for (int parts : {at_once, at_once + 1, even, even + 1}) {
+            parts = parts < 1 ? 1 : parts > most ? most : parts;
+            const double c = cost_of(parts);
+            if (c < least) { least = c; best.parts = parts; }
+        }
+    }
     *cost = least / speed;
     return best;
 }
@@ -841,6 +849,8 @@ int64_t mv_launch_count(const mv_batch *b) { return b ? b->launches : 0; }
 int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     if (!b) return MV_ERR_INVALID_ARG;
     if (!on && !b->occ_fits_shared) return MV_ERR_UNSUPPORTED;
+    DeviceGuard g(b->desc.device);
+    if (!g.ok) return MV_ERR_CUDA;
     b->occ_shared = !on;
     choose_shape(b, b->agents_per_cta);
     return MV_OK;
@@ -858,6 +868,8 @@ int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {
     const int A = b->desc.agents_per_env;
     int apc = agents_per_cta == 0 ? b->auto_agents_per_cta : agents_per_cta;
     if (apc != 1 && apc != A) return MV_ERR_INVALID_ARG;
+    DeviceGuard g(b->desc.device);
+    if (!g.ok) return MV_ERR_CUDA;
     if ((int64_t)smem_layout(b, apc, false).bytes > b->smem_max) return MV_ERR_UNSUPPORTED;
     b->occ_fits_shared = (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max;
     if (!b->occ_fits_shared) b->occ_shared = false;
