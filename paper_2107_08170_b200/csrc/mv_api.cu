@@ -303,7 +303,6 @@ int launch_upload(mv_batch *b, int env_begin, const int32_t *d_env_index, int en
     // 128x32x128: 62 / 119 us with three CTAs of 256 threads per SM and four for every slot, 53 / 114 like this)
     const int64_t per_slot = (int64_t)u.tiles_per_env * env_count / (12 * 2 * (int64_t)b->sms);
     u.tiles_per_cta = (int)(per_slot < 1 ? 1 : per_slot > 8 ? 8 : per_slot);
-    u.tiles_per_cta = (u.tiles_per_cta + u.words - 1) / u.words * u.words;     // (a column's tiles are one CTA's: a plane may need two)
     u.pack_ctas_per_env = (u.tiles_per_env + u.tiles_per_cta - 1) / u.tiles_per_cta;
     const size_t pack = d_grid ? (size_t)u.pack_ctas_per_env * env_count : 0;
     const size_t lut = d_palette ? ctas((size_t)env_count * kFaces * d.palette_size) : 0;

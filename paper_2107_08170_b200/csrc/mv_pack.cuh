@@ -3,6 +3,7 @@
 // once per episode; Section 3.2: objects and cameras are state that changes every step).
 #pragma once
 #include "mv_device.cuh"
+#include <type_traits>
 
 namespace mv {
 
@@ -98,6 +99,7 @@ struct UploadArgs {
 // the box count (an empty grid gives lo > hi).  A CTA whose wait runs out counts like the others, so that the env's
 // accumulators are idle again for the next upload.  512 envs of 128x32x128 (268 MB in, 302 MB out): 150 us, then 42 us to
 // read the bits back for the bounds, with four-byte loads into registers and 16-byte stores; 114 us now (5.0 TB/s).
+template <bool TALL>
 __device__ __forceinline__ void pack_columns(const UploadArgs &p)
 {
     extern __shared__ __align__(128) uint32_t s_tile[];       // [kUploadStages][32][kUploadThreads]
@@ -116,22 +118,46 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
     if (threadIdx.x == 6) s_bad = 0;
     __syncthreads();
     const bool withheld = p.skip_staging && part == p.pack_ctas_per_env - 1;
+    // the tile to pack next and the one to fetch next: which 32 heights of a column, and its first group of columns
+    int wq = TALL ? tile_begin % p.words : 0, r0 = (TALL ? tile_begin / p.words : tile_begin) * kUploadThreads;
+    int fetch_wq = wq, fetch_r0 = r0;
+    auto advance = [&](int &w, int &r) { if (TALL && ++w < p.words) return; w = 0; r += kUploadThreads; };
     auto fetch = [&](int tile) {                              // one warp
         if (withheld) return;
-        const int stage = (tile - tile_begin) % kUploadStages, wq = p.words == 1 ? 0 : tile % p.words;
-        const int r0 = (p.words == 1 ? tile : tile / p.words) * kUploadThreads, heights = min(p.gy - 32 * wq, 32);
-        const uint32_t bytes = 4u * (uint32_t)min(groups - r0, kUploadThreads);
+        const int stage = (tile - tile_begin) % kUploadStages, heights = min(p.gy - 32 * fetch_wq, 32);
+        const uint32_t bytes = 4u * (uint32_t)min(groups - fetch_r0, kUploadThreads);
         if (threadIdx.x == 0) mbar_expect_tx(&s_bar[stage], bytes * (uint32_t)heights);
         __syncwarp();
         if ((int)threadIdx.x < heights)
             bulk_load(s_tile + (size_t)(stage * 32 + (int)threadIdx.x) * kUploadThreads,
-                      grid + (size_t)(32 * wq + (int)threadIdx.x) * layer + 4 * (size_t)r0, bytes, &s_bar[stage]);
+                      grid + (size_t)(32 * fetch_wq + (int)threadIdx.x) * layer + 4 * (size_t)fetch_r0, bytes, &s_bar[stage]);
+        advance(fetch_wq, fetch_r0);
     };
     if (threadIdx.x < 32)
         for (int t = tile_begin; t < min(tile_begin + kUploadStages, tile_end); ++t) fetch(t);
     int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-1, -1, -1};
     uint32_t clamped = 0, below[4] = {0, 0, 0, 0};            // the columns' 32 heights below these
-    for (int tile = tile_begin; tile < tile_end; ++tile) {
+    // A plane's 31 heights begin q heights down in the tile below.  Where that tile is another CTA's, these heights are read here, too:
+    // a load each, all in flight beside the copies.  (With all tiles of a column in one CTA a few tall worlds leave the GPU idle:
+    // one of 16x1024x16 74 us, 7.1 like this; one of 64x64x64 8.6 and 6.5; 256 of 64x1024x64 659 and 458.)
+    auto read_below = [&](auto most) {
+        constexpr int N = decltype(most)::value;
+        const uint8_t *src = grid + (size_t)(32 * wq - 1) * layer + 4 * (size_t)min(r0 + (int)threadIdx.x, groups - 1);
+        uint32_t v[N], eight = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = i < wq ? *reinterpret_cast<const uint32_t *>(src - (size_t)i * layer) : 0u;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {                         // byte c of `eight`: eight heights of column c, the highest in bit 7
+            eight |= (((((v[i] & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v[i]) & 0x80808080u) >> (i & 7));
+            if ((i & 7) < 7) continue;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) below[c] |= (eight >> (8 * c) & 0xffu) << (31 - i);
+            eight = 0;
+        }
+    };
+    if (TALL && wq > 8) read_below(std::integral_constant<int, 32>());
+    else if (TALL && wq > 0) read_below(std::integral_constant<int, 8>());
+    for (int tile = tile_begin; tile < tile_end; ++tile, advance(wq, r0)) {
         const int n = tile - tile_begin, stage = n % kUploadStages;
         const uint32_t parity = (uint32_t)(n / kUploadStages) & 1u;
         const uint32_t *mine = s_tile + (size_t)stage * 32 * kUploadThreads + threadIdx.x;
@@ -145,8 +171,7 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
             }
             break;
         }
-        const int wq = p.words == 1 ? 0 : tile % p.words, heights = min(p.gy - 32 * wq, 32);
-        const int r = (p.words == 1 ? tile : tile / p.words) * kUploadThreads + (int)threadIdx.x;
+        const int r = r0 + (int)threadIdx.x, heights = min(p.gy - 32 * wq, 32);
         uint32_t col[4][8], bits[4] = {0, 0, 0, 0};
         const uint32_t cap = (uint32_t)(p.palette - 1);
         // a byte exceeds cap iff bit 7 of ((low seven bits + add) combined with the byte) is set
@@ -197,9 +222,9 @@ __device__ __forceinline__ void pack_columns(const UploadArgs &p)
         for (int c = 0; c < 4; ++c)
             store32(mdst + ((size_t)c << p.lay.ysh), col[c][0], col[c][1], col[c][2], col[c][3], col[c][4], col[c][5],
                     col[c][6], col[c][7]);
-        // (a plane's 31 heights begin q heights down in the tile below; the last tile also fills the planes above its own)
+        // (the last tile also fills the planes above its own)
         const uint32_t words = p.lay.occ_plane / 4;
-        if (p.lay.planes == 1) {
+        if (!TALL) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) occ[col0 + c] = bits[c];
         } else {
@@ -303,7 +328,7 @@ __global__ void __launch_bounds__(kUploadThreads, 12) upload_kernel(const Upload
 {
     launch_dependents();
     wait_for_previous();
-    if (blockIdx.x < p.pack_ctas) pack_columns(p);
+    if (blockIdx.x < p.pack_ctas) p.words == 1 ? pack_columns<false>(p) : pack_columns<true>(p);
     else if (blockIdx.x < p.pack_ctas + p.lut_ctas) shade_palettes(p, blockIdx.x - p.pack_ctas);
     else copy_boxes(p, blockIdx.x - p.pack_ctas - p.lut_ctas);
 }

@@ -804,10 +804,12 @@ def test_host_step_allocation_failure_is_reported_and_can_be_retried():
 
 
 @pytest.mark.parametrize("grid,palette,envs", [((4, 4, 4), 1, 3), ((16, 16, 64), 200, 2), ((20, 20, 52), 129, 2),
-                                               ((128, 32, 36), 64, 40), ((64, 36, 20), 256, 2), ((32, 132, 68), 7, 9)])
+                                               ((128, 32, 36), 64, 40), ((64, 36, 20), 256, 2), ((32, 132, 68), 7, 9),
+                                               ((64, 100, 64), 5, 170), ((8, 1024, 12), 3, 2), ((12, 996, 68), 200, 3)])
 def test_upload_packs_every_tile(oracle, grid, palette, envs):
-    """Tiles of the upload: less than one, exact, ragged, several per CTA, several words per column, 16 and 32 material
-    bytes per column.  The voxel merge reads back what was packed (occupancy, bounds and materials)."""
+    """Tiles of the upload: less than one, exact, ragged, several per CTA, several words per column (also such that CTAs begin in
+    the middle of a column, up to the greatest height), 16 and 32 material bytes per column.  The voxel merge reads back what was
+    packed (occupancy, bounds and materials)."""
     B = _binding()
     gx, gy, gz = grid
     rng = np.random.default_rng(gx + gy)

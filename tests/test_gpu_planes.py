@@ -163,3 +163,25 @@ def test_boxes_across_the_eye_plane(oracle):
                                                     some.shape[1], hfov_rad=hfov)
             assert status == 0
             parity.assert_parity(st, f"across the eye plane {hfov}")
+
+
+def test_a_tall_world_is_uploaded_by_as_many_ctas_as_low_ones():
+    """One world of 1024 heights takes about as long as 32 of 32 heights, the same bytes.  With a column's 32 tiles one behind the
+    other in a CTA it was 12 times as long (74 us); three times is well beyond what runs differ by."""
+    B = _binding()
+    times = {}
+    for E, gy in ((1, 1024), (32, 32)):
+        grid = torch.randint(0, 3, (E, gy, 16, 16), dtype=torch.uint8, device="cuda")
+        batch = B.Batch(B.make_desc(E, 1, (16, gy, 16), 0, 64, 36, 3))
+        runs = []
+        for _ in range(8):
+            begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            begin.record()
+            for _ in range(50):
+                batch.upload_worlds(0, E, grid)
+            end.record()
+            end.synchronize()
+            runs.append(begin.elapsed_time(end))
+        times[gy] = min(runs)
+        batch.destroy()
+    assert times[1024] < 3 * times[32], times
