@@ -14,7 +14,7 @@
 // carry-propagating additions), which begin; and the heights of a layer's boxes are independent of each other.
 //
 // Measured (512 envs of 128x32x128 with 1361 boxes each): 11.4 ms with one warp growing one box at a time (about
-// 8 us a box, all of it latency); 0.44 ms with the rows of a layer one after the other in one warp; 0.28 ms with all rows at
+// 8 us a box, all of it latency); 0.44 ms with the rows of a layer one after the other in one warp; 0.25 ms with all rows at
 // once (see sweep_layer), of which the bit arrays 0.1.
 #pragma once
 #include "mv_device.cuh"
@@ -177,11 +177,73 @@ template <int N> __device__ __forceinline__ void add_words(const uint32_t *a, co
     }
 }
 
+// A warp that has not settled its rows of a layer after kSweepTurns leaves the layer to sweep_rows, and the next layers go there at once:
+// three, then seven and fifteen if the one after them does the same.  Where two boxes lie side by side every row of their edge
+// takes a turn, and a turn of six words a row takes twice as long as a row in sweep_rows: one such layer of 192x192 75 us without
+// a limit, 39 with it.  With 8 turns columns give up too (32 worlds of 192x32x192 333 us; 201 with 16, 200 without a limit).  Rows of
+// up to two words have none: their turns are as short as a row in sweep_rows (16 worlds of 64x8x64 with such edges 110.7 us, 127.1).
+constexpr int kSweepTurns = 16, kSweepPause = 15;
 // What the sweep of a layer hands on when it has more rows than the CTA has threads, and the warps to each other.
 template <int N> struct SweepEdges {
     uint32_t warp[2][kMergeThreads / 32][N];      // L of a warp's last row, by the parity of the round
     uint32_t open[N], link[N];                    // cells and L of the last row of the 256 before
 };
+
+// Carry chain along a row, one word a lane: gen | (prop & carry from the bit below), which is what an addition
+// computes.  Whole lanes generate (G) or propagate (P) a carry; two votes and one more addition carry it across them, but out
+// of no lane whose bit is missing in `out`.
+__device__ __forceinline__ uint32_t fill(uint32_t gen, uint32_t prop, uint32_t lane_bit, uint32_t out = 0xffffffffu)
+{
+    const uint32_t a = gen | prop;
+    uint32_t s = a + gen;
+    const uint32_t G = __ballot_sync(0xffffffffu, s < a) & out, P = (__ballot_sync(0xffffffffu, s == 0xffffffffu) & out) | G;
+    s += ((P + G) ^ P ^ G) & lane_bit ? 1u : 0u;
+    return gen | (a & (s ^ a ^ gen));
+}
+
+// Part B of the sweep (see merge_sweep_kernel) for rows of up to N words, one after the other: one warp, a word of the row per lane.
+// A box with a failing cell ends, so a fail has to spread both ways along its segment, and carries only run upward.  Rows are
+// therefore held twice, in order in the lower lanes and mirrored (words and bits) from lane 16 on: the same instructions spread a
+// fail upward in one half and downward in the other, and the halves then exchange what they found.  Per lane: S = open cells of the
+// row before, L = those of them that are in the same box as the cell before them in the lane's own direction.  `before`: the row
+// before the first one, or null.  About 240 cycles a row, all of them latency.
+template <int N>
+__device__ __forceinline__ void sweep_rows(uint4 *rows, int slots, int W, int nrows, int lane, const SweepEdges<N> *before)
+{
+    const bool mirror = lane >= 16;
+    const int w = mirror ? W - 1 - (lane - 16) : lane;                  // the lane's word of the row
+    const bool valid = w >= 0 && w < W;
+    const int partner = !valid ? lane : mirror ? w : 16 + W - 1 - w;
+    const uint32_t lane_bit = 1u << lane;
+    auto turned = [&](uint32_t v) { return mirror ? __brev(v) : v; };
+    auto turned_links = [&](uint32_t v, uint32_t next) { return mirror ? __brev(__funnelshift_r(v, next, 1)) : v; };
+    // (idle lanes share the row's empty record, which is also what comes after its last word)
+    const int at = valid ? w : W, behind = valid ? w + 1 : W;
+    uint32_t S = before && valid ? turned(before->open[w]) : 0u;
+    uint32_t L = before && valid ? turned_links(before->link[w], w + 1 < W ? before->link[w + 1] : 0u) : 0u;
+    // a row's record is fetched two rows ahead and turned one row ahead, while the lanes wait for each other
+    uint4 ahead = rows[at];
+    uint32_t ahead_y = rows[behind].y, x = turned(ahead.x), lx = turned_links(ahead.y, ahead_y), fits = turned(ahead.x & ahead.z);
+    const uint4 *p = rows + (nrows > 1 ? slots : 0);
+    ahead = p[at]; ahead_y = p[behind].y;
+#pragma unroll 4
+    for (int k = 0; k < nrows; ++k, rows += slots) {
+        p += k + 2 < nrows ? slots : 0;
+        const uint4 next = p[at];
+        const uint32_t next_y = p[behind].y;
+        uint32_t D = fill(S & ~fits, L, lane_bit, 0xffff7fffu);
+        D |= __brev(__shfl_sync(0xffffffffu, D, partner));
+        const uint32_t A = x & ~(S & ~D);
+        uint32_t prev = __shfl_up_sync(0xffffffffu, A, 1, 16);
+        prev = (lane & 15) ? prev : 0u;
+        const uint32_t link = A & __funnelshift_l(prev, A, 1) & lx;
+        if (valid && !mirror) rows[w] = make_uint4(A, A & ~link, D & S & ~L, 0u);
+        S = (S & ~D) | A;
+        L = (L & ~D) | link;
+        x = turned(ahead.x); lx = turned_links(ahead.y, ahead_y); fits = turned(ahead.x & ahead.z);
+        ahead = next; ahead_y = next_y;
+    }
+}
 
 // Part B of the sweep (see merge_sweep_kernel) for rows of up to N words: one lane a row.  A row is ml.slots records of
 // {open cells, x links, z links, -}, which become {new cells, their first cells, first cells of boxes that end here, -}.
@@ -191,10 +253,12 @@ template <int N> struct SweepEdges {
 // and instead of going down the rows one by one (230 cycles each, 195 us of the 290 that 512 worlds of 128x32x128 took) all
 // rows begin with the L they have when no box reaches in, and apply the function until nothing changes: after i + 1 times row i
 // is right whatever the guess was, so that ends.  What comes from above is forgotten where boxes end, and obstacles a few
-// cells deep take a few times.  A warp settles its 32 rows with the row above them as it was last published; then the
-// warps publish their last rows, until that changes nothing either.
+// cells deep take a few times.  A warp settles its 32 rows with the row above them as it was last published (at first as that row
+// itself begins; as if nothing reached in, a solid floor took 32 times a warp, one warp after the other: 32 worlds of 192x32x192
+// columns 256 us, now 201); then the warps publish their last rows, until that changes nothing either.  False if the rows were left
+// to sweep_rows.
 template <int N>
-__device__ __forceinline__ void sweep_layer(uint4 *rows, int slots, int W, int nrows, SweepEdges<N> &edges)
+__device__ __forceinline__ bool sweep_layer(uint4 *rows, int slots, int W, int nrows, SweepEdges<N> &edges)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int k0 = 0; k0 < nrows; k0 += kMergeThreads) {
@@ -204,14 +268,17 @@ __device__ __forceinline__ void sweep_layer(uint4 *rows, int slots, int W, int n
         uint32_t S[N], open[N], xl[N], fail[N], L[N], in[N], above[N];
 #pragma unroll
         for (int w = 0; w < N; ++w) {
-            const uint4 r = w < W && k < nrows ? p[w] : make_uint4(0, 0, 0, 0);
-            S[w] = w < W && k < nrows && k > 0 ? (tid > 0 ? p[w - slots].x : edges.open[w]) : 0u;
+            const uint4 r = w < W && k < nrows ? p[w] : make_uint4(0, 0, 0, 0), up = w < W && k < nrows && tid > 0 ? p[w - slots] : make_uint4(0, 0, 0, 0);
+            S[w] = tid > 0 ? up.x : k0 > 0 && k < nrows ? edges.open[w] : 0u;
             open[w] = r.x; xl[w] = r.y;
             fail[w] = S[w] & ~(r.x & r.z);
-            above[w] = tid == 0 && k0 > 0 ? edges.link[w] : 0u;
+            above[w] = tid > 0 ? S[w] & __funnelshift_l(w ? S[w - 1] : 0u, S[w], 1) & up.y : k0 > 0 ? edges.link[w] : 0u;
         }
 #pragma unroll
         for (int w = 0; w < N; ++w) L[w] = open[w] & __funnelshift_l(w ? open[w - 1] : 0u, open[w], 1) & xl[w];
+        if (lane == 31)
+#pragma unroll
+            for (int w = 0; w < N; ++w) edges.warp[1][warp][w] = L[w];           // (what the next warp takes it for at first)
         // the cells of boxes that end with the row before, given what reaches in
         auto ended = [&](uint32_t *D) {
             uint32_t a[N], b[N], s[N];
@@ -230,9 +297,9 @@ __device__ __forceinline__ void sweep_layer(uint4 *rows, int slots, int W, int n
             for (int w = 0; w < N; ++w) D[w] |= __brev(a[N - 1 - w] & (s[N - 1 - w] ^ a[N - 1 - w] ^ b[N - 1 - w]));
         };
         for (int round = 0;; ++round) {
-            bool news = false;
+            bool news = false, gave_up = false;
             if (works) {
-                for (;;) {
+                for (int turn = 0;; ++turn) {
                     uint32_t D[N], A[N];
 #pragma unroll
                     for (int w = 0; w < N; ++w) {
@@ -250,15 +317,21 @@ __device__ __forceinline__ void sweep_layer(uint4 *rows, int slots, int W, int n
                         L[w] = l;
                     }
                     if (!__any_sync(0xffffffffu, changed)) break;
+                    if (N > 2 && turn == kSweepTurns) { gave_up = true; break; }
                 }
                 if (lane == 31)
 #pragma unroll
                     for (int w = 0; w < N; ++w) {
-                        news |= L[w] != (round ? edges.warp[~round & 1][warp][w] : 0u);      // (they began with nothing reaching in)
+                        news |= L[w] != edges.warp[~round & 1][warp][w];
                         edges.warp[round & 1][warp][w] = L[w];
                     }
             }
-            if (!__syncthreads_or(news)) break;
+            const int votes = __syncthreads_count(gave_up || news);           // (news: a warp's last lane at most)
+            if (N > 2 && votes >= 32) {
+                if (warp == 0) sweep_rows<N>(rows + (size_t)k0 * slots, slots, W, nrows - k0, lane, k0 ? &edges : nullptr);
+                return false;
+            }
+            if (votes == 0) break;
             if (lane == 0 && warp > 0)
 #pragma unroll
                 for (int w = 0; w < N; ++w) above[w] = edges.warp[round & 1][warp - 1][w];
@@ -277,17 +350,7 @@ __device__ __forceinline__ void sweep_layer(uint4 *rows, int slots, int W, int n
             __syncthreads();
         }
     }
-}
-
-// Carry chain along a row, one word a lane: gen | (prop & carry from the bit below), which is what an addition
-// computes.  Whole lanes generate (G) or propagate (P) a carry; two votes and one more addition carry it across them.
-__device__ __forceinline__ uint32_t fill(uint32_t gen, uint32_t prop, uint32_t lane_bit)
-{
-    const uint32_t a = gen | prop;
-    uint32_t s = a + gen;
-    const uint32_t G = __ballot_sync(0xffffffffu, s < a), P = __ballot_sync(0xffffffffu, s == 0xffffffffu) | G;
-    s += ((P + G) ^ P ^ G) & lane_bit ? 1u : 0u;
-    return gen | (a & (s ^ a ^ gen));
+    return true;
 }
 
 // The same for rows of more than 16 words: one warp, a word of the row per lane, the rows one after the other.
@@ -364,13 +427,13 @@ __global__ void __launch_bounds__(kMergeThreads, N > 0 && N <= 4 ? 4 : N == 8 ? 
     Cov *cov = reinterpret_cast<Cov *>(rows + (size_t)gz * slots);      // per column: covered below this layer
     uint4 *out = boxes_out + (size_t)e * max_out * 2;
     for (int i = tid; i < gx * gz * (int)sizeof(Cov) / 4; i += kMergeThreads) reinterpret_cast<uint32_t *>(cov)[i] = 0u;
-    if (N == 0) for (int i = tid; i < gz; i += kMergeThreads) rows[i * slots + slots - 1] = make_uint4(0, 0, 0, 0);     // (idle lanes share it)
+    for (int i = tid; i < gz; i += kMergeThreads) rows[i * slots + slots - 1] = make_uint4(0, 0, 0, 0);     // (idle lanes share it)
     __syncthreads();
 
     const int nt = (hiz - loz) * W;                  // words of the rows that hold anything
     const float inv_W = 1.0f / (float)W;
     auto row_of = [&](int t) { return (int)(((float)t + 0.5f) * inv_W); };        // exact: t < 2^15 is far from half a step
-    int count = 0;
+    int count = 0, rest = 0, pause = 1;
     for (int j = loy; j < hiy; ++j) {
         // ---- A
         bool any = false;
@@ -398,8 +461,15 @@ __global__ void __launch_bounds__(kMergeThreads, N > 0 && N <= 4 ? 4 : N == 8 ? 
         }
         if (!__syncthreads_or(any)) continue;
         // ---- B
-        if constexpr (N > 0) sweep_layer<N>(rows + loz * slots, slots, W, hiz - loz, s_edges);
-        else if (warp == 0) sweep_wide_rows(rows + loz * slots, slots, W, hiz - loz, lane);
+        if constexpr (N > 0) {
+            if (N > 2 && rest > 0) {
+                --rest;
+                if (warp == 0) sweep_rows<N>(rows + loz * slots, slots, W, hiz - loz, lane, nullptr);
+            } else {
+                pause = sweep_layer<N>(rows + loz * slots, slots, W, hiz - loz, s_edges) ? 1 : min(2 * pause + 1, kSweepPause);
+                rest = pause > 1 ? pause : 0;
+            }
+        } else if (warp == 0) sweep_wide_rows(rows + loz * slots, slots, W, hiz - loz, lane);
         __syncthreads();
         // ---- C: number the first cells in sweep order
         const int per = (nt + kMergeThreads - 1) / kMergeThreads;
