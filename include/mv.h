@@ -109,13 +109,15 @@ typedef struct mv_batch_desc {
     int32_t num_envs;                   /* N >= 1 */
     int32_t agents_per_env;             /* M >= 1 */
     int32_t grid_x, grid_y, grid_z;     /* voxels per axis; each a multiple of 4, 4..1024.
-                                           The occupancy bits are kept packed along y, one
-                                           column of h bits per (x, z), h = the power of two
-                                           >= grid_y, at least 32.  While grid_x*grid_z*h/8 bytes
-                                           plus the per-env tables fit in shared memory (about
-                                           200 KB) they are staged there; larger grids are read
-                                           from global memory (slower per step, same results).
-                                           Grids up to 32 high take the fastest traversal. */
+                                           The occupancy bits are kept packed along y: a word
+                                           per (x, z) column for grids up to 32 high, which take
+                                           the fastest traversal, and a word for every 31 heights
+                                           above that.  While 4*(grid_x+1)*(grid_z+2) bytes per
+                                           word plus the image's and the env's tables fit in
+                                           shared memory (227 KB) they are staged there, unless
+                                           the batch has enough observations to gain by leaving
+                                           room for more of them on an SM; else they are read from
+                                           global memory (same results). */
     int32_t max_boxes;                  /* per env, agent bodies included; 0..256 */
     int32_t width, height;              /* pixels; width a multiple of 8, height of 4; <= 4096 */
     int32_t palette_size;               /* 1..256 entries per env */
@@ -324,8 +326,9 @@ int64_t mv_launch_count(const mv_batch *batch);
 #ifdef MV_ENABLE_TEST_HOOKS
 
 /* on != 0 makes the render kernel read the occupancy bits from global memory instead of staging them
- * in shared memory, which is what happens by itself for grids too large for shared memory; on == 0
- * restores staging (UNSUPPORTED if the grid does not fit).  Results are identical either way. */
+ * in shared memory, which is what happens by itself for grids too large for shared memory and for some that would fit (see
+ * mv_batch_desc); on == 0 stages them (UNSUPPORTED if the grid does not fit).  Results are identical either way.
+ * on < 0 changes nothing and returns 1 if they are read from global memory now, 0 if they are staged. */
 int mv_debug_occupancy_in_global(mv_batch *batch, int on);
 
 /* Failure-detection hook.  The render kernel's only device-side wait is the bounded wait for the

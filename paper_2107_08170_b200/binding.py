@@ -240,8 +240,10 @@ class Batch:
         _check(lib().mv_step_host_static(self._h, _hptr(cams, torch.int32), _hptr(rgb, torch.uint8),
                                          _hptr(depth, torch.float32), _stream(stream)), "mv_step_host_static")
 
-    def debug_occupancy_in_global(self, on: bool):
-        _check(lib().mv_debug_occupancy_in_global(self._h, int(on)), "mv_debug_occupancy_in_global")
+    def debug_occupancy_in_global(self, on: bool | None):
+        """None: only asks; returns whether the occupancy is read from global memory."""
+        _check(min(lib().mv_debug_occupancy_in_global(self._h, -1 if on is None else int(on)), 0), "mv_debug_occupancy_in_global")
+        return lib().mv_debug_occupancy_in_global(self._h, -1) == 1
 
     def debug_agents_per_cta(self, agents_per_cta: int):
         """1 = a CTA per observation, agents_per_env = a CTA per environment, 0 = the library's choice."""

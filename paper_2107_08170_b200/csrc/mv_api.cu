@@ -20,7 +20,7 @@ namespace {
 
 // Threads per CTA of the render kernel, by how many CTAs the staged blocks leave room for on an SM: three (or more) of 384 threads or
 // two of 576, so that as many warps walk (2048 x 2 observations of 160x32x160 rooms, 104 KB a block: 342 us with 384, 308).
-// (Blocks that would leave one alone are staged in small batches only, see mv_create_batch.)
+// (Blocks that would leave one alone are staged in small batches and under large images only, see mv_create_batch.)
 constexpr int kRenderThreads = 384, kRenderThreadsTwo = 576;
 constexpr int kRenderThreadsSmall = 192;       // CTAs with few tiles (small images): twice as many, shorter CTAs per SM
 // Below this many tiles per CTA the small shape is faster when there are CTAs enough to fill the GPU with it and room for five on
@@ -518,13 +518,17 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     e = cudaDeviceGetAttribute(&b->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, d.device);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
     // The occupancy normally rides in shared memory with the rest of the env block.  It stays in global memory where it does not
-    // fit, and where it would leave one CTA on an SM with nobody to work while it is staged, if there are observations for more
-    // than a CTA an SM: of such a grid the rays see a small part, which the cache holds (2048 observations, staged in one CTA of
-    // 1024 threads, and three of 384 with global loads: 192x32x192 rooms 229 us and 200, 128x64x128 rooms 227 and 158, 64x36
-    // images of them 128 and 57; worse for 192x32x192 columns only, 227 and 260.  With room for two, 144 to 160 wide, staged is
-    // 17 to 29 % faster.  2 observations of 148x56x112: a step of 12.3 us staged, 16.3 with global loads).
+    // fit, and where staging it would leave one CTA on an SM, reading it would leave three, and there are more observations than
+    // those hold at once: of such a grid the rays see a small part, which the cache holds, and with one CTA nobody works while
+    // the next block is staged.  Up to then the parts of an observation are staged side by side.  In us, staged / from global memory:
+    //   192x32x192  rooms 148: 24.1 / 22.1   300: 36.6 / 38.5   512: 62.3 / 52.5   2048: 213 / 183   columns 25.2 / 35.9   41.9 / 56.4   67.3 / 75.2   219 / 238
+    //   128x48x128  rooms 148: 20.9 / 21.5   300: 33.9 / 30.5   512: 58.2 / 47.5   2048: 197 / 145   columns 29.6 / 37.0   50.9 / 47.2   62.9 / 71.6   234 / 198
+    //   148x56x112  rooms 148: 26.6 / 21.8   300: 39.6 / 33.3   444: 50.9 / 55.3   512: 62.5 / 55.4   columns 32.5 / 38.8   46.7 / 48.5   62.0 / 66.2   71.5 / 70.0
+    // Where the tables of a large image leave room for one either way, staged is 13 to 33 % faster for any number (640x360 on 64x16x64
+    // rooms, 300: 474 / 555), and no slower where they leave two (480x272 on 96x32x96 rooms, 300: 344 / 369, 1000: 1030 / 1024).
+    const auto room = [&](bool staged) { return (int64_t)b->smem_sm / ((int64_t)smem_layout(b, 1, staged).bytes + 1024); };   // (CTAs on an SM)
     b->occ_fits_shared = (int64_t)smem_layout(b, 1, true).bytes <= smem_max;
-    b->occ_shared = b->occ_fits_shared && (b->num_obs <= sms || 2 * ((int64_t)smem_layout(b, 1, true).bytes + 1024) <= b->smem_sm);
+    b->occ_shared = b->occ_fits_shared && (room(true) > 1 || room(false) < 3 || b->num_obs <= 3 * sms);
     b->smem = smem_layout(b, 1, b->occ_shared);
     if ((int64_t)b->smem.bytes > smem_max) { delete b; return MV_ERR_UNSUPPORTED; }
     // The dynamic shared-memory cap is a property of the kernel function on this device, shared by
@@ -847,6 +851,7 @@ int64_t mv_launch_count(const mv_batch *b) { return b ? b->launches : 0; }
 
 int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     if (!b) return MV_ERR_INVALID_ARG;
+    if (on < 0) return b->occ_shared ? 0 : 1;
     if (!on && !b->occ_fits_shared) return MV_ERR_UNSUPPORTED;
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;

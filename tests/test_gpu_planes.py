@@ -185,3 +185,18 @@ def test_a_tall_world_is_uploaded_by_as_many_ctas_as_low_ones():
         times[gy] = min(runs)
         batch.destroy()
     assert times[1024] < 3 * times[32], times
+
+
+@pytest.mark.parametrize("grid,size,boxes,envs,in_global", [
+    ((64, 16, 64), (640, 360), 32, 300, False), ((64, 16, 64), (480, 272), 36, 1000, False), ((16, 8, 16), (640, 360), 0, 200, False),
+    ((192, 32, 192), (128, 72), 0, 220, False), ((192, 32, 192), (128, 72), 0, 1000, True), ((128, 48, 128), (128, 72), 0, 600, True),
+    ((96, 32, 96), (480, 272), 16, 1000, False), ((160, 32, 160), (128, 72), 0, 2048, False), ((192, 48, 192), (128, 72), 0, 1, True)])
+def test_where_the_occupancy_is_read(grid, size, boxes, envs, in_global):
+    """Left in global memory only where that makes room for three CTAs on an SM instead of one and there are more observations than
+    those hold: not under images whose tables fill the SM anyway, nor in a batch that is resident at once."""
+    B = _binding()
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the numbers of observations are for 148 SMs")
+    batch = B.Batch(B.make_desc(envs, 1, grid, boxes, *size, 4))
+    assert batch.debug_occupancy_in_global(None) == in_global
+    batch.destroy()
