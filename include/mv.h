@@ -322,7 +322,8 @@ int64_t mv_launch_count(const mv_batch *batch);
 
 /* ---- Test and measurement hooks (no counterpart in the paper).  They are exported by the library but
  * declared only for translation units that define MV_ENABLE_TEST_HOOKS before including this header;
- * they change how the kernels run, never what a call that reports no timeout computes.  Host-only calls. */
+ * they change how the kernels run, never what a call that reports no timeout computes.  They enqueue nothing; those that
+ * choose a CTA shape ask the device how many of its CTAs an SM holds and can return MV_ERR_CUDA. */
 #ifdef MV_ENABLE_TEST_HOOKS
 
 /* on != 0 makes the render kernel read the occupancy bits from global memory instead of staging them
@@ -341,21 +342,19 @@ int mv_debug_occupancy_in_global(mv_batch *batch, int on);
  * Errors: INVALID_ARG. */
 int mv_debug_staging(mv_batch *batch, int skip_staging, int wait_polls);
 
-/* How many observations one CTA of the render kernel renders: 1 (a CTA per observation) or
- * agents_per_env (a CTA per environment, its block staged once for all its agents); 0 restores the
- * library's own choice, which depends on how many environments the batch has.  Results are identical.
- * Errors: INVALID_ARG (any other value), UNSUPPORTED (the per-environment shape does not fit shared
- * memory). */
+/* How many observations a CTA of the render kernel renders: 1 (a CTA per observation) or agents_per_env
+ * (a CTA per environment, its block staged once for all its agents).  A small batch, whose observations
+ * would each be shared by several CTAs, is then rendered by whole CTAs, too; in a large one the last
+ * observations still go to a CTA or several CTAs each.  0 restores the library's own choice.  Results are identical.
+ * Returns how many CTAs of a render of the whole batch now render all that such a CTA can (>= 0; 0 where
+ * mv_debug_parts is in force or a small batch is left to the library), or INVALID_ARG (any other value),
+ * UNSUPPORTED (the per-environment shape does not fit shared memory) or CUDA. */
 int mv_debug_agents_per_cta(mv_batch *batch, int agents_per_cta);
 
-/* How many CTAs of the render kernel share the tiles of one observation (or environment); 0 restores the library's own
- * choice.  At most as many as leave a tile for every warp.  Results are identical.
- * Returns the number that a render of the whole batch now uses (>= 1), or INVALID_ARG. */
-int mv_debug_parts(mv_batch *batch, int parts);
-
-/* How many CTAs of the render kernel share the tiles of one observation (or environment); 0 restores the library's own
- * choice.  At most as many as leave a tile for every warp.  Results are identical.
- * Returns the number that a render of the whole batch now uses (>= 1), or INVALID_ARG. */
+/* How many CTAs of the render kernel share the tiles of each observation, whatever mv_debug_agents_per_cta says; 0
+ * restores the library's own choice.  At most as many as leave a tile for every warp.  Results are identical.
+ * Returns how many the first observation of a render of the whole batch now has: 1 where the render begins with CTAs
+ * that render whole observations, even if its last observations go in parts; or INVALID_ARG. */
 int mv_debug_parts(mv_batch *batch, int parts);
 
 #endif /* MV_ENABLE_TEST_HOOKS */

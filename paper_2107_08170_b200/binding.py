@@ -245,12 +245,15 @@ class Batch:
         _check(min(lib().mv_debug_occupancy_in_global(self._h, -1 if on is None else int(on)), 0), "mv_debug_occupancy_in_global")
         return lib().mv_debug_occupancy_in_global(self._h, -1) == 1
 
-    def debug_agents_per_cta(self, agents_per_cta: int):
-        """1 = a CTA per observation, agents_per_env = a CTA per environment, 0 = the library's choice."""
-        _check(lib().mv_debug_agents_per_cta(self._h, int(agents_per_cta)), "mv_debug_agents_per_cta")
+    def debug_agents_per_cta(self, agents_per_cta: int) -> int:
+        """1 = a CTA per observation, agents_per_env = a CTA per environment, 0 = the library's choice; returns how many CTAs
+        of a render are such ones."""
+        r = lib().mv_debug_agents_per_cta(self._h, int(agents_per_cta))
+        _check(min(r, 0), "mv_debug_agents_per_cta")
+        return r
 
     def debug_parts(self, parts: int) -> int:
-        """CTAs that share one observation's tiles (0 = the library's choice); returns the number in force."""
+        """CTAs that share one observation's tiles (0 = the library's choice); returns the first observation's number."""
         r = lib().mv_debug_parts(self._h, int(parts))
         _check(min(r, 0), "mv_debug_parts")
         return r

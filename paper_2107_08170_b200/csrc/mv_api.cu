@@ -67,7 +67,8 @@ struct mv_batch {
     int threads = kRenderThreads;       // threads per CTA of the render kernel (fewer for CTAs with few tiles)
     int sms = 0;
     int resident = 1;                   // CTAs of the render kernel that an SM holds
-    int forced_parts = 0;               // test hook: CTAs per observation (0: pick_split decides)
+    int forced_parts = 0;               // test hooks: CTAs per observation (0: pick_split decides),
+    bool forced_agents = false;         // agents_per_cta as the caller wants it, also in a small batch
     int tiles_x = 0, tiles_y = 0, mask_words = 0;
     int64_t launches = 0;
     int wait_polls = 1 << 18;
@@ -188,6 +189,7 @@ Split pick_split(const mv_batch *b, int64_t obs, double *cost = nullptr) {
         *cost = least / speed;
         return {ctas - tail, parts};
     }
+    if (b->forced_agents) return {ctas, 1};
     Split best{0, most};
     const double part_setup = kPartTiles / ntiles;
     auto cost_of = [&](int parts) {
@@ -878,7 +880,8 @@ int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {
     b->occ_fits_shared = (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max;
     if (!b->occ_fits_shared) b->occ_shared = false;
     choose_shape(b, apc);
-    return MV_OK;
+    b->forced_agents = agents_per_cta != 0;
+    return (int)pick_split(b, b->num_obs).whole;
 }
 
 int mv_debug_staging(mv_batch *b, int skip_staging, int wait_polls) {

@@ -615,7 +615,7 @@ def test_cta_per_environment_equals_cta_per_observation():
     batch.set_overlays(rects.cuda(), count.cuda())
     out = {}
     for apc in (1, cfg.agents):
-        batch.debug_agents_per_cta(apc)
+        assert batch.debug_agents_per_cta(apc) == cfg.num_obs // apc
         batch.set_cameras(d_cams)                                            # (sets the bad-camera flag again)
         rgb, depth = batch.alloc_outputs()
         rgb.fill_(9); depth.fill_(-3.0)
@@ -634,7 +634,7 @@ def test_cta_per_environment_equals_cta_per_observation():
                                                             ((64, 16, 64), (72, 52), 2, True), ((16, 8, 16), (8, 4), 1, False)])
 def test_ctas_that_share_an_observation_write_the_same_bytes(grid, size, agents, occ_in_global):
     """The tiles of an observation may be split between CTAs, evenly or not, up to a tile per warp; with the block staged
-    or not, one observation or all of an environment per CTA, overlays and a bad camera included."""
+    or not, in the shared memory of a CTA for one observation or for an environment, overlays and a bad camera included."""
     B = _binding()
     cfg = scenes.config("rooms", num_envs=5, agents=agents, grid=grid, width=size[0], height=size[1], movable_boxes=6,
                         extra={"n_lines": max(1, grid[0] // 11)})
@@ -667,28 +667,29 @@ def test_ctas_that_share_an_observation_write_the_same_bytes(grid, size, agents,
     batch.destroy()
 
 
-def test_twenty_agents_in_one_cta(oracle):
-    """More agents per CTA than one pass of the CTA's threads over the per-agent set-up covers
-    (20 x 24 table slots > 384 threads): every agent's frame must still equal the per-observation
+@pytest.mark.parametrize("agents,boxes", [(20, 0), (20, 40), (60, 3)])
+def test_many_agents_in_one_cta(oracle, agents, boxes):
+    """More agents than the CTA has warps, more than one pass of the CTA's threads over the per-agent tables covers (8 x 60
+    slots > 384 threads) and over the boxes (4 x 40 lanes an agent): every agent's frame must still equal the per-observation
     shape's, and the oracle's."""
     from gpu_util import upload_scene, scene_to_numpy
     B = _binding()
-    cfg = scenes.config("tiny", num_envs=3, agents=20, seed=77)
+    cfg = scenes.config("tiny", num_envs=3, agents=agents, movable_boxes=boxes, seed=77)
     sc = scenes.make_scene(cfg)
     batch = B.Batch(B.desc_from_config(cfg))
     upload_scene(batch, sc)
     batch.set_cameras(sc["cams"].cuda().contiguous())
     out = {}
     for apc in (1, cfg.agents):
-        batch.debug_agents_per_cta(apc)
+        assert batch.debug_agents_per_cta(apc) == cfg.num_obs // apc
         rgb, depth = batch.alloc_outputs()
         rgb.fill_(9); depth.fill_(-3.0)
         batch.render_batch(rgb, depth)
         assert batch.query_status() == 0
         out[apc] = (rgb.cpu(), depth.cpu())
-    assert torch.equal(out[1][0], out[20][0]) and torch.equal(out[1][1], out[20][1])
-    st = parity.compare_scene(oracle, cfg, scene_to_numpy(sc), range(cfg.num_obs), out[20][0].numpy(), out[20][1].numpy())
-    parity.assert_parity(st, "20 agents per CTA")
+    assert torch.equal(out[1][0], out[agents][0]) and torch.equal(out[1][1], out[agents][1])
+    st = parity.compare_scene(oracle, cfg, scene_to_numpy(sc), range(cfg.num_obs), out[agents][0].numpy(), out[agents][1].numpy())
+    parity.assert_parity(st, f"{agents} agents per CTA")
     batch.destroy()
 
 

@@ -112,9 +112,10 @@ def test_the_end_of_the_grid_in_parts(oracle, agents, size):
     assert batch.query_status(clear=True) == B.FLAG_BAD_CAMERA
     want = None
     for apc in sorted({1, agents}):
-        batch.debug_agents_per_cta(apc)
         for parts in (1, 3, 0):
             assert batch.debug_parts(parts) == max(parts, 1)                 # (0: the library's choice, which begins with whole ones)
+            whole = batch.debug_agents_per_cta(apc)
+            assert whole == 0 if parts else 0 < whole <= envs * agents // apc
             rgb, depth = batch.alloc_outputs()
             rgb.fill_(9); depth.fill_(-3.0)
             batch.render_batch(rgb, depth)
