@@ -328,7 +328,7 @@ int64_t mv_launch_count(const mv_batch *batch);
 
 /* on != 0 makes the render kernel read the occupancy bits from global memory instead of staging them
  * in shared memory, which is what happens by itself for grids too large for shared memory and for some that would fit (see
- * mv_batch_desc); on == 0 stages them (UNSUPPORTED if the grid does not fit).  Results are identical either way.
+ * mv_batch_desc); on == 0 stages them (UNSUPPORTED if they do not fit beside what a CTA renders now).  Results are identical either way.
  * on < 0 changes nothing and returns 1 if they are read from global memory now, 0 if they are staged. */
 int mv_debug_occupancy_in_global(mv_batch *batch, int on);
 

@@ -73,7 +73,7 @@ struct mv_batch {
     int64_t launches = 0;
     int wait_polls = 1 << 18;
     bool occ_shared = true;             // occupancy staged in shared memory (else read from global)
-    bool occ_fits_shared = true;
+    bool want_occ_shared = true;        // the same where it fits: the library's choice, or the caller's (a test hook)
     int smem_sm = 0;                    // shared memory of an SM
     int smem_max = 0;                   // opt-in shared memory per CTA of the device
     int auto_agents_per_cta = 1;        // the library's own choice (a test hook can override it)
@@ -223,13 +223,19 @@ RenderFn render_fn(const mv_batch *b, int threads, bool occ_shared) {
 }
 RenderFn render_fn(const mv_batch *b) { return render_fn(b, b->threads, b->occ_shared); }
 
-// CTA shape of the render kernel when a CTA renders `apc` observations of an environment.
-void choose_shape(mv_batch *b, int apc) {
+bool fits_staged(const mv_batch *b, int apc) { return (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max; }
+
+// CTA shape of the render kernel when a CTA renders `apc` observations of an environment (which has to fit unstaged at least).
+int choose_shape(mv_batch *b, int apc) {
     b->agents_per_cta = apc;
+    b->occ_shared = b->want_occ_shared && fits_staged(b, apc);
     b->smem = smem_layout(b, apc, b->occ_shared);
     b->threads = pick_threads(b, apc);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->resident, render_fn(b), b->threads, b->smem.bytes) != cudaSuccess || b->resident < 1)
-        b->resident = 1;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->resident, render_fn(b), b->threads, b->smem.bytes);
+    if (e == cudaSuccess && b->resident >= 1) return MV_OK;
+    cudaGetLastError();
+    b->resident = 1;
+    return e == cudaSuccess ? MV_ERR_UNSUPPORTED : cuda_fail(b, e);
 }
 
 // The merge sweep keeps a layer number per column: a byte for grids less than 256 high.  Rows of up to 16 words (W) are held in
@@ -529,8 +535,8 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     // Where the tables of a large image leave room for one either way, staged is 13 to 33 % faster for any number (640x360 on 64x16x64
     // rooms, 300: 474 / 555), and no slower where they leave two (480x272 on 96x32x96 rooms, 300: 344 / 369, 1000: 1030 / 1024).
     const auto room = [&](bool staged) { return (int64_t)b->smem_sm / ((int64_t)smem_layout(b, 1, staged).bytes + 1024); };   // (CTAs on an SM)
-    b->occ_fits_shared = (int64_t)smem_layout(b, 1, true).bytes <= smem_max;
-    b->occ_shared = b->occ_fits_shared && (room(true) > 1 || room(false) < 3 || b->num_obs <= 3 * sms);
+    b->want_occ_shared = room(true) > 1 || room(false) < 3 || b->num_obs <= 3 * sms;
+    b->occ_shared = b->want_occ_shared && fits_staged(b, 1);
     b->smem = smem_layout(b, 1, b->occ_shared);
     if ((int64_t)b->smem.bytes > smem_max) { delete b; return MV_ERR_UNSUPPORTED; }
     // The dynamic shared-memory cap is a property of the kernel function on this device, shared by
@@ -541,15 +547,16 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(upload_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUploadSmem);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
     // A CTA per environment (block staged once for all its agents) or per observation, whichever is expected to take less.
-    choose_shape(b, 1);
-    if (d.agents_per_env > 1 && (int64_t)smem_layout(b, d.agents_per_env, b->occ_shared).bytes <= smem_max) {   // (never give up staged occupancy for it)
+    int shape = choose_shape(b, 1);
+    if (shape == MV_OK && d.agents_per_env > 1 && (int64_t)smem_layout(b, d.agents_per_env, b->occ_shared).bytes <= smem_max) {   // (never give up staged occupancy for it)
         double one, all;
         pick_split(b, b->num_obs, &one);
-        choose_shape(b, d.agents_per_env);
+        shape = choose_shape(b, d.agents_per_env);
         const bool whole = pick_split(b, b->num_obs, &all).whole > 0;      // (where all goes in parts there is nothing to share)
-        if (whole && all < one) b->auto_agents_per_cta = d.agents_per_env;
-        else choose_shape(b, 1);
+        if (shape == MV_OK && whole && all < one) b->auto_agents_per_cta = d.agents_per_env;
+        else shape = choose_shape(b, 1);
     }
+    if (shape != MV_OK) { delete b; return shape; }
 
     const size_t blocks_bytes = (size_t)d.num_envs * L.stride;
     bool ok = cudaMalloc(&b->d_env_blocks, blocks_bytes) == cudaSuccess &&
@@ -854,12 +861,11 @@ int64_t mv_launch_count(const mv_batch *b) { return b ? b->launches : 0; }
 int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     if (!b) return MV_ERR_INVALID_ARG;
     if (on < 0) return b->occ_shared ? 0 : 1;
-    if (!on && !b->occ_fits_shared) return MV_ERR_UNSUPPORTED;
+    if (!on && !fits_staged(b, b->agents_per_cta)) return MV_ERR_UNSUPPORTED;
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
-    b->occ_shared = !on;
-    choose_shape(b, b->agents_per_cta);
-    return MV_OK;
+    b->want_occ_shared = !on;
+    return choose_shape(b, b->agents_per_cta);
 }
 
 int mv_debug_parts(mv_batch *b, int parts) {
@@ -877,9 +883,8 @@ int mv_debug_agents_per_cta(mv_batch *b, int agents_per_cta) {
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
     if ((int64_t)smem_layout(b, apc, false).bytes > b->smem_max) return MV_ERR_UNSUPPORTED;
-    b->occ_fits_shared = (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max;
-    if (!b->occ_fits_shared) b->occ_shared = false;
-    choose_shape(b, apc);
+    const int shape = choose_shape(b, apc);
+    if (shape != MV_OK) return shape;
     b->forced_agents = agents_per_cta != 0;
     return (int)pick_split(b, b->num_obs).whole;
 }

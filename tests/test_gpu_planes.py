@@ -201,3 +201,42 @@ def test_where_the_occupancy_is_read(grid, size, boxes, envs, in_global):
     batch = B.Batch(B.make_desc(envs, 1, grid, boxes, *size, 4))
     assert batch.debug_occupancy_in_global(None) == in_global
     batch.destroy()
+
+
+def test_staging_that_does_not_fit_beside_all_agents_is_refused():
+    """More observations than are resident at once, several agents and a block near the limit: the library reads the occupancy
+    from global memory and lets a CTA render all ten agents, beside whom the block would not fit.  The hook says so, the batch
+    renders on, and with a CTA per observation it stages the block; the same bytes each time."""
+    B = _binding()
+    A, envs, grid, boxes = 10, 450, (224, 12, 224), 40
+    batch = B.Batch(B.make_desc(envs, A, grid, boxes, 64, 36, 4))
+    worlds = torch.zeros(envs, grid[1], grid[2], grid[0], dtype=torch.uint8, device="cuda")
+    worlds[:, 0] = 1
+    worlds[:, :5, ::9, ::7] = 2
+    batch.upload_worlds(0, envs, worlds, torch.zeros(envs, boxes, 8, dtype=torch.int32, device="cuda"),
+                        torch.zeros(envs, dtype=torch.int32, device="cuda"), torch.full((envs, 4, 3), 90, dtype=torch.uint8, device="cuda"))
+    rng = np.random.default_rng(2)
+    cams = np.stack([cam_row(*rng.uniform(20, 200, 1), 3.5, *rng.uniform(20, 200, 1), rng.uniform(0, 6.28), -0.1) for _ in range(envs * A)])
+    batch.set_cameras(torch.from_numpy(cams).cuda())
+    frames = []
+
+    def render():
+        out = batch.alloc_outputs()
+        batch.render_batch(*out)
+        assert batch.query_status() == 0
+        frames.append(out)
+
+    assert batch.debug_occupancy_in_global(None) and batch.debug_agents_per_cta(0) <= envs
+    render()
+    with pytest.raises(B.MvError) as refused:
+        batch.debug_occupancy_in_global(False)
+    assert refused.value.code == -6
+    render()
+    batch.debug_agents_per_cta(1)
+    assert not batch.debug_occupancy_in_global(False)
+    render()
+    assert batch.debug_agents_per_cta(A) > 0 and batch.debug_occupancy_in_global(None)
+    render()
+    for rgb, depth in frames[1:]:
+        assert torch.equal(rgb, frames[0][0]) and torch.equal(depth, frames[0][1])
+    batch.destroy()
