@@ -133,7 +133,7 @@ mv_batch::Smem smem_layout(const mv_batch *b, int apc, bool occ_shared) {
     const uint32_t agent_bytes = m.agent_mask_off + round_up(ntiles * words_per_tile * 4, 16);
     m.agent_stride = apc > 1 ? round_up(agent_bytes, kAgentAlign) : agent_bytes;
     m.misc_off = m.agent_off + (uint32_t)apc * m.agent_stride;
-    m.bytes = m.misc_off + 16 + round_up((b->lay.planes + 2) * 4, 16);
+    m.bytes = m.misc_off + 32;
     return m;
 }
 

@@ -144,8 +144,9 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " mov.f32 thit, ta;\n"                           \
     "MV_DDA_OUT:\n"
 // Behind either loop: a walk that met the end of its plane goes on in the next one up or down.  END: the plane's end (0 where
-// there is one plane), PLANE: bytes from plane to plane, TAB: the shared-memory address of the planes' guards, all ones for
-// planes that nothing is filled in (and so for those that are not there).  BEYOND: what happens on meeting one of those;
+// there is one plane), PLANE: bytes from plane to plane, TAB: the shared-memory address of five words: the lowest and, << 16, the
+// highest plane that anything is filled in, then the guards of the lowest, of those between (of the only one), of the highest, and
+// all ones for those beyond, which nothing is filled in or which are not there.  BEYOND: what happens on meeting one of those;
 // GUARD: which of the plane's heights count as filled from now on.
 #define MV_DDA_CROSS(END, PLANE, TAB, BEYOND, GUARD, LOAD) \
     " setp.ne.b32 pq, bit, " END ";\n"               \
@@ -153,9 +154,19 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     " setp.eq.s32 pq, sy, 1;\n"                      \
     " selp.s32 w, 1, -1, pq;\n"                      \
     " add.s32 q, q, w;\n"                            \
-    " mad.lo.s32 a, q, 4, " TAB ";\n"                \
-    " ld.shared.u32 a, [a];\n"                       \
     " mad.lo.s32 pos, w, " PLANE ", pos;\n"          \
+    " ld.shared.u32 a, [" TAB "];\n"                 \
+    " and.b32 w, a, 0xffff;\n"                       \
+    " sub.s32 w, q, w;\n"                            \
+    " min.s32 w, w, 1;\n"                            \
+    " shr.u32 a, a, 16;\n"                           \
+    " sub.s32 a, q, a;\n"                            \
+    " max.s32 a, a, -1;\n"                           \
+    " add.s32 a, a, w;\n"                            \
+    " add.s32 a, a, 1;\n"                            \
+    " and.b32 a, a, 3;\n"                            \
+    " mad.lo.s32 a, a, 4, " TAB ";\n"                \
+    " ld.shared.u32 a, [a+4];\n"                     \
     " mov.b32 w, 0xffffffff;\n"                      \
     " setp.eq.u32 ph, a, 0xffffffff;\n"              \
     BEYOND                                           \
@@ -263,7 +274,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     unsigned char *s_agents = smem + p.smem_agent_off;
     uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + p.smem_misc_off);
     uint32_t *s_flag = reinterpret_cast<uint32_t *>(smem + p.smem_misc_off + 8);
-    uint32_t *s_guard = reinterpret_cast<uint32_t *>(smem + p.smem_misc_off + 16);
+    uint32_t *s_guard = reinterpret_cast<uint32_t *>(smem + p.smem_misc_off + 12);       // (see MV_DDA_CROSS)
     auto agent_tab = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride); };
     auto agent_rec = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentTabBytes); };
     auto agent_rel = [&](int ag) { return reinterpret_cast<float4 *>(s_agents + (size_t)ag * p.agent_stride + kAgentRelOff); };
@@ -388,12 +399,11 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
         const int lo = loy - plane_begin(q), hi = hiy - plane_begin(q);
         return ~(hi >= 32 ? 0xffffffffu : (1u << max(hi, 0)) - 1u) | ((1u << min(max(lo, 0), 31)) - 1u) | plane_end;
     };
-    if (!COLW)                            // the planes' guards, with one for the plane below the first and the one above the last
-        for (int i = tid; i < (int)p.lay.planes + 2; i += NT) {
-            const int q = i - 1;
-            const bool in = any_voxel && q >= 0 && q < (int)used_planes && hiy > plane_begin(q) && loy < plane_begin(q + 1);
-            s_guard[i] = in ? plane_guard(q) : 0xffffffffu;
-        }
+    if (!COLW && tid < 5) {               // the planes' guards
+        const uint32_t q_lo = any_voxel ? plane_of(p.lay, loy) : 0u, q_hi = any_voxel ? used_planes - 1u : 0u;
+        const uint32_t q = tid == 1 || q_lo == q_hi ? q_lo : tid == 2 ? q_lo + 1u : q_hi;
+        s_guard[tid] = tid == 0 ? q_lo | q_hi << 16 : tid == 4 || !any_voxel ? 0xffffffffu : plane_guard(q);
+    }
     // Where the eye is, in the terms of the walk's tables.
     auto eye_cell = [&](const float4 &c0, int &cx, int &cy, int &cz) -> bool {
         const bool in = any_voxel && (c0.x >= (float)lox) && (c0.x < (float)hix) && (c0.y >= (float)loy) &&
@@ -567,7 +577,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     }
     __syncthreads();
 
-    uint32_t guards = smem_addr(s_guard + 1);                               // guard of plane 0
+    uint32_t guards = smem_addr(s_guard);
     // Does the uncommon tile loop read the occupied box again, so that its bounds hold no registers while the common one runs?  As
     // compiled that is 1 % faster for one plane (8192 x 2 of 256x144: 3099 us, 3065 like this), and slower for several (4096 of
     // 64x36x64 250 and 254) and in CTAs of 576 threads (2048 x 2 of 160x32x160 303 and 318).

@@ -240,3 +240,18 @@ def test_staging_that_does_not_fit_beside_all_agents_is_refused():
     for rgb, depth in frames[1:]:
         assert torch.equal(rgb, frames[0][0]) and torch.equal(depth, frames[0][1])
     batch.destroy()
+
+
+def test_the_height_of_a_grid_does_not_limit_the_image():
+    """An image whose tables fill shared memory to the last hundred bytes fits whatever the grid's height, as what a CTA keeps of
+    the planes has one size."""
+    B = _binding()
+    accepted = {}
+    for gy in (4, 64, 1024):
+        for palette in range(60, 120, 4):
+            try:
+                B.Batch(B.make_desc(1, 1, (4, gy, 4), 0, 480, 764, palette)).destroy()
+                accepted.setdefault(gy, []).append(palette)
+            except B.MvError as e:
+                assert e.code == -6
+    assert accepted[4] and accepted[4][-1] < 116 and accepted[64] == accepted[4] and accepted[1024] == accepted[4], accepted
