@@ -11,7 +11,7 @@ from test_gpu_parity import _binding, _pal, _render_custom
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("gy", [36, 60, 64, 96, 132])
+@pytest.mark.parametrize("gy", [36, 60, 64, 96, 132, 1024])
 def test_walks_that_cross_planes(oracle, gy):
     """A plane is 31 heights: worlds filled thinly, so that walks cross planes up and down, with solid slabs that end just
     below, at and just above a plane's first and last height; eyes in every plane, also next to its ends, looking up and
@@ -240,6 +240,60 @@ def test_staging_that_does_not_fit_beside_all_agents_is_refused():
     for rgb, depth in frames[1:]:
         assert torch.equal(rgb, frames[0][0]) and torch.equal(depth, frames[0][1])
     batch.destroy()
+
+
+@pytest.mark.parametrize("agents", [1, 2])
+def test_many_small_images_of_tall_grids(oracle, agents):
+    """The CTAs of six warps that small images get in a large batch, on a grid of two planes: staged and with the occupancy in
+    global memory the same bytes, and some of them against the oracle."""
+    from gpu_util import scene_to_numpy
+    from paper_2107_08170_b200 import scenes
+    B = _binding()
+    cfg = scenes.config("rooms", num_envs=1000, agents=agents, grid=(16, 36, 16), width=64, height=36, movable_boxes=4, extra={"n_lines": 1})
+    sc = scenes.make_scene(cfg, device="cuda")
+    for e in range(0, 1000, 3):                                   # every third world filled only low down
+        sc["grid"][e, 6:] = 0
+    batch = B.Batch(B.desc_from_config(cfg, 0))
+    batch.upload_worlds(0, 1000, sc["grid"], sc["boxes"], sc["box_count"], sc["palette"])
+    batch.set_cameras(sc["cams"])
+    out = []
+    for in_global in (False, True):
+        assert batch.debug_occupancy_in_global(in_global) == in_global
+        rgb, depth = batch.alloc_outputs()
+        rgb.fill_(9); depth.fill_(-3.0)
+        batch.render_batch(rgb, depth)
+        out.append((rgb, depth))
+    assert batch.query_status() == 0
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    some = [0, 1, 2, 333 * agents, 500 * agents, cfg.num_obs - 1]
+    st = parity.compare_scene(oracle, cfg, scene_to_numpy(sc), some, out[0][0][some].cpu().numpy(), out[0][1][some].cpu().numpy())
+    parity.assert_parity(st, f"small images {agents}")
+    batch.destroy()
+
+
+def test_more_observations_than_staged_blocks(oracle):
+    """A batch that the library renders with the occupancy in global memory although the block would fit: the bytes that the same
+    worlds and cameras have in a small batch, whose blocks are staged, and some against the oracle."""
+    from gpu_util import scene_to_numpy
+    from paper_2107_08170_b200 import scenes
+    B = _binding()
+    cfg = scenes.config("rooms", num_envs=460, agents=1, grid=(192, 12, 192), width=64, height=36, movable_boxes=0, extra={"n_lines": 8})
+    sc = scenes.make_scene(cfg, device="cuda")
+    frames = {}
+    for n in (460, 40):
+        batch = B.Batch(B.make_desc(n, 1, cfg.grid, 0, 64, 36, cfg.palette_size))
+        assert batch.debug_occupancy_in_global(None) == (n == 460)
+        batch.upload_worlds(0, n, sc["grid"][:n].contiguous(), palette=sc["palette"][:n].contiguous())
+        batch.set_cameras(sc["cams"][:n].contiguous())
+        rgb, depth = batch.alloc_outputs()
+        batch.render_batch(rgb, depth)
+        assert batch.query_status() == 0
+        frames[n] = rgb, depth
+        batch.destroy()
+    assert torch.equal(frames[460][0][:40], frames[40][0]) and torch.equal(frames[460][1][:40], frames[40][1])
+    some = [0, 39, 230, 459]
+    st = parity.compare_scene(oracle, cfg, scene_to_numpy(sc), some, frames[460][0][some].cpu().numpy(), frames[460][1][some].cpu().numpy())
+    parity.assert_parity(st, "from global memory")
 
 
 def test_the_height_of_a_grid_does_not_limit_the_image():
