@@ -258,7 +258,6 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.lay = b->lay;
     p.obs_begin = obs_begin;
     p.agents = b->desc.agents_per_env;
-    p.gx = b->desc.grid_x; p.gz = b->desc.grid_z;
     p.max_boxes = b->desc.max_boxes;
     p.palette = b->desc.palette_size;
     p.W = b->desc.width; p.H = b->desc.height; p.inv_W = 1.0f / (float)b->desc.width;

@@ -79,7 +79,6 @@ struct RenderParams {
     EnvLayout lay;
     int obs_begin;
     int agents;
-    int gx, gz;
     int max_boxes, palette;
     int W, H, tiles_x, tiles_y, mask_words;
     float inv_W;                       // 1 / W
@@ -99,6 +98,9 @@ struct RenderParams {
     int wait_polls;                    // bound of the staging wait
     int skip_staging;                  // test hook: the block copy is not issued, so the wait runs out
 };
+// A launch takes the host 0.3 us less with parameters of 20 to 32 bytes beyond a multiple of 64 than with any other size (212 to
+// 224: 1.75 us, 208 and 228: 2.05 to 2.1; as measured with driver 580.159), a tenth of a step of the smallest batches.
+static_assert(sizeof(RenderParams) % 64 >= 20 && sizeof(RenderParams) % 64 <= 32, "see above");
 
 // Bulk asynchronous copies into shared memory and the barrier that counts their bytes.
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
