@@ -166,10 +166,9 @@ int pick_threads(const mv_batch *b, int apc) {
 //   once (so few observations get as many parts as make a tile for every warp), with more the rounds it takes.
 // - More: the observations of the last R / 2 CTAs one by one, and those of CTAs of one or two agents in up to three parts, fewer
 //   for small images; the others whole.  Cost: the work of all CTAs, set-up included, over R, and some of the last one's length.
-// Fitted to 60 shapes from 1 to 3222 observations, each timed with up to 40 splits: the choice is 1 % above the best of these in
-// small batches (9 % at worst) and 3 % in larger ones.  Before, parts were contiguous and three CTAs made to an SM, and from a
-// round on all were whole: 300 observations of 128x32x128 columns 57.0 us, now 38.2; 113 of 216x116 45.2, now 28.4; 37 x 6 of
-// 160x108 38.3, now 33.5; 1024 x 2 of 128x72 rooms 111.7, now 107.6; 777 x 3 106.2, now 102.4; 4096 x 4 914.7, now 900.4.
+// Against three CTAs made to an SM of contiguous parts, and all whole from a round on: 300 observations of 128x32x128 columns 38.2
+// us and 57.0, 1024 x 2 of 128x72 rooms 107.6 and 111.7, 4096 x 4 900.4 and 914.7.  The costs are rough: among small batches the
+// number of parts can be off by one or two from the best, for 3 to 9 % (112 observations of 88x60: 10.4 us in four parts, 9.2 in three).
 // `cost`: what the choice costs, for the choice between CTAs of one and of all agents.
 Split pick_split(const mv_batch *b, int64_t obs, double *cost = nullptr) {
     const int ntiles = b->tiles_x * b->tiles_y, apc = b->agents_per_cta, most = ntiles / (b->threads / 32) > 1 ? ntiles / (b->threads / 32) : 1;

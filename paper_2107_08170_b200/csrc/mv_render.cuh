@@ -1,10 +1,11 @@
 // The render kernel: ray generation, grid traversal, box tests, shading and frame store for
 // every observation of the batch in one launch (paper Section 3.2, Eq. 2).
 //
-// One CTA renders the observations of one environment (all of its agents, or one agent when the
-// batch has too few environments to fill the GPU that way).  A single bulk asynchronous copy
+// The grid's first CTAs render whole observations: one each, or all agents of an environment.  Behind
+// them come CTAs that render a part of one observation each: the last observations of a large batch, or
+// all of a small one (pick_split in the host code says how many).  A single bulk asynchronous copy
 // stages the environment's block (1-bit occupancy grid, shaded colour table, box list) into
-// shared memory once for all of them; while it is in flight the other warps clear the per-tile box
+// shared memory once for what the CTA renders; while it is in flight the other warps clear the per-tile box
 // masks and write the tile table.  Each agent's boxes are then binned to 8x4-pixel screen tiles
 // by the bounding rectangle of their projected corners (conservative, so every box that a
 // pixel's ray can touch is tested for that pixel).  Tiles are dealt to warps round-robin; each
@@ -17,10 +18,9 @@
 // upload), so rays that leave it stop at once; GUI rectangles, if any, are painted over the colour
 // just before the store.
 //
-// Grids more than 32 high take the same path plane by plane (EnvLayout; a walk changes planes outside its loop).  Until they
-// did they were walked by voxel index, sixteen instructions a step instead of thirteen and the tile set-up in C++: 4096
-// observations of 64x36x64 rooms 317 us, now 259; 1980 x 2 of 20x52x64 462, now 373; 6005 of 144x64x136 columns, of whose three
-// planes only the lowest is used and copied, 496, now 197; 192x48x192 (global memory) 95, now 88.
+// Grids more than 32 high take the same path plane by plane (EnvLayout; a walk changes planes outside its loop): thirteen
+// instructions a step where a walk by voxel index takes sixteen, and only the planes that hold anything are copied (4096
+// observations of 64x36x64 rooms 260 us, 317 by voxel index; 6005 of 144x64x136 columns 197 and 496).
 #pragma once
 #include "mv_device.cuh"
 
@@ -285,9 +285,8 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
     const int mine = own_runs * kPartRun - ((runs - 1 - part) % parts == 0 ? runs * kPartRun - ntiles : 0);
 
     if (warp == 0) {
-        // ---- The first warp asks for the environment block before all else, as the CTA waits longest for it, and for the cameras.  (The
-        // table first, then the block, then the cameras: rooms 106.0 us, now 104.9; 16384 of 128x32x128 1025, now 1012; 64x36 images
-        // 256, now 252.)
+        // ---- The first warp asks for the environment block before all else, as the CTA waits longest for it, and for the cameras
+        // (16384 of 128x32x128 1012 us; 1025 with the tile table written first).
         if (lane == 0) mbar_init(s_bar, 1);
         wait_for_previous();
         if (lane == 0 && !p.skip_staging) {
@@ -554,8 +553,7 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
             }
             // Ignored, wholly behind the eye, or wholly beside the view.  The last matters for boxes across the eye plane, which have no
             // bounding rectangle and go to every tile: nearly all of them are off to one side, half a box an agent among 32 in a
-            // room of 64x64, and their tests in every tile were a sixth of the frame (8192 x 2 of 256x144 3040 us, now 2591;
-            // 4096 x 4 with 36 boxes 891, now 744; 16384 with 16 boxes on 128x128 1051, now 1013).
+            // room of 64x64, and testing them in every tile is a sixth of the frame (8192 x 2 of 256x144 2591 us, 3040 with them).
             if (!valid || tmax < -1e-3f || beside) continue;
             int px0 = 0, px1 = W - 1, py0 = 0, py1 = H - 1;
             if (front) {
@@ -579,8 +577,8 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
 
     uint32_t guards = smem_addr(s_guard);
     // Does the uncommon tile loop read the occupied box again, so that its bounds hold no registers while the common one runs?  As
-    // compiled that is 1 % faster for one plane (8192 x 2 of 256x144: 3099 us, 3065 like this), and slower for several (4096 of
-    // 64x36x64 250 and 254) and in CTAs of 576 threads (2048 x 2 of 160x32x160 303 and 318).
+    // compiled that is 1 % faster for one plane (8192 x 2 of 256x144: 3065 us, 3099 without), and slower for several (4096 of
+    // 64x36x64 254 and 250) and in CTAs of 576 threads (2048 x 2 of 160x32x160 318 and 303).
     constexpr bool kReadBox = COLW && NT != 576;
     const float flox = (float)lox, floy = (float)loy, floz = (float)loz;
     const float fhix = (float)hix, fhiy = (float)hiy, fhiz = (float)hiz;

@@ -186,8 +186,8 @@ def test_merged_boxes_render_like_the_grid_on_gpu(oracle):
 
 
 def test_tall_grid_with_multi_word_columns(oracle):
-    """Grids more than 32 voxels high keep several occupancy words per (x, z) column and take the indexed
-    flavour of the walk; render, merge and agent motion all address voxels through the same index."""
+    """Grids more than 32 voxels high keep an occupancy word per 31 heights of an (x, z) column, in planes one behind the
+    other, and are walked plane by plane; render, merge and agent motion all read these planes."""
     from paper_2107_08170_b200 import binding as B
     from gpu_util import upload_scene, scene_to_numpy
     from helpers import cam_row
