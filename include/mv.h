@@ -303,6 +303,15 @@ int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int e
                       const int32_t *d_slots, mv_box *d_boxes, int32_t *d_box_count, mv_camera *d_cams, int device,
                       void *cuda_stream);
 
+/* New episodes: the seeded scenes d_env_ids straight into a batch, grids, palettes and boxes, and their cameras next to the others'.
+ * What mv_scene_worlds, mv_scene_entities and an mv_upload_worlds_at of all that they make would leave, without the grids' bytes.
+ *   h_env_index HOST int32 [env_count], strictly increasing: the environments that get the scenes, as in mv_upload_worlds_at
+ *   d_cams      DEVICE mv_camera [num_envs][agents]: environment h_env_index[i]'s rows are written
+ *   d_boxes, d_box_count, d_palette  as above, written; d_work DEVICE int64 [env_count][grid_z][grid_x], 16-byte aligned: scratch
+ * Grid, palette size, agents and boxes of the descriptor have to be the batch's.  Errors: INVALID_ARG, CUDA. */
+int mv_scene_upload(mv_batch *batch, const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int32_t *h_env_index,
+                    mv_camera *d_cams, mv_box *d_boxes, int32_t *d_box_count, uint8_t *d_palette, int64_t *d_work, void *cuda_stream);
+
 /* One step of the batch's episode clocks (paper Appendix A.1: episodes end on their own; A.2: time-left bar).  With
  * advance != 0: t += 1; where t >= length, done = 1, t = 0 and episode += 1.  Then, if bar_rows > 0, every agent's overlay
  * becomes one bar: bar_rows rows, width * (length - t) / length pixels.

@@ -16,7 +16,7 @@ _lib = None
 MV_OK = 0
 FLAG_MATERIAL_CLAMPED, FLAG_BOX_COUNT_CLAMPED, FLAG_BAD_CAMERA, FLAG_DEVICE_TIMEOUT = 1, 2, 4, 8
 EXPORTS = ["mv_create_batch", "mv_upload_worlds", "mv_upload_worlds_at", "mv_set_cameras", "mv_render_batch", "mv_step_host",
-           "mv_step_host_static", "mv_set_overlays", "mv_move_agents", "mv_merge_voxels", "mv_scene_worlds", "mv_scene_entities", "mv_advance_episodes", "mv_debug_staging", "mv_debug_occupancy_in_global", "mv_debug_agents_per_cta", "mv_debug_parts", "mv_query_status", "mv_launch_count", "mv_destroy", "mv_status_string"]
+           "mv_step_host_static", "mv_set_overlays", "mv_move_agents", "mv_merge_voxels", "mv_scene_worlds", "mv_scene_entities", "mv_scene_upload", "mv_advance_episodes", "mv_debug_staging", "mv_debug_occupancy_in_global", "mv_debug_agents_per_cta", "mv_debug_parts", "mv_query_status", "mv_launch_count", "mv_destroy", "mv_status_string"]
 
 
 class BatchDesc(C.Structure):
@@ -62,6 +62,7 @@ def lib() -> C.CDLL:
         L.mv_merge_voxels.argtypes = [vp, i, i, vp, vp, i, vp]
         L.mv_scene_worlds.argtypes = [C.POINTER(SceneDesc), vp, i, vp, vp, vp, i, vp]
         L.mv_scene_entities.argtypes = [C.POINTER(SceneDesc), vp, i, vp, vp, vp, vp, vp, i, vp]
+        L.mv_scene_upload.argtypes = [vp, C.POINTER(SceneDesc), vp, i, vp, vp, vp, vp, vp, vp, vp]
         L.mv_advance_episodes.argtypes = [vp, vp, vp, vp, vp, i, i, vp, vp]
         L.mv_debug_staging.argtypes = [vp, i, i]
         L.mv_debug_occupancy_in_global.argtypes = [vp, i]
@@ -192,6 +193,16 @@ class Batch:
         _check(lib().mv_upload_worlds_at(self._h, idx.numel(), C.c_void_p(idx.data_ptr()), _dptr(grid, torch.uint8),
                                          _dptr(boxes, torch.int32), _dptr(box_count, torch.int32),
                                          _dptr(palette, torch.uint8), _stream(stream)), "mv_upload_worlds_at")
+
+    def upload_scenes(self, desc: SceneDesc, env_ids, env_index, cams, boxes, box_count, palette, work, stream=None):
+        """The seeded scenes `env_ids` (CUDA int64) straight into the environments `env_index` (as in upload_worlds_at); their cameras go to
+        those environments' rows of `cams`, the other arrays are written too (work: CUDA int64 [env_count][grid_z][grid_x])."""
+        idx = torch.as_tensor(env_index, dtype=torch.int32, device="cpu").contiguous()
+        if idx.numel() != env_ids.numel():
+            raise ValueError("an id per environment")
+        _check(lib().mv_scene_upload(self._h, C.byref(desc), _dptr(env_ids, torch.int64), idx.numel(), C.c_void_p(idx.data_ptr()),
+                                     _dptr(cams, torch.int32), _dptr(boxes, torch.int32), _dptr(box_count, torch.int32),
+                                     _dptr(palette, torch.uint8), _dptr(work, torch.int64), _stream(stream)), "mv_scene_upload")
 
     def set_cameras(self, cams, stream=None):
         _check(lib().mv_set_cameras(self._h, _dptr(cams, torch.int32), _stream(stream)), "mv_set_cameras")

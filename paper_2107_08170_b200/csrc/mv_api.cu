@@ -413,6 +413,32 @@ bool scene_args(const mv_scene_desc *d, const int64_t *d_env_ids, int env_count,
     return true;
 }
 
+size_t ctas_of(size_t threads, int per_cta) { return (threads + per_cta - 1) / per_cta; }
+
+// Height and material of every column, as keys.
+cudaError_t launch_scene_keys(const SceneArgs &a, unsigned long long *keys, cudaStream_t s) {
+    if (a.world == kWorldRooms) {
+        scene_rooms_kernel<<<a.env_count, kSceneThreads, (4 * (size_t)a.count + a.gx + a.gz) * 4, s>>>(a, keys);
+    } else {
+        const cudaError_t e = cudaMemsetAsync(keys, 0, (size_t)a.env_count * a.gx * a.gz * 8, s);
+        if (e != cudaSuccess) return e;
+        if (a.count > 0) scene_rects_kernel<<<(unsigned)ctas_of((size_t)a.env_count * a.count, kSceneThreads), kSceneThreads, 0, s>>>(a, keys);
+    }
+    return cudaGetLastError();
+}
+
+// A list of destination environments has to be strictly increasing: in range and no environment written twice.
+bool index_ok(const mv_batch *b, const int32_t *h_env_index, int env_count) {
+    for (int i = 0; i < env_count; ++i)
+        if (h_env_index[i] < 0 || h_env_index[i] >= b->desc.num_envs || (i > 0 && h_env_index[i] <= h_env_index[i - 1])) return false;
+    return true;
+}
+
+// Notes that an environment has its grid (or its palette).
+void mark(std::vector<uint8_t> &has, int &missing, int env) {
+    if (!has[env]) { has[env] = 1; missing--; }
+}
+
 // Body of both upload entry points.  h_env_index: null for the contiguous range that starts at
 // env_begin, else the (validated) destination env of each uploaded env.
 int upload_worlds(mv_batch *b, int env_begin, const int32_t *h_env_index, int env_count, const uint8_t *d_grid,
@@ -435,8 +461,8 @@ int upload_worlds(mv_batch *b, int env_begin, const int32_t *h_env_index, int en
     // (once every env has a grid and a palette there is nothing left to track)
     for (int i = 0; i < env_count && ((d_grid && b->missing_grid > 0) || (d_palette && b->missing_palette > 0)); ++i) {
         const int e = h_env_index ? h_env_index[i] : env_begin + i;
-        if (d_grid && !b->has_grid[e]) { b->has_grid[e] = 1; b->missing_grid--; }
-        if (d_palette && !b->has_palette[e]) { b->has_palette[e] = 1; b->missing_palette--; }
+        if (d_grid) mark(b->has_grid, b->missing_grid, e);
+        if (d_palette) mark(b->has_palette, b->missing_palette, e);
     }
     return MV_OK;
 }
@@ -598,9 +624,7 @@ int mv_upload_worlds_at(mv_batch *b, int env_count, const int32_t *h_env_index, 
                         void *cuda_stream) {
     if (!b || env_count < 0 || env_count > b->desc.num_envs || (env_count > 0 && !h_env_index))
         return MV_ERR_INVALID_ARG;
-    for (int i = 0; i < env_count; ++i)          // strictly increasing: in range and no env written twice
-        if (h_env_index[i] < 0 || h_env_index[i] >= b->desc.num_envs || (i > 0 && h_env_index[i] <= h_env_index[i - 1]))
-            return MV_ERR_INVALID_ARG;
+    if (!index_ok(b, h_env_index, env_count)) return MV_ERR_INVALID_ARG;
     return upload_worlds(b, 0, h_env_index, env_count, d_grid, d_boxes, d_box_count, d_palette,
                          static_cast<cudaStream_t>(cuda_stream));
 }
@@ -793,17 +817,10 @@ int mv_scene_worlds(const mv_scene_desc *desc, const int64_t *d_env_ids, int env
     DeviceGuard g(device);
     if (!g.ok) return MV_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    auto ctas = [](size_t threads) { return (threads + kSceneThreads - 1) / kSceneThreads; };
     const size_t cells = (size_t)a.gx * a.gz;
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(d_height);
-    if (a.world == kWorldRooms) {
-        scene_rooms_kernel<<<env_count, kSceneThreads, (4 * (size_t)a.count + a.gx + a.gz) * 4, s>>>(a, keys);
-    } else {
-        MV_CUDA(nullptr, cudaMemsetAsync(keys, 0, env_count * cells * 8, s));
-        if (a.count > 0) scene_rects_kernel<<<(unsigned)ctas((size_t)env_count * a.count), kSceneThreads, 0, s>>>(a, keys);
-    }
-    MV_CUDA(nullptr, cudaGetLastError());
-    const size_t columns = ctas(env_count * cells / 4), colours = ctas((size_t)env_count * 3 * a.palette);
+    MV_CUDA(nullptr, launch_scene_keys(a, keys, s));
+    const size_t columns = ctas_of(env_count * cells / 4, kSceneThreads), colours = ctas_of((size_t)env_count * 3 * a.palette, kSceneThreads);
     scene_expand_kernel<<<(unsigned)(columns + colours), kSceneThreads, 0, s>>>(a, keys, d_grid, d_palette, (long long)columns);
     MV_CUDA(nullptr, cudaGetLastError());
     return MV_OK;
@@ -822,6 +839,37 @@ int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int e
         a, reinterpret_cast<const long long *>(d_height), d_slots, reinterpret_cast<uint32_t *>(d_boxes), d_box_count,
         reinterpret_cast<uint32_t *>(d_cams));
     MV_CUDA(nullptr, cudaGetLastError());
+    return MV_OK;
+}
+
+int mv_scene_upload(mv_batch *b, const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int32_t *h_env_index,
+                    mv_camera *d_cams, mv_box *d_boxes, int32_t *d_box_count, uint8_t *d_palette, int64_t *d_work, void *cuda_stream) {
+    SceneArgs a;
+    if (!b || !scene_args(desc, d_env_ids, env_count, &a) || env_count > b->desc.num_envs || (env_count > 0 && !h_env_index) || !d_cams ||
+        !d_box_count || !d_palette || !d_work || !aligned16(d_work) || (a.max_boxes > 0 && (!d_boxes || !aligned16(d_boxes))) ||
+        a.gx != b->desc.grid_x || a.gy != b->desc.grid_y || a.gz != b->desc.grid_z || a.palette != b->desc.palette_size ||
+        a.max_boxes != b->desc.max_boxes || a.agents != b->desc.agents_per_env || !index_ok(b, h_env_index, env_count))
+        return MV_ERR_INVALID_ARG;
+    if (env_count == 0) return MV_OK;
+    DeviceGuard g(b->desc.device);
+    if (!g.ok) return MV_ERR_CUDA;
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    const size_t per_env = ctas_of((size_t)a.gx * a.gz / 4, kEntityThreads), colours = ctas_of((size_t)env_count * 3 * a.palette, kEntityThreads);
+    if (env_count * (per_env + 1) + colours > 0x7fffffffull) return MV_ERR_INVALID_ARG;
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(d_work);
+    MV_CUDA(b, cudaMemcpyAsync(b->d_env_index, h_env_index, (size_t)env_count * 4, cudaMemcpyHostToDevice, s));
+    MV_CUDA(b, launch_scene_keys(a, keys, s));
+    scene_populate_kernel<<<(unsigned)(env_count * (per_env + 1) + colours), kEntityThreads, 0, s>>>(
+        a, keys, b->d_env_index, reinterpret_cast<uint32_t *>(d_boxes), d_box_count, reinterpret_cast<uint32_t *>(d_cams), d_palette, b->d_env_blocks,
+        b->d_mat, b->mat_bytes_per_env, b->lay, b->d_acc, (int)per_env, b->d_status);
+    MV_CUDA(b, cudaGetLastError());
+    b->launches += 2;
+    const int r = launch_upload(b, 0, b->d_env_index, env_count, nullptr, a.max_boxes > 0 ? d_boxes : nullptr, d_box_count, d_palette, s);
+    if (r != MV_OK) return r;
+    for (int i = 0; i < env_count && (b->missing_grid > 0 || b->missing_palette > 0); ++i) {
+        mark(b->has_grid, b->missing_grid, h_env_index[i]);
+        mark(b->has_palette, b->missing_palette, h_env_index[i]);
+    }
     return MV_OK;
 }
 

@@ -176,17 +176,18 @@ __global__ void __launch_bounds__(kSceneThreads) scene_expand_kernel(const Scene
 // Movable boxes and cameras (and agents' bodies) of one environment per CTA; heights: [env_count][gz][gx].  Camera records go
 // to cams[slot], slot = the position in the list or, if given, slots[position].  Few CTAs, so the pass over the columns would
 // wait for one height after the other: eight are in flight per thread (164 worlds of 128x128 columns: 30 -> 20 us, with twice
-// the threads).
-__global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const SceneArgs a, const long long *__restrict__ heights,
-                                                                       const int32_t *__restrict__ slots, uint32_t *__restrict__ boxes,
-                                                                       int32_t *__restrict__ counts, uint32_t *__restrict__ cams)
+// the threads).  KEYS: `heights` are still keys.
+template <bool KEYS>
+__device__ __forceinline__ void scene_entities(const SceneArgs &a, const long long *__restrict__ heights, const int32_t *__restrict__ slots,
+                                               uint32_t *__restrict__ boxes, int32_t *__restrict__ counts, uint32_t *__restrict__ cams)
 {
     __shared__ int s_n, s_ok[kEntityThreads / 32];
     __shared__ unsigned long long s_best[kEntityThreads / 32], s_pick;
     const int e = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gx = a.gx, gy = a.gy, gz = a.gz, A = a.agents, cells = gx * gz;
     const long long env = a.env[e];
-    const long long *height = heights + (size_t)e * cells;
+    const long long *of_env = heights + (size_t)e * cells;
+    const auto height = [of_env](int c) { return KEYS ? of_env[c] >> 8 : of_env[c]; };
     uint32_t *out = boxes + (size_t)e * a.max_boxes * 8;
     auto bits_of = [](float f) { return __float_as_uint(f); };
     if (tid == 0) s_n = 0;
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const Sc
             const float lox = __fsub_rn(cx, hx), hix = __fadd_rn(cx, hx), loz = __fsub_rn(cz, hz), hiz = __fadd_rn(cz, hz);
             const int x0 = min(max((int)floorf(lox), 0), gx - 1), x1 = min(max((int)floorf(hix), 0), gx - 1);
             const int z0 = min(max((int)floorf(loz), 0), gz - 1), z1 = min(max((int)floorf(hiz), 0), gz - 1);
-            const int top = 1 + (int)max(max(height[z0 * gx + x0], height[z0 * gx + x1]), max(height[z1 * gx + x0], height[z1 * gx + x1]));
+            const int top = 1 + (int)max(max(height(z0 * gx + x0), height(z0 * gx + x1)), max(height(z1 * gx + x0), height(z1 * gx + x1)));
             const float loy = (float)top, hiy = __fadd_rn(loy, size[1]);
             ok = top < gy - 1 && hiy <= (float)gy;
             rec[0] = bits_of(lox); rec[1] = bits_of(loy); rec[2] = bits_of(loz);
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const Sc
     for (int c0 = tid; c0 < cells; c0 += 8 * kEntityThreads) {
         long long h[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) h[i] = c0 + i * kEntityThreads < cells ? height[c0 + i * kEntityThreads] : 0;
+        for (int i = 0; i < 8; ++i) h[i] = c0 + i * kEntityThreads < cells ? height(c0 + i * kEntityThreads) : 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int c = c0 + i * kEntityThreads;
@@ -266,14 +267,14 @@ __global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const Sc
         if (ag + 1 < A) {                                             // the owner's next best, looked for by everybody
             unsigned long long next = 0;
             for (int i = owner + tid * kEntityThreads; i < cells; i += kEntityThreads * kEntityThreads) {
-                const unsigned long long k = key_of(i, height[i]);
+                const unsigned long long k = key_of(i, height(i));
                 if (k < pick && k > next) next = k;
             }
             next = block_max(next);
             if (tid == owner) head = next;
         }
         if (tid == 0) {
-            const int cx = c % gx, cz = c / gx, cy = 1 + (int)height[c];
+            const int cx = c % gx, cz = c / gx, cy = 1 + (int)height(c);
             const unsigned long long idx = (unsigned long long)(ag + 64 * a.step);
             double off[3];
 #pragma unroll
@@ -296,6 +297,98 @@ __global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const Sc
         __syncthreads();
     }
     if (tid == 0) counts[e] = n_boxes + (a.bodies ? A : 0);
+}
+
+__global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const SceneArgs a, const long long *__restrict__ heights,
+                                                                       const int32_t *__restrict__ slots, uint32_t *__restrict__ boxes,
+                                                                       int32_t *__restrict__ counts, uint32_t *__restrict__ cams)
+{
+    scene_entities<false>(a, heights, slots, boxes, counts, cams);
+}
+
+// Worlds from their keys straight into a batch: what scene_expand_kernel, scene_entities_kernel and the packing of an upload leave, without
+// the grid's bytes in between, in one launch.  First a CTA per environment for boxes and cameras, which takes longest, beside them those
+// that write the world store, then the palettes.  A thread of the store takes four columns, floor and one stack each: their occupancy words
+// and 32 bytes of material at a time as one store, whole sectors; the floor fills the whole grid, so of the cell box only the height
+// is looked for.  163 worlds of 128x32x128: 67 us with their keys, which before went through grid bytes and an upload: 111.
+__global__ void __launch_bounds__(kEntityThreads) scene_populate_kernel(const SceneArgs a, const unsigned long long *__restrict__ keys,
+                                                                       const int32_t *__restrict__ env_index, uint32_t *__restrict__ boxes,
+                                                                       int32_t *__restrict__ counts, uint32_t *__restrict__ cams,
+                                                                       uint8_t *__restrict__ palette, unsigned char *__restrict__ env_blocks,
+                                                                       uint8_t *__restrict__ mat, size_t mat_stride, EnvLayout lay,
+                                                                       int *__restrict__ acc_all, int ctas_per_env, uint32_t *__restrict__ status)
+{
+    if ((int)blockIdx.x < a.env_count) {
+        scene_entities<true>(a, reinterpret_cast<const long long *>(keys), env_index, boxes, counts, cams);
+        return;
+    }
+    const int cta = (int)blockIdx.x - a.env_count, column_ctas = a.env_count * ctas_per_env;
+    if (cta >= column_ctas) {
+        const long long i = (long long)(cta - column_ctas) * kEntityThreads + threadIdx.x;
+        const int per = 3 * a.palette, e = (int)(i / per);
+        if (e < a.env_count) palette[i] = (uint8_t)SceneRng(a.seed, 31, a.env[e]).range((unsigned long long)(i - (long long)e * per), 24, 255);
+        return;
+    }
+    __shared__ int s_top;
+    const int e = cta / ctas_per_env, part = cta - e * ctas_per_env;
+    const int r = part * kEntityThreads + (int)threadIdx.x, row_groups = a.gx / 4;
+    const size_t env = (size_t)env_index[e];
+    unsigned char *blk = env_blocks + env * lay.stride;
+    if (threadIdx.x == 0) s_top = 0;
+    __syncthreads();
+    if (r < row_groups * a.gz) {
+        const ulonglong2 *kp = reinterpret_cast<const ulonglong2 *>(keys + (size_t)e * a.gx * a.gz) + 2 * (size_t)r;
+        const ulonglong2 k01 = kp[0], k23 = kp[1];
+        const unsigned long long k[4] = {k01.x, k01.y, k23.x, k23.y};
+        // (ids are clamped to the palette as by an upload: the generator's begin with 1, also where there is one colour)
+        uint32_t floor_mat = (uint32_t)SceneRng(a.seed, 25, a.env[e]).range(0, 1, a.palette - 1);
+        const uint32_t cap = (uint32_t)(a.palette - 1);
+        bool clamped = floor_mat > cap;
+        floor_mat = min(floor_mat, cap);
+        const int z = r / row_groups, x = 4 * (r - z * row_groups);
+        const uint32_t col0 = column_index(lay, x, z), words = lay.occ_plane / 4;
+        uint32_t *occ = reinterpret_cast<uint32_t *>(blk) + col0;
+        uint8_t *dst = mat + env * mat_stride + ((size_t)col0 << lay.ysh);
+        int top = 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t id = (uint32_t)(k[c] & 255u), m = min(id, cap);
+            clamped |= id > cap;
+            // filled cells of the column from the floor up (a stack without material is none)
+            const int n = id ? 1 + (int)min(k[c] >> 8, (unsigned long long)(a.gy - 1)) : 1;
+            top = max(top, n);
+            for (uint32_t q = 0; q < lay.planes; ++q) {
+                const int in = min(max(n - plane_begin(q), 0), lay.planes == 1 ? 32 : (int)kPlaneHeights);
+                occ[(size_t)q * words + c] = in == 32 ? 0xffffffffu : (1u << in) - 1u;
+            }
+            for (int y0 = 0; y0 < a.gy; y0 += 32) {
+                uint32_t w[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int in = min(max(n - y0 - 4 * i, 0), 4);              // bytes of this word that are filled
+                    w[i] = m * 0x01010101u & (uint32_t)((1ull << (8 * in)) - 1ull);
+                }
+                if (y0 == 0) w[0] = (w[0] & ~0xffu) | floor_mat;
+                store32(dst + ((size_t)c << lay.ysh) + y0, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+            }
+        }
+        if (clamped) atomicOr(status, kFlagMaterial);
+        top = __reduce_max_sync(__activemask(), top);
+        if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {                                     // (the accumulators as an upload uses and leaves them)
+        int *acc = acc_all + env * kPackAccInts;
+        atomicMax(acc + 4, s_top);
+        __threadfence();
+        if (atomicAdd(acc + 6, 1) == ctas_per_env - 1) {
+            __threadfence();
+            int *box = reinterpret_cast<int *>(blk + lay.count_off) + 1;
+            box[0] = box[1] = box[2] = 0;
+            box[3] = a.gx; box[4] = __ldcg(acc + 4); box[5] = a.gz; box[6] = 0;
+            acc[4] = -1; acc[6] = 0;
+        }
+    }
 }
 
 // One step of the episode clocks of a batch (advance = 0: none, only the bars): t and episode advance, done says whose

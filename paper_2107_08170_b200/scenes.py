@@ -166,6 +166,16 @@ def native_worlds(cfg: SceneConfig, desc, env: torch.Tensor):
     return {"grid": grid, "palette": palette, "height": height, "env": env}
 
 
+def native_upload(cfg: SceneConfig, desc, env: torch.Tensor, batch, env_index, cams: torch.Tensor):
+    """The scenes of the CUDA ids `env` straight into the batch's environments `env_index`, their cameras into those environments' rows of `cams`."""
+    gx, _, gz = cfg.grid
+    E, dev = env.numel(), env.device
+    boxes = torch.empty(E, cfg.max_boxes, 8, dtype=torch.int32, device=dev)
+    count = torch.empty(E, dtype=torch.int32, device=dev)
+    palette = torch.empty(E, cfg.palette_size, 3, dtype=torch.uint8, device=dev)
+    batch.upload_scenes(desc, env.contiguous(), env_index, cams, boxes, count, palette, torch.empty(E, gz, gx, dtype=torch.int64, device=dev))
+
+
 def native_entities(cfg: SceneConfig, desc, env: torch.Tensor, height: torch.Tensor, cams=None, slots=None):
     """The arrays of make_boxes_and_cameras, likewise.  With `cams` and `slots` (CUDA int32) the cameras go straight to those environments' rows of an existing array."""
     from . import binding

@@ -102,12 +102,12 @@ class VecRenderEnv:
             host[1].view(np.int32)[:len(chunk)] = chunk
             ids, dst = torch.from_numpy(host).pin_memory().to(self.device, non_blocking=True)
             dst = dst.view(torch.int32)[:len(chunk)]
-            w = scenes.make_worlds(self.cfg, device=self.device, env_ids=ids)
             if self._native is not None:
-                e = scenes.native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst)
-            else:
-                e = scenes.make_boxes_and_cameras(self.cfg, w)
-                self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
+                scenes.native_upload(self.cfg, self._native, ids, self.batch, chunk.astype(np.int32), self.cams)
+                continue
+            w = scenes.make_worlds(self.cfg, device=self.device, env_ids=ids)
+            e = scenes.make_boxes_and_cameras(self.cfg, w)
+            self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
             boxes = count = None
             if self.cfg.max_boxes > 0:
                 boxes, count = e["boxes"], e["box_count"]

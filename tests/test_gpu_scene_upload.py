@@ -1,0 +1,59 @@
+"""Seeded scenes made straight in a batch: what an upload of their grids, boxes and palettes leaves, over environments that held something else."""
+from __future__ import annotations
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("grid,world,extra,palette,agents,boxes", [
+    ((128, 32, 128), "columns", {}, 64, 1, 16), ((16, 64, 24), "rooms", {"n_lines": 1}, 7, 2, 3), ((20, 4, 12), "segments", {}, 2, 1, 0),
+    ((8, 100, 1024), "columns", {}, 256, 3, 1), ((64, 36, 4), "rooms", {"n_lines": 0}, 1, 1, 4), ((4, 8, 4), "columns", {"n_rects": 0}, 3, 1, 0),
+    ((36, 32, 44), "rooms", {"n_lines": 3}, 17, 4, 0)])
+def test_scenes_made_in_the_batch(grid, world, extra, palette, agents, boxes):
+    from paper_2107_08170_b200 import binding as B, scenes
+    cfg = scenes.config("rooms", num_envs=9, agents=agents, grid=grid, width=40, height=24, palette_size=palette, movable_boxes=boxes,
+                        body_boxes=agents > 1, world=world, extra=extra)
+    desc = scenes.native_desc(cfg)
+    ids = torch.tensor([5, 70001, 3, 12], device="cuda")
+    at = [0, 3, 4, 8]
+    slots = torch.tensor(at, dtype=torch.int32, device="cuda")
+    results = []
+    for direct in (False, True):
+        batch = B.Batch(B.desc_from_config(cfg, 0))
+        old = torch.full((9, grid[1], grid[2], grid[0]), min(1, palette - 1), dtype=torch.uint8, device="cuda")
+        batch.upload_worlds(0, 9, old, palette=torch.full((9, palette, 3), 77, dtype=torch.uint8, device="cuda"))       # everything filled, for one thing
+        cams = torch.zeros(9 * agents, 6, dtype=torch.int32, device="cuda")
+        for _ in range(2):                                                       # (the second time over scenes made the same way)
+            if direct:
+                scenes.native_upload(cfg, desc, ids, batch, at, cams)
+            else:
+                w = scenes.make_worlds(cfg, device="cuda", env_ids=ids)
+                e = scenes.native_entities(cfg, desc, ids, w["height"], cams, slots)
+                batch.upload_worlds_at(at, w["grid"], e["boxes"] if cfg.max_boxes else None, e["box_count"] if cfg.max_boxes else None, w["palette"])
+        batch.set_cameras(cams)
+        rgb, depth = batch.alloc_outputs()
+        batch.render_batch(rgb, depth)
+        merged, count = batch.merge_voxels(0, 9, 4096)
+        results.append((rgb, depth, merged, count, cams, torch.tensor(batch.query_status())))
+        batch.destroy()
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
+
+
+def test_scenes_that_do_not_fit_the_batch_are_refused():
+    from paper_2107_08170_b200 import binding as B, scenes
+    make = lambda **over: scenes.config("rooms", **{**dict(num_envs=3, agents=1, grid=(16, 8, 16), movable_boxes=2, extra={"n_lines": 1}), **over})
+    cfg = make()
+    batch = B.Batch(B.desc_from_config(cfg, 0))
+    ids = torch.tensor([1, 2], device="cuda")
+    cams = torch.zeros(8, 6, dtype=torch.int32, device="cuda")
+    for c, at in [(cfg, [1, 1]), (cfg, [2, 3]), (cfg, [-1, 0]), (make(grid=(16, 8, 20)), [0, 1]), (make(palette_size=9), [0, 1]),
+                  (make(movable_boxes=3), [0, 1]), (make(agents=2), [0, 1])]:
+        with pytest.raises(B.MvError) as refused:
+            scenes.native_upload(c, scenes.native_desc(c), ids, batch, at, cams)
+        assert refused.value.code == -1
+    with pytest.raises(ValueError):
+        scenes.native_upload(cfg, scenes.native_desc(cfg), ids, batch, [0], cams)
+    batch.destroy()
