@@ -308,6 +308,9 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 // one after the other, and a line from HBM takes twice as long as one from L2.  In us, without / with: 192x48x192 columns 64
                 // observations 59.3 / 41.0, 148: 71.7 / 53.3, 512: 114.8 / 107.0, 2048: 245.8 / 222.2; rooms, whose rays are short,
                 // 22.6 / 22.6, 32.8 / 31.2, 59.4 / 55.5, 157.8 / 155.7.  (Two or three dozen rows around the eye are too few for that.)
+                // These are for bits that other work has pushed out of L2 since the last step.  Rendered again and again with nothing in
+                // between, batches whose planes together are a little more than L2 (512 here) pay for lines that no ray touches: columns
+                // 80.5 / 86.4, rooms 47.6 / 57.9; smaller ones the same either way, 2048 247.1 / 221.7.
                 if (OCC == kOccGlobal && part == 0) {
                     const int *bounds = reinterpret_cast<const int *>(env_block + p.lay.count_off);
                     const uint32_t used = bounds[2] < bounds[5] ? (plane_of(p.lay, bounds[5] - 1) + 1u) * p.lay.occ_plane : 0u;
