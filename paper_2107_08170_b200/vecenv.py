@@ -68,7 +68,9 @@ class VecRenderEnv:
     """The clocks t, episode and episode_len (CUDA int64 [num_envs]) may be changed between steps, in place by torch
     operations or by assignment, for instance t[i] = episode_len[i] - 1 to end an episode with the next step; that step then
     reads them back once.  (A write that torch does not see, through `.data` or another library's pointer, is made known
-    by assigning the tensor to its own name: env.t = env.t.)"""
+    by assigning the tensor to its own name: env.t = env.t.)
+    cfg may be changed between steps as far as the batch's sizes allow: the grids and palettes of episodes that begin later
+    follow it; boxes and cameras are drawn as the object was made to."""
 
     t = _clock_property("t", "steps taken in the present episode")
     episode = _clock_property("episode", "episodes finished; env e in its k-th episode shows the seeded scene e + k * num_envs")
@@ -94,6 +96,12 @@ class VecRenderEnv:
         """Fresh worlds for the env indices in `envs` (sorted int64 array), each in its current episode: env e in its
         k-th episode uses the seeded scene id e + k * num_envs."""
         A = self.cfg.agents
+        # straight into the batch while the configuration is the one that this object was made with
+        desc = scenes.native_desc(self.cfg)
+        direct = desc is not None and self._native is not None and bytes(desc) == bytes(self._native)
+        made = self.batch.desc
+        if not direct and (tuple(self.cfg.grid), self.cfg.palette_size) != ((made.grid_x, made.grid_y, made.grid_z), made.palette_size):
+            raise ValueError("the grid's size and the number of colours are fixed when the environment is made")
         for c0 in range(0, len(envs), _GEN_CHUNK):
             chunk = envs[c0:c0 + _GEN_CHUNK]
             # ids and destinations (as int32) in one pinned copy that nothing waits for
@@ -102,12 +110,15 @@ class VecRenderEnv:
             host[1].view(np.int32)[:len(chunk)] = chunk
             ids, dst = torch.from_numpy(host).pin_memory().to(self.device, non_blocking=True)
             dst = dst.view(torch.int32)[:len(chunk)]
-            if self._native is not None:
+            if direct:
                 scenes.native_upload(self.cfg, self._native, ids, self.batch, chunk.astype(np.int32), self.cams)
                 continue
             w = scenes.make_worlds(self.cfg, device=self.device, env_ids=ids)
-            e = scenes.make_boxes_and_cameras(self.cfg, w)
-            self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
+            if self._native is not None:
+                e = scenes.native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst)
+            else:
+                e = scenes.make_boxes_and_cameras(self.cfg, w)
+                self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
             boxes = count = None
             if self.cfg.max_boxes > 0:
                 boxes, count = e["boxes"], e["box_count"]

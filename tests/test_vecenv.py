@@ -145,3 +145,46 @@ def test_clocks_set_by_the_caller_end_episodes(inference):
         env.t = env.t
         step({1: 3, 2: 8, 3: 3})
     env.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("change", [{"extra": {"n_lines": 1, "n_pillars": 200}}, {"world": "columns", "extra": {"n_rects": 30}}, {"seed": 77}, {}])
+def test_worlds_follow_a_changed_configuration(change):
+    """A configuration changed between steps (a curriculum): the episodes that begin then have its grids and palettes; boxes and cameras
+    are dealt out over those as the object was made to."""
+    from paper_2107_08170_b200 import binding as B
+    make = lambda **over: scenes.config("rooms_boxes", num_envs=3, agents=2, **over)
+    cfg, A = make(), 2
+    desc = scenes.native_desc(cfg)
+    env = vecenv.VecRenderEnv(cfg, 2, time_bar=False)
+    env.reset()
+    still = torch.zeros(cfg.num_obs, 4, device="cuda")
+    env.step(still)
+    for name, value in change.items():
+        setattr(cfg, name, value)
+    rgb, depth, done = env.step(still)
+    assert done.all()
+    ids = torch.arange(3, 6, device="cuda")
+    w = scenes.make_worlds(make(**change), device="cuda", env_ids=ids)
+    e = scenes.native_entities(make(), desc, ids, w["height"])
+    batch = B.Batch(B.desc_from_config(make()))
+    batch.upload_worlds(0, 3, w["grid"], e["boxes"], e["box_count"], w["palette"])
+    batch.set_cameras(e["cams"])
+    want = batch.alloc_outputs()
+    batch.render_batch(*want)
+    assert torch.equal(env.cams, e["cams"]) and torch.equal(rgb, want[0]) and torch.equal(depth, want[1])
+    batch.destroy()
+    env.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("change,refused", [({"grid": (64, 16, 60)}, ValueError), ({"palette_size": 63}, ValueError), ({"world": "maze"}, ValueError)])
+def test_configurations_the_batch_was_not_made_for_are_refused(change, refused):
+    cfg = scenes.config("rooms_boxes", num_envs=3, agents=2)
+    env = vecenv.VecRenderEnv(cfg, 1, time_bar=False)
+    env.reset()
+    for name, value in change.items():
+        setattr(cfg, name, value)
+    with pytest.raises(refused):
+        env.step(torch.zeros(cfg.num_obs, 4, device="cuda"))
+    env.close()
