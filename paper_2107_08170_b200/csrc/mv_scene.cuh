@@ -336,6 +336,7 @@ __global__ void __launch_bounds__(kEntityThreads) scene_populate_kernel(const Sc
     unsigned char *blk = env_blocks + env * lay.stride;
     if (threadIdx.x == 0) s_top = 0;
     __syncthreads();
+    int top = 0;                                                 // (of threads without columns too)
     if (r < row_groups * a.gz) {
         const ulonglong2 *kp = reinterpret_cast<const ulonglong2 *>(keys + (size_t)e * a.gx * a.gz) + 2 * (size_t)r;
         const ulonglong2 k01 = kp[0], k23 = kp[1];
@@ -349,7 +350,6 @@ __global__ void __launch_bounds__(kEntityThreads) scene_populate_kernel(const Sc
         const uint32_t col0 = column_index(lay, x, z), words = lay.occ_plane / 4;
         uint32_t *occ = reinterpret_cast<uint32_t *>(blk) + col0;
         uint8_t *dst = mat + env * mat_stride + ((size_t)col0 << lay.ysh);
-        int top = 0;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const uint32_t id = (uint32_t)(k[c] & 255u), m = min(id, cap);
@@ -373,9 +373,9 @@ __global__ void __launch_bounds__(kEntityThreads) scene_populate_kernel(const Sc
             }
         }
         if (clamped) atomicOr(status, kFlagMaterial);
-        top = __reduce_max_sync(__activemask(), top);
-        if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
     }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
     __syncthreads();
     if (threadIdx.x == 0) {                                     // (the accumulators as an upload uses and leaves them)
         int *acc = acc_all + env * kPackAccInts;

@@ -64,3 +64,10 @@ def test_zero_light_is_rejected(mvlib):
     d = mvlib.make_desc(4, 1, (16, 8, 16), 0, 64, 36, 16, light_dir=(0.0, 0.0, 0.0))
     h = C.c_void_p()
     assert mvlib.lib().mv_create_batch(C.byref(d), C.byref(h)) == -1
+
+
+def test_warp_votes_name_their_lanes():
+    """A mask of whoever happens to be active is not the mask of whoever should take part: a warp that was split would lose part of a
+    result without a word."""
+    for source in sorted((ROOT / "paper_2107_08170_b200" / "csrc").iterdir()):
+        assert "__activemask" not in source.read_text(), source.name
