@@ -854,14 +854,22 @@ int mv_scene_upload(mv_batch *b, const mv_scene_desc *desc, const int64_t *d_env
     DeviceGuard g(b->desc.device);
     if (!g.ok) return MV_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t per_env = ctas_of((size_t)a.gx * a.gz / 4, kEntityThreads), colours = ctas_of((size_t)env_count * 3 * a.palette, kEntityThreads);
-    if (env_count * (per_env + 1) + colours > 0x7fffffffull) return MV_ERR_INVALID_ARG;
+    const size_t columns = ctas_of((size_t)a.gx * a.gz / 4, kEntityThreads), colours = ctas_of((size_t)env_count * 3 * a.palette, kEntityThreads);
+    // Few high worlds have few columns and many bytes, more than an SM writes in the time that boxes and cameras take: their heights are dealt to as
+    // many CTAs as leave each one an SM of its own (more would share those that place boxes).  64x1024x64, 1 world: 89 -> 25 us (by its arrays
+    // and an upload 61), 8: 90 -> 30; 64x256x64, 8: 39 -> 24; from 64 worlds on, and where grids are at most 32 high, nothing changes.
+    const int64_t idle = (int64_t)b->sms - (int64_t)(env_count + colours), most = (a.gy + 31) / 32;
+    int64_t slabs = idle / (int64_t)(columns * env_count);
+    slabs = slabs < 1 ? 1 : slabs > most ? most : slabs;
+    const size_t ctas = env_count * (columns * slabs + 1) + colours;
+    if (ctas > 0x7fffffffull) return MV_ERR_INVALID_ARG;
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(d_work);
     MV_CUDA(b, cudaMemcpyAsync(b->d_env_index, h_env_index, (size_t)env_count * 4, cudaMemcpyHostToDevice, s));
     MV_CUDA(b, launch_scene_keys(a, keys, s));
-    scene_populate_kernel<<<(unsigned)(env_count * (per_env + 1) + colours), kEntityThreads, 0, s>>>(
+    const auto populate = slabs > 1 ? scene_populate_kernel<true> : scene_populate_kernel<false>;
+    populate<<<(unsigned)ctas, kEntityThreads, 0, s>>>(
         a, keys, b->d_env_index, reinterpret_cast<uint32_t *>(d_boxes), d_box_count, reinterpret_cast<uint32_t *>(d_cams), d_palette, b->d_env_blocks,
-        b->d_mat, b->mat_bytes_per_env, b->lay, b->d_acc, (int)per_env, b->d_status);
+        b->d_mat, b->mat_bytes_per_env, b->lay, b->d_acc, (int)columns, (int)slabs, b->d_status);
     MV_CUDA(b, cudaGetLastError());
     b->launches += 2;
     const int r = launch_upload(b, 0, b->d_env_index, env_count, nullptr, a.max_boxes > 0 ? d_boxes : nullptr, d_box_count, d_palette, s);

@@ -310,28 +310,31 @@ __global__ void __launch_bounds__(kEntityThreads) scene_entities_kernel(const Sc
 // the grid's bytes in between, in one launch.  First a CTA per environment for boxes and cameras, which takes longest, beside them those
 // that write the world store, then the palettes.  A thread of the store takes four columns, floor and one stack each: their occupancy words
 // and 32 bytes of material at a time as one store, whole sectors; the floor fills the whole grid, so of the cell box only the height
-// is looked for.  163 worlds of 128x32x128: 67 us with their keys, which before went through grid bytes and an upload: 111.
+// is looked for.  SLABS: every CTA of columns is `slabs` ones, each with every slabs-th 32 heights and plane (few high worlds, see
+// mv_scene_upload).  163 worlds of 128x32x128: 67 us with their keys, which before went through grid bytes and an upload: 111.
+template <bool SLABS>
 __global__ void __launch_bounds__(kEntityThreads) scene_populate_kernel(const SceneArgs a, const unsigned long long *__restrict__ keys,
                                                                        const int32_t *__restrict__ env_index, uint32_t *__restrict__ boxes,
                                                                        int32_t *__restrict__ counts, uint32_t *__restrict__ cams,
                                                                        uint8_t *__restrict__ palette, unsigned char *__restrict__ env_blocks,
                                                                        uint8_t *__restrict__ mat, size_t mat_stride, EnvLayout lay,
-                                                                       int *__restrict__ acc_all, int ctas_per_env, uint32_t *__restrict__ status)
+                                                                       int *__restrict__ acc_all, int column_ctas, int slabs, uint32_t *__restrict__ status)
 {
     if ((int)blockIdx.x < a.env_count) {
         scene_entities<true>(a, reinterpret_cast<const long long *>(keys), env_index, boxes, counts, cams);
         return;
     }
-    const int cta = (int)blockIdx.x - a.env_count, column_ctas = a.env_count * ctas_per_env;
-    if (cta >= column_ctas) {
-        const long long i = (long long)(cta - column_ctas) * kEntityThreads + threadIdx.x;
+    const int n_slabs = SLABS ? slabs : 1, ctas_per_env = column_ctas * n_slabs;
+    const int cta = (int)blockIdx.x - a.env_count, store_ctas = a.env_count * ctas_per_env;
+    if (cta >= store_ctas) {
+        const long long i = (long long)(cta - store_ctas) * kEntityThreads + threadIdx.x;
         const int per = 3 * a.palette, e = (int)(i / per);
         if (e < a.env_count) palette[i] = (uint8_t)SceneRng(a.seed, 31, a.env[e]).range((unsigned long long)(i - (long long)e * per), 24, 255);
         return;
     }
     __shared__ int s_top;
-    const int e = cta / ctas_per_env, part = cta - e * ctas_per_env;
-    const int r = part * kEntityThreads + (int)threadIdx.x, row_groups = a.gx / 4;
+    const int e = cta / ctas_per_env, part = cta - e * ctas_per_env, slab = SLABS ? part / column_ctas : 0;
+    const int r = (part - slab * column_ctas) * kEntityThreads + (int)threadIdx.x, row_groups = a.gx / 4;
     const size_t env = (size_t)env_index[e];
     unsigned char *blk = env_blocks + env * lay.stride;
     if (threadIdx.x == 0) s_top = 0;
@@ -357,11 +360,11 @@ __global__ void __launch_bounds__(kEntityThreads) scene_populate_kernel(const Sc
             // filled cells of the column from the floor up (a stack without material is none)
             const int n = id ? 1 + (int)min(k[c] >> 8, (unsigned long long)(a.gy - 1)) : 1;
             top = max(top, n);
-            for (uint32_t q = 0; q < lay.planes; ++q) {
+            for (uint32_t q = slab; q < lay.planes; q += n_slabs) {
                 const int in = min(max(n - plane_begin(q), 0), lay.planes == 1 ? 32 : (int)kPlaneHeights);
                 occ[(size_t)q * words + c] = in == 32 ? 0xffffffffu : (1u << in) - 1u;
             }
-            for (int y0 = 0; y0 < a.gy; y0 += 32) {
+            for (int y0 = 32 * slab; y0 < a.gy; y0 += 32 * n_slabs) {
                 uint32_t w[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {

@@ -57,3 +57,61 @@ def test_scenes_that_do_not_fit_the_batch_are_refused():
     with pytest.raises(ValueError):
         scenes.native_upload(cfg, scenes.native_desc(cfg), ids, batch, [0], cams)
     batch.destroy()
+
+
+def _both_ways(cfg, at):
+    """The scenes 3, 10, 17 ... in the environments `at`: (direct, by their arrays) as functions of a batch and its cameras."""
+    from paper_2107_08170_b200 import scenes
+    desc = scenes.native_desc(cfg)
+    ids = 3 + 7 * torch.arange(len(at), device="cuda")
+    slots = torch.tensor(at, dtype=torch.int32, device="cuda")
+
+    def by_arrays(batch, cams):
+        w = scenes.make_worlds(cfg, device="cuda", env_ids=ids)
+        e = scenes.native_entities(cfg, desc, ids, w["height"], cams, slots)
+        batch.upload_worlds_at(at, w["grid"], e["boxes"], e["box_count"], w["palette"])
+
+    return lambda batch, cams: scenes.native_upload(cfg, desc, ids, batch, at, cams), by_arrays
+
+
+@pytest.mark.parametrize("grid,n", [((16, 1024, 16), 12), ((16, 1024, 16), 48), ((16, 1024, 16), 100), ((64, 1024, 64), 1), ((64, 256, 64), 21), ((20, 64, 12), 150)])
+def test_high_worlds_in_slabs(grid, n):
+    """Worlds stored by several CTAs above one another, as many as there are 32 heights and fewer (every slabs-th 32 heights and plane)."""
+    from paper_2107_08170_b200 import binding as B, scenes
+    cfg = scenes.config("rooms", num_envs=n, agents=1, grid=grid, width=40, height=24, palette_size=9, movable_boxes=2, world="segments", extra={"n_rects": 40})
+    results = []
+    for make in _both_ways(cfg, list(range(n))):
+        batch = B.Batch(B.desc_from_config(cfg, 0))
+        cams = torch.zeros(n, 6, dtype=torch.int32, device="cuda")
+        make(batch, cams)
+        batch.set_cameras(cams)
+        rgb, depth = batch.alloc_outputs()
+        batch.render_batch(rgb, depth)
+        results.append((rgb, depth, cams, *batch.merge_voxels(0, n, 512)))
+        batch.destroy()
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("grid,n", [((64, 1024, 64), 1), ((64, 1024, 64), 8), ((128, 32, 128), 1)])
+def test_straight_into_the_batch_is_not_the_longer_way(grid, n):
+    """One to a few worlds, also high ones, whose store is many bytes for few columns: no longer than their arrays made and uploaded."""
+    from paper_2107_08170_b200 import binding as B, scenes
+    cfg = scenes.config("rooms", num_envs=n, agents=1, grid=grid, width=40, height=24, movable_boxes=4, world="columns", extra={"n_rects": 200})
+    batch = B.Batch(B.desc_from_config(cfg, 0))
+    cams = torch.zeros(n, 6, dtype=torch.int32, device="cuda")
+    best = [float("inf")] * 2
+    for _ in range(6):
+        for i, make in enumerate(_both_ways(cfg, list(range(n)))):
+            make(batch, cams)
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            torch.cuda._sleep(4000000)                                           # (so that the host's share does not count)
+            start.record()
+            for _ in range(8):
+                make(batch, cams)
+            end.record()
+            torch.cuda.synchronize()
+            best[i] = min(best[i], start.elapsed_time(end))
+    assert best[0] <= 1.1 * best[1], best
+    batch.destroy()
