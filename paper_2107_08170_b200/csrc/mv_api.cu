@@ -866,12 +866,13 @@ int mv_scene_upload(mv_batch *b, const mv_scene_desc *desc, const int64_t *d_env
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(d_work);
     MV_CUDA(b, cudaMemcpyAsync(b->d_env_index, h_env_index, (size_t)env_count * 4, cudaMemcpyHostToDevice, s));
     MV_CUDA(b, launch_scene_keys(a, keys, s));
+    if (a.world == kWorldRooms || a.count > 0) b->launches++;
     const auto populate = slabs > 1 ? scene_populate_kernel<true> : scene_populate_kernel<false>;
     populate<<<(unsigned)ctas, kEntityThreads, 0, s>>>(
         a, keys, b->d_env_index, reinterpret_cast<uint32_t *>(d_boxes), d_box_count, reinterpret_cast<uint32_t *>(d_cams), d_palette, b->d_env_blocks,
         b->d_mat, b->mat_bytes_per_env, b->lay, b->d_acc, (int)columns, (int)slabs, b->d_status);
     MV_CUDA(b, cudaGetLastError());
-    b->launches += 2;
+    b->launches++;
     const int r = launch_upload(b, 0, b->d_env_index, env_count, nullptr, a.max_boxes > 0 ? d_boxes : nullptr, d_box_count, d_palette, s);
     if (r != MV_OK) return r;
     for (int i = 0; i < env_count && (b->missing_grid > 0 || b->missing_palette > 0); ++i) {

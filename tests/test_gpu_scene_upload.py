@@ -115,3 +115,17 @@ def test_straight_into_the_batch_is_not_the_longer_way(grid, n):
             best[i] = min(best[i], start.elapsed_time(end))
     assert best[0] <= 1.1 * best[1], best
     batch.destroy()
+
+
+@pytest.mark.parametrize("world,extra,keys", [("columns", {"n_rects": 5}, 1), ("columns", {"n_rects": 0}, 0), ("segments", {"n_rects": 0}, 0), ("rooms", {"n_lines": 0}, 1)])
+def test_launches_are_counted(world, extra, keys):
+    """Every kernel that was launched and no other: keys (without rectangles there is nothing to launch), the world store, palettes and boxes."""
+    from paper_2107_08170_b200 import binding as B, scenes
+    cfg = scenes.config("rooms", num_envs=3, agents=1, grid=(16, 8, 16), movable_boxes=2, world=world, extra=extra)
+    batch = B.Batch(B.desc_from_config(cfg, 0))
+    cams = torch.zeros(3, 6, dtype=torch.int32, device="cuda")
+    before = batch.launch_count()
+    scenes.native_upload(cfg, scenes.native_desc(cfg), torch.tensor([1, 2], device="cuda"), batch, [0, 2], cams)
+    assert batch.launch_count() - before == keys + 2
+    torch.cuda.synchronize()
+    batch.destroy()
