@@ -341,6 +341,11 @@ int64_t mv_launch_count(const mv_batch *batch);
  * on < 0 changes nothing and returns 1 if they are read from global memory now, 0 if they are staged. */
 int mv_debug_occupancy_in_global(mv_batch *batch, int on);
 
+/* on == 0 / 1: occupancy bits that are read from global memory are not / are asked for in L2 as a render begins; on == 2 restores the
+ * library's own choice; on < 0 changes nothing.  Results are identical.  Returns 1 if a render now asks for them, 0 if not (or they are
+ * staged), or INVALID_ARG. */
+int mv_debug_prefetch(mv_batch *batch, int on);
+
 /* Failure-detection hook.  The render kernel's only device-side wait is the bounded wait for the
  * staged env block; with skip_staging != 0 the copy is not issued, so every CTA's wait runs out after
  * wait_polls polls, the kernel returns without touching the outputs and MV_FLAG_DEVICE_TIMEOUT is set

@@ -16,7 +16,7 @@ _lib = None
 MV_OK = 0
 FLAG_MATERIAL_CLAMPED, FLAG_BOX_COUNT_CLAMPED, FLAG_BAD_CAMERA, FLAG_DEVICE_TIMEOUT = 1, 2, 4, 8
 EXPORTS = ["mv_create_batch", "mv_upload_worlds", "mv_upload_worlds_at", "mv_set_cameras", "mv_render_batch", "mv_step_host",
-           "mv_step_host_static", "mv_set_overlays", "mv_move_agents", "mv_merge_voxels", "mv_scene_worlds", "mv_scene_entities", "mv_scene_upload", "mv_advance_episodes", "mv_debug_staging", "mv_debug_occupancy_in_global", "mv_debug_agents_per_cta", "mv_debug_parts", "mv_query_status", "mv_launch_count", "mv_destroy", "mv_status_string"]
+           "mv_step_host_static", "mv_set_overlays", "mv_move_agents", "mv_merge_voxels", "mv_scene_worlds", "mv_scene_entities", "mv_scene_upload", "mv_advance_episodes", "mv_debug_staging", "mv_debug_occupancy_in_global", "mv_debug_prefetch", "mv_debug_agents_per_cta", "mv_debug_parts", "mv_query_status", "mv_launch_count", "mv_destroy", "mv_status_string"]
 
 
 class BatchDesc(C.Structure):
@@ -66,6 +66,7 @@ def lib() -> C.CDLL:
         L.mv_advance_episodes.argtypes = [vp, vp, vp, vp, vp, i, i, vp, vp]
         L.mv_debug_staging.argtypes = [vp, i, i]
         L.mv_debug_occupancy_in_global.argtypes = [vp, i]
+        L.mv_debug_prefetch.argtypes = [vp, i]
         L.mv_debug_agents_per_cta.argtypes = [vp, i]
         L.mv_debug_parts.argtypes = [vp, i]
         L.mv_query_status.argtypes = [vp, i, vp]
@@ -255,6 +256,12 @@ class Batch:
         """None: only asks; returns whether the occupancy is read from global memory."""
         _check(min(lib().mv_debug_occupancy_in_global(self._h, -1 if on is None else int(on)), 0), "mv_debug_occupancy_in_global")
         return lib().mv_debug_occupancy_in_global(self._h, -1) == 1
+
+    def debug_prefetch(self, on: bool | None, ask=False) -> bool:
+        """None: the library's choice; returns whether a render asks for occupancy in L2 (with `ask` nothing is changed)."""
+        r = lib().mv_debug_prefetch(self._h, -1 if ask else 2 if on is None else int(on))
+        _check(min(r, 0), "mv_debug_prefetch")
+        return r == 1
 
     def debug_agents_per_cta(self, agents_per_cta: int) -> int:
         """1 = a CTA per observation, agents_per_env = a CTA per environment, 0 = the library's choice; returns how many CTAs

@@ -78,6 +78,7 @@ struct mv_batch {
     int smem_max = 0;                   // opt-in shared memory per CTA of the device
     int auto_agents_per_cta = 1;        // the library's own choice (a test hook can override it)
     int skip_staging = 0;
+    bool prefetch = false;              // occupancy in global memory is asked for in L2 (prefetch_pays, or a test hook)
     int last_cuda_error = 0;
     // mv_step_host resources (allocated on first use)
     uint8_t *d_rgb = nullptr;
@@ -222,6 +223,23 @@ RenderFn render_fn(const mv_batch *b, int threads, bool occ_shared) {
 }
 RenderFn render_fn(const mv_batch *b) { return render_fn(b, b->threads, b->occ_shared); }
 
+// Is a plane of occupancy per environment asked for in L2 as a render begins, where it is read from global memory?  A render finds
+// its lines in HBM if other work has pushed them out of L2 since the last one, or if the batch itself does; rendered again and again with
+// nothing in between, a batch that L2 holds has no use for it, and lines that no ray sees push out what is used.  So, with figures in us
+// without / with, first after other work, then again and again (images of 128x72 but where it says so):
+// - few environments, whose planes and frames L2 holds side by side, so that asking pushes nothing out.  192x48x192 columns 64 of them 60.4 /
+//   43.2, 28.4 / 28.3; 320: 120.1 / 93.0, 68.4 / 68.6; 128 with 4 agents 118.5 / 105.3, 86.4 / 86.7; rooms 148: 33.8 / 29.7, 21.0 / 21.3; 320 of 64x36
+//   39.9 / 33.8, 21.5 / 21.7.  More lose: 512 columns 115 / 106 but 78 / 86, 640: 84 / 113, 300 of 256x144 126 / 145, 400 rooms (both planes) 41.8 / 46.9.
+// - more frames than L2 holds, which push everything out in every step, as long as the planes are not much beside the frames and an
+//   image has few rays to share their lines.  2048 columns 248.4 / 222.2, 243.4 / 217.1; rooms 158.9 / 155.2, 153.2 / 149.7; 512 with 4 agents 236.4 / 211.8,
+//   230.7 / 206.8; 4096 of 128x48x128 360.8 / 348.9, 355.4 / 343.0.  Not: planes four times the frames (2048 rooms of 256x64x256 152.7 / 166.5);
+//   2048 rooms of 64x36 (both planes) 55.9 / 82.7; 1024 of 256x144 (both) 240.7 / 243.0.
+bool prefetch_pays(const mv_batch *b) {
+    const int64_t px = (int64_t)b->desc.width * b->desc.height, frames = 7 * px * b->num_obs, planes = (int64_t)b->desc.num_envs * b->lay.occ_plane;
+    constexpr int64_t MB = 1 << 20;
+    return (planes <= 46 * MB && planes + frames <= 68 * MB) || (frames >= 120 * MB && 2 * planes <= 5 * frames && px <= 1 << 14);
+}
+
 bool fits_staged(const mv_batch *b, int apc) { return (int64_t)smem_layout(b, apc, true).bytes <= b->smem_max; }
 
 // CTA shape of the render kernel when a CTA renders `apc` observations of an environment (which has to fit unstaged at least).
@@ -274,6 +292,7 @@ int launch_render(mv_batch *b, uint8_t *d_rgb, float *d_depth, int obs_begin, in
     p.max_overlay = b->desc.max_overlay_rects;
     p.wait_polls = b->wait_polls;
     p.skip_staging = b->skip_staging;
+    p.prefetch = b->prefetch;
     const Split split = pick_split(b, obs_count);         // (callers pass whole environments when a CTA renders one)
     p.whole_ctas = (unsigned)split.whole; p.parts = (unsigned)split.parts;
     const int64_t ctas = split.whole + (obs_count - split.whole * b->agents_per_cta) * split.parts;
@@ -553,9 +572,11 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
     // fit, and where staging it would leave one CTA on an SM, reading it would leave three, and there are more observations than
     // those hold at once: of such a grid the rays see a small part, which the cache holds, and with one CTA nobody works while
     // the next block is staged.  Up to then the parts of an observation are staged side by side.  In us, staged / from global memory:
-    //   192x32x192  rooms 148: 24.1 / 22.1   300: 36.6 / 38.5   512: 62.3 / 52.5   2048: 213 / 183   columns 25.2 / 35.9   41.9 / 56.4   67.3 / 75.2   219 / 238
-    //   128x48x128  rooms 148: 20.9 / 21.5   300: 33.9 / 30.5   512: 58.2 / 47.5   2048: 197 / 145   columns 29.6 / 37.0   50.9 / 47.2   62.9 / 71.6   234 / 198
+    //   192x32x192  rooms 148: 25.7 / 24.2   300: 38.1 / 41.0   512: 64.5 / 54.5   2048: 216 / 183   columns 26.9 / 38.9   43.8 / 59.0   69.8 / 77.7   223 / 217
+    //   128x48x128  rooms 148: 23.2 / 23.2   300: 36.2 / 34.3   512: 60.3 / 47.2   2048: 201 / 146   columns 31.6 / 37.5   53.1 / 50.8   65.3 / 73.6   238 / 190
     //   148x56x112  rooms 148: 26.6 / 21.8   300: 39.6 / 33.3   444: 50.9 / 55.3   512: 62.5 / 55.4   columns 32.5 / 38.8   46.7 / 48.5   62.0 / 66.2   71.5 / 70.0
+    // (These again and again with nothing in between.  After other work 192x32x192 rooms take 33.8 / 33.7, 48.2 / 52.1, 70.7 / 68.7, 222 / 188, but columns,
+    // whose rays look far, 34.0 / 59.7, 54.3 / 79.7, 74.8 / 116, 228 / 222.)
     // Where the tables of a large image leave room for one either way, staged is 13 to 33 % faster for any number (640x360 on 64x16x64
     // rooms, 300: 474 / 555), and no slower where they leave two (480x272 on 96x32x96 rooms, 300: 344 / 369, 1000: 1030 / 1024).
     const auto room = [&](bool staged) { return (int64_t)b->smem_sm / ((int64_t)smem_layout(b, 1, staged).bytes + 1024); };   // (CTAs on an SM)
@@ -570,6 +591,7 @@ int mv_create_batch(const mv_batch_desc *desc, mv_batch **out) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(upload_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUploadSmem);
     if (e != cudaSuccess) { delete b; return MV_ERR_CUDA; }
+    b->prefetch = prefetch_pays(b);
     // A CTA per environment (block staged once for all its agents) or per observation, whichever is expected to take less.
     int shape = choose_shape(b, 1);
     if (shape == MV_OK && d.agents_per_env > 1 && (int64_t)smem_layout(b, d.agents_per_env, b->occ_shared).bytes <= smem_max) {   // (never give up staged occupancy for it)
@@ -921,6 +943,12 @@ int mv_debug_occupancy_in_global(mv_batch *b, int on) {
     if (!g.ok) return MV_ERR_CUDA;
     b->want_occ_shared = !on;
     return choose_shape(b, b->agents_per_cta);
+}
+
+int mv_debug_prefetch(mv_batch *b, int on) {
+    if (!b || on > 2) return MV_ERR_INVALID_ARG;
+    if (on >= 0) b->prefetch = on == 2 ? prefetch_pays(b) : on == 1;
+    return b->prefetch && !b->occ_shared ? 1 : 0;
 }
 
 int mv_debug_parts(mv_batch *b, int parts) {

@@ -97,6 +97,7 @@ struct RenderParams {
     int max_overlay;
     int wait_polls;                    // bound of the staging wait
     int skip_staging;                  // test hook: the block copy is not issued, so the wait runs out
+    int prefetch;                      // occupancy that is read from global memory is asked for in L2
 };
 // A launch takes the host 0.3 us less with parameters of 20 to 32 bytes beyond a multiple of 64 than with any other size (212 to
 // 224: 1.75 us, 208 and 228: 2.05 to 2.1; as measured with driver 580.159), a tenth of a step of the smallest batches.

@@ -186,8 +186,6 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 // Threads resident per SM that the registers are laid out for: three CTAs of 384 with 56 registers (16384 observations
 // 1.42 ms when two with 69 took 1.62).
 constexpr int kThreadsPerSm = 3 * 384;
-// Occupancy that is read from global memory is fetched into L2 ahead of the walks up to this many bytes.
-constexpr uint32_t kPrefetchMost = 1u << 20;
 
 constexpr uint32_t kAgentInside = 1u;      // eye inside the occupied cell box
 constexpr uint32_t kAgentBad = 2u;         // non-finite camera: sky frame
@@ -304,18 +302,6 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
                 mbar_expect_tx(s_bar, bytes + p.lay.block_bytes - p.lay.occ_bytes);
                 if (bytes) bulk_load(smem, env_block, bytes, s_bar);
                 bulk_load(smem + stage_occ, env_block + p.lay.occ_bytes, p.lay.block_bytes - p.lay.occ_bytes, s_bar);
-                // Bits that are not staged are asked for in L2, all planes that hold anything: rays that look far touch a new line with every row,
-                // one after the other, and a line from HBM takes twice as long as one from L2.  In us, without / with: 192x48x192 columns 64
-                // observations 59.3 / 41.0, 148: 71.7 / 53.3, 512: 114.8 / 107.0, 2048: 245.8 / 222.2; rooms, whose rays are short,
-                // 22.6 / 22.6, 32.8 / 31.2, 59.4 / 55.5, 157.8 / 155.7.  (Two or three dozen rows around the eye are too few for that.)
-                // These are for bits that other work has pushed out of L2 since the last step.  Rendered again and again with nothing in
-                // between, batches whose planes together are a little more than L2 (512 here) pay for lines that no ray touches: columns
-                // 80.5 / 86.4, rooms 47.6 / 57.9; smaller ones the same either way, 2048 247.1 / 221.7.
-                if (OCC == kOccGlobal && part == 0) {
-                    const int *bounds = reinterpret_cast<const int *>(env_block + p.lay.count_off);
-                    const uint32_t used = bounds[2] < bounds[5] ? (plane_of(p.lay, bounds[5] - 1) + 1u) * p.lay.occ_plane : 0u;
-                    if (used && used <= kPrefetchMost) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(env_block)), "r"(used) : "memory");
-                }
             }
         }
         for (int ag = lane; ag < apc; ag += 32) {
@@ -347,6 +333,14 @@ __global__ void __launch_bounds__(NT, kThreadsPerSm / NT) render_kernel(const Re
         wait_for_previous();
     }
     __syncthreads();
+    // ---- meanwhile: occupancy that is not staged is asked for in L2 once per environment, the plane that the first agent's eye is in: rays
+    // that look far touch a new line with every row, one after the other, and a line from HBM takes twice as long as one from L2.
+    // (For which batches: see prefetch_pays.)
+    if (OCC == kOccGlobal && p.prefetch && tid == 32 && part == 0 && obs0 == env * p.agents) {
+        const int top = plane_begin(p.lay.planes) - 1, y = (int)fminf(fmaxf(agent_rec(0)[3].y, 0.0f), (float)top);
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                     ::"l"(__cvta_generic_to_global(env_block + (size_t)(y / (int)kPlaneHeights) * p.lay.occ_plane)), "r"(p.lay.occ_plane) : "memory");
+    }
     // ---- meanwhile: GUI rectangles
     if (p.overlay) {
         // GUI rectangles of each observation (unpacked to x0,y0,x1,y1 / colour in two slots); the tiles any of them touches
