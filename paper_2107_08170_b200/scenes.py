@@ -166,24 +166,29 @@ def native_worlds(cfg: SceneConfig, desc, env: torch.Tensor):
     return {"grid": grid, "palette": palette, "height": height, "env": env}
 
 
+def _native_boxes(desc) -> int:
+    """Boxes of an environment as the library's kernels count them (the descriptor may be older than a configuration)."""
+    return desc.movable_boxes + (desc.agents if desc.body_boxes else 0)
+
+
 def native_upload(cfg: SceneConfig, desc, env: torch.Tensor, batch, env_index, cams: torch.Tensor):
     """The scenes of the CUDA ids `env` straight into the batch's environments `env_index`, their cameras into those environments' rows of `cams`."""
-    gx, _, gz = cfg.grid
     E, dev = env.numel(), env.device
-    boxes = torch.empty(E, cfg.max_boxes, 8, dtype=torch.int32, device=dev)
+    boxes = torch.empty(E, _native_boxes(desc), 8, dtype=torch.int32, device=dev)
     count = torch.empty(E, dtype=torch.int32, device=dev)
-    palette = torch.empty(E, cfg.palette_size, 3, dtype=torch.uint8, device=dev)
-    batch.upload_scenes(desc, env.contiguous(), env_index, cams, boxes, count, palette, torch.empty(E, gz, gx, dtype=torch.int64, device=dev))
+    palette = torch.empty(E, desc.palette_size, 3, dtype=torch.uint8, device=dev)
+    work = torch.empty(E, desc.grid_z, desc.grid_x, dtype=torch.int64, device=dev)
+    batch.upload_scenes(desc, env.contiguous(), env_index, cams, boxes, count, palette, work)
 
 
 def native_entities(cfg: SceneConfig, desc, env: torch.Tensor, height: torch.Tensor, cams=None, slots=None):
     """The arrays of make_boxes_and_cameras, likewise.  With `cams` and `slots` (CUDA int32) the cameras go straight to those environments' rows of an existing array."""
     from . import binding
     E, dev = env.numel(), env.device
-    boxes = torch.empty(E, cfg.max_boxes, 8, dtype=torch.int32, device=dev)
+    boxes = torch.empty(E, _native_boxes(desc), 8, dtype=torch.int32, device=dev)
     count = torch.empty(E, dtype=torch.int32, device=dev)
     if cams is None:
-        cams = torch.empty(E * cfg.agents, 6, dtype=torch.int32, device=dev)
+        cams = torch.empty(E * desc.agents, 6, dtype=torch.int32, device=dev)
     binding.scene_entities(desc, env.contiguous(), height.contiguous(), boxes, count, cams, slots)
     return {"boxes": boxes, "box_count": count, "cams": cams}
 

@@ -102,6 +102,8 @@ class VecRenderEnv:
         made = self.batch.desc
         if not direct and (tuple(self.cfg.grid), self.cfg.palette_size) != ((made.grid_x, made.grid_y, made.grid_z), made.palette_size):
             raise ValueError("the grid's size and the number of colours are fixed when the environment is made")
+        if self._native is None and (self.cfg.agents, self.cfg.max_boxes) != (made.agents_per_env, made.max_boxes):
+            raise ValueError("the numbers of agents and boxes are fixed when the environment is made")
         for c0 in range(0, len(envs), _GEN_CHUNK):
             chunk = envs[c0:c0 + _GEN_CHUNK]
             # ids and destinations (as int32) in one pinned copy that nothing waits for
@@ -120,7 +122,7 @@ class VecRenderEnv:
                 e = scenes.make_boxes_and_cameras(self.cfg, w)
                 self.cams.view(-1, A, 6)[dst.long()] = e["cams"].view(-1, A, 6)
             boxes = count = None
-            if self.cfg.max_boxes > 0:
+            if made.max_boxes > 0:
                 boxes, count = e["boxes"], e["box_count"]
             self.batch.upload_worlds_at(chunk.astype(np.int32), w["grid"], boxes, count, w["palette"])
 

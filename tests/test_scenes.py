@@ -70,3 +70,21 @@ def test_walk_cameras_moves_only_into_free_cells():
             i, j, k = np.floor(pos[o]).astype(int)
             assert g[o // cfg.agents, j, k, i] == 0
     assert not torch.equal(cams, sc["cams"])
+
+
+def test_arrays_are_as_large_as_the_library_fills_them(monkeypatch):
+    """The kernels write what the descriptor says, also where the configuration has been changed since it was made."""
+    from types import SimpleNamespace
+    from paper_2107_08170_b200 import binding
+    cfg = scenes.config("rooms_boxes", num_envs=3, agents=2, movable_boxes=7)
+    desc, shapes = scenes.native_desc(cfg), {}
+    note = lambda *arrays: shapes.update(zip(("boxes", "count", "cams"), (tuple(a.shape) for a in arrays)))
+    monkeypatch.setattr(binding, "scene_entities", lambda desc, ids, height, boxes, count, cams, slots: note(boxes, count, cams))
+    cfg.movable_boxes, cfg.agents, cfg.body_boxes, cfg.palette_size, cfg.grid = 1, 1, False, 2, (4, 4, 4)
+    scenes.native_entities(cfg, desc, torch.arange(3), torch.zeros(3, 64, 64, dtype=torch.int64))
+    assert shapes == {"boxes": (3, 9, 8), "count": (3,), "cams": (6, 6)}
+
+    def upload_scenes(desc, ids, at, cams, boxes, count, palette, work):
+        assert [tuple(a.shape) for a in (boxes, count, palette, work)] == [(3, 9, 8), (3,), (3, 64, 3), (3, 64, 64)]
+
+    scenes.native_upload(cfg, desc, torch.arange(3), SimpleNamespace(upload_scenes=upload_scenes), [0, 1, 2], torch.zeros(6, 6, dtype=torch.int32))

@@ -148,7 +148,8 @@ def test_clocks_set_by_the_caller_end_episodes(inference):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("change", [{"extra": {"n_lines": 1, "n_pillars": 200}}, {"world": "columns", "extra": {"n_rects": 30}}, {"seed": 77}, {}])
+@pytest.mark.parametrize("change", [{"extra": {"n_lines": 1, "n_pillars": 200}}, {"world": "columns", "extra": {"n_rects": 30}}, {"seed": 77}, {},
+                                    {"movable_boxes": 0}, {"movable_boxes": 40}])
 def test_worlds_follow_a_changed_configuration(change):
     """A configuration changed between steps (a curriculum): the episodes that begin then have its grids and palettes; boxes and cameras
     are dealt out over those as the object was made to."""
