@@ -64,6 +64,11 @@ def _clock_property(name, doc):
     return property(lambda self: self._clocks[name].tensor, lambda self, value: self._clocks[name].assign(value), doc=doc)
 
 
+def _recipe(cfg: scenes.SceneConfig):
+    """What the scenes of a configuration depend on."""
+    return (cfg.world, cfg.seed, tuple(cfg.grid), cfg.palette_size, cfg.agents, cfg.movable_boxes, cfg.body_boxes, cfg.cam_y_fixed, dict(cfg.extra))
+
+
 class VecRenderEnv:
     """The clocks t, episode and episode_len (CUDA int64 [num_envs]) may be changed between steps, in place by torch
     operations or by assignment, for instance t[i] = episode_len[i] - 1 to end an episode with the next step; that step then
@@ -90,15 +95,15 @@ class VecRenderEnv:
         self.cams = torch.zeros(cfg.num_obs, 6, dtype=torch.int32, device=self.device)
         self.rgb, self.depth = self.batch.alloc_outputs()
         self._native = scenes.native_desc(cfg)
+        self._made_by = _recipe(cfg)
         self._started = False
 
     def _load_envs(self, envs):
         """Fresh worlds for the env indices in `envs` (sorted int64 array), each in its current episode: env e in its
         k-th episode uses the seeded scene id e + k * num_envs."""
         A = self.cfg.agents
-        # straight into the batch while the configuration is the one that this object was made with
-        desc = scenes.native_desc(self.cfg)
-        direct = desc is not None and self._native is not None and bytes(desc) == bytes(self._native)
+        # straight into the batch while the scenes' configuration is the one that this object was made with
+        direct = self._native is not None and _recipe(self.cfg) == self._made_by
         made = self.batch.desc
         if not direct and (tuple(self.cfg.grid), self.cfg.palette_size) != ((made.grid_x, made.grid_y, made.grid_z), made.palette_size):
             raise ValueError("the grid's size and the number of colours are fixed when the environment is made")
@@ -106,15 +111,17 @@ class VecRenderEnv:
             raise ValueError("the numbers of agents and boxes are fixed when the environment is made")
         for c0 in range(0, len(envs), _GEN_CHUNK):
             chunk = envs[c0:c0 + _GEN_CHUNK]
-            # ids and destinations (as int32) in one pinned copy that nothing waits for
-            host = np.empty((2, len(chunk)), np.int64)
+            # ids, and destinations (as int32) where an upload does not bring them, in one pinned copy that nothing waits for
+            host = np.empty((1 if direct else 2, len(chunk)), np.int64)
             host[0] = chunk + self._clocks["episode"].host[chunk] * self.cfg.num_envs
-            host[1].view(np.int32)[:len(chunk)] = chunk
-            ids, dst = torch.from_numpy(host).pin_memory().to(self.device, non_blocking=True)
-            dst = dst.view(torch.int32)[:len(chunk)]
+            if not direct:
+                host[1].view(np.int32)[:len(chunk)] = chunk
+            sent = torch.from_numpy(host).pin_memory().to(self.device, non_blocking=True)
+            ids = sent[0]
             if direct:
                 scenes.native_upload(self.cfg, self._native, ids, self.batch, chunk.astype(np.int32), self.cams)
                 continue
+            dst = sent[1].view(torch.int32)[:len(chunk)]
             w = scenes.make_worlds(self.cfg, device=self.device, env_ids=ids)
             if self._native is not None:
                 e = scenes.native_entities(self.cfg, self._native, ids, w["height"], self.cams, dst)

@@ -189,3 +189,38 @@ def test_configurations_the_batch_was_not_made_for_are_refused(change, refused):
     with pytest.raises(refused):
         env.step(torch.zeros(cfg.num_obs, 4, device="cuda"))
     env.close()
+
+
+@pytest.mark.gpu
+def test_resets_send_what_they_need(monkeypatch):
+    """To new episodes that go straight into the batch one id each; elsewhere their destinations, too."""
+    cfg = scenes.config("rooms_boxes", num_envs=5, agents=2)
+    env = vecenv.VecRenderEnv(cfg, 4, time_bar=False, phase=torch.tensor([3, 0, 3, 3, 0]))
+    env.reset()
+    still, sent, real = torch.zeros(cfg.num_obs, 4, device="cuda"), [], torch.from_numpy
+    monkeypatch.setattr(torch, "from_numpy", lambda a: (sent.append(a.nbytes), real(a))[1])
+    env.step(still)
+    assert sent == [3 * 8]
+    cfg.seed = 8
+    env.t.fill_(3)
+    env.step(still)
+    assert sent == [3 * 8, 2 * 5 * 8]
+    env.close()
+
+
+def test_recipe_sees_every_change_of_the_scenes():
+    """Whatever the library's generator is told, changes in place included."""
+    make = lambda: scenes.config("rooms", extra={"n_lines": 2})
+    made = vecenv._recipe(make())
+    assert vecenv._recipe(make()) == made
+    for name, value in dict(world="columns", seed=9, grid=(64, 20, 64), palette_size=9, agents=1, movable_boxes=3, body_boxes=True, cam_y_fixed=0.5).items():
+        cfg = make()
+        before = bytes(scenes.native_desc(cfg))
+        setattr(cfg, name, value)
+        desc = scenes.native_desc(cfg)
+        assert desc is None or bytes(desc) != before
+        assert vecenv._recipe(cfg) != made
+    cfg = make()
+    made = vecenv._recipe(cfg)
+    cfg.extra["n_lines"] = 3
+    assert vecenv._recipe(cfg) != made
