@@ -298,7 +298,7 @@ int mv_scene_worlds(const mv_scene_desc *desc, const int64_t *d_env_ids, int env
  *   d_slots     DEVICE int32 [env_count] or NULL: env i's cameras go to d_cams[slots[i]] (NULL: to d_cams[i])
  *   d_boxes     DEVICE mv_box [env_count][movable_boxes + (body_boxes ? agents : 0)]   d_box_count  DEVICE int32 [env_count]
  *   d_cams      DEVICE mv_camera [...][agents]
- * Errors: INVALID_ARG, CUDA. */
+ * Errors: INVALID_ARG (also where there are more agents than columns), CUDA. */
 int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int64_t *d_height,
                       const int32_t *d_slots, mv_box *d_boxes, int32_t *d_box_count, mv_camera *d_cams, int device,
                       void *cuda_stream);
@@ -308,7 +308,7 @@ int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int e
  *   h_env_index HOST int32 [env_count], strictly increasing: the environments that get the scenes, as in mv_upload_worlds_at
  *   d_cams      DEVICE mv_camera [num_envs][agents]: environment h_env_index[i]'s rows are written
  *   d_boxes, d_box_count, d_palette  as above, written; d_work DEVICE int64 [env_count][grid_z][grid_x], 16-byte aligned: scratch
- * Grid, palette size, agents and boxes of the descriptor have to be the batch's.  Errors: INVALID_ARG, CUDA. */
+ * Grid, palette size, agents and boxes of the descriptor have to be the batch's.  Errors: as for mv_scene_entities. */
 int mv_scene_upload(mv_batch *batch, const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int32_t *h_env_index,
                     mv_camera *d_cams, mv_box *d_boxes, int32_t *d_box_count, uint8_t *d_palette, int64_t *d_work, void *cuda_stream);
 

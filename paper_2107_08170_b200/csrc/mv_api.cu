@@ -432,6 +432,9 @@ bool scene_args(const mv_scene_desc *d, const int64_t *d_env_ids, int env_count,
     return true;
 }
 
+// A cell for every agent's camera?  (Cells that nobody can stand in are dealt out last.)
+bool cameras_fit(const SceneArgs &a) { return a.agents <= a.gx * a.gz; }
+
 size_t ctas_of(size_t threads, int per_cta) { return (threads + per_cta - 1) / per_cta; }
 
 // Height and material of every column, as keys.
@@ -852,7 +855,7 @@ int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int e
                       const int32_t *d_slots, mv_box *d_boxes, int32_t *d_box_count, mv_camera *d_cams, int device,
                       void *cuda_stream) {
     SceneArgs a;
-    if (!scene_args(desc, d_env_ids, env_count, &a) || !d_height || !d_box_count || !d_cams || (a.max_boxes > 0 && !d_boxes))
+    if (!scene_args(desc, d_env_ids, env_count, &a) || !cameras_fit(a) || !d_height || !d_box_count || !d_cams || (a.max_boxes > 0 && !d_boxes))
         return MV_ERR_INVALID_ARG;
     if (env_count == 0) return MV_OK;
     DeviceGuard g(device);
@@ -867,7 +870,7 @@ int mv_scene_entities(const mv_scene_desc *desc, const int64_t *d_env_ids, int e
 int mv_scene_upload(mv_batch *b, const mv_scene_desc *desc, const int64_t *d_env_ids, int env_count, const int32_t *h_env_index,
                     mv_camera *d_cams, mv_box *d_boxes, int32_t *d_box_count, uint8_t *d_palette, int64_t *d_work, void *cuda_stream) {
     SceneArgs a;
-    if (!b || !scene_args(desc, d_env_ids, env_count, &a) || env_count > b->desc.num_envs || (env_count > 0 && !h_env_index) || !d_cams ||
+    if (!b || !scene_args(desc, d_env_ids, env_count, &a) || !cameras_fit(a) || env_count > b->desc.num_envs || (env_count > 0 && !h_env_index) || !d_cams ||
         !d_box_count || !d_palette || !d_work || !aligned16(d_work) || (a.max_boxes > 0 && (!d_boxes || !aligned16(d_boxes))) ||
         a.gx != b->desc.grid_x || a.gy != b->desc.grid_y || a.gz != b->desc.grid_z || a.palette != b->desc.palette_size ||
         a.max_boxes != b->desc.max_boxes || a.agents != b->desc.agents_per_env || !index_ok(b, h_env_index, env_count))

@@ -71,3 +71,13 @@ def test_warp_votes_name_their_lanes():
     result without a word."""
     for source in sorted((ROOT / "paper_2107_08170_b200" / "csrc").iterdir()):
         assert "__activemask" not in source.read_text(), source.name
+
+
+def test_more_agents_than_cells_are_refused(mvlib):
+    """Every camera has a cell of its own: with more agents than a world has columns the last ones would be looked for outside it.  (Refused
+    before a device is asked for; a descriptor that fits gets as far as that.)"""
+    from paper_2107_08170_b200 import scenes
+    L, somewhere = mvlib.lib(), C.c_void_p(4096)
+    for agents, code in ((17, -1), (1 << 16, -1), (16, -3)):
+        desc = scenes.native_desc(scenes.config("rooms", agents=agents, grid=(4, 8, 4), extra={"n_lines": 0}))
+        assert L.mv_scene_entities(C.byref(desc), somewhere, 1, somewhere, None, somewhere, somewhere, somewhere, -1, None) == code

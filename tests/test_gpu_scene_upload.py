@@ -129,3 +129,21 @@ def test_launches_are_counted(world, extra, keys):
     assert batch.launch_count() - before == keys + 2
     torch.cuda.synchronize()
     batch.destroy()
+
+
+def test_more_agents_than_cells_are_refused():
+    from paper_2107_08170_b200 import binding as B, scenes
+    for agents, fits in ((16, True), (17, False)):
+        cfg = scenes.config("rooms", num_envs=1, agents=agents, grid=(4, 8, 4), width=16, height=8, extra={"n_lines": 0, "n_pillars": 0})
+        batch = B.Batch(B.desc_from_config(cfg, 0))
+        cams = torch.zeros(agents, 6, dtype=torch.int32, device="cuda")
+        make = lambda: scenes.native_upload(cfg, scenes.native_desc(cfg), torch.tensor([1], device="cuda"), batch, [0], cams)
+        if fits:
+            make()
+            at = cams.view(torch.float32)[:, [0, 2]].floor().int()
+            assert len(set(map(tuple, at.tolist()))) == agents and at.min() >= 0 and at.max() <= 3
+        else:
+            with pytest.raises(B.MvError) as refused:
+                make()
+            assert refused.value.code == -1
+        batch.destroy()
